@@ -196,6 +196,12 @@ void apply_full(Context &c, double f, const double *xL, double g, const double *
     const double *xl[1] = {xL};
     const double *xm[1] = {xM};
     double *o[1] = {out};
+    if (c.prm.mvp == BEM_MVP_DIRECT) {  // the direct kernel adds the diagonals itself
+        c.stats.n_apply += 1;
+        c.stats.n_apply_rhs += 1;
+        launch_direct<1>(c, c.prm.precision, fa, xl, ga, xm, o, c.ldiag.p, c.mdiag.p);
+        return;
+    }
     offdiag_apply(c, 1, fa, xl, ga, xm, o, c.prm.precision);
     launch_add_diag(c.N, f, xL, g, xM, c.ldiag.p, c.mdiag.p, out, c.stream);
 }

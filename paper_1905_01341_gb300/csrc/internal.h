@@ -439,13 +439,16 @@ void offdiag_apply(Context &c, int R, const double *f, const double *const *xL,
 // p2p.cu
 template <class T, int R>
 void launch_p2p_list(Context &c, const T *q, const T *w, double *near_sorted, bool hq, bool hw, cudaStream_t st);
+
+// direct.cu: the direct all-pairs product; ld / md: the identity diagonals to add, or null
 template <int R>
 void launch_direct(Context &c, int prec, const double *f, const double *const *xL,
-                   const double *g, const double *const *xM, double *const *out);
-
+                   const double *g, const double *const *xM, double *const *out, const double *ld = nullptr,
+                   const double *md = nullptr);
 // Direct FP32 product (k_direct32, one right-hand side) on caller-provided split coordinates.
 void launch_direct32_raw(int64_t N, const float *hi, const float *lo, const double *s, const double *nrm, double f,
-                         const double *xL, double g, const double *xM, double *out, cudaStream_t st);
+                         const double *xL, double g, const double *xM, const double *ld, const double *md, double *out,
+                         cudaStream_t st);
 
 // m2l_tc.cu
 bool m2l_tc_supported(int P);

@@ -5,8 +5,8 @@
 // a device allocation (which synchronises the device) is not acceptable. This entry point
 // serves them: the caller passes inputs and outputs, and the one scratch buffer the direct
 // FP32 kernel needs (the hi + lo split of the coordinates) is a file-scope __device__ array
-// of fixed size, so the call allocates nothing. It launches the same three kernels as a
-// context's direct FP32 product (coordinate split, all-pairs sum, identity diagonals).
+// of fixed size, so the call allocates nothing. It launches the same kernels as a context's
+// direct FP32 product (coordinate split, all-pairs sum with the identity diagonals).
 #include <atomic>
 #include <mutex>
 
@@ -90,8 +90,7 @@ extern "C" int bem_apply_direct_noalloc(int64_t N, const double *xyz, const doub
         float *lo = hi + 3 * N;
         cudaStream_t st = static_cast<cudaStream_t>(stream);
         launch_split_hilo(3 * N, xyz, hi, lo, st);
-        launch_direct32_raw(N, hi, lo, s, n, f, xL, g, xM, out, st);
-        launch_add_diag(N, f, xL, g, xM, ldiag, mdiag, out, st);
+        launch_direct32_raw(N, hi, lo, s, n, f, xL, g, xM, ldiag, mdiag, out, st);
         return BEM_OK;
     } catch (const Error &e) {
         g_create_error = e.msg;  // reported by bem_last_error(NULL)

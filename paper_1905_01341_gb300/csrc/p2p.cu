@@ -1,12 +1,12 @@
-// Near field of the FMM (Section 3.7, A^(sparse) X) and the direct all-pairs product
-// (Section 3.9, brute force), both with the one-point quadrature kernel of Eq. (ns1):
+// Near field of the FMM (Section 3.7, A^(sparse) X) with the one-point quadrature kernel of
+// Eq. (ns1):
 //   u_i += sum_{j != i} [ q_j / |r_i - r_j| + w_j n_j.(r_i - r_j) / |r_i - r_j|^3 ],
 // q_j = f s_j X_L,j / (4 pi), w_j = g s_j X_M,j / (4 pi) (Eqs. (2.13), (3.27)).
 //
 // FP32 variants keep coordinates accurate by construction: the list kernel works in
 // leaf-box units with coordinates relative to each leaf centre (integer box offsets are
-// exact in FP32), the direct kernel splits coordinates into hi + lo FP32 pairs. Sums are
-// formed per shared-memory tile in FP32 and merged with TwoSum compensation.
+// exact in FP32). Sums are formed per shared-memory tile in FP32 and merged with TwoSum
+// compensation.
 //
 // The single-layer kernel of Eq. (ns1) is symmetric in r = |r_i - r_j|, so the FP32 single-RHS,
 // single-layer products (every GMRES product) evaluate every pair of neighbour leaves A < B
@@ -24,8 +24,6 @@
 namespace bem {
 namespace {
 
-constexpr int P2P_THREADS = 128;
-constexpr double kInv4Pi = 0.0795774715459476678844418816862571810;
 
 template <class T>
 __device__ __forceinline__ T rsqrt_t(T x);
@@ -631,128 +629,6 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p_units(
         p2p_unit<T, R, HQ, HW>(stage[warp], lane, units[u], bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out);
 }
 
-template <int R>
-struct DirArgs {
-    double f[R], g[R];
-    const double *xL[R];
-    const double *xM[R];
-    double *out[R];
-};
-
-// Direct sum in FP64 (caller's vertex order).
-template <int R>
-__global__ void __launch_bounds__(P2P_THREADS) k_direct64(int64_t N, const double *__restrict__ xyz, const double *__restrict__ s,
-                                                          const double *__restrict__ nrm, DirArgs<R> a) {
-    __shared__ double sx[P2P_THREADS], sy[P2P_THREADS], sz[P2P_THREADS];
-    __shared__ double snx[P2P_THREADS], sny[P2P_THREADS], snz[P2P_THREADS];
-    __shared__ double sq[R][P2P_THREADS], sw[R][P2P_THREADS];
-    const int64_t i = blockIdx.x * (int64_t)P2P_THREADS + threadIdx.x;
-    const bool vr = i < N;
-    const int64_t ii = vr ? i : 0;
-    const double xi = xyz[ii], yi = xyz[N + ii], zi = xyz[2 * N + ii];
-    double acc[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = 0.0;
-    for (int64_t t0 = 0; t0 < N; t0 += P2P_THREADS) {
-        __syncthreads();
-        int64_t j = t0 + threadIdx.x;
-        if (j < N) {
-            sx[threadIdx.x] = xyz[j];
-            sy[threadIdx.x] = xyz[N + j];
-            sz[threadIdx.x] = xyz[2 * N + j];
-            snx[threadIdx.x] = nrm[j];
-            sny[threadIdx.x] = nrm[N + j];
-            snz[threadIdx.x] = nrm[2 * N + j];
-            double sj = s[j] * kInv4Pi;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                sq[r][threadIdx.x] = a.f[r] != 0.0 ? a.f[r] * sj * a.xL[r][j] : 0.0;
-                sw[r][threadIdx.x] = a.g[r] != 0.0 ? a.g[r] * sj * a.xM[r][j] : 0.0;
-            }
-        }
-        __syncthreads();
-        int ns = (int)((N - t0) < P2P_THREADS ? (N - t0) : P2P_THREADS);
-        if (vr) {
-            for (int sI = 0; sI < ns; ++sI) {
-                double dx = xi - sx[sI], dy = yi - sy[sI], dz = zi - sz[sI];
-                double r2 = dx * dx + dy * dy + dz * dz;
-                double rinv = (t0 + sI == i) ? 0.0 : rsqrt(r2);
-                double rinv3 = rinv * rinv * rinv;
-                double nd3 = (snx[sI] * dx + sny[sI] * dy + snz[sI] * dz) * rinv3;
-#pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] += sq[r][sI] * rinv + sw[r][sI] * nd3;
-            }
-        }
-    }
-    if (vr) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) a.out[r][i] = acc[r];
-    }
-}
-
-// Direct sum in FP32 with hi + lo coordinates and tile-compensated accumulation.
-template <int R>
-__global__ void __launch_bounds__(P2P_THREADS) k_direct32(int64_t N, const float *__restrict__ hi, const float *__restrict__ lo,
-                                                          const double *__restrict__ s, const double *__restrict__ nrm,
-                                                          DirArgs<R> a) {
-    __shared__ float sxh[P2P_THREADS], syh[P2P_THREADS], szh[P2P_THREADS];
-    __shared__ float sxl[P2P_THREADS], syl[P2P_THREADS], szl[P2P_THREADS];
-    __shared__ float snx[P2P_THREADS], sny[P2P_THREADS], snz[P2P_THREADS];
-    __shared__ float sq[R][P2P_THREADS], sw[R][P2P_THREADS];
-    const int64_t i = blockIdx.x * (int64_t)P2P_THREADS + threadIdx.x;
-    const bool vr = i < N;
-    const int64_t ii = vr ? i : 0;
-    const float xh = hi[ii], yh = hi[N + ii], zh = hi[2 * N + ii];
-    const float xl = lo[ii], yl = lo[N + ii], zl = lo[2 * N + ii];
-    Comp<float> acc[R];
-    for (int64_t t0 = 0; t0 < N; t0 += P2P_THREADS) {
-        __syncthreads();
-        int64_t j = t0 + threadIdx.x;
-        if (j < N) {
-            sxh[threadIdx.x] = hi[j];
-            syh[threadIdx.x] = hi[N + j];
-            szh[threadIdx.x] = hi[2 * N + j];
-            sxl[threadIdx.x] = lo[j];
-            syl[threadIdx.x] = lo[N + j];
-            szl[threadIdx.x] = lo[2 * N + j];
-            snx[threadIdx.x] = (float)nrm[j];
-            sny[threadIdx.x] = (float)nrm[N + j];
-            snz[threadIdx.x] = (float)nrm[2 * N + j];
-            double sj = s[j] * kInv4Pi;
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                sq[r][threadIdx.x] = a.f[r] != 0.0 ? (float)(a.f[r] * sj * a.xL[r][j]) : 0.f;
-                sw[r][threadIdx.x] = a.g[r] != 0.0 ? (float)(a.g[r] * sj * a.xM[r][j]) : 0.f;
-            }
-        }
-        __syncthreads();
-        int ns = (int)((N - t0) < P2P_THREADS ? (N - t0) : P2P_THREADS);
-        float part[R];
-#pragma unroll
-        for (int r = 0; r < R; ++r) part[r] = 0.f;
-        if (vr) {
-#pragma unroll 4
-            for (int sI = 0; sI < ns; ++sI) {
-                float dx = (xh - sxh[sI]) + (xl - sxl[sI]);
-                float dy = (yh - syh[sI]) + (yl - syl[sI]);
-                float dz = (zh - szh[sI]) + (zl - szl[sI]);
-                float r2 = dx * dx + dy * dy + dz * dz;
-                float rinv = (t0 + sI == i) ? 0.f : rsqrtf(r2);
-                float rinv3 = rinv * rinv * rinv;
-                float nd3 = (snx[sI] * dx + sny[sI] * dy + snz[sI] * dz) * rinv3;
-#pragma unroll
-                for (int r = 0; r < R; ++r) part[r] += sq[r][sI] * rinv + sw[r][sI] * nd3;
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r) acc[r].add(part[r]);
-    }
-    if (vr) {
-#pragma unroll
-        for (int r = 0; r < R; ++r) a.out[r][i] = acc[r].get();
-    }
-}
-
 }  // namespace
 
 template <class T, int R, bool HQ, bool HW>
@@ -811,42 +687,5 @@ template void launch_p2p_list<double, 1>(Context &, const double *, const double
                                          cudaStream_t);
 template void launch_p2p_list<double, 4>(Context &, const double *, const double *, double *, bool, bool,
                                          cudaStream_t);
-
-template <int R>
-void launch_direct(Context &c, int prec, const double *f, const double *const *xL, const double *g,
-                   const double *const *xM, double *const *out) {
-    DirArgs<R> a{};
-    for (int r = 0; r < R; ++r) {
-        a.f[r] = f[r];
-        a.g[r] = g[r];
-        a.xL[r] = xL[r];
-        a.xM[r] = xM[r];
-        a.out[r] = out[r];
-    }
-    int nb = div_up(c.N, P2P_THREADS);
-    PhaseScope ps(c, PH_DIRECT);
-    if (prec == BEM_PREC_FP64)
-        k_direct64<R><<<nb, P2P_THREADS, 0, c.stream>>>(c.N, c.xyz.p, c.s.p, c.nrm.p, a);
-    else
-        k_direct32<R><<<nb, P2P_THREADS, 0, c.stream>>>(c.N, c.dir_hi.p, c.dir_lo.p, c.s.p, c.nrm.p, a);
-    BEM_LAUNCH_CHECK();
-}
-
-void launch_direct32_raw(int64_t N, const float *hi, const float *lo, const double *s, const double *nrm, double f,
-                         const double *xL, double g, const double *xM, double *out, cudaStream_t st) {
-    DirArgs<1> a{};
-    a.f[0] = f;
-    a.g[0] = g;
-    a.xL[0] = xL;
-    a.xM[0] = xM;
-    a.out[0] = out;
-    k_direct32<1><<<div_up(N, P2P_THREADS), P2P_THREADS, 0, st>>>(N, hi, lo, s, nrm, a);
-    BEM_LAUNCH_CHECK();
-}
-
-template void launch_direct<1>(Context &, int, const double *, const double *const *, const double *,
-                               const double *const *, double *const *);
-template void launch_direct<4>(Context &, int, const double *, const double *const *, const double *,
-                               const double *const *, double *const *);
 
 }  // namespace bem
