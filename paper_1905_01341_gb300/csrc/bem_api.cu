@@ -19,7 +19,6 @@ Context::~Context() {
     if (ev_m2l) cudaEventDestroy(ev_m2l);
     if (side) cudaStreamDestroy(side);
     if (hi) cudaStreamDestroy(hi);
-    for (auto *p : up_chunks) delete p;
     step_free(step);
     mlp_free(mlp);
 }

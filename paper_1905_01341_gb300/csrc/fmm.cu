@@ -530,14 +530,10 @@ __global__ void __launch_bounds__(128) k_p2m_x2(int p, int nleaf, const int32_t 
 }
 
 // ------------------------------------------------------------------------------ translations
-// Class-grouped product: for every pair (src, tgt) of a chunk, Y[tgt] += T_cls X[src], as a
-// tiled GEMM (128 output rows x 128 columns per block in FP32, 64 x 64 in FP64; a column is one
-// pair and one RHS).
+// Class-grouped product: for every pair of a chunk, Y[pair] = T_cls X[src] (one slot per pair,
+// summed later in a fixed order), as a tiled GEMM (128 output rows x 128 columns per block in FP32,
+// 64 x 64 in FP64; a column is one pair and one RHS).
 constexpr int XT_K = 16, XT_THREADS = 256;
-
-// MODE kStorePair: Y[pair] = T X[src] (one slot per pair, summed later in a fixed order).
-// MODE kAddTarget: Y[tgt] += T X[src]; only for launches whose targets are all distinct.
-constexpr int kStorePair = 0, kAddTarget = 1;
 
 // N consecutive elements (16 bytes) from shared memory
 template <int N>
@@ -584,35 +580,28 @@ __device__ __forceinline__ void cp_async_elem(T *dst, const T *src, bool ok) {
                  : "memory");
 }
 
-template <class T, int R, int MODE>
+template <class T, int R>
 __global__ void __launch_bounds__(XT_THREADS, 2) k_xlat(const T *__restrict__ mats, int P, const XChunk *__restrict__ chunks,
-                                                     const int32_t *__restrict__ srcs, const int32_t *__restrict__ tgts,
-                                                     const T *X, T *Y,  // X and Y may be one array (M2M, L2L)
-                                                     const int32_t *__restrict__ cls_K) {
+                                                     const int32_t *__restrict__ srcs, const T *__restrict__ X,
+                                                     T *__restrict__ Y, const int32_t *__restrict__ cls_K) {
     constexpr int RT = xt_rt<T>(), CT = RT, ROWS = xt_rows<T>(), COLS = xt_cols<T>();
     constexpr int AP = xt_apitch<T>(), BP = xt_bpitch<T>(), VW = 16 / (int)sizeof(T);
     // XT_STAGES shared-memory stages of one K tile each: As[st][kk][row], Bs[st][kk][col]
     extern __shared__ __align__(16) unsigned char xt_smem_raw[];
     T *As = reinterpret_cast<T *>(xt_smem_raw);
     T *Bs = As + XT_STAGES * XT_K * AP;
-    __shared__ int s_src[COLS], s_tgt[COLS];
+    __shared__ int s_src[COLS];
     const XChunk ch = chunks[blockIdx.x];
     const int row0 = blockIdx.y * ROWS;
     const T *A = mats + (size_t)ch.cls * P * P;
     // truncated translation of this class (M2L with per-class orders): inputs and outputs of
-    // index < Kt; output rows from Kt on are written as zeros (kStorePair)
+    // index < Kt; output rows from Kt on are neither written nor read
     const int Kt = cls_K ? min(P, cls_K[ch.cls]) : P;
     const int ncol = ch.count * R;
     int tid = threadIdx.x;
     for (int e = tid; e < COLS; e += XT_THREADS) {
         int pr = e / R;
-        if (pr < ch.count) {
-            s_src[e] = srcs[ch.start + pr];
-            s_tgt[e] = tgts[ch.start + pr];
-        } else {
-            s_src[e] = -1;
-            s_tgt[e] = -1;
-        }
+        s_src[e] = pr < ch.count ? srcs[ch.start + pr] : -1;
     }
     __syncthreads();
     // a warp is an 8 x 4 grid of lanes (8 column groups, 4 row groups) and the block 2 x 4 warps;
@@ -693,15 +682,11 @@ __global__ void __launch_bounds__(XT_THREADS, 2) k_xlat(const T *__restrict__ ma
         int col = col_of(j);
         if (col >= ncol) continue;
         int r = col % R;
-        T *yb = (MODE == kStorePair) ? Y + ((size_t)(ch.start + col / R) * R + r) * P
-                                     : Y + ((size_t)s_tgt[col] * R + r) * P;
+        T *yb = Y + ((size_t)(ch.start + col / R) * R + r) * P;
 #pragma unroll
         for (int i = 0; i < RT; ++i) {
             int gr = row0 + row_of(i);
-            if (gr < Kt) {  // truncated rows (Kt < P) are never read
-                if (MODE == kStorePair) yb[gr] = acc[i][j];
-                else yb[gr] += acc[i][j];
-            }
+            if (gr < Kt) yb[gr] = acc[i][j];  // truncated rows (Kt < P) are never read
         }
     }
 }
@@ -1067,12 +1052,6 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p_x2(int p, const int32_t *__
     }
 }
 
-template <class T>
-__global__ void k_zero(size_t n, T *a) {
-    size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i < n) a[i] = (T)0;
-}
-
 // out[perm[k]] = (far_k + near_k) / h_leaf: the far field (L2P) and the near field (P2P, run
 // concurrently on the side stream) meet here, back in the caller's vertex order.
 template <class T>
@@ -1176,34 +1155,6 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
     cudaStream_t fs = ovl ? c.hi : st;
     if (ovl) BEM_CUDA(cudaStreamWaitEvent(fs, c.ev_fork, 0));
 
-    // chunk tables for this R (built once per build)
-    const int per = xt_cols<T>() / R;
-    auto &mch = c.m2l_chunks_h;
-    if (mch.empty() || mch.front().cls != -R) {
-        std::vector<XChunk> all;
-        XChunk tag{-R, 0, 0};
-        all.push_back(tag);  // header: which R the table is for
-        make_chunks(t.m2l_class_off, 0, per, all);
-        for (int l = 3; l <= L; ++l) make_chunks(t.up_class_off[l], t.up_off[l], per, all);
-        mch = all;
-        c.m2l_chunks.resize(all.size());
-        BEM_CUDA(cudaMemcpyAsync(c.m2l_chunks.p, all.data(), all.size() * sizeof(XChunk), cudaMemcpyHostToDevice, fs));
-    }
-    // locate the per-phase ranges in the chunk table
-    int64_t nm2l_chunks = 0;
-    for (size_t cc = 0; cc + 1 < t.m2l_class_off.size(); ++cc)
-        nm2l_chunks += (t.m2l_class_off[cc + 1] - t.m2l_class_off[cc] + per - 1) / per;
-    std::vector<int64_t> up_first(L + 2, 0), up_n(L + 2, 0);
-    int64_t cur = 1 + nm2l_chunks;
-    for (int l = 3; l <= L; ++l) {
-        int64_t k = 0;
-        for (int cc = 0; cc < 8; ++cc) k += (t.up_class_off[l][cc + 1] - t.up_class_off[l][cc] + per - 1) / per;
-        up_first[l] = cur;
-        up_n[l] = k;
-        cur += k;
-    }
-    const int rowblocks = div_up(P, xt_rows<T>());
-
     // P2M at the leaves
     const int nleaf = t.nb[L];
     {
@@ -1230,39 +1181,15 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
         }
         BEM_LAUNCH_CHECK();
     }
-    // zero the multipoles above the leaves and all locals
-    {
-        size_t nup = (size_t)t.base[L] * R * P;
-        if (nup) k_zero<T><<<div_up(nup, tb), tb, 0, fs>>>(nup, mp);
-        k_zero<T><<<div_up(exp_sz, tb), tb, 0, fs>>>(exp_sz, lc);
-        BEM_LAUNCH_CHECK();
-    }
-    // per-pair buffer for the fixed-order reductions
-    T *ypair;
-    {
-        int64_t nup_all = t.up_off[L + 1];
-        size_t need = (size_t)std::max<int64_t>(std::max<int64_t>(t.n_m2l, nup_all), 1) * R * P;
-        if (F64) {
-            c.ypair64.resize(need);
-            ypair = (T *)c.ypair64.p;
-        } else {
-            c.ypair32.resize(need);
-            ypair = (T *)c.ypair32.p;
-        }
-    }
-    // M2M upward, levels L -> 2: per-pair products, then each parent sums its children
+    // zero the locals (boxes without a translation; the multipoles of every level are written whole)
+    BEM_CUDA(cudaMemsetAsync(lc, 0, exp_sz * sizeof(T), fs));
+    // M2M upward, levels L -> 2: each parent sums its children
     for (int l = L; l >= 3; --l) {
         PhaseScope ps(c, PH_M2M, fs);
-        if (!up_n[l]) continue;
-        dim3 grid((unsigned)up_n[l], rowblocks);
-        xlat_smem_attr(k_xlat<T, R, kStorePair>, xt_smem<T>());
-        k_xlat<T, R, kStorePair><<<grid, XT_THREADS, xt_smem<T>(), fs>>>(m2m, P, c.m2l_chunks.p + up_first[l],
-                                                                         t.up_child.p, t.up_parent.p, mp, ypair, nullptr);
-        BEM_LAUNCH_CHECK();
-        launch_reduce_pairs<T, R>(t.base[l - 1], t.nb[l - 1], t.up_par_off.p, t.up_by_par.p, ypair, P, mp, fs);
+        launch_m2m<T, R>(P, t.base[l - 1], t.nb[l - 1], m2m, t.child8.p, mp, fs);
     }
     // M2L, all levels at once, then each target sums its sources
-    if (nm2l_chunks) {
+    if (t.n_m2l > 0) {
         // Single-RHS products (every GMRES product) use the tensor cores with m2l_tensor_cores >= 1;
         // the 4-RHS product behind the diagonals where build decided so (diag_tc): M_ii and L_ii
         // are formed by cancellation (Eqs. (s3), (s5)), which magnifies the far field's rounding.
@@ -1272,6 +1199,17 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
         // product stays pair-major (its target-major form, at 64 targets per tile, was slower and
         // less accurate)
         const bool tm_path = tc_path && R == 1 && c.prm.m2l_target_major;
+        T *ypair = nullptr;  // per-pair products of the pair-major forms, for the fixed-order sums
+        if (!tm_path) {
+            const size_t need = (size_t)t.n_m2l * R * P;
+            if (F64) {
+                c.ypair64.resize(need);
+                ypair = (T *)c.ypair64.p;
+            } else {
+                c.ypair32.resize(need);
+                ypair = (T *)c.ypair32.p;
+            }
+        }
         if (tm_path) {
             PhaseScope ps(c, PH_M2L, fs);
             launch_m2l_tm<1>(c, opr, (const float *)mp, (int64_t)t.nbox, c.tc_err.p, fs);
@@ -1302,11 +1240,21 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
                                  (float *)ypair, c.tc_err.p, fs);
         } else {
             PhaseScope ps(c, PH_M2L_CC, fs);
-            dim3 grid((unsigned)nm2l_chunks, rowblocks);
-            xlat_smem_attr(k_xlat<T, R, kStorePair>, xt_smem<T>());
-            k_xlat<T, R, kStorePair><<<grid, XT_THREADS, xt_smem<T>(), fs>>>(m2l, P, c.m2l_chunks.p + 1,
-                                                                             t.m2l_src.p, t.m2l_tgt.p, mp, ypair,
-                                                                             opr.margin >= 0 ? opr.cls_K.p : nullptr);
+            // chunk table for this column count (built once per build)
+            const int per = xt_cols<T>() / R;
+            auto &mch = c.m2l_chunks_h;
+            if (mch.empty() || mch.front().cls != -per) {
+                std::vector<XChunk> all;
+                all.push_back(XChunk{-per, 0, 0});  // header: the pairs per chunk of the table
+                make_chunks(t.m2l_class_off, 0, per, all);
+                mch = all;
+                c.m2l_chunks.resize(all.size());
+                BEM_CUDA(cudaMemcpyAsync(c.m2l_chunks.p, mch.data(), mch.size() * sizeof(XChunk), cudaMemcpyHostToDevice, fs));
+            }
+            dim3 grid((unsigned)(mch.size() - 1), div_up(P, xt_rows<T>()));
+            xlat_smem_attr(k_xlat<T, R>, xt_smem<T>());
+            k_xlat<T, R><<<grid, XT_THREADS, xt_smem<T>(), fs>>>(m2l, P, c.m2l_chunks.p + 1, t.m2l_src.p, mp, ypair,
+                                                                 opr.margin >= 0 ? opr.cls_K.p : nullptr);
             BEM_LAUNCH_CHECK();
         }
         if (omode == 2) {  // the M2L is queued: the near field may start (after the multipoles)
@@ -1330,13 +1278,8 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
     }
     // L2L downward, levels 3 -> L: every child has exactly one parent, so it adds in place
     for (int l = 3; l <= L; ++l) {
-        if (!up_n[l]) continue;
         PhaseScope ps(c, PH_L2L, fs);
-        dim3 grid((unsigned)up_n[l], rowblocks);
-        xlat_smem_attr(k_xlat<T, R, kAddTarget>, xt_smem<T>());
-        k_xlat<T, R, kAddTarget><<<grid, XT_THREADS, xt_smem<T>(), fs>>>(l2l, P, c.m2l_chunks.p + up_first[l],
-                                                                         t.up_parent.p, t.up_child.p, lc, lc, nullptr);
-        BEM_LAUNCH_CHECK();
+        launch_l2l<T, R>(P, t.base[l - 1], t.nb[l - 1], l2l, t.child8.p, lc, fs);
     }
     // L2P
     {

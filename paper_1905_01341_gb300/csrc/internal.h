@@ -127,14 +127,10 @@ struct Tree {
     DevBuf<int32_t> m2l_src, m2l_tgt;  // global box indices
     DevBuf<uint32_t> m2l_cls;          // offset class of each pair (ascending)
     std::vector<int64_t> m2l_class_off;  // [kNumM2LClasses+1] host copy
-    // M2M / L2L: per level l (1..L), child->parent pairs sorted by child octant
-    std::vector<int64_t> up_off;       // per level: offset into up_child/up_parent
-    std::vector<std::vector<int64_t>> up_class_off;  // per level: [9]
-    DevBuf<int32_t> up_child, up_parent;
-    // target-major views of the pair lists, for the fixed-order reductions: for every box,
-    // the pair indices that write to it, ascending (CSR over all boxes)
+    DevBuf<int32_t> child8;            // [nbox][8] children of a box by octant (global indices), -1 where empty
+    // target-major view of the M2L pairs, for the fixed-order reductions: for every box, the pair
+    // indices that write to it, ascending (CSR over all boxes)
     DevBuf<int32_t> m2l_tgt_off, m2l_by_tgt;  // [nbox+1], [n_m2l]
-    DevBuf<int32_t> up_par_off, up_by_par;    // [nbox+1], [n_up]
     // leaf-local coordinates of sorted points in units of the leaf box (range [-1/2, 1/2))
     DevBuf<double> loc64;      // [3][N]
     DevBuf<float> loc32;       // [3][N]
@@ -355,8 +351,6 @@ struct Context {
     // flags of the finiteness and mesh checks, one per check site, and the diagonal product's output
     DevBuf<int> chk[4];
     DevBuf<double> diag_tmp;
-    std::vector<DevBuf<XChunk> *> up_chunks;  // per level
-    std::vector<std::vector<XChunk>> up_chunks_h;
     DevBuf<double> ones;
 
     // direct-sum work arrays
@@ -435,6 +429,13 @@ std::vector<int> m2l_class_orders(int p, int margin);
 void offdiag_apply(Context &c, int R, const double *f, const double *const *xL,
                    const double *g, const double *const *xM, double *const *out, int prec,
                    const Operators *ops = nullptr);
+
+// updown.cu: M2M into the parents pbase .. pbase + np - 1 (global boxes of one level) and L2L out
+// of them; mats [8][P][P] by child octant, child8 as in Tree
+template <class T, int R>
+void launch_m2m(int P, int pbase, int np, const T *mats, const int32_t *child8, T *mp, cudaStream_t st);
+template <class T, int R>
+void launch_l2l(int P, int pbase, int np, const T *mats, const int32_t *child8, T *lc, cudaStream_t st);
 
 // p2p.cu
 template <class T, int R>

@@ -500,21 +500,11 @@ __global__ void k_hist_small(int64_t n, const uint32_t *__restrict__ k, int nbin
     if (i < n) atomicAdd(&h[k[i]], 1);
 }
 
-// Octant keys of the children at one level, for the child -> parent translation pairs.
-__global__ void k_octants(int n, const uint32_t *__restrict__ key, uint32_t *__restrict__ oct, int32_t *__restrict__ id) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    oct[i] = key[i] & 7u;
-    id[i] = i;
-}
-
-__global__ void k_up_pairs(int n, const int32_t *__restrict__ id, int base, const int32_t *__restrict__ parent,
-                           int32_t *__restrict__ child, int32_t *__restrict__ par) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int g = base + id[i];
-    child[i] = g;
-    par[i] = parent[g];
+// child8[box][8]: the children of every box by octant (the low bits of their keys), -1 where empty
+__global__ void k_child8(int first, int nbox, const uint32_t *__restrict__ bkey, const int32_t *__restrict__ parent,
+                         int32_t *__restrict__ child8) {
+    const int i = first + blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nbox) child8[(int64_t)parent[i] * 8 + (bkey[i] & 7u)] = i;
 }
 
 // Sorted-order point data: leaf-local coordinates (units of the leaf box, centred), normals
@@ -868,66 +858,36 @@ void build_tree(Context &c) {
         for (int k = 0; k < kNumM2LClasses; ++k) t.m2l_class_off[k + 1] = t.m2l_class_off[k] + hh[k];
     }
 
-    // 7. child -> parent pairs per level (levels 3..L), sorted by child octant
-    t.up_off.assign(L + 2, 0);
-    t.up_class_off.assign(L + 1, std::vector<int64_t>(9, 0));
-    int64_t nup = 0;
-    for (int l = 3; l <= L; ++l) {
-        t.up_off[l] = nup;
-        nup += t.nb[l];
-    }
-    t.up_off[L + 1] = nup;
-    t.up_child.resize(nup);
-    t.up_parent.resize(nup);
-    for (int l = 3; l <= L; ++l) {
-        int n = t.nb[l];
-        DevBuf<uint32_t> &ok = t.s_u32[2], &oktmp = t.s_u32[3];
-        DevBuf<int32_t> &id = t.s_i32[17], &idtmp = t.s_i32[18], &h8 = t.s_i32[19];
-        ok.resize(n);
-        oktmp.resize(n);
-        id.resize(n);
-        idtmp.resize(n);
-        h8.resize(8);
-        k_octants<<<div_up(n, tb), tb, 0, st>>>(n, t.bkey.p + t.base[l], ok.p, id.p);
-        BEM_LAUNCH_CHECK();
-        BEM_CUDA(cudaMemsetAsync(h8.p, 0, 8 * sizeof(int32_t), st));
-        k_hist_small<<<div_up(n, tb), tb, 0, st>>>(n, ok.p, 8, h8.p);
-        BEM_LAUNCH_CHECK();
-        radix_sort_u32(ok.p, id.p, n, 3, oktmp.p, idtmp.p, st);
-        k_up_pairs<<<div_up(n, tb), tb, 0, st>>>(n, id.p, t.base[l], t.parent.p, t.up_child.p + t.up_off[l],
-                                                  t.up_parent.p + t.up_off[l]);
-        BEM_LAUNCH_CHECK();
-        int32_t hh[8];
-        BEM_CUDA(cudaMemcpyAsync(hh, h8.p, sizeof(hh), cudaMemcpyDeviceToHost, st));
-        BEM_CUDA(cudaStreamSynchronize(st));
-        for (int k = 0; k < 8; ++k) t.up_class_off[l][k + 1] = t.up_class_off[l][k] + hh[k];
-    }
+    // 7. children of every box by octant (M2M, L2L)
+    t.child8.resize((size_t)t.nbox * 8);
+    BEM_CUDA(cudaMemsetAsync(t.child8.p, 0xff, (size_t)t.nbox * 8 * sizeof(int32_t), st));
+    k_child8<<<div_up(t.nbox - t.base[1], tb), tb, 0, st>>>(t.base[1], t.nbox, t.bkey.p, t.parent.p, t.child8.p);
+    BEM_LAUNCH_CHECK();
 
-    // 8. target-major CSR of the M2L and child->parent pairs (stable: ascending pair index)
-    auto target_csr = [&](const int32_t *tgt, int64_t np, DevBuf<int32_t> &off, DevBuf<int32_t> &by) {
+    // 8. target-major CSR of the M2L pairs (stable: ascending pair index)
+    {
+        DevBuf<int32_t> &off = t.m2l_tgt_off, &by = t.m2l_by_tgt;
         off.resize((size_t)t.nbox + 1);
-        by.resize(np > 0 ? np : 1);
+        by.resize(nm2l > 0 ? nm2l : 1);
         DevBuf<int32_t> &cnt2 = t.s_i32[20];
         cnt2.resize((size_t)t.nbox + 1);
         BEM_CUDA(cudaMemsetAsync(cnt2.p, 0, ((size_t)t.nbox + 1) * sizeof(int32_t), st));
-        if (np > 0) {
+        if (nm2l > 0) {
             DevBuf<uint32_t> &k = t.s_u32[4], &ktmp2 = t.s_u32[5];
             DevBuf<int32_t> &vtmp2 = t.s_i32[21];
-            k.resize(np);
-            ktmp2.resize(np);
-            vtmp2.resize(np);
-            k_copy_keys<<<div_up(np, tb), tb, 0, st>>>(np, tgt, k.p, cnt2.p);
+            k.resize(nm2l);
+            ktmp2.resize(nm2l);
+            vtmp2.resize(nm2l);
+            k_copy_keys<<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, t.m2l_tgt.p, k.p, cnt2.p);
             BEM_LAUNCH_CHECK();
-            k_iota<<<div_up(np, tb), tb, 0, st>>>(np, by.p);
+            k_iota<<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, by.p);
             BEM_LAUNCH_CHECK();
             int bits = 1;
             while ((1ll << bits) <= (long long)t.nbox) ++bits;
-            radix_sort_u32(k.p, by.p, np, bits, ktmp2.p, vtmp2.p, st);
+            radix_sort_u32(k.p, by.p, nm2l, bits, ktmp2.p, vtmp2.p, st);
         }
         exclusive_scan_i32(cnt2.p, off.p, (int64_t)t.nbox + 1, nullptr, st);
-    };
-    target_csr(t.m2l_tgt.p, nm2l, t.m2l_tgt_off, t.m2l_by_tgt);
-    target_csr(t.up_parent.p, nup, t.up_par_off, t.up_by_par);
+    }
 
     // 9. sorted point data
     t.loc64.resize(3 * N);
