@@ -142,6 +142,12 @@ struct Tree {
     DevBuf<int2> p2p_units;
     int64_t n_p2p_units = 0;
     DevBuf<int32_t> p2p_ucnt;  // [nleaf] units per leaf
+    // FP32 near-field work items (leaf, first receiver, first and end position in the unit's list of
+    // neighbour points; first = -1: the list from 0 and the leaf's own points): [0] symmetric (the neighbours f > leaf), [1] one-way (all but the leaf); the
+    // items of unit u are p2p_ioff[u] .. p2p_ioff[u + 1] - 1
+    DevBuf<int4> p2p_items[2];
+    DevBuf<int32_t> p2p_ioff[2];
+    int64_t n_p2p_items[2] = {0, 0};
     // symmetric near field (FP32 single-RHS products): a pair of neighbour leaves A < B is
     // evaluated once, by A's units; each unit of A writes B's share (one float per point of B)
     // into its own region of `back`, and a gather adds those shares to B's points in a fixed order
@@ -152,7 +158,7 @@ struct Tree {
     int64_t n_back = 0;
     // scratch of the build, kept between builds so that a rebuild allocates (and synchronises)
     // nothing once the sizes have settled; each slot has one use
-    DevBuf<int32_t> s_i32[22];
+    DevBuf<int32_t> s_i32[24];
     DevBuf<uint32_t> s_u32[6];
     DevBuf<int64_t> s_i64[1];
     DevBuf<double> s_f64[3];
@@ -318,6 +324,7 @@ struct Context {
     DevBuf<double> far64;          // far-field potential [R][N] (sorted)
     DevBuf<float> far32;
     DevBuf<double> near_out;       // combined potential [R][N] (sorted)
+    DevBuf<float2> p2p_fwd;        // FP32 near field: sums of every item [items][R][64]
     DevBuf<XChunk> m2l_chunks;
     std::vector<XChunk> m2l_chunks_h;
     // M2L chunks of <= 256/R pairs for the tensor-core kernel: [0] for R = 1, [1] for R = 4

@@ -236,14 +236,23 @@ __device__ __forceinline__ void p2p_unit(P2PStage<T, R, HQ, HW> &sg, int lane, i
 }
 
 // FP32 form with packed two-wide arithmetic (add/mul/fma .f32x2: one instruction for two
-// lanes' worth of FP32 work). The near field is issue-bound, so each lane takes its two
-// receivers against two sources at a time: a staged tile holds 16 source pairs, each as
-// (-x, -x', -y, -y'), (-z, -z', q, q') (and (n_x, n_x', n_y, n_y'), (n_z, n_z', w, w') for the
-// double layer); a receiver's coordinate is a broadcast pair, so x_i - x_j is one packed add of
-// the negated source coordinate (exactly the scalar difference) and r^2, the sums and the
-// double layer's n.(r_i - r_j) / r^3 are packed products; the reciprocal square roots stay
-// scalar. Lanes past a tile's end stage a source of zero strength far outside the leaf's
-// neighbourhood (finite r^2), so a partial tile runs whole pairs.
+// lanes' worth of FP32 work): each lane takes its two receivers against two sources at a time. A
+// staged tile holds 16 source pairs, each as (-x, -x', -y, -y'), (-z, -z', q, q') (and
+// (n_x, n_x', n_y, n_y'), (n_z, n_z', w, w') for the double layer); a receiver's coordinate is a
+// broadcast pair, so x_i - x_j is one packed add of the negated source coordinate (exactly the
+// scalar difference) and r^2, the sums and the double layer's n.(r_i - r_j) / r^3 are packed
+// products; the reciprocal square roots stay scalar. Lanes past a tile's end stage a source of zero
+// strength far outside the leaf's neighbourhood (finite r^2), so a partial tile runs whole pairs.
+//
+// Work items (Tree::p2p_items): the neighbour leaves that a unit evaluates, one after another in its
+// neighbour list, count as one list of sources; an item is a unit and a range of that list, of about
+// the same length for all items (the unit's own leaf belongs to its first item). Tiles run across
+// the borders of the leaves (every staged source gets its own leaf's offset), so only an item's last
+// tile is partial: with a tile per 32 sources of each leaf, about a sixth of the pair slots were
+// empty at 90 to 130 points a leaf. And a small product has enough items of equal size to fill the
+// chip: one warp per unit left the SMs active 59 % of the kernel's time at 192600 points. An item's
+// sums go to its own row of `fwd`, joined per point by k_p2p_gather. Symmetric single-layer kernel
+// with its gather, 192600 points: 207 -> 124 us; 3.21M points: 2.51 -> 2.35 ms.
 template <int R, bool HQ, bool HW>
 struct P2PStageX2 {
     float4 a[16];               // -x, -x', -y, -y'
@@ -252,7 +261,12 @@ struct P2PStageX2 {
     float4 d[HW ? 16 : 1];      // n_z, n_z', w, w' (first RHS)
     float q[(R > 1 && HQ) ? R - 1 : 1][32];
     float w[(R > 1 && HW) ? R - 1 : 1][32];
-    float tr[R == 1 ? 32 : 1][20];  // symmetric form: per-lane rows of the sources' shares, transposed
+    float4 tab[27];  // per neighbour: box offset x, y, z and (as an integer) first point - list position
+    int32_t tend[27];  // per neighbour: end in the item's source list
+};
+template <int R, bool HQ, bool HW, bool SYM>
+struct P2PStageSym : P2PStageX2<R, HQ, HW> {
+    float tr[SYM ? 32 : 1][20];  // symmetric form: per-lane rows of the sources' shares, transposed
 };
 
 template <bool SELF>
@@ -309,16 +323,17 @@ __device__ __forceinline__ void p2p_source_x2(const P2PStageX2<R, HQ, HW> &sg, i
     }
 }
 
-// A staged tile of an owned neighbour leaf (symmetric form, one RHS): the forward sums as in
-// p2p_tile_x2 and, per batch of up to 16 sources of a group, each source's share summed over the
-// unit's receivers (every group holds all of them), written to back[s] for the tile's source s.
-// The sum over lanes goes through shared memory: every lane stores its row of the batch's
-// values, then lane rs adds up column rs over its group's rows (for one group of 32 lanes, each
-// half of the warp takes half the rows and one shuffle joins them). The groups read their rows
-// in skewed orders so that their columns fall in different banks; the order of every sum is
-// fixed, so the result is deterministic.
+// A staged tile in the symmetric form (one RHS): the forward sums and, per batch of up to 16
+// sources of a group, each source's share summed over the unit's receivers (every group holds all
+// of them), written to back[s] for the tile's sources s < ns. The sum over lanes goes through
+// shared memory: every lane stores its row of the batch's values. One group of 32 lanes: lane
+// (rg, cq) adds the rows rg + 8 i of the four columns of quad cq with 16-byte loads (the quads of a
+// row rotate with the row, so neither the stores nor the loads conflict), then three exchanges join
+// the row groups. More groups: lane rs adds up column rs over its group's rows, the groups' rows
+// skewed so that their columns fall in different banks. The order of every sum is fixed, so the
+// result is deterministic.
 template <int G, bool HQ, bool HW>
-__device__ __forceinline__ void p2p_tile_x2_sym(P2PStageX2<1, HQ, HW> &sg, int ns, int gi, int lane,
+__device__ __forceinline__ void p2p_tile_x2_sym(P2PStageSym<1, HQ, HW, true> &sg, int ns, int gi, int lane,
                                                 const float2 *X, const float2 *Y, const float2 *Z, const RecvX2 &rv,
                                                 Comp<float> (*acc)[1], float *__restrict__ back) {
     constexpr int SP = 16 / G, LG = 32 / G;
@@ -329,51 +344,62 @@ __device__ __forceinline__ void p2p_tile_x2_sym(P2PStageX2<1, HQ, HW> &sg, int n
     float2 part[2][1];
     part[0][0] = part[1][0] = make_float2(0.f, 0.f);
     const int p0 = gi * SP;
-    const int e = min(SP, (ns + 1) / 2 - p0);  // pairs of this group holding sources
 #pragma unroll
     for (int h0 = 0; h0 < SP; h0 += HP) {
-        if (ns == 32) {
-            float2 bk[HP];
+        float2 bk[HP];
 #pragma unroll
-            for (int t = 0; t < HP; ++t) bk[t] = make_float2(0.f, 0.f);
+        for (int t = 0; t < HP; ++t) bk[t] = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int t = 0; t < HP; ++t) p2p_source_x2<1, HQ, HW, false, true>(sg, p0 + h0 + t, X, Y, Z, part, &rv, &bk[t]);
+        for (int t = 0; t < HP; ++t) p2p_source_x2<1, HQ, HW, false, true>(sg, p0 + h0 + t, X, Y, Z, part, &rv, &bk[t]);
+        if constexpr (G == 1) {
+            float4 *tr = reinterpret_cast<float4 *>(&sg.tr[0][0]);  // [32 rows][4 quads]
+            const int sw = (lane >> 1) & 3;
+#pragma unroll
+            for (int c4 = 0; c4 < 4; ++c4)
+                tr[lane * 4 + (c4 ^ sw)] = make_float4(bk[2 * c4].x, bk[2 * c4].y, bk[2 * c4 + 1].x, bk[2 * c4 + 1].y);
+            __syncwarp();
+            const int cq = lane & 3, rg = lane >> 2;
+            float2 u = make_float2(0.f, 0.f), v = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int row = rg + 8 * i;
+                const float4 t4 = tr[row * 4 + (cq ^ ((row >> 1) & 3))];
+                u = __fadd2_rn(u, make_float2(t4.x, t4.y));
+                v = __fadd2_rn(v, make_float2(t4.z, t4.w));
+            }
+            // join the row groups (lane bits 4, 3, 2); bits 4 and 3 choose the column kept
+            const bool b4 = lane & 16, b3 = lane & 8;
+            const float s0 = b4 ? u.x : v.x, s1 = b4 ? u.y : v.y;
+            const float k0 = (b4 ? v.x : u.x) + __shfl_xor_sync(0xffffffffu, s0, 16);
+            const float k1 = (b4 ? v.y : u.y) + __shfl_xor_sync(0xffffffffu, s1, 16);
+            float tot = (b3 ? k1 : k0) + __shfl_xor_sync(0xffffffffu, b3 ? k0 : k1, 8);
+            tot += __shfl_xor_sync(0xffffffffu, tot, 4);
+            __syncwarp();  // the next batch rewrites the rows
+            const int src = 2 * h0 + 4 * cq + (b4 ? 2 : 0) + (b3 ? 1 : 0);
+            if (!(lane & 4) && src < ns) back[src] = tot;
+        } else {
             float4 *row = reinterpret_cast<float4 *>(&sg.tr[lane][0]);
 #pragma unroll
             for (int c4 = 0; c4 < NV / 4; ++c4)
                 row[c4] = make_float4(bk[2 * c4].x, bk[2 * c4].y, bk[2 * c4 + 1].x, bk[2 * c4 + 1].y);
-        } else {  // a partial tile: a rolled loop (small code), each pair's shares stored as it goes
-#pragma unroll 1
-            for (int t = 0; t < HP; ++t) {
-                float2 b = make_float2(0.f, 0.f);
-                if (h0 + t < e) p2p_source_x2<1, HQ, HW, false, true>(sg, p0 + h0 + t, X, Y, Z, part, &rv, &b);
-                *reinterpret_cast<float2 *>(&sg.tr[lane][2 * t]) = b;
-            }
-        }
-        __syncwarp();
-        float tot = 0.f;
-        if constexpr (G == 1) {
-            const int half = lane >> 4, col = lane & 15;
-#pragma unroll
-            for (int r = 0; r < 16; ++r) tot += sg.tr[half * 16 + ((r + 4 * half) & 15)][col];
-            tot += __shfl_xor_sync(0xffffffffu, tot, 16);
-        } else {
+            __syncwarp();
+            float tot = 0.f;
             const int sk = G == 8 ? (gi >> 1) : SK * gi;
 #pragma unroll
             for (int r = 0; r < LG; ++r) tot += sg.tr[gi * LG + ((r + sk) & (LG - 1))][rs];
+            __syncwarp();  // the next batch rewrites the rows
+            const int src = 2 * (p0 + h0) + (rs & (NV - 1));
+            if (rs < NV && src < ns) back[src] = tot;
         }
-        __syncwarp();  // the next batch rewrites the rows
-        const int src = 2 * (p0 + h0) + (rs & (NV - 1));
-        if (rs < NV && src < ns) back[src] = tot;
     }
 #pragma unroll
     for (int k = 0; k < 2; ++k) acc[k][0].add(part[k][0].x + part[k][0].y);
 }
 
-// one staged tile (up to 16 source pairs) against a lane's two receivers; group gi of G takes
-// the pairs gi * 16/G .. (gi + 1) * 16/G - 1
+// one staged tile (16 source pairs, those past the tile's end of zero strength) against a lane's
+// two receivers; group gi of G takes the pairs gi * 16/G .. (gi + 1) * 16/G - 1
 template <int R, int G, bool HQ, bool HW, bool SELF>
-__device__ __forceinline__ void p2p_tile_x2(const P2PStageX2<R, HQ, HW> &sg, int ns, int gi, const float2 *X,
+__device__ __forceinline__ void p2p_tile_x2(const P2PStageX2<R, HQ, HW> &sg, int gi, const float2 *X,
                                             const float2 *Y, const float2 *Z, Comp<float> (*acc)[R]) {
     constexpr int SP = 16 / G;  // source pairs per group and tile
     float2 part[2][R];
@@ -382,41 +408,83 @@ __device__ __forceinline__ void p2p_tile_x2(const P2PStageX2<R, HQ, HW> &sg, int
 #pragma unroll
         for (int r = 0; r < R; ++r) part[k][r] = make_float2(0.f, 0.f);
     const int p0 = gi * SP;
-    if (ns == 32) {
-#pragma unroll 4
-        for (int t = 0; t < SP; ++t) p2p_source_x2<R, HQ, HW, SELF>(sg, p0 + t, X, Y, Z, part);
-    } else {
-        const int e = min(SP, (ns + 1) / 2 - p0);
-#pragma unroll 1
-        for (int t = 0; t < e; ++t) p2p_source_x2<R, HQ, HW, SELF>(sg, p0 + t, X, Y, Z, part);
-    }
+#pragma unroll(SELF ? 2 : 4)
+    for (int t = 0; t < SP; ++t) p2p_source_x2<R, HQ, HW, SELF>(sg, p0 + t, X, Y, Z, part);
 #pragma unroll
     for (int k = 0; k < 2; ++k)
 #pragma unroll
         for (int r = 0; r < R; ++r) acc[k][r].add(part[k][r].x + part[k][r].y);
 }
 
-// Symmetric form (SYM, one RHS): a neighbour leaf f > b is owned: its tiles also produce the
-// shares of f's points, written at back + back_unit + (owned points before f) + tile offset; a
-// neighbour f < b is skipped (f's units evaluate the pair and b's points get their shares by
-// the gather); the leaf's own tiles are evaluated one way, all pairs i != j.
+// lane `lane` stages source j (in: the slot holds a source), displaced by the box offset o
+template <int R, bool HQ, bool HW>
+__device__ __forceinline__ void p2p_stage_x2(P2PStageX2<R, HQ, HW> &sg, int lane, bool in, int64_t j, float ox, float oy,
+                                             float oz, int64_t N, const float *__restrict__ loc,
+                                             const float *__restrict__ nrm, const float *__restrict__ q,
+                                             const float *__restrict__ w) {
+    const int sp = lane >> 1, h = lane & 1;
+    float *a = reinterpret_cast<float *>(&sg.a[sp]), *b = reinterpret_cast<float *>(&sg.b[sp]);
+    if (in) {
+        a[h] = -(loc[j] + ox);
+        a[2 + h] = -(loc[N + j] + oy);
+        b[h] = -(loc[2 * N + j] + oz);
+        b[2 + h] = HQ ? q[j] : 0.f;
+        if (HW) {
+            float *c = reinterpret_cast<float *>(&sg.c[sp]), *d = reinterpret_cast<float *>(&sg.d[sp]);
+            c[h] = nrm[j];
+            c[2 + h] = nrm[N + j];
+            d[h] = nrm[2 * N + j];
+            d[2 + h] = w[j];
+        }
+#pragma unroll
+        for (int r = 1; r < R; ++r) {
+            if (HQ) sg.q[r - 1][lane] = q[r * N + j];
+            if (HW) sg.w[r - 1][lane] = w[r * N + j];
+        }
+    } else {  // zero strength, 1e4 leaf widths away
+        a[h] = -1e4f;
+        a[2 + h] = -1e4f;
+        b[h] = -1e4f;
+        b[2 + h] = 0.f;
+        if (HW) {
+            float *c = reinterpret_cast<float *>(&sg.c[sp]), *d = reinterpret_cast<float *>(&sg.d[sp]);
+            c[h] = 0.f;
+            c[2 + h] = 0.f;
+            d[h] = 0.f;
+            d[2 + h] = 0.f;
+        }
+#pragma unroll
+        for (int r = 1; r < R; ++r) {
+            if (HQ) sg.q[r - 1][lane] = 0.f;
+            if (HW) sg.w[r - 1][lane] = 0.f;
+        }
+    }
+}
+
+// Symmetric form (SYM, one RHS): the list holds the neighbour leaves f > b; their tiles also
+// produce the shares of the sources, written at back + the unit's region + list position; a
+// neighbour f < b is left out (f's units evaluate the pair and b's points get their shares by the
+// gather). Otherwise the list holds all neighbours. The leaf's own tiles are evaluated one way,
+// all pairs i != j.
 struct BackArgs {
     float *back;
     const int32_t *S;
     const int64_t *base;
 };
 
-// the packed counterpart of p2p_unit_g (same units, lanes, groups and merge)
-template <int R, int G, bool HQ, bool HW, bool SYM = false>
-__device__ __forceinline__ void p2p_unit_gx2(P2PStageX2<R, HQ, HW> &sg, int lane, int b, int r0, int nr,
+// One item by one warp, its lanes split into G groups (G = 1 for 33..64 receivers, 2 for 17..32, 4
+// for 9..16, 8 for 1..8): lane = gi * (32/G) + rs holds the receivers rs and rs + 32/G and takes
+// group gi's share of every source tile.
+template <int R, int G, bool HQ, bool HW, bool SYM>
+__device__ __forceinline__ void p2p_item_gx2(P2PStageSym<R, HQ, HW, SYM> &sg, int lane, int4 it, int nr,
                                              const int32_t *__restrict__ bstart, const int32_t *__restrict__ bcount,
                                              const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
                                              const int8_t *__restrict__ nd, int64_t N, const float *__restrict__ loc,
                                              const float *__restrict__ nrm, const float *__restrict__ q,
-                                             const float *__restrict__ w, double *__restrict__ out,
-                                             BackArgs ba = BackArgs{}) {
+                                             const float *__restrict__ w, float2 *__restrict__ fwd, BackArgs ba) {
     constexpr int LG = 32 / G;
     const int rs = lane & (LG - 1), gi = lane / LG;
+    const int b = it.x, r0 = it.y;
     const int s0 = bstart[b];
     float2 X[2], Y[2], Z[2];
     RecvX2 rv;
@@ -435,76 +503,62 @@ __device__ __forceinline__ void p2p_unit_gx2(P2PStageX2<R, HQ, HW> &sg, int lane
             rv.q[k] = make_float2(qi, qi);
         }
     }
-    float *back_unit = nullptr;
-    if (SYM) back_unit = ba.back + ba.base[b] + (int64_t)(r0 / P2P_UNIT) * ba.S[b];
-    int boff = 0;  // owned points before the current neighbour
-    const int nn = ncnt[b];
-    int my_f = 0;
-    float my_d[3] = {0.f, 0.f, 0.f};
-    if (lane < nn) {
-        my_f = nbr[b * 27 + lane];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) my_d[d] = (float)nd[(b * 27 + lane) * 4 + d];
-    }
-    const int sp = lane >> 1, h = lane & 1;  // this lane's slot when staging
-    for (int k = 0; k < nn; ++k) {
-        const int f = __shfl_sync(0xffffffffu, my_f, k);
-        const float ox = __shfl_sync(0xffffffffu, my_d[0], k);
-        const float oy = __shfl_sync(0xffffffffu, my_d[1], k);
-        const float oz = __shfl_sync(0xffffffffu, my_d[2], k);
-        if (SYM && f < b) continue;  // uniform in the warp
-        const int fs = bstart[f], fc = bcount[f];
-        const bool self = (f == b);
+    if (it.z < 0) {  // the unit's first item: its own leaf, then the list from 0
+        const int fc = bcount[b];
         for (int t0 = 0; t0 < fc; t0 += 32) {
-            float *a = reinterpret_cast<float *>(&sg.a[sp]);
-            float *bq = reinterpret_cast<float *>(&sg.b[sp]);
-            if (t0 + lane < fc) {
-                const int64_t j = fs + t0 + lane;
-                a[h] = -(loc[j] + ox);
-                a[2 + h] = -(loc[N + j] + oy);
-                bq[h] = -(loc[2 * N + j] + oz);
-                bq[2 + h] = HQ ? q[j] : 0.f;
-                if (HW) {
-                    float *c = reinterpret_cast<float *>(&sg.c[sp]);
-                    float *dd = reinterpret_cast<float *>(&sg.d[sp]);
-                    c[h] = nrm[j];
-                    c[2 + h] = nrm[N + j];
-                    dd[h] = nrm[2 * N + j];
-                    dd[2 + h] = w[j];
-                }
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    if (HQ) sg.q[r - 1][lane] = q[r * N + j];
-                    if (HW) sg.w[r - 1][lane] = w[r * N + j];
-                }
-            } else {  // zero strength, 1e4 leaf widths away
-                a[h] = -1e4f;
-                a[2 + h] = -1e4f;
-                bq[h] = -1e4f;
-                bq[2 + h] = 0.f;
-                if (HW) {
-                    float *c = reinterpret_cast<float *>(&sg.c[sp]);
-                    float *dd = reinterpret_cast<float *>(&sg.d[sp]);
-                    c[h] = 0.f;
-                    c[2 + h] = 0.f;
-                    dd[h] = 0.f;
-                    dd[2 + h] = 0.f;
-                }
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    if (HQ) sg.q[r - 1][lane] = 0.f;
-                    if (HW) sg.w[r - 1][lane] = 0.f;
-                }
-            }
+            p2p_stage_x2<R, HQ, HW>(sg, lane, t0 + lane < fc, (int64_t)s0 + t0 + lane, 0.f, 0.f, 0.f, N, loc, nrm, q, w);
             __syncwarp();
-            const int ns = min(32, fc - t0);
-            if (self) p2p_tile_x2<R, G, HQ, HW, true>(sg, ns, gi, X, Y, Z, acc);
-            else if constexpr (SYM) p2p_tile_x2_sym<G, HQ, HW>(sg, ns, gi, lane, X, Y, Z, rv, acc, back_unit + boff + t0);
-            else p2p_tile_x2<R, G, HQ, HW, false>(sg, ns, gi, X, Y, Z, acc);
+            p2p_tile_x2<R, G, HQ, HW, true>(sg, gi, X, Y, Z, acc);
             __syncwarp();
         }
-        if (SYM && !self) boff += fc;
     }
+    const int lbeg = max(it.z, 0), lend = it.w;
+    if (lbeg < lend) {
+        // the list: per neighbour its end position and the shift from positions to points
+        const int nn = ncnt[b];
+        int cnt = 0, st = 0;
+        float4 tb = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (lane < nn) {
+            const int f = nbr[b * 27 + lane];
+            if (SYM ? f > b : f != b) cnt = bcount[f];
+            st = bstart[f];
+            tb.x = (float)nd[(b * 27 + lane) * 4];
+            tb.y = (float)nd[(b * 27 + lane) * 4 + 1];
+            tb.z = (float)nd[(b * 27 + lane) * 4 + 2];
+        }
+        int end = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += v;
+        }
+        if (lane < 27) {
+            tb.w = __int_as_float(st - (end - cnt));
+            sg.tab[lane] = tb;
+            sg.tend[lane] = end;
+        }
+        __syncwarp();
+        float *back_unit = nullptr;
+        if (SYM) back_unit = ba.back + ba.base[b] + (int64_t)(r0 / P2P_UNIT) * ba.S[b];
+        int k = 0, kend = sg.tend[0];
+        float4 cur = sg.tab[0];
+        for (int t0 = lbeg; t0 < lend; t0 += 32) {
+            const int s = t0 + lane;
+            const bool in = s < lend;
+            if (in && s >= kend) {
+                do kend = sg.tend[++k];
+                while (s >= kend);
+                cur = sg.tab[k];
+            }
+            p2p_stage_x2<R, HQ, HW>(sg, lane, in, (int64_t)__float_as_int(cur.w) + s, cur.x, cur.y, cur.z, N, loc, nrm, q,
+                                    w);
+            __syncwarp();
+            if constexpr (SYM) p2p_tile_x2_sym<G, HQ, HW>(sg, min(32, lend - t0), gi, lane, X, Y, Z, rv, acc, back_unit + t0);
+            else p2p_tile_x2<R, G, HQ, HW, false>(sg, gi, X, Y, Z, acc);
+            __syncwarp();
+        }
+    }
+    // merge the groups' partial sums into group 0 (a fixed butterfly: deterministic)
 #pragma unroll
     for (int off = LG; off < 32; off <<= 1)
 #pragma unroll
@@ -521,93 +575,119 @@ __device__ __forceinline__ void p2p_unit_gx2(P2PStageX2<R, HQ, HW> &sg, int lane
         for (int k = 0; k < 2; ++k) {
             const int li = rs + k * LG;
             if (li < nr) {
-                const int64_t i = s0 + r0 + li;
 #pragma unroll
-                for (int r = 0; r < R; ++r) out[r * N + i] = acc[k][r].get();
+                for (int r = 0; r < R; ++r) fwd[r * P2P_UNIT + li] = make_float2(acc[k][r].s, acc[k][r].c);
             }
         }
     }
 }
 
+// Each warp takes the items blockIdx.x * P2P_WARPS + warp, then every gridDim.x * P2P_WARPS further:
+// one item per warp when the grid covers all items, or a persistent grid of a fixed number of
+// blocks per SM (leaving room on every SM for the far-field kernels that run concurrently on the
+// other stream). Every item writes its own row, so the result does not depend on the grid.
 template <int R, bool HQ, bool HW, bool SYM>
-__global__ void __launch_bounds__(P2P_WARPS * 32, SYM ? 6 : (R == 1 ? 5 : 4)) k_p2p_units_x2(
-    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ bstart,
+__global__ void __launch_bounds__(P2P_WARPS * 32, SYM ? 6 : (R == 1 ? 5 : 4)) k_p2p_items_x2(
+    const int4 *__restrict__ items, int64_t nitems, const int32_t *__restrict__ bstart,
     const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
     const int8_t *__restrict__ nd, int64_t N, const float *__restrict__ loc, const float *__restrict__ nrm,
-    const float *__restrict__ q, const float *__restrict__ w, double *__restrict__ out, BackArgs ba) {
+    const float *__restrict__ q, const float *__restrict__ w, float2 *__restrict__ fwd, BackArgs ba) {
     static_assert(!SYM || (R == 1 && !HW), "the symmetric form is single-RHS, single-layer");
-    __shared__ P2PStageX2<R, HQ, HW> stage[P2P_WARPS];
+    __shared__ P2PStageSym<R, HQ, HW, SYM> stage[P2P_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * P2P_WARPS;
-    for (int64_t u = (int64_t)blockIdx.x * P2P_WARPS + warp; u < nunits; u += stride) {
-        const int2 un = units[u];
-        const int b = un.x, r0 = un.y;
-        const int nr = min(P2P_UNIT, bcount[b] - r0);  // uniform in the warp
-        auto &sg = stage[warp];
-        if (nr > 32) p2p_unit_gx2<R, 1, HQ, HW, SYM>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out, ba);
-        else if (nr > 16) p2p_unit_gx2<R, 2, HQ, HW, SYM>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out, ba);
-        else if (nr > 8) p2p_unit_gx2<R, 4, HQ, HW, SYM>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out, ba);
-        else p2p_unit_gx2<R, 8, HQ, HW, SYM>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out, ba);
+    auto &sg = stage[warp];
+    for (int64_t u = (int64_t)blockIdx.x * P2P_WARPS + warp; u < nitems; u += stride) {
+        const int4 it = items[u];
+        const int nr = min(P2P_UNIT, bcount[it.x] - it.y);  // uniform in the warp
+        float2 *f = fwd + u * (R * P2P_UNIT);
+        if (nr > 32) p2p_item_gx2<R, 1, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
+        else if (nr > 16) p2p_item_gx2<R, 2, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
+        else if (nr > 8) p2p_item_gx2<R, 4, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
+        else p2p_item_gx2<R, 8, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
     }
 }
 
-// Symmetric near field, second pass: one warp per work unit (up to 64 points of leaf B, two per
-// lane); every point j adds the shares that the units of B's neighbours A < B wrote for it,
-// neighbour by neighbour in B's list, unit by unit, in a compensated FP32 sum (TwoSum; FP64
-// arithmetic is slow on this part). Lane k first looks up neighbour k's region; shuffles
-// broadcast it.
+// Second pass: one warp per work unit (up to 64 points of leaf B, two per lane); every point adds
+// its unit's items in order and, in the symmetric form, the shares that the units of B's neighbours
+// A < B wrote for it, neighbour by neighbour in B's list, unit by unit, in a compensated FP32 sum
+// (TwoSum; FP64 arithmetic is slow on this part). Lane k first looks up neighbour k's region;
+// shuffles broadcast it.
 constexpr int GATHER_WARPS = 8;
-__global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_back_gather(
-    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ bstart,
-    const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
-    const int32_t *__restrict__ gofs, const int32_t *__restrict__ ucnt, const int32_t *__restrict__ S,
-    const int64_t *__restrict__ base, const float *__restrict__ back, double *__restrict__ out) {
+template <int R, bool SYM>
+__global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_gather(
+    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ ioff, const float2 *__restrict__ fwd,
+    const int32_t *__restrict__ bstart, const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr,
+    const int32_t *__restrict__ ncnt, const int32_t *__restrict__ gofs, const int32_t *__restrict__ ucnt,
+    const int32_t *__restrict__ S, const int64_t *__restrict__ base, const float *__restrict__ back, int64_t N,
+    double *__restrict__ out) {
     const int64_t uw = (int64_t)blockIdx.x * GATHER_WARPS + (threadIdx.x >> 5);
     const int lane = threadIdx.x & 31;
     if (uw >= nunits) return;  // uniform in the warp
     const int2 un = units[uw];
     const int b = un.x, r0 = un.y;
-    const int nn = ncnt[b];
-    int64_t my_off = 0;
-    int my_S = 0, my_n = 0;
-    if (lane < nn) {
-        const int g = gofs[b * 27 + lane];
-        if (g >= 0) {
-            const int a = nbr[b * 27 + lane];
-            my_off = base[a] + g;
-            my_S = S[a];
-            my_n = ucnt[a];
-        }
-    }
     const int nr = min(P2P_UNIT, bcount[b] - r0);
-    const int j0 = r0 + lane, j1 = r0 + lane + 32;
     const bool v0 = lane < nr, v1 = lane + 32 < nr;
-    Comp<float> a0, a1;
-    for (int k = 0; k < nn; ++k) {
-        const int nk = __shfl_sync(0xffffffffu, my_n, k);
-        if (nk == 0) continue;
-        const int64_t off = __shfl_sync(0xffffffffu, my_off, k);
-        const int sk = __shfl_sync(0xffffffffu, my_S, k);
-        const float *p = back + off;
-        int u = 0;
-        for (; u + 2 <= nk; u += 2) {  // the loads of two units issued before their (ordered) sums
-            const float *pu = p + (int64_t)u * sk, *pv = pu + sk;
-            const float x0 = v0 ? pu[j0] : 0.f, x1 = v1 ? pu[j1] : 0.f;
-            const float y0 = v0 ? pv[j0] : 0.f, y1 = v1 ? pv[j1] : 0.f;
-            a0.add(x0);
-            a1.add(x1);
-            a0.add(y0);
-            a1.add(y1);
-        }
-        for (; u < nk; ++u) {
-            const float *pu = p + (int64_t)u * sk;
-            a0.add(v0 ? pu[j0] : 0.f);
-            a1.add(v1 ? pu[j1] : 0.f);
+    const int64_t i0 = (int64_t)bstart[b] + r0 + lane;
+    Comp<float> a0[R], a1[R];
+    for (int i = ioff[uw], e = ioff[uw + 1]; i < e; ++i) {
+        const float2 *f = fwd + (int64_t)i * (R * P2P_UNIT) + lane;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (v0) {
+                const float2 x = f[r * P2P_UNIT];
+                a0[r].add(x.x);
+                a0[r].c += x.y;
+            }
+            if (v1) {
+                const float2 x = f[r * P2P_UNIT + 32];
+                a1[r].add(x.x);
+                a1[r].c += x.y;
+            }
         }
     }
-    const int64_t i0 = bstart[b];
-    if (v0) out[i0 + j0] += a0.get();
-    if (v1) out[i0 + j1] += a1.get();
+    if constexpr (SYM) {
+        const int nn = ncnt[b];
+        int64_t my_off = 0;
+        int my_S = 0, my_n = 0;
+        if (lane < nn) {
+            const int g = gofs[b * 27 + lane];
+            if (g >= 0) {
+                const int a = nbr[b * 27 + lane];
+                my_off = base[a] + g;
+                my_S = S[a];
+                my_n = ucnt[a];
+            }
+        }
+        const int j0 = r0 + lane, j1 = r0 + lane + 32;
+        for (int k = 0; k < nn; ++k) {
+            const int nk = __shfl_sync(0xffffffffu, my_n, k);
+            if (nk == 0) continue;
+            const int64_t off = __shfl_sync(0xffffffffu, my_off, k);
+            const int sk = __shfl_sync(0xffffffffu, my_S, k);
+            const float *p = back + off;
+            int u = 0;
+            for (; u + 2 <= nk; u += 2) {  // the loads of two units issued before their (ordered) sums
+                const float *pu = p + (int64_t)u * sk, *pv = pu + sk;
+                const float x0 = v0 ? pu[j0] : 0.f, x1 = v1 ? pu[j1] : 0.f;
+                const float y0 = v0 ? pv[j0] : 0.f, y1 = v1 ? pv[j1] : 0.f;
+                a0[0].add(x0);
+                a1[0].add(x1);
+                a0[0].add(y0);
+                a1[0].add(y1);
+            }
+            for (; u < nk; ++u) {
+                const float *pu = p + (int64_t)u * sk;
+                a0[0].add(v0 ? pu[j0] : 0.f);
+                a1[0].add(v1 ? pu[j1] : 0.f);
+            }
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (v0) out[r * N + i0] = a0[r].get();
+        if (v1) out[r * N + i0 + 32] = a1[r].get();
+    }
 }
 
 // Each warp takes the units u = blockIdx.x * P2P_WARPS + warp, then every gridDim.x * P2P_WARPS
@@ -647,21 +727,24 @@ static void launch_units(Context &c, const T *q, const T *w, double *out_sorted,
     // every launch; about a microsecond.)
     const int32_t *bst = t.bstart.p + t.base[L], *bcn = t.bcount.p + t.base[L];
     if constexpr (std::is_same<T, float>::value) {
-        // FP32: the packed kernel, symmetric for one RHS (then the gather of the shares)
+        // FP32: the packed kernel over the work items, symmetric for one RHS and the single layer
         constexpr bool SYM = R == 1 && !HW;
-        auto kern = k_p2p_units_x2<R, HQ, HW, SYM>;
+        constexpr int li = SYM ? 0 : 1;
+        auto kern = k_p2p_items_x2<R, HQ, HW, SYM>;
         if (c.tuned_overlap)
             BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                           (int)cudaSharedmemCarveoutMaxShared));
+        const int64_t ni = t.n_p2p_items[li];
+        blocks = div_up(ni, P2P_WARPS);
+        if (c.tuned_p2p_blocks > 0) blocks = std::min<int64_t>(blocks, (int64_t)c.num_sms * c.tuned_p2p_blocks);
+        c.p2p_fwd.resize((size_t)ni * R * P2P_UNIT);
         const BackArgs ba{SYM ? t.back.p : nullptr, t.back_S.p, t.back_base.p};
-        kern<<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(t.p2p_units.p, nu, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.nbr_d.p,
-                                                           c.N, loc, nrm, q, w, out_sorted, ba);
+        kern<<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(t.p2p_items[li].p, ni, bst, bcn, t.nbr.p, t.nbr_cnt.p,
+                                                           t.nbr_d.p, c.N, loc, nrm, q, w, c.p2p_fwd.p, ba);
         BEM_LAUNCH_CHECK();
-        if (SYM) {
-            k_p2p_back_gather<<<(unsigned)div_up(nu, GATHER_WARPS), GATHER_WARPS * 32, 0, st>>>(
-                t.p2p_units.p, nu, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.back_gofs.p, t.p2p_ucnt.p, t.back_S.p,
-                t.back_base.p, t.back.p, out_sorted);
-        }
+        k_p2p_gather<R, SYM><<<(unsigned)div_up(nu, GATHER_WARPS), GATHER_WARPS * 32, 0, st>>>(
+            t.p2p_units.p, nu, t.p2p_ioff[li].p, c.p2p_fwd.p, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.back_gofs.p, t.p2p_ucnt.p,
+            t.back_S.p, t.back_base.p, t.back.p, c.N, out_sorted);
     } else {
         if (c.tuned_overlap)
             BEM_CUDA(cudaFuncSetAttribute(k_p2p_units<T, R, HQ, HW>, cudaFuncAttributePreferredSharedMemoryCarveout,

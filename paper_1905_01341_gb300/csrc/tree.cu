@@ -535,6 +535,7 @@ __global__ void k_sorted_points(int64_t N, int L, int deep, const int32_t *__res
     }
     s_sorted[i] = s[j];
 }
+constexpr int P2P_ITEM_RECV = 64;  // receivers of a near-field unit
 // Near-field work units: leaf b gets ceil(n_b / 64) units (b, 64 u).
 __global__ void k_p2p_unit_count(int nleaf, const int32_t *__restrict__ bcount, int32_t *__restrict__ cnt) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -551,19 +552,54 @@ __global__ void k_p2p_unit_emit(int nleaf, const int32_t *__restrict__ bcount, c
 
 // Symmetric near field: leaf A owns its pairs with the neighbours B > A. S_A = the floats one
 // unit of A writes (the points of its owned neighbours, in neighbour-list order); the leaf's
-// region holds its units' shares one after another, padded to 32 floats.
+// region holds its units' shares one after another, padded to 32 floats. all_A = the points of all
+// neighbours but A itself.
 __global__ void k_back_sizes(int nleaf, const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
                              const int32_t *__restrict__ bcount, const int32_t *__restrict__ ucnt,
-                             int32_t *__restrict__ S, int32_t *__restrict__ blk32) {
+                             int32_t *__restrict__ S, int32_t *__restrict__ all, int32_t *__restrict__ blk32) {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a >= nleaf) return;
-    int s = 0;
+    int s = 0, n = 0;
     for (int k = 0; k < ncnt[a]; ++k) {
         const int f = nbr[a * 27 + k];
         if (f > a) s += bcount[f];
+        if (f != a) n += bcount[f];
     }
     S[a] = s;
+    all[a] = n;
     blk32[a] = (int32_t)(((int64_t)ucnt[a] * s + 31) / 32);
+}
+
+// Items of a near-field unit (leaf b, receivers r0 ..): `len` list positions cut every `chunk` (times
+// the lane groups that a small unit splits its tiles over); the first item also takes the leaf's
+// own points, and so much less of the list.
+struct UnitCut {
+    int first, chunk, n;
+};
+__device__ __forceinline__ UnitCut unit_cut(int own, int r0, int len, int chunk) {
+    const int nr = min(64, own - r0);
+    const int c = chunk * (nr > 32 ? 1 : (nr > 16 ? 2 : (nr > 8 ? 4 : 8)));
+    const int first = min(len, max(0, c - (own + 31) / 32 * 32));
+    return {first, c, 1 + (len - first + c - 1) / c};
+}
+__global__ void k_p2p_item_count(int64_t nu, const int2 *__restrict__ units, const int32_t *__restrict__ bcount,
+                                 const int32_t *__restrict__ len, int chunk, int32_t *__restrict__ cnt) {
+    const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (u >= nu) return;
+    const int2 un = units[u];
+    cnt[u] = unit_cut(bcount[un.x], un.y, len[un.x], chunk).n;
+}
+__global__ void k_p2p_item_emit(int64_t nu, const int2 *__restrict__ units, const int32_t *__restrict__ bcount,
+                                const int32_t *__restrict__ len, int chunk, const int32_t *__restrict__ off,
+                                int4 *__restrict__ items) {
+    const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (u >= nu) return;
+    const int2 un = units[u];
+    const int L = len[un.x];
+    const UnitCut uc = unit_cut(bcount[un.x], un.y, L, chunk);
+    items[off[u]] = make_int4(un.x, un.y, -1, uc.first);  // -1: from 0, and the leaf's own points
+    for (int i = 1; i < uc.n; ++i)
+        items[off[u] + i] = make_int4(un.x, un.y, uc.first + (i - 1) * uc.chunk, min(L, uc.first + i * uc.chunk));
 }
 
 __global__ void k_back_base(int nleaf, const int32_t *__restrict__ blkoff, int64_t *__restrict__ base) {
@@ -750,40 +786,71 @@ void build_tree(Context &c) {
         DevBuf<int32_t> &ucnt = t.s_i32[4], &uoff = t.s_i32[5], &utot = t.s_i32[6];
         ucnt.resize(nleaf + 1);
         uoff.resize(nleaf + 1);
-        utot.resize(1);
+        utot.resize(4);  // units, 32-float blocks of shares, items of either list
         k_p2p_unit_count<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.bcount.p + t.base[L], ucnt.p);
         BEM_LAUNCH_CHECK();
         exclusive_scan_i32(ucnt.p, uoff.p, nleaf, utot.p, st);
-        int32_t nu = 0;
-        BEM_CUDA(cudaMemcpyAsync(&nu, utot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        // symmetric near field: per-leaf regions of the shares
+        DevBuf<int32_t> &blk = t.s_i32[7], &blkoff = t.s_i32[8], &all = t.s_i32[22];
+        blk.resize(nleaf + 1);
+        blkoff.resize(nleaf + 1);
+        all.resize(nleaf);
+        t.back_S.resize(nleaf);
+        t.back_base.resize(nleaf);
+        t.back_gofs.resize((size_t)nleaf * 27);
+        k_back_sizes<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.nbr.p, t.nbr_cnt.p, t.bcount.p + t.base[L], ucnt.p,
+                                                        t.back_S.p, all.p, blk.p);
+        BEM_LAUNCH_CHECK();
+        exclusive_scan_i32(blk.p, blkoff.p, nleaf, utot.p + 1, st);
+        k_back_base<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, blkoff.p, t.back_base.p);
+        BEM_LAUNCH_CHECK();
+        k_back_gofs<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.nbr.p, t.nbr_cnt.p, t.bcount.p + t.base[L],
+                                                       t.back_gofs.p);
+        BEM_LAUNCH_CHECK();
+        int32_t tot2[2] = {0, 0};
+        unsigned long long hpairs = 0;
+        BEM_CUDA(cudaMemcpyAsync(tot2, utot.p, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        BEM_CUDA(cudaMemcpyAsync(&hpairs, pairs.p, sizeof(hpairs), cudaMemcpyDeviceToHost, st));
         BEM_CUDA(cudaStreamSynchronize(st));
+        const int64_t nu = tot2[0];
+        t.p2p_pairs = (int64_t)hpairs;
         t.n_p2p_units = nu;
         t.p2p_units.resize(std::max<int64_t>(nu, 1));
         k_p2p_unit_emit<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.bcount.p + t.base[L], uoff.p, t.p2p_units.p);
         BEM_LAUNCH_CHECK();
         t.p2p_ucnt.resize(nleaf);
         BEM_CUDA(cudaMemcpyAsync(t.p2p_ucnt.p, ucnt.p, nleaf * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
-        // symmetric near field: per-leaf regions of the shares
-        DevBuf<int32_t> &blk = t.s_i32[7], &blkoff = t.s_i32[8];
-        blk.resize(nleaf + 1);
-        blkoff.resize(nleaf + 1);
-        t.back_S.resize(nleaf);
-        t.back_base.resize(nleaf);
-        t.back_gofs.resize((size_t)nleaf * 27);
-        k_back_sizes<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.nbr.p, t.nbr_cnt.p, t.bcount.p + t.base[L], ucnt.p,
-                                                        t.back_S.p, blk.p);
-        BEM_LAUNCH_CHECK();
-        exclusive_scan_i32(blk.p, blkoff.p, nleaf, utot.p, st);
-        k_back_base<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, blkoff.p, t.back_base.p);
-        BEM_LAUNCH_CHECK();
-        k_back_gofs<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.nbr.p, t.nbr_cnt.p, t.bcount.p + t.base[L],
-                                                       t.back_gofs.p);
-        BEM_LAUNCH_CHECK();
-        int32_t nblk = 0;
-        BEM_CUDA(cudaMemcpyAsync(&nblk, utot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        BEM_CUDA(cudaStreamSynchronize(st));
-        t.n_back = 32 * (int64_t)nblk;
+        t.n_back = 32 * (int64_t)tot2[1];
         t.back.resize(std::max<int64_t>(t.n_back, 1));
+        // FP32 items. The list length of an item: enough items for about six rounds of the warps that
+        // the chip holds (24 per SM), so that the last round is a small part, but at least 64 and at
+        // most 4096 positions (an item's set-up is about a quarter of a 64-source item's time, and
+        // beyond 4096 nearly every unit is one item). Half the pairs in the symmetric list.
+        const double per_item = (double)t.p2p_pairs / P2P_ITEM_RECV / ((double)c.num_sms * 24 * 6);
+        DevBuf<int32_t> &icnt = t.s_i32[23];
+        icnt.resize(std::max<int64_t>(nu, 1));
+        int chunk[2];
+        const int32_t *len[2] = {t.back_S.p, all.p};
+        for (int k = 0; k < 2; ++k) {
+            const double want = k == 0 ? 0.5 * per_item : per_item;
+            chunk[k] = std::min(4096, std::max(64, ((int)std::min(want, 1e6) + 31) / 32 * 32));
+            t.p2p_ioff[k].resize(nu + 1);
+            k_p2p_item_count<<<div_up(nu, tb), tb, 0, st>>>(nu, t.p2p_units.p, t.bcount.p + t.base[L], len[k], chunk[k],
+                                                            icnt.p);
+            BEM_LAUNCH_CHECK();
+            exclusive_scan_i32(icnt.p, t.p2p_ioff[k].p, nu, utot.p + 2 + k, st);
+            BEM_CUDA(cudaMemcpyAsync(t.p2p_ioff[k].p + nu, utot.p + 2 + k, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
+        }
+        int32_t ni[2] = {0, 0};
+        BEM_CUDA(cudaMemcpyAsync(ni, utot.p + 2, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        BEM_CUDA(cudaStreamSynchronize(st));
+        for (int k = 0; k < 2; ++k) {
+            t.n_p2p_items[k] = ni[k];
+            t.p2p_items[k].resize(std::max<int64_t>(ni[k], 1));
+            k_p2p_item_emit<<<div_up(nu, tb), tb, 0, st>>>(nu, t.p2p_units.p, t.bcount.p + t.base[L], len[k], chunk[k],
+                                                           t.p2p_ioff[k].p, t.p2p_items[k].p);
+            BEM_LAUNCH_CHECK();
+        }
     }
 
     // 6. M2L pairs of levels 2..L, then sorted by offset class
@@ -900,10 +967,7 @@ void build_tree(Context &c) {
                                                    clusters ? c.vcid.p : nullptr, t.loc64.p, t.loc32.p, t.nrm64.p,
                                                    t.nrm32.p, t.s_sorted.p, t.ih.p);
     BEM_LAUNCH_CHECK();
-    unsigned long long hpairs = 0;
-    BEM_CUDA(cudaMemcpyAsync(&hpairs, pairs.p, sizeof(hpairs), cudaMemcpyDeviceToHost, st));
     BEM_CUDA(cudaStreamSynchronize(st));
-    t.p2p_pairs = (int64_t)hpairs;
 }
 
 }  // namespace bem
