@@ -336,7 +336,7 @@ struct Context {
     // target-major tensor-core M2L, one state per RHS count R (index 0: R = 1, index 1: R = 4;
     // the products use R = 1, the 4-RHS diagonal product the pair-major kernel): target boxes
     // grouped by octant into tiles of 256 / R targets (256 rows of (target, rhs)); per tile the
-    // offset classes present, by truncated size (ascending), cut into items of a few classes;
+    // offset classes present, by truncated size (ascending), cut into items of equal cost;
     // each item's partial local expansions, summed per target
     struct TmState {
         bool ok = false;                 // built for the current tree and the operators `ops`
@@ -348,7 +348,7 @@ struct Context {
         DevBuf<int32_t> item_off;        // [tiles + 1] first item of each tile
         DevBuf<int4> items;              // [items] (tile, first class slot, classes, largest truncated size)
         DevBuf<float> part;              // [items][256][N_pad] partial local expansions
-        DevBuf<int32_t> s_i32[8];        // scratch of the table build (kept between builds)
+        DevBuf<int32_t> s_i32[9];        // scratch of the table build (kept between builds)
         DevBuf<uint32_t> s_u32[2];
     };
     TmState tm[2];

@@ -75,18 +75,23 @@ __global__ void k_build_tc_table(int P, int Npad, const double *__restrict__ T, 
     }
 }
 
-// Multipoles X [rows][P] (FP32) -> three BF16 planes [3][rows][Kp], zero-padded to Kp.
+// Multipoles X [rows][P] (FP32, P a multiple of 4) -> three BF16 planes [3][rows][Kp], zero-padded to
+// Kp; one thread per four coefficients.
 __global__ void k_split_x(int64_t rows, int P, int Kp, const float *__restrict__ X, __nv_bfloat16 *__restrict__ Xs) {
+    const int quads = Kp / 4;
     const int64_t plane = rows * Kp;
-    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < plane; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = e / Kp;
-        const int k = (int)(e % Kp);
-        const float v = k < P ? X[r * P + k] : 0.f;
-        __nv_bfloat16 b0, b1, b2;
-        split3_f(v, b0, b1, b2);
-        Xs[e] = b0;
-        Xs[plane + e] = b1;
-        Xs[2 * plane + e] = b2;
+    for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < rows * quads; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = e / quads;
+        const int k = (int)(e - r * quads) * 4;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (k < P) v = *reinterpret_cast<const float4 *>(X + r * P + k);
+        const float x[4] = {v.x, v.y, v.z, v.w};
+        alignas(8) __nv_bfloat16 b[3][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) split3_f(x[i], b[0][i], b[1][i], b[2][i]);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            *reinterpret_cast<uint2 *>(Xs + c * plane + r * Kp + k) = *reinterpret_cast<const uint2 *>(b[c]);
     }
 }
 
@@ -343,20 +348,22 @@ void build_tc_tables(Context &c, Operators &o) {
     BEM_LAUNCH_CHECK();
 }
 
+// the multipoles, split once for all translations of a product
+static __nv_bfloat16 *split_multipoles(Context &c, const Operators &o, const float *X, int64_t xrows, cudaStream_t st) {
+    const int Npad = o.tc_Npad;
+    c.xsplit.resize((size_t)3 * xrows * Npad);
+    __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(c.xsplit.p);
+    const int nb = (int)std::min<int64_t>(div_up(xrows * (Npad / 4), 256), 152 * 16);
+    k_split_x<<<nb, 256, 0, st>>>(xrows, o.P, Npad, X, xs);
+    BEM_LAUNCH_CHECK();
+    return xs;
+}
+
 template <int R>
 void launch_m2l_tc(Context &c, const Operators &o, const XChunk *chunks, int64_t nchunks, const float *X,
                    int64_t xrows, float *Ypair, int *err, cudaStream_t st) {
     const int Npad = o.tc_Npad;
-    // split the multipoles once for all translations of this product
-    const size_t nxs = (size_t)3 * xrows * Npad;
-    c.xsplit.resize(nxs);
-    __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(c.xsplit.p);
-    {
-        const int64_t plane = xrows * Npad;
-        const int nb = (int)std::min<int64_t>(div_up(plane, 256), 152 * 16);
-        k_split_x<<<nb, 256, 0, st>>>(xrows, o.P, Npad, X, xs);
-        BEM_LAUNCH_CHECK();
-    }
+    __nv_bfloat16 *xs = split_multipoles(c, o, X, xrows, st);
     // pipeline depth: the context's choice (parameter or autotuner), else three stages (as many as
     // fit at the four-tile stage size)
     const int stages = c.tuned_stages == 2 ? 2 : 3;
@@ -388,14 +395,14 @@ template void launch_m2l_tc<4>(Context &, const Operators &, const XChunk *, int
 // by truncated size ascending (the far classes, whose translations are the smallest), and within
 // a class the K steps from the highest degrees down. A target's items are summed by k_tm_reduce
 // in a fixed order with TwoSum compensation, so the FP32 accumulation in tensor memory spans at
-// most a few classes (8 for one RHS, 4 for four). Target boxes are grouped by octant (their
+// most an item. Target boxes are grouped by octant (their
 // position in the parent), since the 189 classes a box can have depend on it: a tile's classes
 // are then about two thirds full. The products use it with one RHS; with four (the diagonal
 // product, 64 targets per tile) it was slower than the pair-major kernel.
 namespace {
 
 constexpr int TM_ROWS = 2 * TC_M;  // rows per tile: (target, rhs)
-constexpr int TM_MAXCLS = 8;       // classes per item at most
+constexpr int TM_MAXCLS = 32;      // classes per item at most (an item's cost limits them before)
 constexpr size_t TM_STAGE_BYTES = 3 * TM_ROWS * 16 * 2 + 3 * 256 * 16 * 2;  // A (two tiles) + B (K_c <= 256)
 
 // target boxes: the boxes of levels 2.. with at least one M2L translation, key = octant
@@ -455,21 +462,39 @@ __global__ void __launch_bounds__(512) k_tm_classes(int TT, const int32_t *__res
     if (f) tcls[(int64_t)tile * kNumM2LClasses + idx] = order[k];
     if (k == 511) ncls[tile] = before + v;
 }
-__global__ void k_tm_item_count(int64_t ntiles, int per, const int32_t *__restrict__ ncls, int32_t *__restrict__ cnt) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t < ntiles) cnt[t] = (ncls[t] + per - 1) / per;
-}
-__global__ void k_tm_item_emit(int64_t ntiles, int per, const int32_t *__restrict__ ncls,
-                               const int32_t *__restrict__ off, const int32_t *__restrict__ tcls,
-                               const int32_t *__restrict__ cls_K, int Npad, int4 *__restrict__ items) {
+// Time of one class in an item, in arbitrary units: K_c / 16 K steps, whose shared-memory traffic (the
+// MMAs' operand reads and the staged copies: about 576 + 3.75 K_c clocks) bounds a step.
+__device__ __forceinline__ int tm_cost(int Kc) { return Kc / TC_K * (Kc + 160); }
+__global__ void k_tm_tile_cost(int64_t ntiles, const int32_t *__restrict__ ncls, const int32_t *__restrict__ tcls,
+                               const int32_t *__restrict__ cls_K, int Npad, int32_t *__restrict__ cost) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= ntiles) return;
-    const int n = ncls[t];
-    for (int c0 = 0, i = 0; c0 < n; c0 += per, ++i) {
-        const int nc = min(per, n - c0);
-        const int last = tcls[t * kNumM2LClasses + c0 + nc - 1];  // the largest truncated size
-        items[off[t] + i] = make_int4((int)t, c0, nc, cls_K ? cls_K[last] : Npad);
+    int c = 0;
+    for (int i = 0; i < ncls[t]; ++i) c += tm_cost(cls_K ? cls_K[tcls[t * kNumM2LClasses + i]] : Npad);
+    cost[t] = c;
+}
+// The tile's classes cut into items of about equal cost, n = cost / target of them (rounded up), of
+// fewer than TM_MAXCLS classes. Pass 0 counts the items, pass 1 writes them from off[tile] on.
+__global__ void k_tm_items(int64_t ntiles, int target, const int32_t *__restrict__ ncls, const int32_t *__restrict__ tcls,
+                           const int32_t *__restrict__ cls_K, int Npad, const int32_t *__restrict__ cost, int pass,
+                           int32_t *__restrict__ cnt, const int32_t *__restrict__ off, int4 *__restrict__ items) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= ntiles) return;
+    const int n = ncls[t], parts = max(1, (cost[t] + target - 1) / target);
+    int64_t run = 0;  // cost so far
+    int nit = 0, c0 = 0;
+    for (int i = 0; i < n; ++i) {
+        const int Kc = cls_K ? cls_K[tcls[t * kNumM2LClasses + i]] : Npad;
+        run += tm_cost(Kc);
+        // the share of the items that ends nearest to here is full, or the item is
+        const bool cut = (run + tm_cost(Kc) / 2) * parts >= (int64_t)cost[t] * (nit + 1);
+        if (cut || i + 1 - c0 == TM_MAXCLS || i + 1 == n) {
+            if (pass) items[off[t] + nit] = make_int4((int)t, c0, i + 1 - c0, Kc);  // K_c: the largest of the item
+            ++nit;
+            c0 = i + 1;
+        }
     }
+    if (!pass) cnt[t] = nit;
 }
 
 __device__ __forceinline__ void two_sum_add(float &s, float &c, float v) {
@@ -481,7 +506,7 @@ __device__ __forceinline__ void two_sum_add(float &s, float &c, float v) {
 // lc[box][rhs][col] = sum over the tile's items of the partial row (fixed order, compensated)
 // (the loads of four items are issued before their sums, which stay in item order; a row's
 // coefficients past an item's size read as zero and leave the TwoSum unchanged)
-constexpr int TM_MAXITEMS = (kNumM2LClasses + 3) / 4;  // items of one tile at most (4 classes per item)
+constexpr int TM_MAXITEMS = kNumM2LClasses;  // items of one tile at most
 template <int R>
 __global__ void k_tm_reduce(int P, int Npad, const int32_t *__restrict__ tm_box, const int32_t *__restrict__ item_off,
                             const int4 *__restrict__ items, const float *__restrict__ part, float *__restrict__ lc) {
@@ -514,7 +539,7 @@ __global__ void k_tm_reduce(int P, int Npad, const int32_t *__restrict__ tm_box,
 }
 
 template <int R, int TC_STAGES>
-__global__ void __launch_bounds__(TC_THREADS) k_m2l_tm(int P, int Npad, const __nv_bfloat16 *__restrict__ tcB,
+__global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const __nv_bfloat16 *__restrict__ tcB,
                                                        const int4 *__restrict__ items, const int32_t *__restrict__ tab,
                                                        const int32_t *__restrict__ tcls, int64_t xrows,
                                                        const __nv_bfloat16 *__restrict__ Xs, float *__restrict__ part,
@@ -531,7 +556,6 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tm(int P, int Npad, const __
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bfull + TC_STAGES);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     constexpr int NPROD = TC_THREADS - 32;
-    __shared__ int s_src[TM_MAXCLS * TT];
     __shared__ int s_cls[TM_MAXCLS], s_K[TM_MAXCLS];
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -544,13 +568,6 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tm(int P, int Npad, const __
         s_cls[tid] = cl;
         s_K[tid] = cls_K ? cls_K[cl] : Npad;
     }
-    __syncthreads();
-    for (int e = tid; e < nc * TT; e += TC_THREADS) {
-        const int j = e / TT, r = e % TT;
-        s_src[e] = tab[(tile * kNumM2LClasses + s_cls[j]) * TT + r];
-    }
-    int nsteps = 0;
-    for (int j = 0; j < nc; ++j) nsteps += s_K[j] / TC_K;
     if (tid == 0) {
         for (int s = 0; s < TC_STAGES; ++s) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[s])));
@@ -585,6 +602,8 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tm(int P, int Npad, const __
         __syncthreads();
         asm volatile("tcgen05.fence::after_thread_sync;");
     }
+    int nsteps = 0;
+    for (int j = 0; j < nc; ++j) nsteps += s_K[j] / TC_K;
     const int Kp = Npad;
     const int64_t plane = xrows * Kp;
     const uint32_t sbase = smem_u32(smem);
@@ -640,6 +659,17 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tm(int P, int Npad, const __
             const int row2 = u >> 1, jh = u & 1;
             a_dst[i] = (uint32_t)((row2 / TC_M) * atile + kmajor_off(row2 % TC_M, jh * 8) * 2);
         }
+        // rows of Xs of the next class, read while the current one is moved; -1: a target without the
+        // class, a zero row
+        int nxt[AU];
+        auto rows_of = [&](int j) {
+#pragma unroll
+            for (int i = 0; i < AU; ++i) {
+                const int row2 = (pt + i * NPROD) >> 1;  // (target slot, rhs) = (row2 / R, row2 % R)
+                nxt[i] = row2 < TM_ROWS && j < nc ? tab[(tile * kNumM2LClasses + s_cls[j]) * TT + row2 / R] : -1;
+            }
+        };
+        rows_of(0);
         const bool bulk = pt == 0;
         int issued = -1, ks = 0;
         bool stop = false;
@@ -651,12 +681,11 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tm(int P, int Npad, const __
             uint32_t a_sz[AU];
 #pragma unroll
             for (int i = 0; i < AU; ++i) {
-                const int u = pt + i * NPROD;
-                const int row2 = u >> 1;  // (target slot, rhs) = (row2 / R, row2 % R)
-                const int sidx = u < 2 * TM_ROWS ? s_src[j * TT + row2 / R] : -1;
-                a_src[i] = Xs + ((size_t)(sidx >= 0 ? sidx : 0) * R + row2 % R) * Kp + (u & 1) * 8;
-                a_sz[i] = sidx >= 0 ? 16u : 0u;  // a target without this class: a zero row
+                const int u = pt + i * NPROD, row2 = u >> 1;
+                a_src[i] = Xs + ((size_t)max(nxt[i], 0) * R + row2 % R) * Kp + (u & 1) * 8;
+                a_sz[i] = nxt[i] >= 0 ? 16u : 0u;
             }
+            rows_of(j + 1);
             for (int s = 0; s < Kj / TC_K; ++s, ++ks) {
                 const int st = ks % TC_STAGES;
                 if (ks >= TC_STAGES &&
@@ -743,13 +772,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tm(int P, int Npad, const __
 
 }  // namespace
 
-// classes per item: 8 for one RHS; 4 for four (the diagonal product's identities cancel O(1)
-// sums down to O(h), which magnifies the rounding of the FP32 accumulation)
+// Items: whole rounds of the SMs (one block per SM), of equal cost. The rounds are those that 8
+// average classes per item would take, rounded up: cutting every tile into items of 8 classes gave
+// 307 items at 192600 points, three rounds for the work of two (M2L 191 us, 144 us since), and 80 items for 152
+// SMs at 40962 (97 us, 45 us since).
 template <int R>
 static void build_tm_tables(Context &c, const Operators &o, cudaStream_t st) {
     Context::TmState &S = c.tm[R == 1 ? 0 : 1];
     constexpr int TT = TM_ROWS / R;
-    const int per = R == 1 ? 8 : 4;
     Tree &t = c.tree;
     const int tb = 256;
     const int64_t first = t.base[2], n = (int64_t)t.nbox - first;
@@ -805,7 +835,34 @@ static void build_tm_tables(Context &c, const Operators &o, cudaStream_t st) {
     S.item_off.resize(ntiles + 1);
     k_tm_classes<<<(unsigned)ntiles, 512, 0, st>>>(TT, S.src.p, dorder.p, S.cls.p, ncls.p);
     BEM_LAUNCH_CHECK();
-    k_tm_item_count<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, per, ncls.p, icnt.p);
+    const int32_t *clsK = o.margin >= 0 ? o.cls_K.p : nullptr;
+    DevBuf<int32_t> &cost = S.s_i32[8];
+    cost.resize(ntiles);
+    k_tm_tile_cost<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, ncls.p, S.cls.p, clsK, P16, cost.p);
+    BEM_LAUNCH_CHECK();
+    std::vector<int32_t> hcost(ntiles);
+    BEM_CUDA(cudaMemcpyAsync(hcost.data(), cost.p, ntiles * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    BEM_CUDA(cudaStreamSynchronize(st));
+    int64_t total = 0, mean8 = 0;  // mean8: 8 average classes
+    for (int32_t v : hcost) total += v;
+    for (int k = 0; k < kNumM2LClasses; ++k) mean8 += 8 * (int64_t)(Kof(k) / TC_K * (Kof(k) + 160));
+    mean8 /= kNumM2LClasses;
+    const int64_t rounds = std::max<int64_t>(1, div_up(total, c.num_sms * mean8));
+    // the smallest target that gives at most rounds x SMs items (a tile's last item is its own)
+    auto count = [&](int64_t target) {
+        int64_t n = 0;
+        for (int32_t v : hcost) n += std::max<int64_t>(1, (v + target - 1) / target);
+        return n;
+    };
+    int64_t lo = 1, hi = std::max<int64_t>(1, total);
+    while (lo < hi) {
+        const int64_t mid = (lo + hi) / 2;
+        if (count(mid) <= rounds * c.num_sms) hi = mid;
+        else lo = mid + 1;
+    }
+    const int target = (int)lo;
+    k_tm_items<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, target, ncls.p, S.cls.p, clsK, P16, cost.p, 0, icnt.p, nullptr,
+                                                  nullptr);
     BEM_LAUNCH_CHECK();
     exclusive_scan_i32(icnt.p, S.item_off.p, ntiles, tot.p, st);
     BEM_CUDA(cudaMemcpyAsync(S.item_off.p + ntiles, tot.p, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
@@ -814,8 +871,8 @@ static void build_tm_tables(Context &c, const Operators &o, cudaStream_t st) {
     BEM_CUDA(cudaStreamSynchronize(st));
     S.nitems = nitems;
     S.items.resize(std::max(nitems, 1));
-    k_tm_item_emit<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, per, ncls.p, S.item_off.p, S.cls.p,
-                                                       o.margin >= 0 ? o.cls_K.p : nullptr, P16, S.items.p);
+    k_tm_items<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, target, ncls.p, S.cls.p, clsK, P16, cost.p, 1, nullptr,
+                                                  S.item_off.p, S.items.p);
     BEM_LAUNCH_CHECK();
     S.part.resize(std::max<size_t>((size_t)nitems * TM_ROWS * P16, 1));
     BEM_CUDA(cudaStreamSynchronize(st));  // dorder is freed on return
@@ -828,15 +885,7 @@ void launch_m2l_tm(Context &c, const Operators &o, const float *X, int64_t xrows
     Context::TmState &S = c.tm[R == 1 ? 0 : 1];
     if (!S.ok || S.ops != &o) build_tm_tables<R>(c, o, st);
     const int Npad = o.tc_Npad;
-    const size_t nxs = (size_t)3 * xrows * Npad;
-    c.xsplit.resize(nxs);
-    __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(c.xsplit.p);
-    {
-        const int64_t plane = xrows * Npad;
-        const int nb = (int)std::min<int64_t>(div_up(plane, 256), 152 * 16);
-        k_split_x<<<nb, 256, 0, st>>>(xrows, o.P, Npad, X, xs);
-        BEM_LAUNCH_CHECK();
-    }
+    __nv_bfloat16 *xs = split_multipoles(c, o, X, xrows, st);
     if (S.nitems == 0) return;
     const int stages = 3;
     const size_t epi = (size_t)TC_M * Npad * 4;
