@@ -215,7 +215,8 @@ __global__ void k_strengths(int64_t N, const int32_t *__restrict__ perm, const d
 }
 
 // ------------------------------------------------------------------------------ P2M
-// One block per leaf. Points are taken 32 at a time: their regular harmonics R_n^m (m >= 0)
+// FP64, and four right-hand sides in FP32 (the FP32 single-RHS form is in p2m_l2p.cu: with four, the
+// 16 moments of its charges cost twice this kernel's time). One block per leaf. Points are taken 32 at a time: their regular harmonics R_n^m (m >= 0)
 // are built column by column (the recurrence in n for each m) into shared memory, then each
 // thread owns one complex coefficient (n, m) and accumulates
 //   M_n^m += q conj(R_n^m) + w conj(n . grad R_n^m),
@@ -390,141 +391,6 @@ __global__ void __launch_bounds__(256) k_p2m(int p, int nleaf, const int32_t *__
                 dst[n * n + 2 * m - 1] = are[o][r];
                 dst[n * n + 2 * m] = aim[o][r];
             }
-        }
-    }
-}
-
-// FP32 single-RHS, single-layer P2M (every GMRES product) in packed two-wide arithmetic
-// (add/mul/fma .f32x2). The same two phases as k_p2m, with the harmonics of a chunk stored as
-// planes re[ntri][P2MX_RS], im[ntri][P2MX_RS] (point index fastest, rows padded against bank
-// conflicts): a recurrence task (order m, four points) runs as two packed pairs of points and
-// stores each pair with one 8-byte store; a coefficient's thread sums q x R over the chunk's
-// points two at a time (q of the points past the chunk's end is zero, their harmonics finite).
-constexpr int P2MX_RS = P2M_PC + 2;
-__global__ void __launch_bounds__(128) k_p2m_x2(int p, int nleaf, const int32_t *__restrict__ bstart,
-                                                const int32_t *__restrict__ bcount, int64_t N,
-                                                const float *__restrict__ loc, const float *__restrict__ q,
-                                                float *__restrict__ mp) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int P = p * p;
-    const int ntri = p * (p + 1) / 2;
-    float *re = reinterpret_cast<float *>(smraw);  // [ntri][P2MX_RS]
-    float *im = re + ntri * P2MX_RS;               // [ntri][P2MX_RS]
-    float *pq = im + ntri * P2MX_RS;               // [P2M_PC]
-    float2 *tk = reinterpret_cast<float2 *>(pq + P2M_PC);  // [p]: -1 / (2k)
-    float2 *c2t = tk + p;                                  // [p]: 2n - 1
-    float2 *tnm = c2t + p;                                 // [ntri]: 1 / ((n + m)(n - m)), n >= m + 2
-    for (int e = threadIdx.x; e < p; e += blockDim.x) {
-        const float v = e > 0 ? -0.5f / (float)e : 0.f, c = (float)(2 * e - 1);
-        tk[e] = make_float2(v, v);
-        c2t[e] = make_float2(c, c);
-    }
-    for (int e = threadIdx.x; e < ntri; e += blockDim.x) {
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= e) ++n;
-        const int m = e - n * (n + 1) / 2;
-        const float v = n >= m + 2 ? 1.f / ((float)(n + m) * (float)(n - m)) : 0.f;
-        tnm[e] = make_float2(v, v);
-    }
-    const int b = blockIdx.x;
-    const int s0 = bstart[b], cnt = bcount[b];
-    constexpr int MAXC = 2;  // complex coefficients per thread (ntri <= 2 * blockDim)
-    int cn[MAXC], cm[MAXC];
-    float2 accr[MAXC], acci[MAXC];
-#pragma unroll
-    for (int o = 0; o < MAXC; ++o) {
-        const int c = threadIdx.x + o * blockDim.x;
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= c) ++n;
-        cn[o] = (c < ntri) ? n : -1;
-        cm[o] = c - n * (n + 1) / 2;
-        accr[o] = acci[o] = make_float2(0.f, 0.f);
-    }
-    for (int c0 = 0; c0 < cnt; c0 += P2M_PC) {
-        const int pc = min(P2M_PC, cnt - c0);
-        __syncthreads();
-        for (int jj = threadIdx.x; jj < P2M_PC; jj += blockDim.x) pq[jj] = jj < pc ? q[s0 + c0 + jj] : 0.f;
-        // recurrence tasks: (order m, four points), the point groups fastest
-        constexpr int NG = P2M_PC / 4;
-        for (int task = threadIdx.x; task < NG * p; task += blockDim.x) {
-            const int g = task % NG, m = task / NG;
-            float2 X[2], Y[2], Z[2], NR2[2], MR[2], MI[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int64_t ia = s0 + c0 + min(g * 4 + 2 * h, pc - 1), ib = s0 + c0 + min(g * 4 + 2 * h + 1, pc - 1);
-                X[h] = make_float2(loc[ia], loc[ib]);
-                Y[h] = make_float2(loc[N + ia], loc[N + ib]);
-                Z[h] = make_float2(loc[2 * N + ia], loc[2 * N + ib]);
-                const float2 r2 = __ffma2_rn(Z[h], Z[h], __ffma2_rn(Y[h], Y[h], __fmul2_rn(X[h], X[h])));
-                NR2[h] = make_float2(-r2.x, -r2.y);
-                MR[h] = make_float2(1.f, 1.f);
-                MI[h] = make_float2(0.f, 0.f);
-            }
-            for (int k = 1; k <= m; ++k) {
-                const float2 F = tk[k];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float2 a = __ffma2_rn(X[h], MR[h], __fmul2_rn(make_float2(-Y[h].x, -Y[h].y), MI[h]));
-                    const float2 bb = __ffma2_rn(X[h], MI[h], __fmul2_rn(Y[h], MR[h]));
-                    MR[h] = __fmul2_rn(F, a);
-                    MI[h] = __fmul2_rn(F, bb);
-                }
-            }
-            float2 P2R[2], P2I[2], P1R[2], P1I[2];
-            const int rmm = tri_idx(m, m) * P2MX_RS + g * 4, rm1 = tri_idx(m + 1, m) * P2MX_RS + g * 4;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                *reinterpret_cast<float2 *>(re + rmm + 2 * h) = MR[h];
-                *reinterpret_cast<float2 *>(im + rmm + 2 * h) = MI[h];
-                P2R[h] = MR[h];
-                P2I[h] = MI[h];
-                P1R[h] = __fmul2_rn(Z[h], MR[h]);
-                P1I[h] = __fmul2_rn(Z[h], MI[h]);
-                if (m + 1 < p) {
-                    *reinterpret_cast<float2 *>(re + rm1 + 2 * h) = P1R[h];
-                    *reinterpret_cast<float2 *>(im + rm1 + 2 * h) = P1I[h];
-                }
-            }
-            for (int n = m + 2; n < p; ++n) {
-                const int idx = tri_idx(n, m);
-                const float2 D = tnm[idx], C2 = c2t[n];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const float2 C2Z = __fmul2_rn(C2, Z[h]);
-                    const float2 CR = __fmul2_rn(__ffma2_rn(C2Z, P1R[h], __fmul2_rn(NR2[h], P2R[h])), D);
-                    const float2 CI = __fmul2_rn(__ffma2_rn(C2Z, P1I[h], __fmul2_rn(NR2[h], P2I[h])), D);
-                    *reinterpret_cast<float2 *>(re + idx * P2MX_RS + g * 4 + 2 * h) = CR;
-                    *reinterpret_cast<float2 *>(im + idx * P2MX_RS + g * 4 + 2 * h) = CI;
-                    P2R[h] = P1R[h];
-                    P2I[h] = P1I[h];
-                    P1R[h] = CR;
-                    P1I[h] = CI;
-                }
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int o = 0; o < MAXC; ++o) {
-            if (cn[o] < 0) continue;
-            const int row = tri_idx(cn[o], cm[o]) * P2MX_RS;
-#pragma unroll 4
-            for (int jj = 0; jj < P2M_PC; jj += 2) {
-                const float2 Q = *reinterpret_cast<const float2 *>(pq + jj);
-                accr[o] = __ffma2_rn(Q, *reinterpret_cast<const float2 *>(re + row + jj), accr[o]);
-                acci[o] = __ffma2_rn(Q, *reinterpret_cast<const float2 *>(im + row + jj), acci[o]);
-            }
-        }
-    }
-#pragma unroll
-    for (int o = 0; o < MAXC; ++o) {
-        const int n = cn[o], m = cm[o];
-        if (n < 0) continue;
-        float *dst = mp + (size_t)b * P;
-        if (m == 0) {
-            dst[n * n] = accr[o].x + accr[o].y;
-        } else {
-            dst[n * n + 2 * m - 1] = accr[o].x + accr[o].y;
-            dst[n * n + 2 * m] = -(acci[o].x + acci[o].y);
         }
     }
 }
@@ -816,8 +682,8 @@ void launch_reduce_pairs(int t0, int ntg, const int32_t *off, const int32_t *by,
     BEM_LAUNCH_CHECK();
 }
 
-// ------------------------------------------------------------------------------ L2P
-// One warp per leaf: leaves hold about 70-150 points, and a 128-thread block left most of its
+// ------------------------------------------------------------------------------ L2P (FP64)
+// One warp per leaf (the FP32 form is in p2m_l2p.cu): leaves hold about 70-150 points, and a 128-thread block left most of its
 // lanes idle on the second pass over a leaf's points.
 constexpr int L2P_THREADS = 32;
 
@@ -948,110 +814,6 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p(int p, const int32_t *__res
     }
 }
 
-// FP32 form of k_l2p with packed two-wide arithmetic (add/mul/fma .f32x2): each lane's two
-// points are the two halves of every recurrence and sum, so one instruction advances both. The
-// tables are stored as broadcast pairs: the local expansion with the real form's factors folded
-// in (m = 0: 1; m > 0: 2 Re, -2 Im), -1/(2k), 1/((n+m)(n-m)) and 2n - 1. Same recurrences, same
-// column order and the same TwoSum over the columns as k_l2p.
-template <int R>
-__global__ void __launch_bounds__(L2P_THREADS) k_l2p_x2(int p, const int32_t *__restrict__ bstart,
-                                                        const int32_t *__restrict__ bcount, int64_t N,
-                                                        const float *__restrict__ loc, const float *__restrict__ lc,
-                                                        float *__restrict__ far) {
-    extern __shared__ __align__(16) unsigned char smraw[];
-    const int P = p * p, ntri = p * (p + 1) / 2;
-    float2 *Ls = reinterpret_cast<float2 *>(smraw);  // [R][P]
-    float2 *tk = Ls + R * P;                          // [p]
-    float2 *tnm = tk + p;                             // [ntri]
-    float2 *c2t = tnm + ntri;                         // [p]: 2n - 1
-    const int b = blockIdx.x;
-    for (int e = threadIdx.x; e < R * P; e += L2P_THREADS) {
-        const int k = e % P;
-        int n = 0;
-        while ((n + 1) * (n + 1) <= k) ++n;
-        const int j = k - n * n;
-        const float f = j == 0 ? 1.f : ((j & 1) ? 2.f : -2.f);
-        const float v = f * lc[(size_t)b * R * P + e];
-        Ls[e] = make_float2(v, v);
-    }
-    for (int e = threadIdx.x; e < p; e += L2P_THREADS) {
-        const float v = e > 0 ? -0.5f / (float)e : 0.f;
-        tk[e] = make_float2(v, v);
-        const float c = (float)(2 * e - 1);
-        c2t[e] = make_float2(c, c);
-    }
-    for (int e = threadIdx.x; e < ntri; e += L2P_THREADS) {
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= e) ++n;
-        const int m = e - n * (n + 1) / 2;
-        const float v = n >= m + 2 ? 1.f / ((float)(n + m) * (float)(n - m)) : 0.f;
-        tnm[e] = make_float2(v, v);
-    }
-    __syncthreads();
-    const int s0 = bstart[b], cnt = bcount[b];
-    for (int c0 = threadIdx.x; c0 < cnt; c0 += 2 * L2P_THREADS) {
-        const bool two = c0 + L2P_THREADS < cnt;
-        const int64_t i0 = s0 + c0, i1 = s0 + (two ? c0 + L2P_THREADS : c0);
-        const float2 X = make_float2(loc[i0], loc[i1]), Y = make_float2(loc[N + i0], loc[N + i1]),
-                     Z = make_float2(loc[2 * N + i0], loc[2 * N + i1]);
-        const float2 NY = make_float2(-Y.x, -Y.y);
-        const float2 R2 = __ffma2_rn(Z, Z, __ffma2_rn(Y, Y, __fmul2_rn(X, X)));
-        const float2 NR2 = make_float2(-R2.x, -R2.y);
-        CompSum<float> acc[2][R];
-        float2 MR = make_float2(1.f, 1.f), MI = make_float2(0.f, 0.f);
-        for (int m = 0; m < p; ++m) {
-            if (m > 0) {
-                const float2 F = tk[m];
-                const float2 a = __ffma2_rn(X, MR, __fmul2_rn(NY, MI));  // x mr - y mi
-                const float2 bb = __ffma2_rn(X, MI, __fmul2_rn(Y, MR));  // x mi + y mr
-                MR = __fmul2_rn(F, a);
-                MI = __fmul2_rn(F, bb);
-            }
-            float2 col[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) col[r] = make_float2(0.f, 0.f);
-            auto term = [&](int n, float2 cr, float2 ci) {
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float2 *Lr = Ls + r * P + n * n;
-                    if (m == 0) {
-                        col[r] = __ffma2_rn(Lr[0], cr, col[r]);
-                    } else {
-                        col[r] = __ffma2_rn(Lr[2 * m - 1], cr, col[r]);
-                        col[r] = __ffma2_rn(Lr[2 * m], ci, col[r]);
-                    }
-                }
-            };
-            term(m, MR, MI);
-            if (m + 1 < p) {
-                float2 P2R = MR, P2I = MI, P1R = __fmul2_rn(Z, MR), P1I = __fmul2_rn(Z, MI);
-                term(m + 1, P1R, P1I);
-                for (int n = m + 2; n < p; ++n) {
-                    const float2 D = tnm[tri_idx(n, m)];
-                    const float2 C2Z = __fmul2_rn(c2t[n], Z);
-                    const float2 CR = __fmul2_rn(__ffma2_rn(C2Z, P1R, __fmul2_rn(NR2, P2R)), D);
-                    const float2 CI = __fmul2_rn(__ffma2_rn(C2Z, P1I, __fmul2_rn(NR2, P2I)), D);
-                    term(n, CR, CI);
-                    P2R = P1R;
-                    P2I = P1I;
-                    P1R = CR;
-                    P1I = CI;
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r) {
-                acc[0][r].add(col[r].x);
-                acc[1][r].add(col[r].y);
-            }
-        }
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            far[r * N + i0] = acc[0][r].get();
-            if (two) far[r * N + i1] = acc[1][r].get();
-        }
-    }
-}
-
 // out[perm[k]] = (far_k + near_k) / h_leaf: the far field (L2P) and the near field (P2P, run
 // concurrently on the side stream) meet here, back in the caller's vertex order.
 template <class T>
@@ -1159,27 +921,25 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
     const int nleaf = t.nb[L];
     {
         PhaseScope ps(c, PH_P2M, fs);
-        const int ntri = p * (p + 1) / 2;
-        size_t sm = ((size_t)2 * P2M_PC * ntri + P2M_PC * 3 + 2 * P2M_PC * R + p + ntri) * sizeof(T);
-        const int threads = ntri <= 256 ? 128 : 256;  // ntri <= 2 * threads
-        bool hw = false;
-        for (int r = 0; r < R; ++r) hw = hw || a.g[r] != 0.0;
-        if (!F64 && R == 1 && !hw && ntri <= 256) {  // packed FP32x2 form (every GMRES product)
-            const size_t smx = (size_t)2 * ntri * P2MX_RS * sizeof(float) + P2M_PC * sizeof(float) +
-                               (size_t)(2 * p + ntri) * sizeof(float2);
-            if (smx > 48 * 1024)
-                BEM_CUDA(cudaFuncSetAttribute(k_p2m_x2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smx));
-            k_p2m_x2<<<nleaf, 128, smx, fs>>>(p, nleaf, t.bstart.p + t.base[L], t.bcount.p + t.base[L], N,
-                                              (const float *)loc, (const float *)q,
-                                              (float *)mp + (size_t)t.base[L] * P);
-        } else {
+        const int32_t *bst = t.bstart.p + t.base[L], *bcn = t.bcount.p + t.base[L];
+        T *leaf_mp = mp + (size_t)t.base[L] * R * P;
+        bool hq = false, hw = false;
+        for (int r = 0; r < R; ++r) {
+            hq = hq || a.f[r] != 0.0;
+            hw = hw || a.g[r] != 0.0;
+        }
+        if constexpr (F64 || R > 1) {
+            const int ntri = p * (p + 1) / 2;
+            const size_t sm = ((size_t)2 * P2M_PC * ntri + P2M_PC * 3 + 2 * P2M_PC * R + p + ntri) * sizeof(T);
+            const int threads = ntri <= 256 ? 128 : 256;  // ntri <= 2 * threads
             auto kern = hw ? k_p2m<T, R, true> : k_p2m<T, R, false>;
             if (sm > 48 * 1024)
                 BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-            kern<<<nleaf, threads, sm, fs>>>(p, nleaf, t.bstart.p + t.base[L], t.bcount.p + t.base[L], N, loc, nrm, q,
-                                             w, mp + (size_t)t.base[L] * R * P);
+            kern<<<nleaf, threads, sm, fs>>>(p, nleaf, bst, bcn, N, loc, nrm, q, w, leaf_mp);
+            BEM_LAUNCH_CHECK();
+        } else {
+            launch_p2m32<R>(p, nleaf, bst, bcn, N, loc, nrm, q, w, hq, hw, leaf_mp, fs);
         }
-        BEM_LAUNCH_CHECK();
     }
     // zero the locals (boxes without a translation; the multipoles of every level are written whole)
     BEM_CUDA(cudaMemsetAsync(lc, 0, exp_sz * sizeof(T), fs));
@@ -1284,17 +1044,15 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
     // L2P
     {
         PhaseScope ps(c, PH_L2P, fs);
+        const int32_t *bst = t.bstart.p + t.base[L], *bcn = t.bcount.p + t.base[L];
+        const T *leaf_lc = lc + (size_t)t.base[L] * R * P;
         if constexpr (F64) {
-            size_t sm = ((size_t)R * P + p + (size_t)p * (p + 1) / 2) * sizeof(T);  // expansion + divisor tables
-            k_l2p<T, R><<<nleaf, L2P_THREADS, sm, fs>>>(p, t.bstart.p + t.base[L], t.bcount.p + t.base[L], N, loc,
-                                                        lc + (size_t)t.base[L] * R * P, far);
-        } else {  // packed FP32x2: the expansion and the tables as broadcast pairs
-            size_t sm = ((size_t)R * P + 2 * p + (size_t)p * (p + 1) / 2) * sizeof(float2);
-            k_l2p_x2<R><<<nleaf, L2P_THREADS, sm, fs>>>(p, t.bstart.p + t.base[L], t.bcount.p + t.base[L], N,
-                                                        (const float *)loc, (const float *)lc + (size_t)t.base[L] * R * P,
-                                                        (float *)far);
+            const size_t sm = ((size_t)R * P + p + (size_t)p * (p + 1) / 2) * sizeof(T);  // expansion + divisor tables
+            k_l2p<T, R><<<nleaf, L2P_THREADS, sm, fs>>>(p, bst, bcn, N, loc, leaf_lc, far);
+            BEM_LAUNCH_CHECK();
+        } else {
+            launch_l2p32<R>(p, nleaf, bst, bcn, N, loc, leaf_lc, far, fs);
         }
-        BEM_LAUNCH_CHECK();
     }
     launch_near(c.ev_fork);  // (no M2L pairs: the near field has not started yet)
     BEM_CUDA(cudaEventRecord(c.ev_far, fs));

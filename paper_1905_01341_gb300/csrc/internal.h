@@ -444,6 +444,15 @@ void launch_m2m(int P, int pbase, int np, const T *mats, const int32_t *child8, 
 template <class T, int R>
 void launch_l2l(int P, int pbase, int np, const T *mats, const int32_t *child8, T *lc, cudaStream_t st);
 
+// p2m_l2p.cu: FP32 points -> leaf multipoles [leaf][R][p^2] (hq / hw: any single- / double-layer
+// strengths) and leaf local expansions -> far-field potential [R][N]
+template <int R>
+void launch_p2m32(int p, int nleaf, const int32_t *bstart, const int32_t *bcount, int64_t N, const float *loc,
+                  const float *nrm, const float *q, const float *w, bool hq, bool hw, float *mp, cudaStream_t st);
+template <int R>
+void launch_l2p32(int p, int nleaf, const int32_t *bstart, const int32_t *bcount, int64_t N, const float *loc,
+                  const float *lc, float *far, cudaStream_t st);
+
 // p2p.cu
 template <class T, int R>
 void launch_p2p_list(Context &c, const T *q, const T *w, double *near_sorted, bool hq, bool hw, cudaStream_t st);
