@@ -14,11 +14,14 @@
 // |y - (c(q) - c(q_prev)) / tscale|^2 / 2 over recorded solves with Adam.
 //
 // The matrix products run on the tensor cores (tcgen05.mma kind::f16, BF16 operands, FP32
-// accumulation in tensor memory); weights keep an FP32 master copy. Operands are loaded with
-// arbitrary strides into the K-major core-matrix layout, which covers the transposed products
-// of the backward pass. Waits on the MMA barrier are bounded.
+// accumulation in tensor memory); weights keep an FP32 master copy. Every operand exists with its
+// summation index contiguous (weights and, in training, activations and errors also transposed,
+// written by the kernels that make them), in rows padded to 16 bytes, so all products of the forward
+// and the backward pass are filled by 16-byte asynchronous copies. Waits on the MMA barriers are
+// bounded.
 #include "internal.h"
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -26,25 +29,35 @@
 #include <cstring>
 #include <random>
 
+namespace cg = cooperative_groups;
+
 namespace bem {
 
 struct Mlp {
     bool ready = false;
     int lmax = 10, Psh = 121;
     int dims[5] = {0, 0, 0, 0, 0};
-    DevBuf<float> W[4], b[4], mW[4], vW[4], mb[4], vb[4], gW[4], gb[4];
-    DevBuf<__nv_bfloat16> Wb[4];
+    DevBuf<float> W[4], b[4], mW[4], vW[4], mb[4], vb[4];
+    DevBuf<float> grad;           // gradients in parameter order: W1, b1, ..., W4, b4
+    DevBuf<__nv_bfloat16> Wb[4], WTb[4];  // BF16 weights [out][ld(in)] and transposed [in][ld(out)]
+    float *gW(int i) const { return grad.p + goff[2 * i]; }
+    float *gb(int i) const { return grad.p + goff[2 * i + 1]; }
+    int64_t goff[9] = {0};        // offsets of W1, b1, ... in the parameter vector
     int64_t adam_t = 0;
     // recorded samples
     DevBuf<float> SF, ST;
     int64_t ns = 0, cap = 0;
     // work space (batch rows)
     int64_t wrows = 0;
-    DevBuf<__nv_bfloat16> Hb[5];  // layer inputs in BF16 (Hb[0] = features)
+    DevBuf<__nv_bfloat16> Hb[5];  // layer inputs in BF16 [rows][ld(dim)] (Hb[0] = features)
+    DevBuf<__nv_bfloat16> HT[4];  // ... and transposed [dim][ld(rows)] (training)
     DevBuf<float> Z[4];           // pre-activations
-    DevBuf<float> G;              // gradient w.r.t. a layer's output
-    DevBuf<__nv_bfloat16> Gb;
-    DevBuf<float> loss;
+    // gradient w.r.t. a layer's output (two: a layer's is read while the one below is written), in
+    // FP32 [rows][dim], BF16 [rows][ld(dim)] and transposed [dim][ld(rows)]
+    DevBuf<float> G[2];
+    DevBuf<__nv_bfloat16> Gb[2], GT[2];
+    DevBuf<float> loss;           // partial sums of the loss
+    HostPinned<float> hloss;      // the same on the host, then the error flag
     ShBasis feat;
     DevBuf<double> qprev, cphi, cqp, cq, cqp_last;  // q_prev [N]; coefficients [M][Psh]
     bool have_last = false;
@@ -63,10 +76,20 @@ void mlp_free(Mlp *m) { delete m; }
 namespace {
 
 constexpr int GM = 128;           // tile rows
+constexpr int GN = 64;            // tile columns
 constexpr int GK = 64;            // K chunk (bf16): 128 bytes per row = 8 core matrices
-constexpr int G_THREADS = 128;
+constexpr int G_STAGES = 4, G_THREADS = 128;
+constexpr int G_STAGE_ELEMS = (GM + GN) * GK;
+constexpr int G_RED_PITCH = GN + 1;
+constexpr int G_SMEM = G_STAGES * G_STAGE_ELEMS * 2 + 1024;  // aligned to 1024 by the kernel
+static_assert(GM * G_RED_PITCH * 4 <= G_STAGES * G_STAGE_ELEMS * 2, "the split sums reuse the stages");
+constexpr int G_SPLIT = 8;        // CTAs sharing a long K (one cluster)
+constexpr int G_SPLIT_K = 512;    // from this K on
+constexpr int LOSS_BLOCKS = 128;
 constexpr uint32_t G_LBO = 128, G_SBO = 1024;
-constexpr long long kWait = 1ll << 24;
+constexpr long long kWait = 1ll << 20;
+
+constexpr int64_t ld8(int64_t n) { return (n + 7) / 8 * 8; }  // row length padded to 16 bytes of BF16
 
 __device__ __forceinline__ uint32_t sa(const void *p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
 
@@ -100,141 +123,228 @@ __device__ __forceinline__ bool wait_bar(uint32_t bar, uint32_t parity) {
 
 enum { EPI_STORE = 0, EPI_BIAS_RELU = 1, EPI_BIAS = 2, EPI_RELU_MASK = 3 };
 
-// C[m][n] = sum_k A(m,k) B(n,k), A(m,k) = A[m*sam + k*sak], B(n,k) = B[n*sbn + k*sbk].
+// C[m][n] = sum_k A(m,k) B(n,k), A(m,k) = A[m*lda + k], B(n,k) = B[n*ldb + k], rows 16-byte aligned.
 // Epilogues: STORE: C = acc; BIAS: C = acc + bias[n]; BIAS_RELU: C = acc + bias[n] and
-// H = bf16(relu(C)); RELU_MASK: C = acc where Zm[m*ldc + n] > 0, else 0 (and H = bf16(C)).
-template <int NT>
+// H = bf16(relu(C)); RELU_MASK: C = acc where Zm[m*ldc + n] > 0, else 0, and H = bf16(C). HT (when set):
+// H transposed.
+//
+// One 128 x 64 tile per CTA; K in chunks of 64, four of them in flight. The layers are at most a few
+// hundred wide, so a product is a few dozen CTAs and bound by latency: a product of 1000 x 256 with
+// K = 363 took 166 us as 8 CTAs that copied each chunk element by element between two barriers. Weight
+// gradients (K = the batch, a small result) split K over the 8 CTAs of a cluster, whose sums are
+// joined through distributed shared memory in rank order.
+struct GemmOut {
+    float *C;
+    int64_t ldc;
+    int epi;
+    const float *bias, *Zm;
+    __nv_bfloat16 *H, *HT;
+    int64_t ldh, ldt;
+};
+__device__ __forceinline__ void gemm_store(const GemmOut &o, int m, int n, float a) {
+    const int64_t ix = (int64_t)m * o.ldc + n;
+    if (o.epi == EPI_BIAS || o.epi == EPI_BIAS_RELU) a += o.bias[n];
+    if (o.epi == EPI_RELU_MASK) a = o.Zm[ix] > 0.f ? a : 0.f;
+    o.C[ix] = a;
+    if (o.H) {
+        const __nv_bfloat16 h = __float2bfloat16(o.epi == EPI_BIAS_RELU ? fmaxf(a, 0.f) : a);
+        o.H[(int64_t)m * o.ldh + n] = h;
+        if (o.HT) o.HT[(int64_t)n * o.ldt + m] = h;
+    }
+}
+
+template <bool SPLIT>
 __global__ void __launch_bounds__(G_THREADS) k_gemm_bf16(int M, int N, int K, const __nv_bfloat16 *__restrict__ A,
-                                                         int64_t sam, int64_t sak, const __nv_bfloat16 *__restrict__ B,
-                                                         int64_t sbn, int64_t sbk, float *__restrict__ C, int64_t ldc,
-                                                         int epi, const float *__restrict__ bias,
-                                                         const float *__restrict__ Zm, __nv_bfloat16 *__restrict__ H,
-                                                         int *__restrict__ err) {
-    __shared__ __align__(1024) __nv_bfloat16 As[GM * GK];
-    __shared__ __align__(1024) __nv_bfloat16 Bs[NT * GK];
-    __shared__ uint64_t bar;
+                                                         int64_t lda, const __nv_bfloat16 *__restrict__ B, int64_t ldb,
+                                                         GemmOut out, int *__restrict__ err) {
+    extern __shared__ unsigned char g_smem[];
+    __shared__ uint64_t bars[G_STAGES];  // a stage's MMAs are done
     __shared__ uint32_t tslot;
+    unsigned char *smem = g_smem + ((1024u - (sa(g_smem) & 1023u)) & 1023u);
+    __nv_bfloat16 *st0 = reinterpret_cast<__nv_bfloat16 *>(smem);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int m0 = blockIdx.x * GM, n0 = blockIdx.y * NT;
+    int rank = 0, nr = 1, tile_m = blockIdx.x;
+    if constexpr (SPLIT) {
+        cg::cluster_group cl = cg::this_cluster();
+        rank = (int)cl.block_rank();
+        nr = (int)cl.num_blocks();
+        tile_m = blockIdx.x / nr;
+    }
+    const int m0 = tile_m * GM, n0 = blockIdx.y * GN;
     if (tid == 0) {
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sa(&bar)));
+        for (int i = 0; i < G_STAGES; ++i) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sa(&bars[i])));
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sa(&tslot)), "r"(NT));
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sa(&tslot)), "n"(GN));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tslot;
-    uint32_t phase = 0;
-    bool ok = true;
-    const int nchunk = (K + GK - 1) / GK;
-    for (int kc = 0; kc < nchunk && ok; ++kc) {
-        // stage: 16-byte units (8 consecutive k of one row) in the canonical layout
-        for (int u = tid; u < (GM + NT) * (GK / 8); u += G_THREADS) {
-            const bool isA = u < GM * (GK / 8);
-            const int uu = isA ? u : u - GM * (GK / 8);
-            const int row = uu / (GK / 8), j = uu % (GK / 8);
-            __nv_bfloat16 v[8];
-            const int k0 = kc * GK + j * 8;
+    const int nall = (K + GK - 1) / GK;
+    const int c0 = rank * nall / nr, nc = (rank + 1) * nall / nr - c0;  // this CTA's chunks
+    // 16-byte units (8 consecutive k of one row) into the canonical layout; past the edges zeros
+    auto load = [&](int i) {
+        if (i < nc) {
+            __nv_bfloat16 *As = st0 + (i % G_STAGES) * G_STAGE_ELEMS, *Bs = As + GM * GK;
+            const int k0 = (c0 + i) * GK;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int k = k0 + e;
-                __nv_bfloat16 x = __float2bfloat16(0.f);
-                if (isA) {
-                    const int m = m0 + row;
-                    if (m < M && k < K) x = A[(int64_t)m * sam + (int64_t)k * sak];
-                } else {
-                    const int n = n0 + row;
-                    if (n < N && k < K) x = B[(int64_t)n * sbn + (int64_t)k * sbk];
-                }
-                v[e] = x;
+            for (int v = 0; v < (GM + GN) * (GK / 8) / G_THREADS; ++v) {
+                const int u = tid + v * G_THREADS, j = u % (GK / 8), k = k0 + j * 8;
+                const bool isA = v < GM * (GK / 8) / G_THREADS;
+                const int row = isA ? u / (GK / 8) : u / (GK / 8) - GM, g = (isA ? m0 : n0) + row;
+                const bool in = g < (isA ? M : N) && k < K;
+                const __nv_bfloat16 *src = isA ? A + (in ? (int64_t)g * lda + k : 0) : B + (in ? (int64_t)g * ldb + k : 0);
+                __nv_bfloat16 *dst = (isA ? As : Bs) + (row / 8) * 512 + j * 64 + (row % 8) * 8;
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa(dst)), "l"(src),
+                             "r"(in ? min(16, 2 * (K - k)) : 0)
+                             : "memory");
             }
-            __nv_bfloat16 *dst = (isA ? As : Bs) + (row / 8) * 512 + j * 64 + (row % 8) * 8;  // elements
-            *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(v);
         }
+        asm volatile("cp.async.commit_group;" ::: "memory");  // one group per call, empty past the end
+    };
+    bool ok = true;
+    for (int i = 0; i < G_STAGES; ++i) load(i);
+    for (int i = 0; i < nc; ++i) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(G_STAGES - 2) : "memory");  // chunk i (this thread's part)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
         if (tid == 0) {
             asm volatile("tcgen05.fence::after_thread_sync;");
-            const int ksteps = (min(GK, K - kc * GK) + 15) / 16;
+            const __nv_bfloat16 *As = st0 + (i % G_STAGES) * G_STAGE_ELEMS, *Bs = As + GM * GK;
+            const int ksteps = (min(GK, K - (c0 + i) * GK) + 15) / 16;
             for (int s = 0; s < ksteps; ++s) {
                 const uint32_t o = s * 2 * G_LBO;
-                const uint32_t acc = (kc > 0 || s > 0) ? 1u : 0u;
+                const uint32_t acc = (i > 0 || s > 0) ? 1u : 0u;
                 asm volatile(
                     "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                     "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(tmem),
-                    "l"(desc(sa(As) + o)), "l"(desc(sa(Bs) + o)), "r"(idesc_bf16(GM, NT)), "r"(acc));
+                    "l"(desc(sa(As) + o)), "l"(desc(sa(Bs) + o)), "r"(idesc_bf16(GM, GN)), "r"(acc));
             }
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(sa(&bar))
+            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                             sa(&bars[i % G_STAGES]))
                          : "memory");
         }
         __syncwarp();
-        const int bad = __syncthreads_or(wait_bar(sa(&bar), phase) ? 0 : 1);
-        if (bad) {
-            wait_bar(sa(&bar), phase);
-            if (tid == 0) atomicOr(err, 1);
-            ok = false;
+        // refill the stage of chunk i - 1, once its MMAs are done
+        if (i >= 1 && i - 1 + G_STAGES < nc) {
+            ok = ok && wait_bar(sa(&bars[(i - 1) % G_STAGES]), ((i - 1) / G_STAGES) & 1);
+            if (ok) load(i - 1 + G_STAGES);
+            else asm volatile("cp.async.commit_group;" ::: "memory");
+        } else {
+            asm volatile("cp.async.commit_group;" ::: "memory");
         }
-        phase ^= 1u;
-        __syncthreads();
     }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    // the last commit covers every MMA before it
+    if (nc > 0) ok = wait_bar(sa(&bars[(nc - 1) % G_STAGES]), ((nc - 1) / G_STAGES) & 1) && ok;
+    ok = __syncthreads_and(ok);
+    if (!ok && tid == 0) atomicOr(err, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
+    const int row = warp * 32 + lane, m = m0 + row;
+    float *red = reinterpret_cast<float *>(smem);  // SPLIT: [row][G_RED_PITCH], in the free stages
     if (ok) {
-        const int m = m0 + warp * 32 + lane;
-        for (int c0 = 0; c0 < NT; c0 += 16) {
+        for (int q = 0; q < GN; q += 16) {
             uint32_t v[16];
             asm volatile(
                 "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
                   "=r"(v[15])
-                : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0));
+                : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)q));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (m < M) {
+            if constexpr (SPLIT) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int n = n0 + c0 + i;
-                    if (n >= N) continue;
-                    float a = __uint_as_float(v[i]);
-                    const int64_t ix = (int64_t)m * ldc + n;
-                    if (epi == EPI_BIAS || epi == EPI_BIAS_RELU) a += bias[n];
-                    if (epi == EPI_RELU_MASK) a = Zm[ix] > 0.f ? a : 0.f;
-                    C[ix] = a;
-                    if (epi == EPI_BIAS_RELU) H[ix] = __float2bfloat16(fmaxf(a, 0.f));
-                    if (epi == EPI_RELU_MASK && H) H[ix] = __float2bfloat16(a);
-                }
+                for (int i = 0; i < 16; ++i) red[row * G_RED_PITCH + q + i] = nc > 0 ? __uint_as_float(v[i]) : 0.f;
+            } else if (m < M) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (n0 + q + i < N) gemm_store(out, m, n0 + q + i, __uint_as_float(v[i]));
             }
         }
     }
+    if constexpr (SPLIT) {
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        // rank r joins the rows r, r + nr, ... of the tile (a CTA whose wait ran out has set the flag)
+        for (int e = tid; e < GM / nr * GN; e += G_THREADS) {
+            const int rr = rank + e / GN * nr, q = e % GN;
+            if (m0 + rr >= M || n0 + q >= N) continue;
+            float a = 0.f;
+            for (int c = 0; c < nr; ++c) a += cl.map_shared_rank(red, c)[rr * G_RED_PITCH + q];
+            gemm_store(out, m0 + rr, n0 + q, a);
+        }
+        cl.sync();  // no CTA leaves while another still reads its sums
+    }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NT));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(GN));
 }
 
-__global__ void k_f2bf(int64_t n, const float *__restrict__ x, __nv_bfloat16 *__restrict__ y) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) y[i] = __float2bfloat16(x[i]);
+// H[r][c] = bf16(x[r][c] / scale[c]) (scale may be null), rows of ldh; HT (when set) transposed, rows of
+// ldt. Tiles of 32 x 32 through shared memory.
+template <class T>
+__global__ void k_to_bf16(int rows, int cols, const T *__restrict__ x, const float *__restrict__ scale,
+                          __nv_bfloat16 *__restrict__ H, int64_t ldh, __nv_bfloat16 *__restrict__ HT, int64_t ldt) {
+    __shared__ __nv_bfloat16 t[32][34];
+    const int r0 = blockIdx.y * 32, q0 = blockIdx.x * 32;
+    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+        const int r = r0 + i, q = q0 + threadIdx.x;
+        if (r < rows && q < cols) {
+            const float v = (float)x[(int64_t)r * cols + q];
+            const __nv_bfloat16 h = __float2bfloat16(scale ? v / scale[q] : v);
+            H[(int64_t)r * ldh + q] = h;
+            t[i][threadIdx.x] = h;
+        }
+    }
+    if (!HT) return;
+    __syncthreads();
+    for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+        const int q = q0 + i, r = r0 + threadIdx.x;
+        if (r < rows && q < cols) HT[(int64_t)q * ldt + r] = t[threadIdx.x][i];
+    }
 }
 
-__global__ void k_d2bf(int64_t n, const double *__restrict__ x, __nv_bfloat16 *__restrict__ y) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) y[i] = __float2bfloat16((float)x[i]);
+template <class S, class D>
+__global__ void k_convert(int64_t n, const S *__restrict__ x, D *__restrict__ y) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        y[i] = (D)x[i];
 }
 
-// G = (Y - T) / B (also bf16), loss partial sums per block
-__global__ void k_loss_grad(int64_t n, int B, const float *__restrict__ Y, const float *__restrict__ T,
-                            float *__restrict__ G, __nv_bfloat16 *__restrict__ Gb, float *__restrict__ loss) {
+// G = (Y - T) / B (also BF16 and transposed); partial sums of the loss, one per block (LOSS_BLOCKS of
+// them, added up in order on the host). Tiles of 32 rows x 32 columns.
+__global__ void __launch_bounds__(256) k_loss_grad(int rows, int cols, const float *__restrict__ Y,
+                                                   const float *__restrict__ T, float *__restrict__ G,
+                                                   __nv_bfloat16 *__restrict__ Gb, int64_t ldh,
+                                                   __nv_bfloat16 *__restrict__ GT, int64_t ldt, float *__restrict__ loss) {
     __shared__ float red[256];
+    __shared__ __nv_bfloat16 t[32][34];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int tc = (cols + 31) / 32, nt = tc * ((rows + 31) / 32);
     float s = 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        float d = Y[i] - T[i];
-        s += d * d;
-        float g = d / (float)B;
-        G[i] = g;
-        Gb[i] = __float2bfloat16(g);
+    for (int tile = blockIdx.x; tile < nt; tile += gridDim.x) {
+        const int r0 = tile / tc * 32, q0 = tile % tc * 32;
+        __syncthreads();
+        for (int i = ty; i < 32; i += 8) {
+            const int r = r0 + i, q = q0 + tx;
+            if (r < rows && q < cols) {
+                const int64_t ix = (int64_t)r * cols + q;
+                const float d = Y[ix] - T[ix];
+                s += d * d;
+                const float g = d / (float)rows;
+                G[ix] = g;
+                const __nv_bfloat16 h = __float2bfloat16(g);
+                Gb[(int64_t)r * ldh + q] = h;
+                t[i][tx] = h;
+            }
+        }
+        __syncthreads();
+        for (int i = ty; i < 32; i += 8) {
+            const int q = q0 + i, r = r0 + tx;
+            if (r < rows && q < cols) GT[(int64_t)q * ldt + r] = t[tx][i];
+        }
     }
     red[threadIdx.x] = s;
     __syncthreads();
@@ -242,21 +352,30 @@ __global__ void k_loss_grad(int64_t n, int B, const float *__restrict__ Y, const
         if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) atomicAdd(loss, 0.5f * red[0] / (float)B);
+    if (threadIdx.x == 0) loss[blockIdx.x] = 0.5f * red[0] / (float)rows;
 }
 
-// db[n] = sum_rows G[row][n]
-__global__ void k_colsum(int rows, int cols, const float *__restrict__ G, float *__restrict__ db) {
-    int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= cols) return;
+// db[n] = sum_rows G[row][n]: 32 columns per block, 32 rows at a time, joined in a fixed order
+__global__ void __launch_bounds__(1024) k_colsum(int rows, int cols, const float *__restrict__ G, float *__restrict__ db) {
+    __shared__ float red[32][33];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5, n = blockIdx.x * 32 + tx;
     float s = 0.f;
-    for (int r = 0; r < rows; ++r) s += G[(int64_t)r * cols + n];
-    db[n] = s;
+    if (n < cols)
+        for (int r = ty; r < rows; r += 32) s += G[(int64_t)r * cols + n];
+    red[ty][tx] = s;
+    __syncthreads();
+    if (ty == 0 && n < cols) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < 32; ++k) t += red[k][tx];
+        db[n] = t;
+    }
 }
 
+// pb, pt (when set): the BF16 copies of a weight matrix with `din` columns, [out][ldb] and transposed
 __global__ void k_adam(int64_t n, float *__restrict__ p, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, float lr, float b1, float b2, float c1, float c2, float eps,
-                       __nv_bfloat16 *__restrict__ pb) {
+                       float *__restrict__ v, float lr, float b1, float b2, float c1, float c2, float eps, int din,
+                       __nv_bfloat16 *__restrict__ pb, int64_t ldb, __nv_bfloat16 *__restrict__ pt, int64_t ldt) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     float mm = b1 * m[i] + (1.f - b1) * g[i];
@@ -265,7 +384,12 @@ __global__ void k_adam(int64_t n, float *__restrict__ p, const float *__restrict
     v[i] = vv;
     float x = p[i] - lr * (mm / c1) / (sqrtf(vv / c2) + eps);
     p[i] = x;
-    if (pb) pb[i] = __float2bfloat16(x);
+    if (pb) {
+        const int64_t o = i / din, k = i - o * din;
+        const __nv_bfloat16 h = __float2bfloat16(x);
+        pb[o * ldb + k] = h;
+        pt[k * ldt + o] = h;
+    }
 }
 
 // out[m][p] = sum_i Gp_m[p][i] x[a_m + i]  (per-bubble SH coefficients; one block per bubble)
@@ -313,13 +437,6 @@ __global__ void k_col_rms(int64_t rows, int cols, const float *__restrict__ X, f
     out[j] = rms > 0.0 ? (float)rms : 1.f;
 }
 
-// y[r][j] = bf16(x[r][j] / scale[j]) for the network input
-__global__ void k_f2bf_scaled(int64_t n, int cols, const float *__restrict__ x, const float *__restrict__ scale,
-                              __nv_bfloat16 *__restrict__ y) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) y[i] = __float2bfloat16(x[i] / scale[i % cols]);
-}
-
 // y[r][j] = x[r][j] / scale[j] (training targets)
 __global__ void k_div_cols(int64_t n, int cols, const float *__restrict__ x, const float *__restrict__ scale,
                            float *__restrict__ y) {
@@ -353,61 +470,103 @@ Mlp &mlp_of(Context &c) {
     return *c.mlp;
 }
 
-void gemm(Context &c, Mlp &m, int M, int N, int K, const __nv_bfloat16 *A, int64_t sam, int64_t sak,
-          const __nv_bfloat16 *B, int64_t sbn, int64_t sbk, float *C, int64_t ldc, int epi, const float *bias,
-          const float *Zm, __nv_bfloat16 *H) {
-    if (N > 128) {
-        dim3 grid((M + GM - 1) / GM, (N + 255) / 256);
-        k_gemm_bf16<256><<<grid, G_THREADS, 0, c.stream>>>(M, N, K, A, sam, sak, B, sbn, sbk, C, ldc, epi, bias, Zm, H,
-                                                          m.err.p);
-    } else {
-        dim3 grid((M + GM - 1) / GM, (N + 127) / 128);
-        k_gemm_bf16<128><<<grid, G_THREADS, 0, c.stream>>>(M, N, K, A, sam, sak, B, sbn, sbk, C, ldc, epi, bias, Zm, H,
-                                                          m.err.p);
-    }
+void gemm(Context &c, Mlp &m, int M, int N, int K, const __nv_bfloat16 *A, int64_t lda, const __nv_bfloat16 *B,
+          int64_t ldb, const GemmOut &out) {
+    const bool split = K >= G_SPLIT_K;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(div_up(M, GM) * (split ? G_SPLIT : 1)), (unsigned)div_up(N, GN));
+    cfg.blockDim = dim3(G_THREADS);
+    cfg.dynamicSmemBytes = G_SMEM;
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = G_SPLIT;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = split ? 1 : 0;
+    auto kern = split ? k_gemm_bf16<true> : k_gemm_bf16<false>;
+    BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, G_SMEM));
+    BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, M, N, K, A, lda, B, ldb, out, m.err.p));
+    BEM_LAUNCH_CHECK();
+}
+
+template <class T>
+void to_bf16(Context &c, int rows, int cols, const T *x, const float *scale, __nv_bfloat16 *H, __nv_bfloat16 *HT) {
+    dim3 grid(div_up(cols, 32), div_up(rows, 32));
+    k_to_bf16<T><<<grid, dim3(32, 8), 0, c.stream>>>(rows, cols, x, scale, H, ld8(cols), HT, ld8(rows));
     BEM_LAUNCH_CHECK();
 }
 
 void ensure_work(Mlp &m, int64_t rows) {
     if (rows <= m.wrows) return;
     m.wrows = rows;
-    for (int i = 0; i <= 4; ++i) m.Hb[i].resize((size_t)rows * m.dims[i]);
-    for (int i = 0; i < 4; ++i) m.Z[i].resize((size_t)rows * m.dims[i + 1]);
-    int dmax = *std::max_element(m.dims, m.dims + 5);
-    m.G.resize((size_t)rows * dmax);
-    m.Gb.resize((size_t)rows * dmax);
+    const int dmax = *std::max_element(m.dims, m.dims + 5);
+    for (int i = 0; i <= 4; ++i) m.Hb[i].resize((size_t)(rows * ld8(m.dims[i])));
+    for (int i = 0; i < 4; ++i) {
+        m.HT[i].resize((size_t)(m.dims[i] * ld8(rows)));
+        m.Z[i].resize((size_t)rows * m.dims[i + 1]);
+    }
+    for (int i = 0; i < 2; ++i) {
+        m.G[i].resize((size_t)rows * dmax);
+        m.Gb[i].resize((size_t)(rows * ld8(dmax)));
+        m.GT[i].resize((size_t)(dmax * ld8(rows)));
+    }
+    m.loss.resize(LOSS_BLOCKS);
 }
 
-// Forward pass on Hb[0] (rows x dims[0]); Z[3] holds the output y.
-void forward(Context &c, Mlp &m, int rows) {
+// BF16 copies of the weights of layer i, also transposed
+void refresh_weights(Context &c, Mlp &m, int i) {
+    to_bf16(c, m.dims[i + 1], m.dims[i], m.W[i].p, (const float *)nullptr, m.Wb[i].p, m.WTb[i].p);
+}
+
+// Forward pass on Hb[0] (rows x dims[0]); Z[3] holds the output y. train: also the transposed
+// activations that the backward pass reads.
+void forward(Context &c, Mlp &m, int rows, bool train) {
     for (int i = 0; i < 4; ++i) {
         const bool last = i == 3;
-        gemm(c, m, rows, m.dims[i + 1], m.dims[i], m.Hb[i].p, m.dims[i], 1, m.Wb[i].p, m.dims[i], 1, m.Z[i].p,
-             m.dims[i + 1], last ? EPI_BIAS : EPI_BIAS_RELU, m.b[i].p, nullptr, last ? nullptr : m.Hb[i + 1].p);
+        const int din = m.dims[i], dout = m.dims[i + 1];
+        GemmOut o{m.Z[i].p, dout, last ? EPI_BIAS : EPI_BIAS_RELU, m.b[i].p, nullptr, nullptr, nullptr, ld8(dout), ld8(rows)};
+        if (!last) {
+            o.H = m.Hb[i + 1].p;
+            o.HT = train ? m.HT[i + 1].p : nullptr;
+        }
+        gemm(c, m, rows, dout, din, m.Hb[i].p, ld8(din), m.Wb[i].p, ld8(din), o);
     }
 }
 
-// Loss and gradients (into gW, gb) for targets T (rows x dims[4], float). Returns loss on device.
+// Gradients (into m.grad) and the loss's partial sums for targets T (rows x dims[4], float).
 void backward(Context &c, Mlp &m, int rows, const float *T) {
-    const int tb = 256;
-    BEM_CUDA(cudaMemsetAsync(m.loss.p, 0, sizeof(float), c.stream));
-    int64_t no = (int64_t)rows * m.dims[4];
-    k_loss_grad<<<std::min<int64_t>(div_up(no, tb), 512), tb, 0, c.stream>>>(no, rows, m.Z[3].p, T, m.G.p, m.Gb.p,
-                                                                              m.loss.p);
+    int cur = 0;
+    k_loss_grad<<<LOSS_BLOCKS, 256, 0, c.stream>>>(rows, m.dims[4], m.Z[3].p, T, m.G[0].p, m.Gb[0].p, ld8(m.dims[4]),
+                                                   m.GT[0].p, ld8(rows), m.loss.p);
     BEM_LAUNCH_CHECK();
-    for (int i = 3; i >= 0; --i) {
+    for (int i = 3; i >= 0; --i, cur ^= 1) {
         const int dout = m.dims[i + 1], din = m.dims[i];
-        // dW_i = G^T H_i  [dout x din]: A(o, r) = G[r*dout + o], B(k, r) = H_i[r*din + k]
-        gemm(c, m, dout, din, rows, m.Gb.p, 1, dout, m.Hb[i].p, 1, din, m.gW[i].p, din, EPI_STORE, nullptr, nullptr,
-             nullptr);
-        k_colsum<<<div_up(dout, 128), 128, 0, c.stream>>>(rows, dout, m.G.p, m.gb[i].p);
+        // dW_i = G^T H_i  [dout x din], summed over the rows
+        gemm(c, m, dout, din, rows, m.GT[cur].p, ld8(rows), m.HT[i].p, ld8(rows),
+             GemmOut{m.gW(i), din, EPI_STORE, nullptr, nullptr, nullptr, nullptr, 0, 0});
+        k_colsum<<<div_up(dout, 32), 1024, 0, c.stream>>>(rows, dout, m.G[cur].p, m.gb(i));
         BEM_LAUNCH_CHECK();
-        if (i > 0) {
-            // G_prev = (G W_i) masked by Z_{i-1} > 0: A(r, o) = G[r*dout + o], B(k, o) = W_i[o*din + k]
-            gemm(c, m, rows, din, dout, m.Gb.p, dout, 1, m.Wb[i].p, 1, din, m.G.p, din, EPI_RELU_MASK, nullptr,
-                 m.Z[i - 1].p, m.Gb.p);
-        }
+        if (i > 0)  // G_prev = (G W_i) masked by Z_{i-1} > 0
+            gemm(c, m, rows, din, dout, m.Gb[cur].p, ld8(dout), m.WTb[i].p, ld8(dout),
+                 GemmOut{m.G[cur ^ 1].p, din, EPI_RELU_MASK, nullptr, m.Z[i - 1].p, m.Gb[cur ^ 1].p, m.GT[cur ^ 1].p,
+                         ld8(din), ld8(rows)});
     }
+}
+
+// The loss of the last backward pass (its partial sums, in order) after everything queued; fails when a
+// product's wait ran out.
+float read_loss(Context &c, Mlp &m) {
+    float *h = m.hloss.get(LOSS_BLOCKS + 1);
+    BEM_CUDA(cudaMemcpyAsync(h, m.loss.p, LOSS_BLOCKS * sizeof(float), cudaMemcpyDeviceToHost, c.stream));
+    BEM_CUDA(cudaMemcpyAsync(h + LOSS_BLOCKS, m.err.p, sizeof(int), cudaMemcpyDeviceToHost, c.stream));
+    BEM_CUDA(cudaStreamSynchronize(c.stream));
+    int bad;
+    std::memcpy(&bad, h + LOSS_BLOCKS, sizeof(int));
+    if (bad) fail(BEM_ERR_TIMEOUT, "tensor-core GEMM wait ran out");
+    double s = 0.0;
+    for (int i = 0; i < LOSS_BLOCKS; ++i) s += h[i];
+    return (float)s;
 }
 
 void check_err(Context &c, Mlp &m) {
@@ -443,19 +602,22 @@ void mlp_init(Context &c, int hidden, int lmax, uint64_t seed, const double *xyz
         std::vector<float> w(nw), bz(dims[i + 1], 0.f);
         const double sc = std::sqrt(2.0 / dims[i]) * (i == 3 ? 0.1 : 1.0);
         for (auto &x : w) x = (float)(nd(rng) * sc);
-        for (auto *bf : {&m.W[i], &m.mW[i], &m.vW[i], &m.gW[i]}) bf->resize(nw);
-        for (auto *bf : {&m.b[i], &m.mb[i], &m.vb[i], &m.gb[i]}) bf->resize(dims[i + 1]);
-        m.Wb[i].resize(nw);
+        for (auto *bf : {&m.W[i], &m.mW[i], &m.vW[i]}) bf->resize(nw);
+        for (auto *bf : {&m.b[i], &m.mb[i], &m.vb[i]}) bf->resize(dims[i + 1]);
+        m.goff[2 * i + 1] = m.goff[2 * i] + nw;
+        m.goff[2 * i + 2] = m.goff[2 * i + 1] + dims[i + 1];
+        m.Wb[i].resize(dims[i + 1] * ld8(dims[i]));
+        m.WTb[i].resize(dims[i] * ld8(dims[i + 1]));
         BEM_CUDA(cudaMemcpyAsync(m.W[i].p, w.data(), nw * sizeof(float), cudaMemcpyHostToDevice, c.stream));
         BEM_CUDA(cudaMemcpyAsync(m.b[i].p, bz.data(), bz.size() * sizeof(float), cudaMemcpyHostToDevice, c.stream));
         BEM_CUDA(cudaMemsetAsync(m.mW[i].p, 0, nw * sizeof(float), c.stream));
         BEM_CUDA(cudaMemsetAsync(m.vW[i].p, 0, nw * sizeof(float), c.stream));
         BEM_CUDA(cudaMemsetAsync(m.mb[i].p, 0, dims[i + 1] * sizeof(float), c.stream));
         BEM_CUDA(cudaMemsetAsync(m.vb[i].p, 0, dims[i + 1] * sizeof(float), c.stream));
-        k_f2bf<<<div_up(nw, 256), 256, 0, c.stream>>>(nw, m.W[i].p, m.Wb[i].p);
-        BEM_LAUNCH_CHECK();
+        refresh_weights(c, m, i);
         BEM_CUDA(cudaStreamSynchronize(c.stream));  // host vectors go out of scope
     }
+    m.grad.resize(m.goff[8]);
     m.adam_t = 0;
     m.ns = 0;
     m.wrows = 0;
@@ -541,9 +703,8 @@ void mlp_before_solve(Context &c, const double *phi, double *q, bool uniform) {
                                  c.stream));
     }
     if (m.use && uniform) {
-        k_f2bf_scaled<<<div_up(M * 3 * P, 256), 256, 0, c.stream>>>(M * 3 * P, 3 * P, F.p, m.fscale.p, m.Hb[0].p);
-        BEM_LAUNCH_CHECK();
-        forward(c, m, (int)M);
+        to_bf16(c, (int)M, 3 * P, F.p, m.fscale.p, m.Hb[0].p, (__nv_bfloat16 *)nullptr);
+        forward(c, m, (int)M, false);
         k_sh_synth_add<<<(unsigned)M, 128, 0, c.stream>>>(M, voff.p, m.feat.shape_of.p, m.feat.g_off.p, P, m.feat.G.p,
                                                           m.Z[3].p, m.tscale.p, m.qprev.p, q);
         BEM_LAUNCH_CHECK();
@@ -588,34 +749,30 @@ double mlp_train(Context &c, int epochs, int batch, double lr) {
         int nb = 0;
         for (int64_t r0 = 0; r0 < m.ns; r0 += batch) {
             const int rows = (int)std::min<int64_t>(batch, m.ns - r0);
-            k_f2bf_scaled<<<div_up((int64_t)rows * 3 * P, 256), 256, 0, c.stream>>>(
-                (int64_t)rows * 3 * P, 3 * P, m.SF.p + r0 * 3 * P, m.fscale.p, m.Hb[0].p);
+            to_bf16(c, rows, 3 * P, m.SF.p + r0 * 3 * P, m.fscale.p, m.Hb[0].p, m.HT[0].p);
             k_div_cols<<<div_up((int64_t)rows * P, 256), 256, 0, c.stream>>>((int64_t)rows * P, P, m.ST.p + r0 * P,
                                                                              m.tscale.p, m.Tb.p);
             BEM_LAUNCH_CHECK();
-            forward(c, m, rows);
+            forward(c, m, rows, true);
             backward(c, m, rows, m.Tb.p);
             m.adam_t += 1;
             const float b1 = 0.9f, b2 = 0.999f;
             const float c1 = 1.f - std::pow(b1, (float)m.adam_t), c2 = 1.f - std::pow(b2, (float)m.adam_t);
             for (int i = 0; i < 4; ++i) {
                 int64_t nw = (int64_t)m.dims[i + 1] * m.dims[i];
-                k_adam<<<div_up(nw, 256), 256, 0, c.stream>>>(nw, m.W[i].p, m.gW[i].p, m.mW[i].p, m.vW[i].p, (float)lr,
-                                                               b1, b2, c1, c2, 1e-8f, m.Wb[i].p);
-                k_adam<<<div_up(m.dims[i + 1], 256), 256, 0, c.stream>>>(m.dims[i + 1], m.b[i].p, m.gb[i].p, m.mb[i].p,
-                                                                          m.vb[i].p, (float)lr, b1, b2, c1, c2, 1e-8f,
-                                                                          nullptr);
+                k_adam<<<div_up(nw, 256), 256, 0, c.stream>>>(nw, m.W[i].p, m.gW(i), m.mW[i].p, m.vW[i].p, (float)lr,
+                                                               b1, b2, c1, c2, 1e-8f, m.dims[i], m.Wb[i].p,
+                                                               ld8(m.dims[i]), m.WTb[i].p, ld8(m.dims[i + 1]));
+                k_adam<<<div_up(m.dims[i + 1], 256), 256, 0, c.stream>>>(m.dims[i + 1], m.b[i].p, m.gb(i), m.mb[i].p,
+                                                                          m.vb[i].p, (float)lr, b1, b2, c1, c2, 1e-8f, 1,
+                                                                          nullptr, 0, nullptr, 0);
                 BEM_LAUNCH_CHECK();
             }
-            float h = 0.f;
-            BEM_CUDA(cudaMemcpyAsync(&h, m.loss.p, sizeof(float), cudaMemcpyDeviceToHost, c.stream));
-            BEM_CUDA(cudaStreamSynchronize(c.stream));
-            tot += h;
+            tot += read_loss(c, m);
             ++nb;
         }
         last = tot / std::max(1, nb);
     }
-    check_err(c, m);
     return last;
 }
 
@@ -626,36 +783,16 @@ double mlp_loss_grad(Context &c, int B, const double *F, const double *T, double
     if (!m.ready) fail(BEM_ERR_NOT_BUILT, "bem_mlp_init has not been called");
     ensure_work(m, B);
     const int din = m.dims[0], dout = m.dims[4];
-    k_d2bf<<<div_up((int64_t)B * din, 256), 256, 0, c.stream>>>((int64_t)B * din, F, m.Hb[0].p);
+    const int64_t nt = (int64_t)B * dout, np = mlp_num_params(m);
+    to_bf16(c, B, din, F, (const float *)nullptr, m.Hb[0].p, m.HT[0].p);
+    m.Tb.resize((size_t)nt);
+    k_convert<double, float><<<std::min(div_up(nt, 256), 1024), 256, 0, c.stream>>>(nt, T, m.Tb.p);
     BEM_LAUNCH_CHECK();
-    DevBuf<float> Tf;
-    Tf.resize((size_t)B * dout);
-    std::vector<double> th((size_t)B * dout);
-    BEM_CUDA(cudaMemcpyAsync(th.data(), T, th.size() * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
-    BEM_CUDA(cudaStreamSynchronize(c.stream));
-    std::vector<float> tf(th.begin(), th.end());
-    BEM_CUDA(cudaMemcpyAsync(Tf.p, tf.data(), tf.size() * sizeof(float), cudaMemcpyHostToDevice, c.stream));
-    forward(c, m, B);
-    backward(c, m, B, Tf.p);
-    float h = 0.f;
-    BEM_CUDA(cudaMemcpyAsync(&h, m.loss.p, sizeof(float), cudaMemcpyDeviceToHost, c.stream));
-    int64_t off = 0;
-    for (int i = 0; i < 4; ++i) {
-        int64_t nw = (int64_t)m.dims[i + 1] * m.dims[i];
-        std::vector<float> a(nw), bb(m.dims[i + 1]);
-        BEM_CUDA(cudaMemcpyAsync(a.data(), m.gW[i].p, nw * sizeof(float), cudaMemcpyDeviceToHost, c.stream));
-        BEM_CUDA(cudaMemcpyAsync(bb.data(), m.gb[i].p, bb.size() * sizeof(float), cudaMemcpyDeviceToHost, c.stream));
-        BEM_CUDA(cudaStreamSynchronize(c.stream));
-        std::vector<double> ad(a.begin(), a.end()), bd(bb.begin(), bb.end());
-        BEM_CUDA(cudaMemcpyAsync(grads_dev + off, ad.data(), nw * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-        off += nw;
-        BEM_CUDA(cudaMemcpyAsync(grads_dev + off, bd.data(), bd.size() * sizeof(double), cudaMemcpyHostToDevice,
-                                 c.stream));
-        off += m.dims[i + 1];
-        BEM_CUDA(cudaStreamSynchronize(c.stream));
-    }
-    check_err(c, m);
-    return h;
+    forward(c, m, B, true);
+    backward(c, m, B, m.Tb.p);
+    k_convert<float, double><<<std::min(div_up(np, 256), 1024), 256, 0, c.stream>>>(np, m.grad.p, grads_dev);
+    BEM_LAUNCH_CHECK();
+    return read_loss(c, m);
 }
 
 // Forward only: Y [B][dout] (device FP64) from F [B][din] (device FP64).
@@ -664,15 +801,11 @@ void mlp_forward(Context &c, int B, const double *F, double *Y) {
     if (!m.ready) fail(BEM_ERR_NOT_BUILT, "bem_mlp_init has not been called");
     ensure_work(m, B);
     const int din = m.dims[0], dout = m.dims[4];
-    k_d2bf<<<div_up((int64_t)B * din, 256), 256, 0, c.stream>>>((int64_t)B * din, F, m.Hb[0].p);
+    to_bf16(c, B, din, F, (const float *)nullptr, m.Hb[0].p, (__nv_bfloat16 *)nullptr);
+    forward(c, m, B, false);
+    const int64_t ny = (int64_t)B * dout;
+    k_convert<float, double><<<std::min(div_up(ny, 256), 1024), 256, 0, c.stream>>>(ny, m.Z[3].p, Y);
     BEM_LAUNCH_CHECK();
-    forward(c, m, B);
-    std::vector<float> y((size_t)B * dout);
-    BEM_CUDA(cudaMemcpyAsync(y.data(), m.Z[3].p, y.size() * sizeof(float), cudaMemcpyDeviceToHost, c.stream));
-    BEM_CUDA(cudaStreamSynchronize(c.stream));
-    std::vector<double> yd(y.begin(), y.end());
-    BEM_CUDA(cudaMemcpyAsync(Y, yd.data(), yd.size() * sizeof(double), cudaMemcpyHostToDevice, c.stream));
-    BEM_CUDA(cudaStreamSynchronize(c.stream));
     check_err(c, m);
 }
 
@@ -704,8 +837,7 @@ void mlp_set_params(Context &c, const double *in) {
         off += m.dims[i + 1];
         BEM_CUDA(cudaMemcpyAsync(m.W[i].p, a.data(), nw * sizeof(float), cudaMemcpyHostToDevice, c.stream));
         BEM_CUDA(cudaMemcpyAsync(m.b[i].p, bb.data(), bb.size() * sizeof(float), cudaMemcpyHostToDevice, c.stream));
-        k_f2bf<<<div_up(nw, 256), 256, 0, c.stream>>>(nw, m.W[i].p, m.Wb[i].p);
-        BEM_LAUNCH_CHECK();
+        refresh_weights(c, m, i);
         BEM_CUDA(cudaStreamSynchronize(c.stream));
     }
 }
