@@ -26,6 +26,11 @@
 // unrelated to the Krylov space, so that a cycle whose estimate met the tolerance could fail the
 // check and restart for no gain; r_0 - A d agrees with the estimate to the rounding of A d, and
 // the next cycle starts from it.
+//
+// Up to about 300000 unknowns the vectors sit in L2 and an iteration's eleven small launches cost
+// more than their work (solve of 642 unknowns, FP64 direct: 3.85 ms, 1.94 ms with it; 160200 unknowns: 15.9 and 14.3 ms). There one cooperative kernel
+// (k_arnoldi) runs the whole Arnoldi step: every CTA keeps its slice of the work vector in shared
+// memory through both projections, and the CTAs join their sums at three grid barriers.
 #include "internal.h"
 
 #include <algorithm>
@@ -35,17 +40,20 @@ namespace bem {
 namespace {
 
 constexpr int RED_THREADS = 256;
-constexpr int RED_BLOCKS = 152 * 3;  // fixed grid: fixed summation order
+constexpr int RED_BLOCKS = 152 * 3;  // most blocks of a reduction
+// blocks of a reduction over N elements: a function of N alone, so the summation order is fixed; one
+// block per 512 elements below the cap (456 blocks of two elements took 20 us at N = 642)
+int red_blocks(int64_t N) { return (int)std::min<int64_t>(RED_BLOCKS, (N + 511) / 512); }
 constexpr int RED_JB = 8;            // basis vectors per pass over w
 
-// partial[j * RED_BLOCKS + block] = sum over the block's slice of V_j . w, j = 0..nv-1.
+// partial[j * gridDim.x + block] = sum over the block's slice of V_j . w, j = 0..nv-1.
 // Each pass reads w once for RED_JB vectors (independent accumulators), then reduces the
 // RED_JB sums across the block in a fixed order.
 __global__ void __launch_bounds__(RED_THREADS) k_multidot(int nv, int64_t N, const double *__restrict__ V,
                                                           size_t ldv, const double *__restrict__ w,
                                                           double *__restrict__ partial) {
     __shared__ double red[RED_THREADS / 32][RED_JB];
-    const int64_t chunk = (N + RED_BLOCKS - 1) / RED_BLOCKS;
+    const int64_t chunk = (N + gridDim.x - 1) / gridDim.x;
     const int64_t i0 = blockIdx.x * chunk, i1 = (N < i0 + chunk) ? N : i0 + chunk;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int j0 = 0; j0 < nv; j0 += RED_JB) {
@@ -70,17 +78,17 @@ __global__ void __launch_bounds__(RED_THREADS) k_multidot(int nv, int64_t N, con
         if (threadIdx.x < nj) {
             double t = 0.0;
             for (int k = 0; k < RED_THREADS / 32; ++k) t += red[k][threadIdx.x];
-            partial[(size_t)(j0 + threadIdx.x) * RED_BLOCKS + blockIdx.x] = t;
+            partial[(size_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
         }
         __syncthreads();
     }
 }
 
 // out[j] = (accumulate ? out[j] : 0) + sum_b partial[j][b]  (one block per j; fixed order)
-__global__ void k_dot_final(const double *__restrict__ partial, double *__restrict__ out, int accumulate) {
+__global__ void k_dot_final(int nb, const double *__restrict__ partial, double *__restrict__ out, int accumulate) {
     __shared__ double red[RED_THREADS];
     double s = 0.0;
-    for (int b = threadIdx.x; b < RED_BLOCKS; b += RED_THREADS) s += partial[(size_t)blockIdx.x * RED_BLOCKS + b];
+    for (int b = threadIdx.x; b < nb; b += RED_THREADS) s += partial[(size_t)blockIdx.x * nb + b];
     red[threadIdx.x] = s;
     __syncthreads();
     for (int k = RED_THREADS / 2; k > 0; k >>= 1) {
@@ -111,13 +119,13 @@ __device__ __forceinline__ void two_sum_acc(float &s, float &c, float p, float e
     s = t;
 }
 
-// k_multidot with an FP32 basis: partial[j * RED_BLOCKS + block] = the block's share of V_j . w,
+// k_multidot with an FP32 basis: partial[j * gridDim.x + block] = the block's share of V_j . w,
 // compensated FP32 per thread, the (sum, compensation) pairs joined in a fixed order
 __global__ void __launch_bounds__(RED_THREADS) k_multidot32(int nv, int64_t N, const float *__restrict__ V,
                                                             size_t ldv, const double *__restrict__ w,
                                                             double *__restrict__ partial) {
     __shared__ float red[2][RED_THREADS / 32][RED_JB];
-    const int64_t chunk = (N + RED_BLOCKS - 1) / RED_BLOCKS;
+    const int64_t chunk = (N + gridDim.x - 1) / gridDim.x;
     const int64_t i0 = blockIdx.x * chunk, i1 = (N < i0 + chunk) ? N : i0 + chunk;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int j0 = 0; j0 < nv; j0 += RED_JB) {
@@ -153,7 +161,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_multidot32(int nv, int64_t N, c
         if (threadIdx.x < nj) {
             double t = 0.0;
             for (int k = 0; k < RED_THREADS / 32; ++k) t += (double)red[0][k][threadIdx.x] + (double)red[1][k][threadIdx.x];
-            partial[(size_t)(j0 + threadIdx.x) * RED_BLOCKS + blockIdx.x] = t;
+            partial[(size_t)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
         }
         __syncthreads();
     }
@@ -219,23 +227,21 @@ __global__ void k_cycle_start(int m, const double *__restrict__ beta, double *__
 
 // Column k of the Hessenberg matrix (h[0..k] from Gram-Schmidt, hk1 = h[k+1]) through the
 // previous rotations, a new rotation that zeroes h[k+1], and the rotated right-hand side.
-// H is stored column-major with leading dimension m+1. resid[0] = |g[k+1]|.
-__global__ void k_givens(int k, int m, const double *__restrict__ h, double *__restrict__ H,
-                         double *__restrict__ cs, double *__restrict__ sn, double *__restrict__ g,
-                         double *__restrict__ resid) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// H is stored column-major with leading dimension m+1. resid[0] = |g[k+1]|. One thread.
+__device__ void givens_step(int k, int m, const double *h, double *H, double *cs, double *sn, double *g, double *resid) {
     double *col = H + (size_t)k * (m + 1);
-    for (int i = 0; i <= k + 1; ++i) col[i] = h[i];
+    double a = h[0];  // entry j, rotated by the rotations before
     for (int j = 0; j < k; ++j) {
-        double t = cs[j] * col[j] + sn[j] * col[j + 1];
-        col[j + 1] = -sn[j] * col[j] + cs[j] * col[j + 1];
-        col[j] = t;
+        const double b = h[j + 1], cj = cs[j], sj = sn[j];
+        col[j] = cj * a + sj * b;
+        a = -sj * a + cj * b;
     }
-    double d = hypot(col[k], col[k + 1]);
+    const double b = h[k + 1];
+    const double d = hypot(a, b);
     double c = 1.0, s = 0.0;
     if (d != 0.0) {
-        c = col[k] / d;
-        s = col[k + 1] / d;
+        c = a / d;
+        s = b / d;
     }
     cs[k] = c;
     sn[k] = s;
@@ -244,6 +250,201 @@ __global__ void k_givens(int k, int m, const double *__restrict__ h, double *__r
     g[k + 1] = -s * g[k];
     g[k] = c * g[k];
     resid[0] = fabs(g[k + 1]);
+}
+__global__ void k_givens(int k, int m, const double *__restrict__ h, double *__restrict__ H,
+                         double *__restrict__ cs, double *__restrict__ sn, double *__restrict__ g,
+                         double *__restrict__ resid) {
+    if (threadIdx.x == 0 && blockIdx.x == 0) givens_step(k, m, h, H, cs, sn, g, resid);
+}
+
+// ------------------------------------------------------------------------------ fused Arnoldi step
+constexpr int AR_THREADS = 512;
+constexpr int AR_SLICE = 2048;             // elements of one CTA at most (its shared-memory slice)
+constexpr int AR_MIN = 64;                 // ... and at least, where that leaves SMs without a share
+constexpr long long kArnoldiWait = 1ll << 22;  // polls before a grid barrier gives up
+
+struct ArnoldiArgs {
+    int k, m;                 // w = A P v_k; basis vectors 0..k are stored, k + 1 is written
+    int64_t N;
+    const double *w;
+    double *partial;          // [nv][CTAs]
+    double *h;                // [k + 2] out: the Hessenberg column, h[k + 1] = |w|
+    double *H, *cs, *sn, *g;
+    double *res;              // res[0] = residual estimate, res[1] = 1 when a barrier gave up
+    unsigned *bar;            // arrivals at grid barriers since the solve began
+    unsigned base;            // ... before this launch
+    double *v64;              // FP32 basis: the exact copy of v_{k+1} for the product
+};
+
+// All CTAs of the grid (co-resident: a cooperative launch) have arrived. false: gave up.
+__device__ __forceinline__ bool grid_barrier(unsigned *bar, unsigned target, int *s_ok) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(bar, 1u);
+        int ok = 0;
+        for (long long it = 0; it < kArnoldiWait; ++it) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+            if ((int)(v - target) >= 0) {
+                ok = 1;
+                break;
+            }
+        }
+        *s_ok = ok;
+    }
+    __syncthreads();
+    return *s_ok != 0;
+}
+
+// sum over the block (fixed order); every thread gets it
+__device__ __forceinline__ double block_sum(double v, double *red) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    double t = 0.0;
+    for (int i = 0; i < AR_THREADS / 32; ++i) t += red[i];
+    return t;
+}
+
+// One Arnoldi step: classical Gram-Schmidt twice, the norm, v_{k+1}, the Hessenberg column and its
+// rotation. VT = float: compensated FP32 products with the (hi, lo) split of w, as k_multidot32.
+template <class VT>
+__global__ void __launch_bounds__(AR_THREADS) k_arnoldi(ArnoldiArgs a, VT *V) {
+    constexpr bool F32 = sizeof(VT) == 4;
+    __shared__ double sw[AR_SLICE];
+    __shared__ float2 swf[F32 ? AR_SLICE : 1];
+    __shared__ double sh[2][128];   // h of the two passes
+    __shared__ float2 shf[F32 ? 128 : 1];
+    __shared__ double red[AR_THREADS / 32];
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, nv = a.k + 1, G = gridDim.x;
+    const int64_t N = a.N, per = (N + G - 1) / G, i0 = blockIdx.x * per;
+    const int n = (int)(i0 >= N ? 0 : (N - i0 < per ? N - i0 : per));
+    for (int e = tid; e < n; e += AR_THREADS) sw[e] = a.w[i0 + e];
+    // lanes per basis vector: the block shared by nv vectors, 4 to 32 lanes each
+    int LJ = 4;
+    while (LJ < 32 && 2 * LJ * nv <= AR_THREADS) LJ *= 2;
+    const int sub = tid & (LJ - 1), grp = tid / LJ, ng = AR_THREADS / LJ;
+    unsigned target = a.base;
+    bool ok = true;
+    for (int pass = 0; pass < 2; ++pass) {
+        __syncthreads();
+        if (F32) {
+            for (int e = tid; e < n; e += AR_THREADS) {
+                const float h = (float)sw[e];
+                swf[e] = make_float2(h, (float)(sw[e] - (double)h));
+            }
+            __syncthreads();
+        }
+        // shares of V_j . w
+        for (int j0 = 0; j0 < nv; j0 += ng) {  // uniform: the shuffles below need every lane
+            const int j = j0 + grp;
+            const VT *vj = V + (size_t)(j < nv ? j : 0) * N + i0;
+            double t;
+            if constexpr (F32) {
+                float s = 0.f, c = 0.f;
+                if (j < nv) {
+#pragma unroll 8
+                    for (int e = sub; e < n; e += LJ) {
+                        const float v = vj[e];
+                        const float2 w = swf[e];
+                        const float p = v * w.x;
+                        two_sum_acc(s, c, p, fmaf(v, w.y, fmaf(v, w.x, -p)));
+                    }
+                }
+                for (int o = LJ / 2; o > 0; o >>= 1) {
+                    const float os = __shfl_xor_sync(0xffffffffu, s, o), oc = __shfl_xor_sync(0xffffffffu, c, o);
+                    two_sum_acc(s, c, os, oc);
+                }
+                t = (double)s + (double)c;
+            } else {
+                t = 0.0;
+                if (j < nv) {
+#pragma unroll 8
+                    for (int e = sub; e < n; e += LJ) t = fma(vj[e], sw[e], t);
+                }
+                for (int o = LJ / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            }
+            if (sub == 0 && j < nv) a.partial[(size_t)j * G + blockIdx.x] = t;
+        }
+        target += G;
+        ok = grid_barrier(a.bar, target, &s_ok);
+        if (!ok) break;
+        // every CTA forms h from the shares, in the same order
+        for (int j0 = 0; j0 < nv; j0 += ng) {
+            const int j = j0 + grp;
+            double t = 0.0;
+            if (j < nv)
+                for (int b = sub; b < G; b += LJ) t += __ldcg(a.partial + (size_t)j * G + b);
+            for (int o = LJ / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+            if (sub == 0 && j < nv) {
+                sh[pass][j] = t;
+                if (F32) {
+                    const float hh = (float)t;
+                    shf[j] = make_float2(hh, (float)(t - (double)hh));
+                }
+            }
+        }
+        __syncthreads();
+        // w -= V h
+        for (int e = tid; e < n; e += AR_THREADS) {
+            const VT *v = V + i0 + e;
+            if constexpr (F32) {
+                float s = 0.f, c = 0.f;
+#pragma unroll 8
+                for (int j = 0; j < nv; ++j) {
+                    const float vv = v[(size_t)j * N];
+                    const float2 h = shf[j];
+                    const float p = h.x * vv;
+                    two_sum_acc(s, c, p, fmaf(h.y, vv, fmaf(h.x, vv, -p)));
+                }
+                sw[e] -= (double)s + (double)c;
+            } else {
+                double acc = 0.0;
+#pragma unroll 8
+                for (int j = 0; j < nv; ++j) acc = fma(sh[pass][j], v[(size_t)j * N], acc);
+                sw[e] -= acc;
+            }
+        }
+        // the shares of the next pass (or of the norm) reuse `partial`: every CTA has read these by the
+        // next barrier only, so they alternate between two halves
+        a.partial += (size_t)128 * G;
+    }
+    double nrm2 = 0.0;
+    if (ok) {
+        double t = 0.0;
+        for (int e = tid; e < n; e += AR_THREADS) t = fma(sw[e], sw[e], t);
+        t = block_sum(t, red);
+        if (tid == 0) a.partial[blockIdx.x] = t;
+        target += G;
+        ok = grid_barrier(a.bar, target, &s_ok);
+    }
+    if (!ok) {  // uniform in the block
+        if (tid == 0) a.res[1] = 1.0;
+        return;
+    }
+    {
+        double t = 0.0;
+        for (int b = tid; b < G; b += AR_THREADS) t += __ldcg(a.partial + b);
+        nrm2 = block_sum(t, red);
+    }
+    const double nn = sqrt(fmax(nrm2, 0.0)), inv = nn > 0.0 ? 1.0 / nn : 0.0;
+    VT *vn = V + (size_t)nv * N + i0;
+    for (int e = tid; e < n; e += AR_THREADS) {
+        const VT f = (VT)(sw[e] * inv);
+        vn[e] = f;
+        if (F32) a.v64[i0 + e] = (double)f;
+    }
+    if (blockIdx.x == 0) {
+        for (int j = tid; j < nv; j += AR_THREADS) a.h[j] = sh[0][j] + sh[1][j];
+        if (tid == 0) a.h[nv] = nn;
+        __syncthreads();
+        if (tid == 0) givens_step(a.k, a.m, a.h, a.H, a.cs, a.sn, a.g, a.res);
+    }
 }
 
 // z = d .* v (right preconditioning by the inverse diagonal)
@@ -268,14 +469,14 @@ __global__ void k_backsolve(int kk, int m, const double *__restrict__ H, const d
 struct Vec {
     Context &c;
     int64_t N;
-    int grid;
-    explicit Vec(Context &cc) : c(cc), N(cc.N) { grid = std::min<int64_t>(div_up(N, 256), 152 * 8); }
+    int grid, rb;
+    explicit Vec(Context &cc) : c(cc), N(cc.N), rb(red_blocks(cc.N)) { grid = std::min<int64_t>(div_up(N, 256), 152 * 8); }
     // out[0..nv) = V_j . w (deterministic)
     void dots(int nv, const double *V, size_t ldv, const double *w, double *out, int accumulate) {
         PhaseScope ps(c, PH_GMRES);
-        k_multidot<<<RED_BLOCKS, RED_THREADS, 0, c.stream>>>(nv, N, V, ldv, w, c.partial.p);
+        k_multidot<<<rb, RED_THREADS, 0, c.stream>>>(nv, N, V, ldv, w, c.partial.p);
         BEM_LAUNCH_CHECK();
-        k_dot_final<<<nv, RED_THREADS, 0, c.stream>>>(c.partial.p, out, accumulate);
+        k_dot_final<<<nv, RED_THREADS, 0, c.stream>>>(rb, c.partial.p, out, accumulate);
         BEM_LAUNCH_CHECK();
     }
     void multiaxpy(int nv, const double *V, size_t ldv, const double *h, double sign, double *w) {
@@ -286,9 +487,9 @@ struct Vec {
     // the same with the FP32 basis
     void dots(int nv, const float *V, size_t ldv, const double *w, double *out, int accumulate) {
         PhaseScope ps(c, PH_GMRES);
-        k_multidot32<<<RED_BLOCKS, RED_THREADS, 0, c.stream>>>(nv, N, V, ldv, w, c.partial.p);
+        k_multidot32<<<rb, RED_THREADS, 0, c.stream>>>(nv, N, V, ldv, w, c.partial.p);
         BEM_LAUNCH_CHECK();
-        k_dot_final<<<nv, RED_THREADS, 0, c.stream>>>(c.partial.p, out, accumulate);
+        k_dot_final<<<nv, RED_THREADS, 0, c.stream>>>(rb, c.partial.p, out, accumulate);
         BEM_LAUNCH_CHECK();
     }
     void multiaxpy(int nv, const float *V, size_t ldv, const double *h, double sign, double *w) {
@@ -318,6 +519,15 @@ double read_scalar(Context &c, const double *dev) {
     BEM_CUDA(cudaMemcpyAsync(h, dev, sizeof(double), cudaMemcpyDeviceToHost, c.stream));
     BEM_CUDA(cudaStreamSynchronize(c.stream));
     return *h;
+}
+
+// the fused step's residual estimate and its barrier status, in one copy
+double read_estimate(Context &c, const double *dev) {
+    double *h = c.hscal.get(2);
+    BEM_CUDA(cudaMemcpyAsync(h, dev, 2 * sizeof(double), cudaMemcpyDeviceToHost, c.stream));
+    BEM_CUDA(cudaStreamSynchronize(c.stream));
+    if (h[1] != 0.0) fail(BEM_ERR_TIMEOUT, "a grid barrier of the Arnoldi step ran out");
+    return h[0];
 }
 
 }  // namespace
@@ -351,16 +561,23 @@ void gmres_solve(Context &c, const double *b, double *x, int *iters_out, double 
     };
     c.wv.resize(N);
     c.rv.resize(N);
-    c.partial.resize((size_t)(m + 2) * RED_BLOCKS);
+    // fused Arnoldi step: CTAs of at least AR_MIN and at most AR_SLICE elements, at most one per SM
+    const int ar_ctas = (int)std::min<int64_t>(c.num_sms, (N + AR_MIN - 1) / AR_MIN);
+    const bool fused = N <= (int64_t)c.num_sms * AR_SLICE;
+    c.partial.resize(std::max((size_t)(m + 2) * RED_BLOCKS, fused ? (size_t)(2 * 128 + 1) * ar_ctas : 0));
+    c.bar.resize(1);
+    if (fused) BEM_CUDA(cudaMemsetAsync(c.bar.p, 0, sizeof(unsigned), c.stream));
+    unsigned bar_base = 0;
     c.hcol.resize(m + 2);
     c.hmat.resize((size_t)(m + 1) * (m + 1));
     c.givens.resize(2 * (m + 1));
     c.gvec.resize(m + 2);
     c.yvec.resize(m + 1);
-    c.scal.resize(8);
+    c.scal.resize(16);
     double *cs = c.givens.p, *sn = c.givens.p + (m + 1);
     double *d_bn2 = c.scal.p, *d_beta2 = c.scal.p + 1, *d_beta = c.scal.p + 2, *d_res = c.scal.p + 3;
-    double *d_tmp = c.scal.p + 4;
+    double *d_tmp = c.scal.p + 4, *d_est = c.scal.p + 8;  // d_est: estimate, barrier error
+    if (fused) BEM_CUDA(cudaMemsetAsync(d_est, 0, 2 * sizeof(double), c.stream));
 
     c.res_hist.clear();
     vec.dots(1, b, N, b, d_bn2, 0);
@@ -413,21 +630,34 @@ void gmres_solve(Context &c, const double *b, double *x, int *iters_out, double 
                 apply_full(c, 1.0, vk, 0.0, nullptr, c.wv.p);
             }
             ++mvps;
-            // classical Gram-Schmidt, twice
-            project(k + 1, c.wv.p, c.hcol.p);
-            update(k + 1, c.hcol.p, -1.0, c.wv.p);
-            project(k + 1, c.wv.p, c.yvec.p);  // second pass into y (free here)
-            update(k + 1, c.yvec.p, -1.0, c.wv.p);
-            k_axpby<<<1, 128, 0, c.stream>>>(k + 1, 1.0, c.yvec.p, 1.0, c.hcol.p);
-            BEM_LAUNCH_CHECK();
-            vec.dots(1, c.wv.p, N, c.wv.p, d_tmp, 0);
-            // h[k+1] = |w|, v_{k+1} = w / |w|
-            vec.normalise(c.wv.p, d_tmp, c.V.p, b32 ? c.V32.p : nullptr, k + 1, c.vk64.p, c.hcol.p + k + 1);
-            k_givens<<<1, 1, 0, c.stream>>>(k, m, c.hcol.p, c.hmat.p, cs, sn, c.gvec.p, d_res);
-            BEM_LAUNCH_CHECK();
+            if (fused) {
+                PhaseScope ps(c, PH_GMRES);
+                ArnoldiArgs ar{k, m, N, c.wv.p, c.partial.p, c.hcol.p, c.hmat.p, cs, sn, c.gvec.p, d_est, c.bar.p, bar_base,
+                               c.vk64.p};
+                double *Vd = c.V.p;
+                float *Vf = c.V32.p;
+                void *args[2] = {&ar, b32 ? (void *)&Vf : (void *)&Vd};
+                BEM_CUDA(cudaLaunchCooperativeKernel(b32 ? (const void *)k_arnoldi<float> : (const void *)k_arnoldi<double>,
+                                                     dim3(ar_ctas), dim3(AR_THREADS), args, 0, c.stream));
+                BEM_LAUNCH_CHECK();
+                bar_base += 3u * ar_ctas;
+            } else {
+                // classical Gram-Schmidt, twice
+                project(k + 1, c.wv.p, c.hcol.p);
+                update(k + 1, c.hcol.p, -1.0, c.wv.p);
+                project(k + 1, c.wv.p, c.yvec.p);  // second pass into y (free here)
+                update(k + 1, c.yvec.p, -1.0, c.wv.p);
+                k_axpby<<<1, 128, 0, c.stream>>>(k + 1, 1.0, c.yvec.p, 1.0, c.hcol.p);
+                BEM_LAUNCH_CHECK();
+                vec.dots(1, c.wv.p, N, c.wv.p, d_tmp, 0);
+                // h[k+1] = |w|, v_{k+1} = w / |w|
+                vec.normalise(c.wv.p, d_tmp, c.V.p, b32 ? c.V32.p : nullptr, k + 1, c.vk64.p, c.hcol.p + k + 1);
+                k_givens<<<1, 1, 0, c.stream>>>(k, m, c.hcol.p, c.hmat.p, cs, sn, c.gvec.p, d_res);
+                BEM_LAUNCH_CHECK();
+            }
             ++iters;
             kk = k + 1;
-            double est = read_scalar(c, d_res) / bnorm;
+            double est = (fused ? read_estimate(c, d_est) : read_scalar(c, d_res)) / bnorm;
             c.res_hist.push_back(est);
             if (est <= tol || iters >= maxit) break;
         }
