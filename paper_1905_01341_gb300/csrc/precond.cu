@@ -26,7 +26,11 @@
 #include "internal.h"
 #include "tcgen05.cuh"
 
+#include <cooperative_groups.h>
+
 #include <cmath>
+
+namespace cg = cooperative_groups;
 
 namespace bem {
 namespace {
@@ -203,20 +207,28 @@ __global__ void __launch_bounds__(BP_THREADS) k_bp_apply(int n, const T *__restr
 
 // Tensor-core form of the block product (mixed precision). For one shape with n vertices and
 // nb bubbles, Z (n x nb) = Inv (n x n) Y (n x nb) with D = A B^T on tcgen05: A = Inv (row r is
-// K-contiguous), B = Y^T (bubble b's segment is K-contiguous), M = 128 rows, N = 256 bubbles
-// per tile, K in steps of 16. Both operands are stored in global memory already in the
+// K-contiguous), B = Y^T (bubble b's segment is K-contiguous), M = 128 rows, NT = 64, 128 or 256
+// bubbles per tile, K in steps of 16. Both operands are stored in global memory already in the
 // canonical K-major blocks of one K step, [piece][K step][rows][16], so that every stage is
 // six contiguous bulk copies (the TMA engine): A from the table split once per build, B from
 // the right-hand side split once per application (k_bp_split_y). Thread 0 fills the stages,
 // thread 32 issues six MMAs per stage (the small cross terms first) and commits each stage to
 // its "empty" barrier; every wait is bounded and raises the error flag when it runs out. The
-// epilogue reads the accumulator tile from TMEM (warp w: lanes 32 (w % 4) .. + 31 = rows,
-// columns 128 (w / 4) .. + 127 = bubbles) and writes z_b[r] = s_b D[r][b] in FP64, 32
-// consecutive rows of one bubble per store instruction.
+// accumulator tile is read from TMEM (warp w: lanes 32 (w % 4) .. + 31 = rows, columns
+// NT/2 (w / 4) .. = bubbles) and z_b[r] = s_b D[r][b] written in FP64, consecutive rows of one
+// bubble together.
+//
+// With few bubbles a shape has few tiles (21 of 128 x 256 for 50 bubbles of 2562 vertices, each
+// walking 161 K steps alone: 100 us an application of a 2562-vertex and a 642-vertex shape, 35 us with the split). The K steps are then shared by the CTAs of a cluster, whose sums
+// are joined through distributed shared memory in rank order, and the tile is no wider than the
+// bubbles need.
 constexpr int BPC_M = 128, BPC_N = 256, BPC_STAGES = 4, BPC_THREADS = 256;
-constexpr uint32_t BPC_A_PIECE = BPC_M * TC_K * 2, BPC_B_PIECE = BPC_N * TC_K * 2;
-constexpr uint32_t BPC_STAGE = 3 * (BPC_A_PIECE + BPC_B_PIECE);
-constexpr size_t BPC_SMEM = (size_t)BPC_STAGES * BPC_STAGE + 2 * BPC_STAGES * 8 + 16 + 1024;
+constexpr uint32_t BPC_A_PIECE = BPC_M * TC_K * 2;
+__host__ __device__ constexpr uint32_t bpc_stage(int NT) { return 3 * (BPC_A_PIECE + (uint32_t)NT * TC_K * 2); }
+constexpr size_t bpc_smem(int NT) { return (size_t)BPC_STAGES * bpc_stage(NT) + 2 * BPC_STAGES * 8 + 16 + 1024; }
+constexpr int BPC_RED = BPC_M + 4;  // row pitch of the split sums [bubble][BPC_RED], in the free stages
+static_assert(BPC_N * BPC_RED * 4 <= BPC_STAGES * bpc_stage(BPC_N) && 64 * BPC_RED * 4 <= BPC_STAGES * bpc_stage(64),
+              "the split sums reuse the stages");
 
 // Inv (row-major n x n, FP64) -> [3][nks][Mpad x 16] K-major blocks; zero past n.
 __global__ void k_bp_split_inv(int n, int nks, int Mpad, const double *__restrict__ inv,
@@ -264,11 +276,12 @@ __global__ void k_bp_split_y(int n, int nks, int nb, int NBpad, const int64_t *_
 }
 
 __global__ void __launch_bounds__(BPC_THREADS, 1)
-    k_bp_apply_tc(int n, int nks, int Mpad, int NBpad, int nb, const __nv_bfloat16 *__restrict__ A,
+    k_bp_apply_tc(int n, int nks, int Mpad, int NBpad, int nb, int NT, const __nv_bfloat16 *__restrict__ A,
                   const __nv_bfloat16 *__restrict__ Ys, const int64_t *__restrict__ voff,
                   const double *__restrict__ scale, double *__restrict__ z, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+    const uint32_t BPC_B_PIECE = (uint32_t)NT * TC_K * 2, BPC_STAGE = bpc_stage(NT);
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + (size_t)BPC_STAGES * BPC_STAGE);
     uint64_t *empty = full + BPC_STAGES;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(empty + BPC_STAGES);
@@ -276,13 +289,16 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
     __shared__ int64_t s_v[BPC_N];
     __shared__ double s_sc[BPC_N];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    __shared__ int s_skip;  // one read of the flag, so that the whole block leaves or stays
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), nr = (int)cl.num_blocks();
+    __shared__ int s_skip;  // one read of the flag, so that the whole block works or not
     if (tid == 0) s_skip = *reinterpret_cast<volatile int *>(err);
     __syncthreads();
-    if (s_skip) return;
-    const int r0 = blockIdx.x * BPC_M, b0 = blockIdx.y * BPC_N;
-    {
-        const int b = b0 + tid;  // BPC_THREADS == BPC_N
+    const bool skip = s_skip != 0;
+    const int r0 = (blockIdx.x / nr) * BPC_M, b0 = blockIdx.y * NT;
+    const int ks0 = rank * nks / nr, nk = (rank + 1) * nks / nr - ks0;  // this CTA's K steps
+    if (tid < NT) {
+        const int b = b0 + tid;
         s_v[tid] = b < nb ? voff[b] : -1;
         s_sc[tid] = b < nb ? scale[b] : 0.0;
     }
@@ -296,7 +312,7 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "n"(BPC_N));
+                     "r"(NT));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -305,9 +321,9 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
     const uint32_t tmem = *tmem_slot;
     const uint32_t sbase = smem_u32(smem);
     __shared__ int s_last;
-    if (tid == 0) {  // producer: six bulk copies per stage
+    if (tid == 0 && !skip) {  // producer: six bulk copies per stage
         int issued = -1;
-        for (int ks = 0; ks < nks; ++ks) {
+        for (int ks = 0; ks < nk; ++ks) {
             const int st = ks % BPC_STAGES;
             if (ks >= BPC_STAGES &&
                 (!mbar_wait(smem_u32(&empty[st]), (uint32_t)((ks / BPC_STAGES - 1) & 1)) || *abort_flag)) {
@@ -317,9 +333,9 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
             const uint32_t sa = sbase + st * BPC_STAGE, sb = sa + 3 * BPC_A_PIECE, fb = smem_u32(&full[st]);
             mbar_expect_tx(fb, BPC_STAGE);
             for (int piece = 0; piece < 3; ++piece) {
-                bulk_g2s(sa + piece * BPC_A_PIECE, A + ((size_t)(piece * nks + ks) * Mpad + r0) * TC_K, BPC_A_PIECE,
+                bulk_g2s(sa + piece * BPC_A_PIECE, A + ((size_t)(piece * nks + ks0 + ks) * Mpad + r0) * TC_K, BPC_A_PIECE,
                          fb);
-                bulk_g2s(sb + piece * BPC_B_PIECE, Ys + ((size_t)(piece * nks + ks) * NBpad + b0) * TC_K,
+                bulk_g2s(sb + piece * BPC_B_PIECE, Ys + ((size_t)(piece * nks + ks0 + ks) * NBpad + b0) * TC_K,
                          BPC_B_PIECE, fb);
             }
             issued = ks;
@@ -328,9 +344,9 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
         for (int k2 = issued; k2 >= 0 && k2 > issued - BPC_STAGES; --k2)
             if (!mbar_wait(smem_u32(&full[k2 % BPC_STAGES]), (uint32_t)((k2 / BPC_STAGES) & 1))) *abort_flag = 1;
     } else if (tid == 32) {  // MMA issuer
-        const uint32_t idesc = make_idesc(BPC_M, BPC_N);
+        const uint32_t idesc = make_idesc(BPC_M, NT);
         int ks = 0;
-        for (; ks < nks; ++ks) {
+        for (; ks < (skip ? 0 : nk); ++ks) {
             const int st = ks % BPC_STAGES;
             if (!mbar_wait(smem_u32(&full[st]), (uint32_t)((ks / BPC_STAGES) & 1)) || *abort_flag) {
                 *abort_flag = 1;
@@ -354,13 +370,14 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
     const int lk = s_last;
     const bool done =
         lk >= 0 && mbar_wait(smem_u32(&empty[lk % BPC_STAGES]), (uint32_t)((lk / BPC_STAGES) & 1));
-    const bool ok = !*abort_flag && lk == nks - 1 && done;
+    const bool ok = !skip && !*abort_flag && lk == nk - 1 && done;
     if (!ok && tid == 0) atomicOr(err, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
+    float *red = reinterpret_cast<float *>(smem);  // the stages are free (split K: the sums to join)
     if (ok) {
         const int q4 = warp & 3, half = warp >> 2;
-        const int row = r0 + q4 * 32 + lane;
-        for (int c0 = half * 128; c0 < half * 128 + 128 && b0 + c0 < nb; c0 += 16) {
+        const int trow = q4 * 32 + lane, row = r0 + trow;
+        for (int c0 = half * (NT / 2); c0 < (half + 1) * (NT / 2) && b0 + c0 < nb; c0 += 16) {
             uint32_t v[16];
             const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)c0;
             asm volatile(
@@ -371,7 +388,10 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
                   "=r"(v[15])
                 : "r"(taddr));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if (row < n) {
+            if (nr > 1) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) red[(c0 + i) * BPC_RED + trow] = __uint_as_float(v[i]);
+            } else if (row < n) {
 #pragma unroll
                 for (int i = 0; i < 16; ++i) {
                     const int64_t vb = s_v[c0 + i];
@@ -380,9 +400,24 @@ __global__ void __launch_bounds__(BPC_THREADS, 1)
             }
         }
     }
+    if (nr > 1) {
+        // every rank joins its share of the rows, the ranks in order (a rank that failed has raised
+        // the error flag: the result is not used)
+        cl.sync();
+        const int share = BPC_M / nr;
+        for (int e = tid; e < share * NT; e += BPC_THREADS) {
+            const int trow = rank * share + e % share, b = e / share, row = r0 + trow;
+            const int64_t vb = s_v[b];
+            if (vb < 0 || row >= n) continue;
+            float t = 0.f;
+            for (int q = 0; q < nr; ++q) t += cl.map_shared_rank(red, q)[b * BPC_RED + trow];
+            z[vb + row] = s_sc[b] * (double)t;
+        }
+        cl.sync();  // no CTA leaves while another still reads its sums
+    }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(BPC_N));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(NT));
 }
 
 // Bubbles whose meshes have the same connectivity (vertex count and triangle list relative to
@@ -510,7 +545,8 @@ void block_precond_prepare(Context &c) {
     auto &bp = c.bp;
     if (c.prm.precision != BEM_PREC_FP64) {
         if (!bp.tc_attr) {
-            BEM_CUDA(cudaFuncSetAttribute(k_bp_apply_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BPC_SMEM));
+            BEM_CUDA(cudaFuncSetAttribute(k_bp_apply_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)bpc_smem(BPC_N)));
             bp.tc_attr = true;
         }
         if (c.tc_err.n == 0) {
@@ -549,16 +585,32 @@ void block_precond_apply(Context &c, const double *y, double *z) {
             k_bp_apply<double><<<grid, BP_THREADS, 0, c.stream>>>(n, bp.inv64.p + bp.inv_off[k], (int)nb, vo, sc, y, z);
         } else {
             const int nks = div_up(n, TC_K), Mpad = div_up(n, BPC_M) * BPC_M;
-            const int NBpad = div_up(nb, BPC_N) * BPC_N;
+            // tile width: the narrowest that still takes all bubbles, so that no MMA column is idle
+            // but the last tile's, at most 256; then the K steps are split while the tiles leave SMs
+            // idle and a share keeps at least four steps (one fill of the pipeline)
+            const int NT = nb <= 64 ? 64 : (nb <= 128 ? 128 : BPC_N);
+            const int NBpad = div_up(nb, NT) * NT;
+            int split = 1;
+            while (split < 8 && (int64_t)(Mpad / BPC_M) * (NBpad / NT) * split * 2 <= c.num_sms && nks >= 8 * split) split *= 2;
             bp.ys.resize((size_t)3 * nks * NBpad * TC_K);
             __nv_bfloat16 *ys = reinterpret_cast<__nv_bfloat16 *>(bp.ys.p);
             k_bp_split_y<<<(unsigned)std::min(div_up((int64_t)NBpad * nks * 2, 256), 152 * 16), 256, 0, c.stream>>>(
                 n, nks, (int)nb, NBpad, vo, y, ys);
             BEM_LAUNCH_CHECK();
-            const dim3 grid((unsigned)(Mpad / BPC_M), (unsigned)(NBpad / BPC_N));
-            k_bp_apply_tc<<<grid, BPC_THREADS, BPC_SMEM, c.stream>>>(
-                n, nks, Mpad, NBpad, (int)nb, reinterpret_cast<const __nv_bfloat16 *>(bp.tcA.p) + bp.tc_off[k], ys, vo,
-                sc, z, c.tc_err.p);
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3((unsigned)(Mpad / BPC_M * split), (unsigned)(NBpad / NT));
+            cfg.blockDim = dim3(BPC_THREADS);
+            cfg.dynamicSmemBytes = bpc_smem(NT);
+            cfg.stream = c.stream;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = (unsigned)split;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            BEM_CUDA(cudaLaunchKernelEx(&cfg, k_bp_apply_tc, n, nks, Mpad, NBpad, (int)nb, NT,
+                                        reinterpret_cast<const __nv_bfloat16 *>(bp.tcA.p) + bp.tc_off[k],
+                                        (const __nv_bfloat16 *)ys, vo, sc, z, c.tc_err.p));
         }
         BEM_LAUNCH_CHECK();
     }
