@@ -22,7 +22,7 @@ namespace bem {
 namespace {
 
 constexpr int SEG_THREADS = 256;
-constexpr int64_t kSeg = 16384;  // vertices per reduction segment
+constexpr int64_t kSeg = 2048;  // vertices per reduction segment
 constexpr int SEG_JB = 8;        // basis vectors per pass over w
 
 // partial[j * nseg + s] = sum over segment s of V_j . w
