@@ -51,25 +51,27 @@ __device__ __forceinline__ void dir_store(const DirArgs<R> &a, int r, int64_t i,
 }
 
 // ------------------------------------------------------------------------------ FP64
-// One lane per receiver, 32 receivers per cluster; the sources are shared by the cluster's 8 CTAs
-// and, tile by tile, by a CTA's 4 warps. FP64 runs at 2 lanes per clock and SM on this part, so
-// the kernel is bound by its FP64 instructions (about 15 per pair for the single layer, 22 for
-// both): what counts is that every SM has a share, which 32-receiver groups x 8 give from a
-// few hundred points on.
-constexpr int D64_THREADS = 128, D64_WARPS = D64_THREADS / 32, D64_RECV = 32, D64_TILE = 128;
+// RECV receivers per cluster, one lane each; the sources are shared by the cluster's 8 CTAs and, tile
+// by tile, by a CTA's 4 warps x 32 / RECV lane groups. FP64 runs at 2 lanes per clock and SM on this
+// part, so the kernel is bound by its FP64 instructions (about 15 per pair for the single layer, 22
+// for both; 5124 points, both: 0.97 ms against 0.92): what counts is that every SM has the same share.
+// 32 receivers where that gives several CTAs per SM; below, 8, for four times as many equal pieces
+// (642 points: 168 CTAs of 32 receivers left 136 SMs waiting for the 16 that had two).
+constexpr int D64_THREADS = 128, D64_WARPS = D64_THREADS / 32, D64_TILE = 128;
 
-template <int R, bool HQ, bool HW>
+template <int R, bool HQ, bool HW, int RECV>
 __global__ void __launch_bounds__(D64_THREADS) k_direct64(int64_t N, const double *__restrict__ xyz,
                                                           const double *__restrict__ s, const double *__restrict__ nrm,
                                                           DirArgs<R> a) {
     __shared__ double sx[D64_TILE], sy[D64_TILE], sz[D64_TILE];
     __shared__ double snx[HW ? D64_TILE : 1], sny[HW ? D64_TILE : 1], snz[HW ? D64_TILE : 1];
     __shared__ double sq[HQ ? R : 1][D64_TILE], sw[HW ? R : 1][D64_TILE];
-    __shared__ double red[D64_WARPS][R][D64_RECV];
+    constexpr int GR = 32 / RECV, PARTS = D64_WARPS * GR;  // shares of a tile's sources
+    __shared__ double red[PARTS][R][RECV];
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), nr = (int)cl.num_blocks();
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int64_t i = (int64_t)(blockIdx.x / nr) * D64_RECV + lane;
+    const int tid = threadIdx.x, part = (tid >> 5) * GR + (tid & 31) / RECV, rl = tid & (RECV - 1);
+    const int64_t i = (int64_t)(blockIdx.x / nr) * RECV + rl;
     const int64_t ii = i < N ? i : N - 1;
     const double xi = xyz[ii], yi = xyz[N + ii], zi = xyz[2 * N + ii];
     const int64_t per = (N + nr - 1) / nr, j0 = rank * per, j1 = N < j0 + per ? N : j0 + per;
@@ -97,7 +99,7 @@ __global__ void __launch_bounds__(D64_THREADS) k_direct64(int64_t N, const doubl
             }
         }
         __syncthreads();
-        const int e0 = warp * ns / D64_WARPS, e1 = (warp + 1) * ns / D64_WARPS;
+        const int e0 = part * ns / PARTS, e1 = (part + 1) * ns / PARTS;
 #pragma unroll 4
         for (int e = e0; e < e1; ++e) {
             const double dx = xi - sx[e], dy = yi - sy[e], dz = zi - sz[e];
@@ -115,18 +117,23 @@ __global__ void __launch_bounds__(D64_THREADS) k_direct64(int64_t N, const doubl
         }
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) red[warp][r][lane] = acc[r];
+    for (int r = 0; r < R; ++r) red[part][r][rl] = acc[r];
+    __syncthreads();
+    // the CTA's own parts in order, then this rank joins the receivers rank, rank + nr, ... of the
+    // group, the ranks in order
+    for (int e = tid; e < R * RECV; e += D64_THREADS) {
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < PARTS; ++w) v += (&red[w][0][0])[e];
+        (&red[0][0][0])[e] = v;
+    }
     cl.sync();
-    // this rank joins the receivers rank, rank + nr, ... of the group: ranks in order, warps in order
-    for (int e = tid; e < R * D64_RECV; e += D64_THREADS) {
-        const int r = e / D64_RECV, l = e % D64_RECV;
-        const int64_t k = (int64_t)(blockIdx.x / nr) * D64_RECV + l;
+    for (int e = tid; e < R * RECV; e += D64_THREADS) {
+        const int r = e / RECV, l = e % RECV;
+        const int64_t k = (int64_t)(blockIdx.x / nr) * RECV + l;
         if (l % nr != rank || k >= N) continue;
         double v = 0.0;
-        for (int c = 0; c < nr; ++c) {
-            const double *p = cl.map_shared_rank(&red[0][0][0], c);
-            for (int w = 0; w < D64_WARPS; ++w) v += p[(w * R + r) * D64_RECV + l];
-        }
+        for (int c = 0; c < nr; ++c) v += cl.map_shared_rank(&red[0][0][0], c)[e];
         dir_store(a, r, k, v);
     }
     cl.sync();  // no CTA leaves while another still reads its sums
@@ -134,12 +141,14 @@ __global__ void __launch_bounds__(D64_THREADS) k_direct64(int64_t N, const doubl
 
 // ------------------------------------------------------------------------------ FP32
 // Coordinates as hi + lo FP32 pairs; packed two-wide arithmetic (add/mul/fma .f32x2) over two
-// sources, two receivers per thread, 256 receivers per cluster. Per pair the FP32 pipe has 9
+// sources, 128 receivers per cluster. Per pair the FP32 pipe has 9
 // additions for the difference of the split coordinates and 4 (single layer) to 11 (both) further
 // operations, the special-function unit one reciprocal square root: FP32-bound, about 0.16 clocks
 // per pair and SM for both layers. Sums run over at most 64 sources per packed half in FP32 and are
 // merged with TwoSum; the cluster's shares are joined in FP64.
-constexpr int D32_THREADS = 128, D32_RI = 2, D32_RECV = D32_THREADS * D32_RI, D32_TILE = 128;
+// One receiver per thread (two save shared-memory loads, but leave half as many warps: 232 against
+// 221 us at 13446 points, 452 against 420 at 20484).
+constexpr int D32_THREADS = 128, D32_RI = 1, D32_RECV = D32_THREADS * D32_RI, D32_TILE = 128;
 
 template <int R, bool HQ, bool HW>
 struct D32Stage {
@@ -223,6 +232,26 @@ __device__ __forceinline__ void dir32_sources(D32Stage<R, HQ, HW> &sg, int64_t N
             }
         }
     };
+    // this thread's source of the next tile, loaded while the current one is evaluated
+    float ph[3], pl[3];
+    double pn[3], ps, pq[R], pw[R];
+    auto fetch = [&](int64_t t0) {
+        if (t0 + tid >= j1) return;
+        const int64_t j = t0 + tid;
+        ps = s[j];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            ph[d] = hi[d * N + j];
+            pl[d] = lo[d * N + j];
+            if (HW) pn[d] = nrm[d * N + j];
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (HQ) pq[r] = a.f[r] != 0.0 ? a.xL[r][j] : 0.0;
+            if (HW) pw[r] = a.g[r] != 0.0 ? a.xM[r][j] : 0.0;
+        }
+    };
+    fetch(j0);
     for (int64_t t0 = j0; t0 < j1; t0 += D32_TILE) {
         const int ns = (int)(j1 - t0 < D32_TILE ? j1 - t0 : D32_TILE);
         __syncthreads();
@@ -231,27 +260,27 @@ __device__ __forceinline__ void dir32_sources(D32Stage<R, HQ, HW> &sg, int64_t N
             float *A = reinterpret_cast<float *>(&sg.a[p]), *B = reinterpret_cast<float *>(&sg.b[p]),
                   *C = reinterpret_cast<float *>(&sg.c[p]);
             const bool in = tid < ns;
-            const int64_t j = in ? t0 + tid : t0;
             // past the share's end: zero strength, far away (a finite r^2)
-            A[h] = in ? -hi[j] : -1e18f;
-            A[2 + h] = in ? -hi[N + j] : -1e18f;
-            B[h] = in ? -hi[2 * N + j] : -1e18f;
-            B[2 + h] = in ? -lo[j] : 0.f;
-            C[h] = in ? -lo[N + j] : 0.f;
-            C[2 + h] = in ? -lo[2 * N + j] : 0.f;
+            A[h] = in ? -ph[0] : -1e18f;
+            A[2 + h] = in ? -ph[1] : -1e18f;
+            B[h] = in ? -ph[2] : -1e18f;
+            B[2 + h] = in ? -pl[0] : 0.f;
+            C[h] = in ? -pl[1] : 0.f;
+            C[2 + h] = in ? -pl[2] : 0.f;
             if (HW) {
                 float *D = reinterpret_cast<float *>(&sg.d[p]), *E = reinterpret_cast<float *>(&sg.e[p]);
-                D[h] = in ? (float)nrm[j] : 0.f;
-                D[2 + h] = in ? (float)nrm[N + j] : 0.f;
-                E[h] = in ? (float)nrm[2 * N + j] : 0.f;
+                D[h] = in ? (float)pn[0] : 0.f;
+                D[2 + h] = in ? (float)pn[1] : 0.f;
+                E[h] = in ? (float)pn[2] : 0.f;
             }
-            const double sj = s[j] * kInv4Pi;
+            const double sj = ps * kInv4Pi;
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                if (HQ) reinterpret_cast<float *>(&sg.q[r][p])[h] = in ? (float)dir_q(a, r, sj, j) : 0.f;
-                if (HW) reinterpret_cast<float *>(&sg.w[r][p])[h] = in ? (float)dir_w(a, r, sj, j) : 0.f;
+                if (HQ) reinterpret_cast<float *>(&sg.q[r][p])[h] = in && a.f[r] != 0.0 ? (float)(a.f[r] * sj * pq[r]) : 0.f;
+                if (HW) reinterpret_cast<float *>(&sg.w[r][p])[h] = in && a.g[r] != 0.0 ? (float)(a.g[r] * sj * pw[r]) : 0.f;
             }
         }
+        fetch(t0 + D32_TILE);
         __syncthreads();
         float2 part[D32_RI][R];
 #pragma unroll
@@ -335,8 +364,12 @@ void launch_cluster(K kern, int64_t groups, int threads, cudaStream_t st, A... a
 }
 
 template <int R, bool HQ, bool HW>
-void launch64(int64_t N, const double *xyz, const double *s, const double *nrm, const DirArgs<R> &a, cudaStream_t st) {
-    launch_cluster(k_direct64<R, HQ, HW>, div_up(N, D64_RECV), D64_THREADS, st, N, xyz, s, nrm, a);
+void launch64(int64_t N, const double *xyz, const double *s, const double *nrm, const DirArgs<R> &a, int num_sms,
+              cudaStream_t st) {
+    if (div_up(N, 32) * DIR_SPLIT >= 8 * num_sms)
+        launch_cluster(k_direct64<R, HQ, HW, 32>, div_up(N, 32), D64_THREADS, st, N, xyz, s, nrm, a);
+    else
+        launch_cluster(k_direct64<R, HQ, HW, 8>, div_up(N, 8), D64_THREADS, st, N, xyz, s, nrm, a);
 }
 template <int R, bool HQ, bool HW>
 void launch32(int64_t N, const float *hi, const float *lo, const double *s, const double *nrm, const DirArgs<R> &a,
@@ -377,7 +410,7 @@ void launch_direct(Context &c, int prec, const double *f, const double *const *x
     PhaseScope ps(c, PH_DIRECT);
     with_layers<R>(a, [&](auto hq, auto hw) {
         constexpr bool HQ = decltype(hq)::value, HW = decltype(hw)::value;
-        if (prec == BEM_PREC_FP64) launch64<R, HQ, HW>(c.N, c.xyz.p, c.s.p, c.nrm.p, a, c.stream);
+        if (prec == BEM_PREC_FP64) launch64<R, HQ, HW>(c.N, c.xyz.p, c.s.p, c.nrm.p, a, c.num_sms, c.stream);
         else launch32<R, HQ, HW>(c.N, c.dir_hi.p, c.dir_lo.p, c.s.p, c.nrm.p, a, c.stream);
     });
 }
