@@ -78,7 +78,7 @@ namespace {
 constexpr int GM = 128;           // tile rows
 constexpr int GN = 64;            // tile columns
 constexpr int GK = 64;            // K chunk (bf16): 128 bytes per row = 8 core matrices
-constexpr int G_STAGES = 4, G_THREADS = 128;
+constexpr int G_STAGES = 4, G_THREADS = 256;
 constexpr int G_STAGE_ELEMS = (GM + GN) * GK;
 constexpr int G_RED_PITCH = GN + 1;
 constexpr int G_SMEM = G_STAGES * G_STAGE_ELEMS * 2 + 1024;  // aligned to 1024 by the kernel
@@ -141,16 +141,14 @@ struct GemmOut {
     __nv_bfloat16 *H, *HT;
     int64_t ldh, ldt;
 };
-__device__ __forceinline__ void gemm_store(const GemmOut &o, int m, int n, float a) {
-    const int64_t ix = (int64_t)m * o.ldc + n;
+// value of C at (m, n) from the sum a
+__device__ __forceinline__ float gemm_epi(const GemmOut &o, int m, int n, float a) {
     if (o.epi == EPI_BIAS || o.epi == EPI_BIAS_RELU) a += o.bias[n];
-    if (o.epi == EPI_RELU_MASK) a = o.Zm[ix] > 0.f ? a : 0.f;
-    o.C[ix] = a;
-    if (o.H) {
-        const __nv_bfloat16 h = __float2bfloat16(o.epi == EPI_BIAS_RELU ? fmaxf(a, 0.f) : a);
-        o.H[(int64_t)m * o.ldh + n] = h;
-        if (o.HT) o.HT[(int64_t)n * o.ldt + m] = h;
-    }
+    if (o.epi == EPI_RELU_MASK) a = o.Zm[(int64_t)m * o.ldc + n] > 0.f ? a : 0.f;
+    return a;
+}
+__device__ __forceinline__ __nv_bfloat16 gemm_h(const GemmOut &o, float c) {
+    return __float2bfloat16(o.epi == EPI_BIAS_RELU ? fmaxf(c, 0.f) : c);
 }
 
 template <bool SPLIT>
@@ -243,26 +241,22 @@ __global__ void __launch_bounds__(G_THREADS) k_gemm_bf16(int M, int N, int K, co
     ok = __syncthreads_and(ok);
     if (!ok && tid == 0) atomicOr(err, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
-    const int row = warp * 32 + lane, m = m0 + row;
-    float *red = reinterpret_cast<float *>(smem);  // SPLIT: [row][G_RED_PITCH], in the free stages
+    const int row = (warp & 3) * 32 + lane, qh = warp >> 2;  // TMEM lanes of a warp; the halves take half the columns
+    // the tile goes through shared memory ([row][G_RED_PITCH], in the free stages), so that every store
+    // below is coalesced: 192 scattered stores per thread took most of a product's 32 us
+    float *red = reinterpret_cast<float *>(smem);
     if (ok) {
-        for (int q = 0; q < GN; q += 16) {
+        for (int q = qh * (GN / 2); q < (qh + 1) * (GN / 2); q += 16) {
             uint32_t v[16];
             asm volatile(
                 "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
                   "=r"(v[15])
-                : "r"(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)q));
+                : "r"(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)q));
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-            if constexpr (SPLIT) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) red[row * G_RED_PITCH + q + i] = nc > 0 ? __uint_as_float(v[i]) : 0.f;
-            } else if (m < M) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    if (n0 + q + i < N) gemm_store(out, m, n0 + q + i, __uint_as_float(v[i]));
-            }
+            for (int i = 0; i < 16; ++i) red[row * G_RED_PITCH + q + i] = nc > 0 ? __uint_as_float(v[i]) : 0.f;
         }
     }
     if constexpr (SPLIT) {
@@ -274,9 +268,30 @@ __global__ void __launch_bounds__(G_THREADS) k_gemm_bf16(int M, int N, int K, co
             if (m0 + rr >= M || n0 + q >= N) continue;
             float a = 0.f;
             for (int c = 0; c < nr; ++c) a += cl.map_shared_rank(red, c)[rr * G_RED_PITCH + q];
-            gemm_store(out, m0 + rr, n0 + q, a);
+            out.C[(int64_t)(m0 + rr) * out.ldc + n0 + q] = a;  // a weight gradient: EPI_STORE
         }
         cl.sync();  // no CTA leaves while another still reads its sums
+    } else {
+        __syncthreads();
+        if (ok) {
+#pragma unroll 4
+            for (int e = tid; e < GM * GN; e += G_THREADS) {
+                const int rr = e / GN, q = e % GN, m = m0 + rr, n = n0 + q;
+                if (m >= M || n >= N) continue;
+                const float a = gemm_epi(out, m, n, red[rr * G_RED_PITCH + q]);
+                red[rr * G_RED_PITCH + q] = a;
+                out.C[(int64_t)m * out.ldc + n] = a;
+                if (out.H) out.H[(int64_t)m * out.ldh + n] = gemm_h(out, a);
+            }
+            if (out.HT) {
+                __syncthreads();
+#pragma unroll 4
+                for (int e = tid; e < GM * GN; e += G_THREADS) {
+                    const int rr = e % GM, q = e / GM, m = m0 + rr, n = n0 + q;
+                    if (m < M && n < N) out.HT[(int64_t)n * out.ldt + m] = gemm_h(out, red[rr * G_RED_PITCH + q]);
+                }
+            }
+        }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
