@@ -435,66 +435,83 @@ __global__ void k_tm_fill(int64_t np, int TT, const int32_t *__restrict__ src, c
     const int64_t tile = r / TT, slot = r % TT;
     tab[(tile * kNumM2LClasses + cls[k]) * TT + slot] = src[k];
 }
-// per tile, the classes present, in the order `order` (truncated size ascending)
-__global__ void __launch_bounds__(512) k_tm_classes(int TT, const int32_t *__restrict__ tab,
-                                                    const int32_t *__restrict__ order, int32_t *__restrict__ tcls,
-                                                    int32_t *__restrict__ ncls) {
-    __shared__ int warp_tot[16];
-    const int tile = blockIdx.x, k = threadIdx.x;
-    int f = 0;
-    if (k < kNumM2LClasses) {
-        const int32_t *col = tab + ((int64_t)tile * kNumM2LClasses + order[k]) * TT;
-        for (int r = 0; r < TT && !f; ++r) f = col[r] >= 0;
-    }
-    // block prefix sum of the flags (warp scans, then the warp totals)
-    const int lane = k & 31, w = k >> 5;
-    int v = f;
+// Time of one class in an item, in arbitrary units: K_c / 16 K steps, whose shared-memory traffic (the
+// MMAs' operand reads and the staged copies: about 576 + 3.75 K_c clocks) bounds a step.
+__device__ __forceinline__ int tm_cost(int Kc) { return Kc / TC_K * (Kc + 160); }
+// inclusive prefix sum over a block of 512 threads
+__device__ __forceinline__ int tm_scan(int v, int *warp_tot) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int t = __shfl_up_sync(0xffffffffu, v, o);
         if (lane >= o) v += t;
     }
+    __syncthreads();
     if (lane == 31) warp_tot[w] = v;
     __syncthreads();
-    int before = 0;
-    for (int i = 0; i < w; ++i) before += warp_tot[i];
-    const int idx = before + v - f;  // exclusive
-    if (f) tcls[(int64_t)tile * kNumM2LClasses + idx] = order[k];
-    if (k == 511) ncls[tile] = before + v;
+    for (int i = 0; i < w; ++i) v += warp_tot[i];
+    return v;
 }
-// Time of one class in an item, in arbitrary units: K_c / 16 K steps, whose shared-memory traffic (the
-// MMAs' operand reads and the staged copies: about 576 + 3.75 K_c clocks) bounds a step.
-__device__ __forceinline__ int tm_cost(int Kc) { return Kc / TC_K * (Kc + 160); }
-__global__ void k_tm_tile_cost(int64_t ntiles, const int32_t *__restrict__ ncls, const int32_t *__restrict__ tcls,
-                               const int32_t *__restrict__ cls_K, int Npad, int32_t *__restrict__ cost) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= ntiles) return;
-    int c = 0;
-    for (int i = 0; i < ncls[t]; ++i) c += tm_cost(cls_K ? cls_K[tcls[t * kNumM2LClasses + i]] : Npad);
-    cost[t] = c;
+// per tile, the classes present, in the order `order` (truncated size ascending), and their cost
+__global__ void __launch_bounds__(512) k_tm_classes(int TT, const int32_t *__restrict__ tab,
+                                                    const int32_t *__restrict__ order,
+                                                    const int32_t *__restrict__ cls_K, int Npad,
+                                                    int32_t *__restrict__ tcls, int32_t *__restrict__ ncls,
+                                                    int32_t *__restrict__ cost) {
+    __shared__ int warp_tot[16];
+    __shared__ uint8_t has[512];
+    const int tile = blockIdx.x, k = threadIdx.x, lane = k & 31;
+    // a warp per class: its 32 lanes look through the class's slots together
+    for (int q = k >> 5; q < kNumM2LClasses; q += 16) {
+        const int32_t *col = tab + ((int64_t)tile * kNumM2LClasses + order[q]) * TT;
+        bool f = false;
+        for (int r = lane; r < TT; r += 32) f = f || col[r] >= 0;
+        const unsigned any = __ballot_sync(0xffffffffu, f);
+        if (lane == 0) has[q] = any != 0;
+    }
+    __syncthreads();
+    const int f = k < kNumM2LClasses && has[k];
+    const int idx = tm_scan(f, warp_tot);  // inclusive
+    if (f) tcls[(int64_t)tile * kNumM2LClasses + idx - 1] = order[k];
+    const int c = tm_scan(f ? tm_cost(cls_K ? cls_K[order[k]] : Npad) : 0, warp_tot);
+    if (k == 511) {
+        ncls[tile] = idx;
+        cost[tile] = c;
+    }
 }
-// The tile's classes cut into items of about equal cost, n = cost / target of them (rounded up), of
-// fewer than TM_MAXCLS classes. Pass 0 counts the items, pass 1 writes them from off[tile] on.
-__global__ void k_tm_items(int64_t ntiles, int target, const int32_t *__restrict__ ncls, const int32_t *__restrict__ tcls,
-                           const int32_t *__restrict__ cls_K, int Npad, const int32_t *__restrict__ cost, int pass,
-                           int32_t *__restrict__ cnt, const int32_t *__restrict__ off, int4 *__restrict__ items) {
-    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= ntiles) return;
-    const int n = ncls[t], parts = max(1, (cost[t] + target - 1) / target);
-    int64_t run = 0;  // cost so far
-    int nit = 0, c0 = 0;
-    for (int i = 0; i < n; ++i) {
-        const int Kc = cls_K ? cls_K[tcls[t * kNumM2LClasses + i]] : Npad;
-        run += tm_cost(Kc);
-        // the share of the items that ends nearest to here is full, or the item is
-        const bool cut = (run + tm_cost(Kc) / 2) * parts >= (int64_t)cost[t] * (nit + 1);
-        if (cut || i + 1 - c0 == TM_MAXCLS || i + 1 == n) {
-            if (pass) items[off[t] + nit] = make_int4((int)t, c0, i + 1 - c0, Kc);  // K_c: the largest of the item
-            ++nit;
-            c0 = i + 1;
+// The tile's classes cut into items of about equal cost, n = cost / target of them (rounded up): a class
+// belongs to the item that the middle of its cost falls into, and an item has at most TM_MAXCLS classes.
+// Pass 0 counts the items, pass 1 writes them from off[tile] on. One block per tile.
+__global__ void __launch_bounds__(512) k_tm_items(int target, const int32_t *__restrict__ ncls,
+                                                  const int32_t *__restrict__ tcls, const int32_t *__restrict__ cls_K,
+                                                  int Npad, const int32_t *__restrict__ cost, int pass,
+                                                  int32_t *__restrict__ cnt, const int32_t *__restrict__ off,
+                                                  int4 *__restrict__ items) {
+    __shared__ int warp_tot[16];
+    __shared__ int part[513], first[513];
+    const int tile = blockIdx.x, i = threadIdx.x, n = ncls[tile];
+    const int64_t total = cost[tile], parts = max((int64_t)1, (total + target - 1) / target);
+    const int Kc = i < n ? (cls_K ? cls_K[tcls[(int64_t)tile * kNumM2LClasses + i]] : Npad) : 0;
+    const int mine = i < n ? tm_cost(Kc) : 0;
+    const int64_t mid = tm_scan(mine, warp_tot) - (mine + 1) / 2;
+    part[i] = i < n ? (int)(mid * parts / total) : -1;
+    __syncthreads();
+    // the first class of i's part, then a cut every TM_MAXCLS classes from there
+    int lo = i;
+    if (i < n)
+        while (lo > 0 && part[lo - 1] == part[i]) --lo;
+    const int f = i < n && (i - lo) % TM_MAXCLS == 0;
+    first[i] = f || i >= n;
+    const int idx = tm_scan(f, warp_tot) - 1;  // (its barriers also publish `first`)
+    if (pass && i < n) {
+        const bool last = i + 1 == n || first[i + 1];
+        if (last) {
+            int c0 = i;
+            while (!first[c0]) --c0;
+            items[off[tile] + idx] = make_int4(tile, c0, i + 1 - c0, Kc);  // K_c: the largest of the item
         }
     }
-    if (!pass) cnt[t] = nit;
+    if (!pass && i == 511) cnt[tile] = idx + 1;
 }
 
 __device__ __forceinline__ void two_sum_add(float &s, float &c, float v) {
@@ -833,12 +850,10 @@ static void build_tm_tables(Context &c, const Operators &o, cudaStream_t st) {
     BEM_CUDA(cudaMemcpyAsync(dorder.p, order.data(), kNumM2LClasses * sizeof(int32_t), cudaMemcpyHostToDevice, st));
     S.cls.resize(std::max<int64_t>(ntiles * kNumM2LClasses, 1));
     S.item_off.resize(ntiles + 1);
-    k_tm_classes<<<(unsigned)ntiles, 512, 0, st>>>(TT, S.src.p, dorder.p, S.cls.p, ncls.p);
-    BEM_LAUNCH_CHECK();
     const int32_t *clsK = o.margin >= 0 ? o.cls_K.p : nullptr;
     DevBuf<int32_t> &cost = S.s_i32[8];
     cost.resize(ntiles);
-    k_tm_tile_cost<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, ncls.p, S.cls.p, clsK, P16, cost.p);
+    k_tm_classes<<<(unsigned)ntiles, 512, 0, st>>>(TT, S.src.p, dorder.p, clsK, P16, S.cls.p, ncls.p, cost.p);
     BEM_LAUNCH_CHECK();
     std::vector<int32_t> hcost(ntiles);
     BEM_CUDA(cudaMemcpyAsync(hcost.data(), cost.p, ntiles * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -861,8 +876,7 @@ static void build_tm_tables(Context &c, const Operators &o, cudaStream_t st) {
         else lo = mid + 1;
     }
     const int target = (int)lo;
-    k_tm_items<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, target, ncls.p, S.cls.p, clsK, P16, cost.p, 0, icnt.p, nullptr,
-                                                  nullptr);
+    k_tm_items<<<(unsigned)ntiles, 512, 0, st>>>(target, ncls.p, S.cls.p, clsK, P16, cost.p, 0, icnt.p, nullptr, nullptr);
     BEM_LAUNCH_CHECK();
     exclusive_scan_i32(icnt.p, S.item_off.p, ntiles, tot.p, st);
     BEM_CUDA(cudaMemcpyAsync(S.item_off.p + ntiles, tot.p, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
@@ -871,8 +885,8 @@ static void build_tm_tables(Context &c, const Operators &o, cudaStream_t st) {
     BEM_CUDA(cudaStreamSynchronize(st));
     S.nitems = nitems;
     S.items.resize(std::max(nitems, 1));
-    k_tm_items<<<div_up(ntiles, tb), tb, 0, st>>>(ntiles, target, ncls.p, S.cls.p, clsK, P16, cost.p, 1, nullptr,
-                                                  S.item_off.p, S.items.p);
+    k_tm_items<<<(unsigned)ntiles, 512, 0, st>>>(target, ncls.p, S.cls.p, clsK, P16, cost.p, 1, nullptr, S.item_off.p,
+                                                 S.items.p);
     BEM_LAUNCH_CHECK();
     S.part.resize(std::max<size_t>((size_t)nitems * TM_ROWS * P16, 1));
     BEM_CUDA(cudaStreamSynchronize(st));  // dorder is freed on return

@@ -4,7 +4,9 @@
 //
 // Everything runs on the device: bounding-cube reduction, 30-bit Morton keys, a stable LSD
 // radix sort written here (8-bit digits, per-warp match ranking), per-level unique boxes by
-// flag + scan, parents and neighbours by binary search over the sorted box keys.
+// flag + scan. The 27 neighbours of every box come from its parent's: the neighbour at d is a
+// child of the parent's neighbour, found in the table of children, so the near-field and M2L
+// lists need no search.
 #include "internal.h"
 
 #include <algorithm>
@@ -226,21 +228,6 @@ __device__ __forceinline__ void demorton(uint32_t k, int &gx, int &gy, int &gz) 
     gy = (int)compact3(k >> 1);
     gz = (int)compact3(k);
 }
-// Index of the first element >= key in the sorted array a[0..n).
-__device__ __forceinline__ int lower_bound_u32(const uint32_t *a, int n, uint32_t key) {
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (a[mid] < key) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-__device__ __forceinline__ int find_box(const uint32_t *a, int n, uint32_t key) {
-    int i = lower_bound_u32(a, n, key);
-    return (i < n && a[i] == key) ? i : -1;
-}
-
 __global__ void k_bbox(int64_t N, const double *__restrict__ xyz, double *__restrict__ part) {
     // part[block][6] = min x,y,z, max x,y,z
     __shared__ double sm[6][256];
@@ -288,12 +275,13 @@ __global__ void k_keys(int64_t N, const double *__restrict__ xyz, double ox, dou
 // so sorting groups clusters and shifting right by 3 (8 - l) gives (cluster << 3l) | box key.
 constexpr int kClusterDeep = 8;
 
+constexpr int CB_PARTS = 16;  // blocks per cluster (one took 219 us for 16 clusters of 359000 points)
 __global__ void k_cluster_bbox(const int64_t *__restrict__ cvoff, int64_t N, const double *__restrict__ xyz,
                                double *__restrict__ out) {
     __shared__ double sm[6][256];
-    const int c = blockIdx.x;
+    const int c = blockIdx.x / CB_PARTS, part = blockIdx.x % CB_PARTS;
     double mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
-    for (int64_t i = cvoff[c] + threadIdx.x; i < cvoff[c + 1]; i += blockDim.x)
+    for (int64_t i = cvoff[c] + part * 256 + threadIdx.x; i < cvoff[c + 1]; i += 256 * CB_PARTS)
         for (int d = 0; d < 3; ++d) {
             double v = xyz[d * N + i];
             mn[d] = fmin(mn[d], v);
@@ -312,7 +300,7 @@ __global__ void k_cluster_bbox(const int64_t *__restrict__ cvoff, int64_t N, con
             }
         __syncthreads();
     }
-    if (threadIdx.x < 6) out[c * 6 + threadIdx.x] = sm[threadIdx.x][0];
+    if (threadIdx.x < 6) out[blockIdx.x * 6 + threadIdx.x] = sm[threadIdx.x][0];
 }
 
 // cube[c] = (origin x, y, z, 1 / size)
@@ -332,17 +320,28 @@ __global__ void k_keys_clusters(int64_t N, const double *__restrict__ xyz, const
     idx[i] = (int32_t)i;
 }
 
-// unique[l] += number of i in [1, N) where the level-l prefix of the key changes
-__global__ void k_level_counts(int64_t N, int deep, const uint32_t *__restrict__ key, int32_t *__restrict__ cnt) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    bool valid = i >= 1 && i < N;
-    uint32_t a = valid ? key[i] : 0u, b = valid ? key[i - 1] : 0u;
-    for (int l = 0; l <= deep; ++l) {
-        int sh = 3 * (deep - l);
-        int f = (valid && (a >> sh) != (b >> sh)) ? 1 : 0;
-        int tot = __reduce_add_sync(0xffffffffu, f);
-        if ((threadIdx.x & 31) == 0 && tot) atomicAdd(&cnt[l], tot);
+// cnt[l] += number of i in [1, N) whose key first differs from the one before at level l (the prefix of
+// every deeper level differs as well)
+__global__ void __launch_bounds__(256) k_level_counts(int64_t N, int deep, const uint32_t *__restrict__ key,
+                                                      int32_t *__restrict__ cnt) {
+    __shared__ int32_t h[kDeepLevel + 1];
+    if (threadIdx.x <= kDeepLevel) h[threadIdx.x] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t b = blockIdx.x * (int64_t)blockDim.x; b < N; b += stride) {  // uniform in the block
+        const int64_t i = b + threadIdx.x;
+        const uint32_t x = i >= 1 && i < N ? key[i] ^ key[i - 1] : 0u;
+        const int l = x ? max(0, deep - (31 - __clz(x)) / 3) : -1;
+        int mine = 0;
+        for (int q = 0; q <= deep; ++q) {
+            const int n = __popc(__ballot_sync(0xffffffffu, l == q));
+            if (lane == q) mine = n;
+        }
+        if (lane <= deep && mine) atomicAdd(&h[lane], mine);
     }
+    __syncthreads();
+    if (threadIdx.x <= deep && h[threadIdx.x]) atomicAdd(&cnt[threadIdx.x], h[threadIdx.x]);
 }
 
 __global__ void k_flags_points(int64_t N, const uint32_t *__restrict__ key, int shift, int32_t *__restrict__ flag) {
@@ -393,35 +392,55 @@ __global__ void k_box_counts(int n, const int32_t *__restrict__ bstart, int32_t 
     bcount[i] = ((i + 1 < n) ? bstart[i + 1] : total) - bstart[i];
 }
 
+// nb27[box][27]: the boxes of the same level (and cluster) around every box, itself included, by offset
+// (dx, dy, dz) in lexicographic order; -1 where empty. One level, from the level above.
+__global__ void k_nb27(int n, int gbase, const uint32_t *__restrict__ bkey, const int32_t *__restrict__ parent,
+                       const int32_t *__restrict__ child8, int32_t *__restrict__ nb27) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= n * 27) return;
+    const int b = gbase + e / 27, k = e % 27;
+    const int d[3] = {k / 9 - 1, k / 3 % 3 - 1, k % 3 - 1};
+    const int par = parent[b];
+    if (par < 0) {  // a root: its cluster has no other box at this level
+        nb27[(int64_t)b * 27 + k] = k == 13 ? b : -1;
+        return;
+    }
+    const uint32_t oct = bkey[b] & 7u;
+    int pk = 0, oc = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int c = (int)((oct >> (2 - a)) & 1u) + d[a];  // -1 .. 2 in the parent's children
+        pk = pk * 3 + (c >> 1) + 1;
+        oc = oc * 2 + (c & 1);
+    }
+    const int pn = nb27[(int64_t)par * 27 + pk];
+    nb27[(int64_t)b * 27 + k] = pn >= 0 ? child8[(int64_t)pn * 8 + oc] : -1;
+}
+
 // Near field (Section 3.7, A^(sparse)): the non-empty leaves among the 27 around each leaf.
-__global__ void k_neighbours(int nleaf, int L, const uint32_t *__restrict__ lkey,
+__global__ void k_neighbours(int nleaf, int gbase, const int32_t *__restrict__ nb27,
                              const int32_t *__restrict__ lcount, int32_t *__restrict__ nbr,
                              int32_t *__restrict__ ncnt, int8_t *__restrict__ nd,
                              unsigned long long *__restrict__ pairs) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    int gx, gy, gz;
-    const uint32_t mask = (1u << (3 * L)) - 1u, pre = lkey[b] & ~mask;  // cluster prefix
-    demorton(lkey[b] & mask, gx, gy, gz);
-    int lim = 1 << L, c = 0;
-    long long src = 0;
-    for (int dx = -1; dx <= 1; ++dx)
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dz = -1; dz <= 1; ++dz) {
-                int x = gx + dx, y = gy + dy, z = gz + dz;
-                if (x < 0 || y < 0 || z < 0 || x >= lim || y >= lim || z >= lim) continue;
-                int f = find_box(lkey, nleaf, pre | morton(x, y, z));
-                if (f < 0) continue;
-                nbr[b * 27 + c] = f;
-                nd[(b * 27 + c) * 4 + 0] = (int8_t)dx;
-                nd[(b * 27 + c) * 4 + 1] = (int8_t)dy;
-                nd[(b * 27 + c) * 4 + 2] = (int8_t)dz;
-                nd[(b * 27 + c) * 4 + 3] = 0;
-                src += lcount[f];
-                ++c;
-            }
-    ncnt[b] = c;
-    atomicAdd(pairs, (unsigned long long)(lcount[b] * (src - 1)));
+    long long mine = 0;
+    if (b < nleaf) {
+        int c = 0;
+        long long src = 0;
+        for (int k = 0; k < 27; ++k) {
+            const int g = nb27[(int64_t)(gbase + b) * 27 + k];
+            if (g < 0) continue;
+            nbr[b * 27 + c] = g - gbase;
+            reinterpret_cast<char4 *>(nd)[b * 27 + c] =
+                make_char4((signed char)(k / 9 - 1), (signed char)(k / 3 % 3 - 1), (signed char)(k % 3 - 1), 0);
+            src += lcount[g - gbase];
+            ++c;
+        }
+        ncnt[b] = c;
+        mine = lcount[b] * (src - 1);
+    }
+    for (int o = 16; o > 0; o >>= 1) mine += __shfl_xor_sync(0xffffffffu, mine, o);
+    if ((threadIdx.x & 31) == 0 && mine) atomicAdd(pairs, (unsigned long long)mine);
 }
 
 // Compact index of an M2L offset (dx,dy,dz) in [-3,3]^3 with max |d| >= 2, in lexicographic
@@ -435,45 +454,47 @@ __device__ __forceinline__ int m2l_class(int dx, int dy, int dz) {
     return full - near_before;
 }
 
-// M2L list of a box: children of the parent's neighbours that are not its own neighbours.
-// pass 0 counts, pass 1 writes (target, source, class) at `off[b]`.
-__global__ void k_m2l_lists(int n, int l, const uint32_t *__restrict__ key, const uint32_t *__restrict__ pkey,
-                            int np, int gbase, int pass, int32_t *__restrict__ cnt,
-                            const int32_t *__restrict__ off, int32_t *__restrict__ tgt,
-                            int32_t *__restrict__ src, uint32_t *__restrict__ cls) {
-    int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= n) return;
-    int gx, gy, gz;
-    const uint32_t mask = (1u << (3 * l)) - 1u;
-    const uint32_t cl = key[b] >> (3 * l);  // cluster id (0 without clusters)
-    const uint32_t pre = cl << (3 * l), ppre = cl << (3 * (l - 1));
-    demorton(key[b] & mask, gx, gy, gz);
-    int px = gx >> 1, py = gy >> 1, pz = gz >> 1;
-    int plim = 1 << (l - 1);
-    int c = 0;
-    int64_t o = pass ? off[b] : 0;
-    for (int dx = -1; dx <= 1; ++dx)
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dz = -1; dz <= 1; ++dz) {
-                int x = px + dx, y = py + dy, z = pz + dz;
-                if (x < 0 || y < 0 || z < 0 || x >= plim || y >= plim || z >= plim) continue;
-                const uint32_t pk = ppre | morton(x, y, z);
-                if (find_box(pkey, np, pk) < 0) continue;
-                // the parent's children are consecutive in key order: key = parent key * 8 + octant
-                for (int f = lower_bound_u32(key, n, pk << 3); f < n && (key[f] >> 3) == pk; ++f) {
-                    const int oc = (int)(key[f] & 7u);
-                    int cx = 2 * x + ((oc >> 2) & 1), cy = 2 * y + ((oc >> 1) & 1), cz = 2 * z + (oc & 1);
-                    int ddx = cx - gx, ddy = cy - gy, ddz = cz - gz;
-                    if (ddx >= -1 && ddx <= 1 && ddy >= -1 && ddy <= 1 && ddz >= -1 && ddz <= 1) continue;
-                    if (pass) {
-                        tgt[o + c] = gbase + b;
-                        src[o + c] = gbase + f;
-                        cls[o + c] = (uint32_t)m2l_class(ddx, ddy, ddz);
-                    }
-                    ++c;
-                }
+// M2L list of a box: children of the parent's neighbours that are not its own neighbours; one warp
+// per box (levels 2 on). The 216 candidates run over the offsets (dx, dy, dz) in lexicographic order,
+// so a box's pairs come out by ascending offset class. pass 0 counts, pass 1 writes (target,
+// source, class) from off[box] on.
+__global__ void __launch_bounds__(256) k_m2l_lists(int first, int nbox, const uint32_t *__restrict__ bkey,
+                                                   const int32_t *__restrict__ parent,
+                                                   const int32_t *__restrict__ nb27, const int32_t *__restrict__ child8,
+                                                   int pass, int32_t *__restrict__ cnt, const int32_t *__restrict__ off,
+                                                   int32_t *__restrict__ tgt, int32_t *__restrict__ src,
+                                                   uint32_t *__restrict__ cls) {
+    const int b = first + blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (b >= nbox) return;  // uniform in the warp
+    const uint32_t oct = bkey[b] & 7u;
+    const int bx = (oct >> 2) & 1, by = (oct >> 1) & 1, bz = oct & 1;
+    const int32_t *pn = nb27 + (int64_t)parent[b] * 27;
+    int n = 0;
+    const int64_t o = pass ? off[b] : 0;
+    for (int c0 = 0; c0 < 216; c0 += 32) {
+        const int c = c0 + lane;
+        int f = -1, dx = 0, dy = 0, dz = 0;
+        if (c < 216) {
+            // per axis i = 0..5: the parent's neighbour (i >> 1) - 1 and its child i & 1
+            const int ix = c / 36, iy = c / 6 % 6, iz = c % 6;
+            dx = ix - 2 - bx;
+            dy = iy - 2 - by;
+            dz = iz - 2 - bz;
+            if (max(abs(dx), max(abs(dy), abs(dz))) > 1) {
+                const int p = pn[(ix >> 1) * 9 + (iy >> 1) * 3 + (iz >> 1)];
+                if (p >= 0) f = child8[(int64_t)p * 8 + (ix & 1) * 4 + (iy & 1) * 2 + (iz & 1)];
             }
-    if (!pass) cnt[b] = c;
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, f >= 0);
+        if (pass && f >= 0) {
+            const int64_t q = o + n + __popc(m & ((1u << lane) - 1u));
+            tgt[q] = b;
+            src[q] = f;
+            cls[q] = (uint32_t)m2l_class(dx, dy, dz);
+        }
+        n += __popc(m);
+    }
+    if (!pass && lane == 0) cnt[b] = n;
 }
 
 __global__ void k_iota(int64_t n, int32_t *a) {
@@ -481,23 +502,27 @@ __global__ void k_iota(int64_t n, int32_t *a) {
     if (i < n) a[i] = (int32_t)i;
 }
 
-template <class T>
-__global__ void k_gather_i32(int64_t n, const int32_t *__restrict__ idx, const T *__restrict__ in, T *__restrict__ out) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) out[i] = in[idx[i]];
-}
-
-__global__ void k_copy_keys(int64_t n, const int32_t *__restrict__ tgt, uint32_t *__restrict__ key,
-                            int32_t *__restrict__ cnt) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+// the pairs in class-sorted order, and every target-major pair's place in it
+__global__ void k_m2l_order(int64_t n, const int32_t *__restrict__ order, const int32_t *__restrict__ ptgt,
+                            const int32_t *__restrict__ psrc, int32_t *__restrict__ tgt, int32_t *__restrict__ src,
+                            int32_t *__restrict__ by_tgt) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    key[i] = (uint32_t)tgt[i];
-    atomicAdd(&cnt[tgt[i]], 1);
+    const int k = order[i];
+    tgt[i] = ptgt[k];
+    src[i] = psrc[k];
+    by_tgt[k] = (int32_t)i;
 }
 
-__global__ void k_hist_small(int64_t n, const uint32_t *__restrict__ k, int nbins, int32_t *__restrict__ h) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i < n) atomicAdd(&h[k[i]], 1);
+__global__ void __launch_bounds__(256) k_class_hist(int64_t n, const uint32_t *__restrict__ k, int32_t *__restrict__ h) {
+    __shared__ int32_t s[kNumM2LClasses];
+    for (int i = threadIdx.x; i < kNumM2LClasses; i += blockDim.x) s[i] = 0;
+    __syncthreads();
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        atomicAdd(&s[k[i]], 1);
+    __syncthreads();
+    for (int i = threadIdx.x; i < kNumM2LClasses; i += blockDim.x)
+        if (s[i]) atomicAdd(&h[i], s[i]);
 }
 
 // child8[box][8]: the children of every box by octant (the low bits of their keys), -1 where empty
@@ -611,26 +636,25 @@ __global__ void k_back_base(int nleaf, const int32_t *__restrict__ blkoff, int64
 // owned neighbours of A before B in A's list, summed)
 __global__ void k_back_gofs(int nleaf, const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
                             const int32_t *__restrict__ bcount, int32_t *__restrict__ gofs) {
-    const int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b >= nleaf) return;
-    for (int k = 0; k < 27; ++k) {
-        int g = -1;
-        if (k < ncnt[b]) {
-            const int a = nbr[b * 27 + k];
-            if (a < b) {
-                int off = 0;
-                for (int k2 = 0; k2 < ncnt[a]; ++k2) {
-                    const int f = nbr[a * 27 + k2];
-                    if (f == b) {
-                        g = off;
-                        break;
-                    }
-                    if (f > a) off += bcount[f];
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= nleaf * 27) return;
+    const int b = e / 27, k = e % 27;
+    int g = -1;
+    if (k < ncnt[b]) {
+        const int a = nbr[e];
+        if (a < b) {
+            int off = 0;
+            for (int k2 = 0; k2 < ncnt[a]; ++k2) {
+                const int f = nbr[a * 27 + k2];
+                if (f == b) {
+                    g = off;
+                    break;
                 }
+                if (f > a) off += bcount[f];
             }
         }
-        gofs[b * 27 + k] = g;
     }
+    gofs[e] = g;
 }
 
 }  // namespace
@@ -679,14 +703,21 @@ void build_tree(Context &c) {
         DevBuf<int64_t> &dcv = t.s_i64[0];
         DevBuf<double> &cb = t.s_f64[2];
         dcv.resize(c.C + 1);
-        cb.resize(6 * c.C);
+        cb.resize(6 * c.C * CB_PARTS);
         BEM_CUDA(cudaMemcpyAsync(dcv.p, cvoff.data(), (c.C + 1) * sizeof(int64_t), cudaMemcpyHostToDevice, st));
-        k_cluster_bbox<<<(unsigned)c.C, 256, 0, st>>>(dcv.p, N, c.xyz.p, cb.p);
+        k_cluster_bbox<<<(unsigned)(c.C * CB_PARTS), 256, 0, st>>>(dcv.p, N, c.xyz.p, cb.p);
         BEM_LAUNCH_CHECK();
-        std::vector<double> hb(6 * c.C);
+        std::vector<double> hb(6 * c.C * CB_PARTS);
         BEM_CUDA(cudaMemcpyAsync(hb.data(), cb.p, hb.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
         BEM_CUDA(cudaStreamSynchronize(st));
         for (int64_t k = 0; k < c.C; ++k) {
+            // the parts' boxes joined into the first one's place
+            for (int q = 0; q < CB_PARTS; ++q)
+                for (int d = 0; d < 3; ++d) {
+                    const double lo = hb[6 * (k * CB_PARTS + q) + d], hi = hb[6 * (k * CB_PARTS + q) + 3 + d];
+                    hb[6 * k + d] = q ? std::min(hb[6 * k + d], lo) : lo;
+                    hb[6 * k + 3 + d] = q ? std::max(hb[6 * k + 3 + d], hi) : hi;
+                }
             double e = 0.0;
             for (int d = 0; d < 3; ++d) e = std::max(e, hb[6 * k + 3 + d] - hb[6 * k + d]);
             if (!(e > 0.0)) e = 1.0;
@@ -716,11 +747,12 @@ void build_tree(Context &c) {
     DevBuf<int32_t> &lc = t.s_i32[1];
     lc.resize(kDeepLevel + 1);
     BEM_CUDA(cudaMemsetAsync(lc.p, 0, (kDeepLevel + 1) * sizeof(int32_t), st));
-    k_level_counts<<<div_up(N, tb), tb, 0, st>>>(N, t.deep, t.key.p, lc.p);
+    k_level_counts<<<(unsigned)std::min<int64_t>(div_up(N, 256), 1024), 256, 0, st>>>(N, t.deep, t.key.p, lc.p);
     BEM_LAUNCH_CHECK();
     int32_t hc[kDeepLevel + 1] = {};
     BEM_CUDA(cudaMemcpyAsync(hc, lc.p, (t.deep + 1) * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     BEM_CUDA(cudaStreamSynchronize(st));
+    for (int l = 1; l <= t.deep; ++l) hc[l] += hc[l - 1];
     int L = 2;
     const int forced = c.level_override > 0 ? c.level_override : c.prm.fixed_level;
     if (forced > 0) {
@@ -771,7 +803,17 @@ void build_tree(Context &c) {
         BEM_LAUNCH_CHECK();
     }
 
-    // 5. near-field lists at the leaf level
+    // 5. children of every box by octant, neighbours of every box, near-field lists at the leaf level
+    t.child8.resize((size_t)t.nbox * 8);
+    BEM_CUDA(cudaMemsetAsync(t.child8.p, 0xff, (size_t)t.nbox * 8 * sizeof(int32_t), st));
+    k_child8<<<div_up(t.nbox - t.base[1], tb), tb, 0, st>>>(t.base[1], t.nbox, t.bkey.p, t.parent.p, t.child8.p);
+    BEM_LAUNCH_CHECK();
+    DevBuf<int32_t> &nb27 = t.s_i32[17];
+    nb27.resize((size_t)t.nbox * 27);
+    for (int l = 0; l <= L; ++l) {
+        k_nb27<<<div_up((int64_t)t.nb[l] * 27, tb), tb, 0, st>>>(t.nb[l], t.base[l], t.bkey.p, t.parent.p, t.child8.p, nb27.p);
+        BEM_LAUNCH_CHECK();
+    }
     int nleaf = t.nb[L];
     t.nbr.resize((size_t)nleaf * 27);
     t.nbr_cnt.resize(nleaf);
@@ -779,8 +821,8 @@ void build_tree(Context &c) {
     DevBuf<unsigned long long> &pairs = t.s_u64[0];
     pairs.resize(1);
     BEM_CUDA(cudaMemsetAsync(pairs.p, 0, sizeof(unsigned long long), st));
-    k_neighbours<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, L, t.bkey.p + t.base[L], t.bcount.p + t.base[L],
-                                                    t.nbr.p, t.nbr_cnt.p, t.nbr_d.p, pairs.p);
+    k_neighbours<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.base[L], nb27.p, t.bcount.p + t.base[L], t.nbr.p,
+                                                    t.nbr_cnt.p, t.nbr_d.p, pairs.p);
     BEM_LAUNCH_CHECK();
     {
         DevBuf<int32_t> &ucnt = t.s_i32[4], &uoff = t.s_i32[5], &utot = t.s_i32[6];
@@ -804,7 +846,7 @@ void build_tree(Context &c) {
         exclusive_scan_i32(blk.p, blkoff.p, nleaf, utot.p + 1, st);
         k_back_base<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, blkoff.p, t.back_base.p);
         BEM_LAUNCH_CHECK();
-        k_back_gofs<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.nbr.p, t.nbr_cnt.p, t.bcount.p + t.base[L],
+        k_back_gofs<<<div_up((int64_t)nleaf * 27, tb), tb, 0, st>>>(nleaf, t.nbr.p, t.nbr_cnt.p, t.bcount.p + t.base[L],
                                                        t.back_gofs.p);
         BEM_LAUNCH_CHECK();
         int32_t tot2[2] = {0, 0};
@@ -853,56 +895,37 @@ void build_tree(Context &c) {
         }
     }
 
-    // 6. M2L pairs of levels 2..L, then sorted by offset class
-    std::vector<int64_t> lvl_off(L + 2, 0);
-    DevBuf<int32_t> &cnt = t.s_i32[9], &off = t.s_i32[10];
-    std::vector<int32_t> level_tot(L + 1, 0);
-    {
-        size_t maxn = 0;
-        for (int l = 2; l <= L; ++l) maxn = std::max<size_t>(maxn, t.nb[l]);
-        cnt.resize(maxn + 1);
-        off.resize(maxn + 1);
-    }
-    DevBuf<int32_t> &tot = t.s_i32[11];
+    // 6. M2L pairs of levels 2..L: counted, then written target by target (m2l_tgt_off is their CSR)
+    DevBuf<int32_t> &cnt = t.s_i32[9], &tot = t.s_i32[11];
+    cnt.resize((size_t)t.nbox + 1);
     tot.resize(1);
-    for (int l = 2; l <= L; ++l) {
-        int n = t.nb[l];
-        k_m2l_lists<<<div_up(n, tb), tb, 0, st>>>(n, l, t.bkey.p + t.base[l], t.bkey.p + t.base[l - 1], t.nb[l - 1],
-                                                   t.base[l], 0, cnt.p, nullptr, nullptr, nullptr, nullptr);
-        BEM_LAUNCH_CHECK();
-        exclusive_scan_i32(cnt.p, off.p, n, tot.p, st);
-        int32_t h;
-        BEM_CUDA(cudaMemcpyAsync(&h, tot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
-        BEM_CUDA(cudaStreamSynchronize(st));
-        level_tot[l] = h;
-    }
-    int64_t nm2l = 0;
-    for (int l = 2; l <= L; ++l) {
-        lvl_off[l] = nm2l;
-        nm2l += level_tot[l];
-    }
+    t.m2l_tgt_off.resize((size_t)t.nbox + 1);
+    BEM_CUDA(cudaMemsetAsync(cnt.p, 0, ((size_t)t.nbox + 1) * sizeof(int32_t), st));
+    const int first2 = t.base[2], lgrid = div_up(t.nbox - first2, 8);
+    k_m2l_lists<<<lgrid, 256, 0, st>>>(first2, t.nbox, t.bkey.p, t.parent.p, nb27.p, t.child8.p, 0, cnt.p, nullptr, nullptr,
+                                       nullptr, nullptr);
+    BEM_LAUNCH_CHECK();
+    exclusive_scan_i32(cnt.p, t.m2l_tgt_off.p, (int64_t)t.nbox + 1, tot.p, st);
+    int32_t hm2l = 0;
+    BEM_CUDA(cudaMemcpyAsync(&hm2l, tot.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    BEM_CUDA(cudaStreamSynchronize(st));
+    const int64_t nm2l = hm2l;
     t.n_m2l = nm2l;
     DevBuf<int32_t> &ptgt = t.s_i32[12], &psrc = t.s_i32[13];
     DevBuf<uint32_t> &pcls = t.m2l_cls;  // sorted in place below: the class of every sorted pair
     ptgt.resize(nm2l);
     psrc.resize(nm2l);
     pcls.resize(std::max<int64_t>(nm2l, 1));
-    for (int l = 2; l <= L; ++l) {
-        int n = t.nb[l];
-        if (!level_tot[l]) continue;
-        k_m2l_lists<<<div_up(n, tb), tb, 0, st>>>(n, l, t.bkey.p + t.base[l], t.bkey.p + t.base[l - 1], t.nb[l - 1],
-                                                   t.base[l], 0, cnt.p, nullptr, nullptr, nullptr, nullptr);
-        BEM_LAUNCH_CHECK();
-        exclusive_scan_i32(cnt.p, off.p, n, nullptr, st);
-        k_m2l_lists<<<div_up(n, tb), tb, 0, st>>>(n, l, t.bkey.p + t.base[l], t.bkey.p + t.base[l - 1], t.nb[l - 1],
-                                                   t.base[l], 1, nullptr, off.p, ptgt.p + lvl_off[l],
-                                                   psrc.p + lvl_off[l], pcls.p + lvl_off[l]);
-        BEM_LAUNCH_CHECK();
-    }
     t.m2l_src.resize(nm2l);
     t.m2l_tgt.resize(nm2l);
+    t.m2l_by_tgt.resize(std::max<int64_t>(nm2l, 1));
     t.m2l_class_off.assign(kNumM2LClasses + 1, 0);
     if (nm2l > 0) {
+        k_m2l_lists<<<lgrid, 256, 0, st>>>(first2, t.nbox, t.bkey.p, t.parent.p, nb27.p, t.child8.p, 1, nullptr,
+                                           t.m2l_tgt_off.p, ptgt.p, psrc.p, pcls.p);
+        BEM_LAUNCH_CHECK();
+        // 7. sorted by offset class (stable: ascending target within a class). A target's pairs were
+        // written by ascending class, so their places in the sorted order ascend as well.
         DevBuf<int32_t> &order = t.s_i32[14], &otmp = t.s_i32[15];
         DevBuf<uint32_t> &ctmp = t.s_u32[1];
         order.resize(nm2l);
@@ -911,13 +934,12 @@ void build_tree(Context &c) {
         DevBuf<int32_t> &hist = t.s_i32[16];
         hist.resize(kNumM2LClasses);
         BEM_CUDA(cudaMemsetAsync(hist.p, 0, kNumM2LClasses * sizeof(int32_t), st));
-        k_hist_small<<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, pcls.p, kNumM2LClasses, hist.p);
+        k_class_hist<<<(unsigned)std::min<int64_t>(div_up(nm2l, 1024), 608), 256, 0, st>>>(nm2l, pcls.p, hist.p);
         BEM_LAUNCH_CHECK();
         k_iota<<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, order.p);
         BEM_LAUNCH_CHECK();
         radix_sort_u32(pcls.p, order.p, nm2l, 9, ctmp.p, otmp.p, st);
-        k_gather_i32<int32_t><<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, order.p, psrc.p, t.m2l_src.p);
-        k_gather_i32<int32_t><<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, order.p, ptgt.p, t.m2l_tgt.p);
+        k_m2l_order<<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, order.p, ptgt.p, psrc.p, t.m2l_tgt.p, t.m2l_src.p, t.m2l_by_tgt.p);
         BEM_LAUNCH_CHECK();
         std::vector<int32_t> hh(kNumM2LClasses);
         BEM_CUDA(cudaMemcpyAsync(hh.data(), hist.p, kNumM2LClasses * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -925,38 +947,7 @@ void build_tree(Context &c) {
         for (int k = 0; k < kNumM2LClasses; ++k) t.m2l_class_off[k + 1] = t.m2l_class_off[k] + hh[k];
     }
 
-    // 7. children of every box by octant (M2M, L2L)
-    t.child8.resize((size_t)t.nbox * 8);
-    BEM_CUDA(cudaMemsetAsync(t.child8.p, 0xff, (size_t)t.nbox * 8 * sizeof(int32_t), st));
-    k_child8<<<div_up(t.nbox - t.base[1], tb), tb, 0, st>>>(t.base[1], t.nbox, t.bkey.p, t.parent.p, t.child8.p);
-    BEM_LAUNCH_CHECK();
-
-    // 8. target-major CSR of the M2L pairs (stable: ascending pair index)
-    {
-        DevBuf<int32_t> &off = t.m2l_tgt_off, &by = t.m2l_by_tgt;
-        off.resize((size_t)t.nbox + 1);
-        by.resize(nm2l > 0 ? nm2l : 1);
-        DevBuf<int32_t> &cnt2 = t.s_i32[20];
-        cnt2.resize((size_t)t.nbox + 1);
-        BEM_CUDA(cudaMemsetAsync(cnt2.p, 0, ((size_t)t.nbox + 1) * sizeof(int32_t), st));
-        if (nm2l > 0) {
-            DevBuf<uint32_t> &k = t.s_u32[4], &ktmp2 = t.s_u32[5];
-            DevBuf<int32_t> &vtmp2 = t.s_i32[21];
-            k.resize(nm2l);
-            ktmp2.resize(nm2l);
-            vtmp2.resize(nm2l);
-            k_copy_keys<<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, t.m2l_tgt.p, k.p, cnt2.p);
-            BEM_LAUNCH_CHECK();
-            k_iota<<<div_up(nm2l, tb), tb, 0, st>>>(nm2l, by.p);
-            BEM_LAUNCH_CHECK();
-            int bits = 1;
-            while ((1ll << bits) <= (long long)t.nbox) ++bits;
-            radix_sort_u32(k.p, by.p, nm2l, bits, ktmp2.p, vtmp2.p, st);
-        }
-        exclusive_scan_i32(cnt2.p, off.p, (int64_t)t.nbox + 1, nullptr, st);
-    }
-
-    // 9. sorted point data
+    // 8. sorted point data
     t.loc64.resize(3 * N);
     t.loc32.resize(3 * N);
     t.nrm64.resize(3 * N);
