@@ -350,6 +350,7 @@ struct Context {
         DevBuf<float> part;              // [items][256][N_pad] partial local expansions
         DevBuf<int32_t> s_i32[9];        // scratch of the table build (kept between builds)
         DevBuf<uint32_t> s_u32[2];
+        DevBuf<uint8_t> has;
     };
     TmState tm[2];
     DevBuf<int> tc_err;              // set by a tensor-core block whose wait ran out

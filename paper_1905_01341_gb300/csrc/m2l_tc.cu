@@ -99,12 +99,17 @@ struct TcLayout {
     size_t stage_bytes, total;
 };
 
+// Row stride (floats) of the epilogue's tile in shared memory: 4 past a multiple of 16, so that the
+// eight rows of a 16-byte store phase fall in different banks (a stride of 256, p = 16, put all of
+// them in one: EPI1)
+__host__ __device__ constexpr int epi_stride(int Npad) { return Npad + 4; }
+
 // ST pipeline stages and three mbarriers per stage (empty, full, bfull); the epilogue reuses
-// the stages for one tile of FP32 rows (at most N_pad floats each)
+// the stages for one tile of FP32 rows
 __host__ __device__ inline TcLayout tc_layout(int Npad, int ST) {
     TcLayout L;
     L.stage_bytes = TC_STAGE_BYTES;
-    const size_t epi = (size_t)TC_M * Npad * 4;
+    const size_t epi = (size_t)TC_M * epi_stride(Npad) * 4;
     L.total = (ST * L.stage_bytes > epi ? ST * L.stage_bytes : epi) + 3 * ST * 8 + 16 + 1024;
     return L;
 }
@@ -122,7 +127,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     // 1024-byte aligned base for the operand stages
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const TcLayout Lo = tc_layout(Npad, TC_STAGES);
-    const size_t epi_bytes = (size_t)TC_M * Npad * 4;
+    const size_t epi_bytes = (size_t)TC_M * epi_stride(Npad) * 4;
     uint64_t *empty = reinterpret_cast<uint64_t *>(
         smem + (TC_STAGES * Lo.stage_bytes > epi_bytes ? TC_STAGES * Lo.stage_bytes : epi_bytes));
     uint64_t *full = empty + TC_STAGES;  // NPROD producer arrivals per use (the gathered A rows)
@@ -278,17 +283,17 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (ok) {
         // epilogue, one tile at a time: warp w holds TMEM lanes 32w..32w+31 = tile rows; each
-        // thread moves its row into shared memory (row stride P floats: conflict-free 16-byte
-        // stores), then the block writes the tile's rows, which are contiguous in Ypair, with
-        // coalesced 16-byte stores
+        // thread moves its row into shared memory, then each warp writes whole rows of Ypair with
+        // coalesced 16-byte stores (the first Kc coefficients; the per-target sums read no more)
+        const int es = epi_stride(Npad), kw = min(Kc, P) / 4;
         float *stage = reinterpret_cast<float *>(smem);  // the operand stages are free now
         for (int t = 0; t < ntiles; ++t) {
             const int rows_t = min(TC_M, nrows - t * TC_M);
             // a warp reads its own quarter of the TMEM lanes (warp % 4); the two warp groups take
             // the lower and the upper half of the 16-column groups
             const int q4 = warp & 3, half = warp >> 2;
-            const int ngroups = Npad / 16, g0 = half ? (ngroups + 1) / 2 : 0, g1 = half ? ngroups : (ngroups + 1) / 2;
-            float *srow = stage + (size_t)(q4 * 32 + lane) * P;
+            const int ngroups = Kc / 16, g0 = half ? (ngroups + 1) / 2 : 0, g1 = half ? ngroups : (ngroups + 1) / 2;
+            float *srow = stage + (size_t)(q4 * 32 + lane) * es;
             for (int c0 = g0 * 16; c0 < g1 * 16; c0 += 16) {
                 if (c0 >= Kc) continue;  // beyond the class's truncation: neither computed nor stored
                 uint32_t v[16];
@@ -310,16 +315,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
             }
             __syncthreads();
             float4 *dst = reinterpret_cast<float4 *>(Ypair + ((size_t)ch.start * R + t * TC_M) * P);
-            const float4 *src = reinterpret_cast<const float4 *>(stage);
-            if (Kc >= P) {
-                const int n4 = rows_t * P / 4;
-                for (int e = tid; e < n4; e += TC_THREADS) dst[e] = src[e];
-            } else {  // the first Kc coefficients of each row; the per-target sums read no more
-                const int k4 = Kc / 4, p4 = P / 4;
-                for (int e = tid; e < rows_t * k4; e += TC_THREADS) {
-                    const int row = e / k4, col = e - row * k4;
-                    dst[row * p4 + col] = src[row * p4 + col];
-                }
+            for (int row = warp; row < rows_t; row += TC_THREADS / 32) {
+                const float4 *src = reinterpret_cast<const float4 *>(stage + (size_t)row * es);
+                for (int col = lane; col < kw; col += 32) dst[(size_t)row * (P / 4) + col] = src[col];
             }
             __syncthreads();
         }
@@ -452,25 +450,24 @@ __device__ __forceinline__ int tm_scan(int v, int *warp_tot) {
     for (int i = 0; i < w; ++i) v += warp_tot[i];
     return v;
 }
+// which classes a tile has: a warp per (tile, class) looks through the class's slots
+__global__ void __launch_bounds__(256) k_tm_has(int64_t n, int TT, const int32_t *__restrict__ tab, uint8_t *__restrict__ has) {
+    const int64_t e = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (e >= n) return;
+    const int lane = threadIdx.x & 31;
+    bool f = false;
+    for (int r = lane; r < TT; r += 32) f = f || tab[e * TT + r] >= 0;
+    const unsigned any = __ballot_sync(0xffffffffu, f);
+    if (lane == 0) has[e] = any != 0;
+}
 // per tile, the classes present, in the order `order` (truncated size ascending), and their cost
-__global__ void __launch_bounds__(512) k_tm_classes(int TT, const int32_t *__restrict__ tab,
-                                                    const int32_t *__restrict__ order,
+__global__ void __launch_bounds__(512) k_tm_classes(const uint8_t *__restrict__ has, const int32_t *__restrict__ order,
                                                     const int32_t *__restrict__ cls_K, int Npad,
                                                     int32_t *__restrict__ tcls, int32_t *__restrict__ ncls,
                                                     int32_t *__restrict__ cost) {
     __shared__ int warp_tot[16];
-    __shared__ uint8_t has[512];
-    const int tile = blockIdx.x, k = threadIdx.x, lane = k & 31;
-    // a warp per class: its 32 lanes look through the class's slots together
-    for (int q = k >> 5; q < kNumM2LClasses; q += 16) {
-        const int32_t *col = tab + ((int64_t)tile * kNumM2LClasses + order[q]) * TT;
-        bool f = false;
-        for (int r = lane; r < TT; r += 32) f = f || col[r] >= 0;
-        const unsigned any = __ballot_sync(0xffffffffu, f);
-        if (lane == 0) has[q] = any != 0;
-    }
-    __syncthreads();
-    const int f = k < kNumM2LClasses && has[k];
+    const int tile = blockIdx.x, k = threadIdx.x;
+    const int f = k < kNumM2LClasses && has[(int64_t)tile * kNumM2LClasses + order[k]];
     const int idx = tm_scan(f, warp_tot);  // inclusive
     if (f) tcls[(int64_t)tile * kNumM2LClasses + idx - 1] = order[k];
     const int c = tm_scan(f ? tm_cost(cls_K ? cls_K[order[k]] : Npad) : 0, warp_tot);
@@ -565,7 +562,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const size_t stage_bytes = TM_STAGE_BYTES;
-    const size_t epi_bytes = (size_t)TC_M * Npad * 4;
+    const size_t epi_bytes = (size_t)TC_M * epi_stride(Npad) * 4;
     uint64_t *empty = reinterpret_cast<uint64_t *>(
         smem + (TC_STAGES * stage_bytes > epi_bytes ? TC_STAGES * stage_bytes : epi_bytes));
     uint64_t *full = empty + TC_STAGES;
@@ -750,10 +747,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
         // the item's partial (the first kmax coefficients; the rest of the row is never read)
         float *stage = reinterpret_cast<float *>(smem);
         float *dst_item = part + (size_t)blockIdx.x * TM_ROWS * Npad;
+        const int es = epi_stride(Npad), kw = kmax / 4, n4 = Npad / 4;
         for (int t = 0; t < 2; ++t) {
             const int q4 = warp & 3, half = warp >> 2;
             const int ngroups = kmax / 16, g0 = half ? (ngroups + 1) / 2 : 0, g1 = half ? ngroups : (ngroups + 1) / 2;
-            float *srow = stage + (size_t)(q4 * 32 + lane) * Npad;
+            float *srow = stage + (size_t)(q4 * 32 + lane) * es;
             for (int c0 = g0 * 16; c0 < g1 * 16; c0 += 16) {
                 uint32_t v[16];
                 const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)t * 256u + (uint32_t)c0;
@@ -772,12 +770,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
                                     __uint_as_float(v[i + 3]));
             }
             __syncthreads();
-            const int k4 = kmax / 4, n4 = Npad / 4;
             float4 *dst = reinterpret_cast<float4 *>(dst_item + (size_t)t * TC_M * Npad);
-            const float4 *src = reinterpret_cast<const float4 *>(stage);
-            for (int e = tid; e < TC_M * k4; e += TC_THREADS) {
-                const int row = e / k4, col = e - row * k4;
-                dst[row * n4 + col] = src[row * n4 + col];
+            for (int row = warp; row < TC_M; row += TC_THREADS / 32) {
+                const float4 *src = reinterpret_cast<const float4 *>(stage + (size_t)row * es);
+                for (int col = lane; col < kw; col += 32) dst[(size_t)row * n4 + col] = src[col];
             }
             __syncthreads();
         }
@@ -853,7 +849,11 @@ static void build_tm_tables(Context &c, const Operators &o, cudaStream_t st) {
     const int32_t *clsK = o.margin >= 0 ? o.cls_K.p : nullptr;
     DevBuf<int32_t> &cost = S.s_i32[8];
     cost.resize(ntiles);
-    k_tm_classes<<<(unsigned)ntiles, 512, 0, st>>>(TT, S.src.p, dorder.p, clsK, P16, S.cls.p, ncls.p, cost.p);
+    const int64_t nhas = ntiles * kNumM2LClasses;
+    S.has.resize(std::max<int64_t>(nhas, 1));
+    k_tm_has<<<div_up(nhas, 8), 256, 0, st>>>(nhas, TT, S.src.p, S.has.p);
+    BEM_LAUNCH_CHECK();
+    k_tm_classes<<<(unsigned)ntiles, 512, 0, st>>>(S.has.p, dorder.p, clsK, P16, S.cls.p, ncls.p, cost.p);
     BEM_LAUNCH_CHECK();
     std::vector<int32_t> hcost(ntiles);
     BEM_CUDA(cudaMemcpyAsync(hcost.data(), cost.p, ntiles * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -902,7 +902,7 @@ void launch_m2l_tm(Context &c, const Operators &o, const float *X, int64_t xrows
     __nv_bfloat16 *xs = split_multipoles(c, o, X, xrows, st);
     if (S.nitems == 0) return;
     const int stages = 3;
-    const size_t epi = (size_t)TC_M * Npad * 4;
+    const size_t epi = (size_t)TC_M * epi_stride(Npad) * 4;
     const size_t sm = (stages * TM_STAGE_BYTES > epi ? stages * TM_STAGE_BYTES : epi) + 3 * stages * 8 + 16 + 1024;
     BEM_CUDA(cudaFuncSetAttribute(k_m2l_tm<R, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     k_m2l_tm<R, 3><<<(unsigned)S.nitems, TC_THREADS, sm, st>>>(
