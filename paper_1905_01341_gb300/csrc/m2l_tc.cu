@@ -2,12 +2,12 @@
 //
 // For one offset class c and a chunk of (source, target) pairs, the product
 //   Y[pair, rhs][n] = sum_k T_c[n][k] X[src, rhs][k]
-// is up to four MMA tiles D_t = A_t B^T with M = 128 rows (pair, rhs) each, N = K = K_c, the
+// is up to three MMA tiles D_t = A_t B^T with M = 128 rows (pair, rhs) each, N = K = K_c, the
 // class's truncated size (p_c^2 rounded up to 16; P rounded up without truncation):
 // A_t = gathered multipole rows, B = T_c (row n of T_c is K-contiguous, i.e. K-major). The
 // tiles share every staged block of T_c, which divides its traffic; a chunk of a class with
-// K_c <= 128 has four tiles (TMEM columns 128 apart), the others two (256 apart), so the small
-// truncated classes amortise a block's set-up and pipeline fill over twice the rows.
+// K_c <= 128 has three tiles (TMEM columns 128 apart), the others two (256 apart), so the small
+// truncated classes amortise a block's set-up and pipeline fill over more rows.
 //
 // Accuracy: both operands are split into three BF16 pieces, x = x0 + x1 + x2 (x0 = bf16(x),
 // x1 = bf16(x - x0), x2 = bf16(x - x0 - x1)), and D accumulates in FP32 the six products with
@@ -18,9 +18,17 @@
 // build from its FP64 values; the multipoles are split once per product (k_split_x).
 //
 // Data movement: K advances 16 at a time (one kind::f16 MMA); each 16-wide K step is one
-// pipeline stage holding A (3 pieces x tiles x 128 x 16) and B (3 pieces x N_pad x 16) in
-// the canonical K-major layout without swizzle (8-row x 16-byte core matrices, K-adjacent core
-// matrices 128 B apart, 8-row groups 256 B apart). The block is warp-specialised: warps 1-7
+// pipeline stage holding A (tiles x 128 rows) and B (3 pieces x N_pad x 16). B has the canonical
+// K-major layout without swizzle (8-row x 16-byte core matrices, K-adjacent core matrices 128 B
+// apart, 8-row groups 256 B apart). The split multipoles lie in memory as they are gathered: per box
+// and right-hand side, per K step, the three pieces side by side in one 128-byte line (96 bytes
+// used); A keeps them so, one 128-byte row per tile row in the 128-byte-swizzled K-major layout (16-byte
+// unit u of row r at u ^ (r % 8)), and an MMA takes piece i by starting 32 i bytes into the rows. A
+// gathered line then arrives in one shared-memory write. With a plane per piece and no swizzle a
+// line brought one 32-byte sector whose halves fell into the same banks: 1536 writes per K step
+// against about 1200 operand reads, which filled the shared-memory pipe to 93 % (M2L of 192600
+// points 144 against 128 us, of 3.21M points 1268 against 963, of the diagonal product at 963000
+// points 3303 against 2908). The block is warp-specialised: warps 1-7
 // fill the stages with cp.async (16-byte copies; rows past the chunk read as zeros), three
 // stages deep (two on request), and let each stage's "full"
 // mbarrier count their copies' arrival (cp.async.mbarrier.arrive.noinc); one thread of warp 0
@@ -42,11 +50,14 @@ namespace bem {
 namespace {
 
 constexpr int TC_M = 128;        // rows per tile
-constexpr int TC_MAXT = 4;       // tiles per block at most (same class, shared B stages)
-constexpr int TC_SMALL_K = 128;  // classes truncated to at most this size take four tiles per block
-// bytes of one pipeline stage: A (3 pieces x tiles x 128 x 16 BF16) and B (3 pieces x K_c x 16),
-// for four tiles with K_c <= 128 or two tiles with K_c <= 256 (the larger of the two)
-constexpr size_t TC_STAGE_BYTES = 3 * 4 * TC_M * 16 * 2 + 3 * 128 * 16 * 2;
+constexpr int TC_MAXT = 3;       // tiles per block at most (same class, shared B stages)
+constexpr int TC_SMALL_K = 128;  // classes truncated to at most this size take three tiles per block
+constexpr uint32_t TC_AROW = 128;           // bytes of one row of A: the three pieces of a K step
+constexpr uint32_t TC_ATILE = TC_M * TC_AROW;
+// bytes of one pipeline stage: A and B (3 pieces x K_c x 16), for three tiles with K_c <= 128 or two
+// tiles with K_c <= 256 (the larger of the two)
+constexpr size_t TC_STAGE_BYTES = 3 * TC_ATILE + 3 * 128 * 16 * 2;
+static_assert(TC_STAGE_BYTES >= 2 * TC_ATILE + 3 * 256 * 16 * 2 && TC_STAGE_BYTES % 1024 == 0, "both forms fit");
 constexpr int TC_THREADS = 256;  // 8 warps: two warp groups share the loads and the epilogue
 
 // Row-major T_c [P][P] (FP64) -> per class, per 16-wide K step, per piece, an N_pad x 16
@@ -75,11 +86,13 @@ __global__ void k_build_tc_table(int P, int Npad, const double *__restrict__ T, 
     }
 }
 
-// Multipoles X [rows][P] (FP32, P a multiple of 4) -> three BF16 planes [3][rows][Kp], zero-padded to
-// Kp; one thread per four coefficients.
+// Multipoles X [rows][P] (FP32, P a multiple of 4) -> Xs [rows][Kp / 16][64]: per K step the three
+// BF16 pieces of 16 coefficients each (zero-padded to Kp) and 16 unused elements; one thread per four
+// coefficients.
+constexpr int XS_STEP = 64;   // elements per row and K step
+constexpr int XS_UNITS = 6;   // 16-byte units of it that are used: (piece, 8-coefficient half)
 __global__ void k_split_x(int64_t rows, int P, int Kp, const float *__restrict__ X, __nv_bfloat16 *__restrict__ Xs) {
     const int quads = Kp / 4;
-    const int64_t plane = rows * Kp;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < rows * quads; e += (int64_t)gridDim.x * blockDim.x) {
         const int64_t r = e / quads;
         const int k = (int)(e - r * quads) * 4;
@@ -89,11 +102,21 @@ __global__ void k_split_x(int64_t rows, int P, int Kp, const float *__restrict__
         alignas(8) __nv_bfloat16 b[3][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) split3_f(x[i], b[0][i], b[1][i], b[2][i]);
+        __nv_bfloat16 *o = Xs + (r * (Kp / TC_K) + k / TC_K) * XS_STEP + k % TC_K;
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
-            *reinterpret_cast<uint2 *>(Xs + c * plane + r * Kp + k) = *reinterpret_cast<const uint2 *>(b[c]);
+        for (int c = 0; c < 3; ++c) *reinterpret_cast<uint2 *>(o + c * TC_K) = *reinterpret_cast<const uint2 *>(b[c]);
     }
 }
+
+// operand A of one K step and piece: rows of 128 bytes, 128-byte swizzle, K-major (8-row groups 1024 B
+// apart); the tile starts on a 1024-byte boundary
+__device__ __forceinline__ uint64_t make_desc_a(uint32_t tile, int piece) {
+    const uint32_t a = tile + 32u * piece;
+    return (uint64_t)((a & 0x3FFFFu) >> 4) | (uint64_t)1 << 16 | (uint64_t)(1024 >> 4) << 32 | (uint64_t)1 << 46 |
+           (uint64_t)2 << 61;
+}
+// byte offset of unit `u` of row `row` within A
+__device__ __forceinline__ uint32_t a_unit(int row, int u) { return (uint32_t)row * TC_AROW + (uint32_t)((u ^ (row & 7)) << 4); }
 
 struct TcLayout {
     size_t stage_bytes, total;
@@ -101,7 +124,7 @@ struct TcLayout {
 
 // Row stride (floats) of the epilogue's tile in shared memory: 4 past a multiple of 16, so that the
 // eight rows of a 16-byte store phase fall in different banks (a stride of 256, p = 16, put all of
-// them in one: EPI1)
+// them in one: 3.77 against 3.30 ms for the diagonal product at 963000 points)
 __host__ __device__ constexpr int epi_stride(int Npad) { return Npad + 4; }
 
 // ST pipeline stages and three mbarriers per stage (empty, full, bfull); the epilogue reuses
@@ -120,7 +143,7 @@ __host__ __device__ inline int tc_tiles_for(int Kc) { return Kc <= TC_SMALL_K ? 
 template <int R, int TC_STAGES>
 __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __nv_bfloat16 *__restrict__ tcB,
                                                        const XChunk *__restrict__ chunks,
-                                                       const int32_t *__restrict__ srcs, int64_t xrows,
+                                                       const int32_t *__restrict__ srcs,
                                                        const __nv_bfloat16 *__restrict__ Xs, float *__restrict__ Ypair,
                                                        const int32_t *__restrict__ cls_K, int *__restrict__ err) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -144,7 +167,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     const int nrows = ch.count * R;
     const int ntiles = (nrows + TC_M - 1) / TC_M;
     // the class's truncated size (a multiple of 16, <= Npad): K steps and output columns; small
-    // classes take four tiles per block (TMEM columns 128 apart), the others two (256 apart)
+    // classes take three tiles per block (TMEM columns 128 apart), the others two (256 apart)
     const int Kc = cls_K ? cls_K[ch.cls] : Npad;
     const int nsteps = Kc / TC_K;
     const int tcap = tc_tiles_for(Kc);
@@ -169,12 +192,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = *tmem_slot;
     const uint32_t idesc = make_idesc(TC_M, Kc);
-    const int Kp = Npad;
-    const int64_t plane = xrows * Kp;
+    const int xrow = Npad / TC_K * XS_STEP;  // elements of one row of Xs
     const __nv_bfloat16 *Bc = tcB + (size_t)ch.cls * (Npad / TC_K) * 3 * Npad * TC_K;  // the class's full table
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t atile = TC_M * TC_K * 2, apiece = (uint32_t)tcap * atile;
-    const uint32_t a_bytes = 3 * apiece;
+    const uint32_t a_bytes = (uint32_t)tcap * TC_ATILE;
     const uint32_t bpiece = (uint32_t)Kc * TC_K * 2;        // one piece's K_c rows in shared memory
     const size_t bpiece_g = (size_t)Npad * TC_K * 2;        // one piece's block in the table
 
@@ -204,14 +225,14 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
                 const uint32_t sb = sa + a_bytes;
                 for (int t = 0; t < ntiles; ++t) {
                     const uint32_t d = tmem + (uint32_t)t * colstride;
-                    const uint32_t a0 = sa + t * atile;
+                    const uint32_t at = sa + t * TC_ATILE;
                     // smallest terms first: (2,0) (1,1) (0,2) (1,0) (0,1) (0,0)
-                    mma_bf16(d, make_desc(a0 + 2 * apiece), make_desc(sb), idesc, ks > 0 ? 1u : 0u);
-                    mma_bf16(d, make_desc(a0 + apiece), make_desc(sb + bpiece), idesc, 1u);
-                    mma_bf16(d, make_desc(a0), make_desc(sb + 2 * bpiece), idesc, 1u);
-                    mma_bf16(d, make_desc(a0 + apiece), make_desc(sb), idesc, 1u);
-                    mma_bf16(d, make_desc(a0), make_desc(sb + bpiece), idesc, 1u);
-                    mma_bf16(d, make_desc(a0), make_desc(sb), idesc, 1u);
+                    mma_bf16(d, make_desc_a(at, 2), make_desc(sb), idesc, ks > 0 ? 1u : 0u);
+                    mma_bf16(d, make_desc_a(at, 1), make_desc(sb + bpiece), idesc, 1u);
+                    mma_bf16(d, make_desc_a(at, 0), make_desc(sb + 2 * bpiece), idesc, 1u);
+                    mma_bf16(d, make_desc_a(at, 1), make_desc(sb), idesc, 1u);
+                    mma_bf16(d, make_desc_a(at, 0), make_desc(sb + bpiece), idesc, 1u);
+                    mma_bf16(d, make_desc_a(at, 0), make_desc(sb), idesc, 1u);
                 }
                 mma_commit(smem_u32(&empty[st]));
             }
@@ -220,20 +241,17 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
         __syncwarp();
     } else {
         const int pt = tid - 32;
-        // this thread's A copies, fixed for the block: unit u = (tile row, 8-element half j) of every
-        // K step; its three pieces are one plane apart in Xs and one piece block apart in a stage
-        constexpr int AU = (TC_MAXT * TC_M * 2 + NPROD - 1) / NPROD;
+        // this thread's A copies, fixed for the block: unit pt % 6 = (piece, 8-element half) of the rows
+        // pt / 6 + PROWS i of every K step (six neighbouring lanes read one row's line)
+        constexpr int PROWS = NPROD / XS_UNITS, AU = (TC_MAXT * TC_M + PROWS - 1) / PROWS;
         const int arows = ntiles * TC_M;
-        const __nv_bfloat16 *a_src[AU];
-        uint32_t a_dst[AU], a_sz[AU];
+        const int unit = pt % XS_UNITS, row0 = pt < PROWS * XS_UNITS ? pt / XS_UNITS : arows;  // the rest copies nothing
+        int a_row[AU];  // row of Xs, -1: a zero row
 #pragma unroll
         for (int i = 0; i < AU; ++i) {
-            const int u = pt + i * NPROD;
-            const int j = u & 1, row2 = u >> 1;
-            const int s = u < 2 * arows ? s_src[row2] : -1;
-            a_src[i] = Xs + ((size_t)(s >= 0 ? s : 0) * R + row2 % R) * Kp + j * 8;
-            a_dst[i] = (uint32_t)((row2 / TC_M) * atile + kmajor_off(row2 % TC_M, j * 8) * 2);
-            a_sz[i] = s >= 0 ? 16u : 0u;  // rows past the chunk: zeros, nothing read
+            const int row2 = row0 + i * PROWS;
+            const int s = row2 < arows ? s_src[row2] : -1;
+            a_row[i] = s >= 0 ? s * R + row2 % R : -1;
         }
         const bool bulk = pt == 0;
         int issued = -1;  // last K step whose block of T_c this thread requested
@@ -256,16 +274,12 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
                     bulk_g2s(sa + a_bytes + piece * bpiece, bsrc + (size_t)piece * bpiece_g, bpiece, bb);
                 issued = ks;
             }
+            const __nv_bfloat16 *xk = Xs + unit * 8 + ks * XS_STEP;
 #pragma unroll
-            for (int i = 0; i < AU; ++i) {
-                if (pt + i * NPROD < 2 * arows) {
-                    const __nv_bfloat16 *src = a_src[i] + ks * TC_K;
-                    const uint32_t dst = sa + a_dst[i];
-                    cp_async16(dst, src, a_sz[i]);
-                    cp_async16(dst + apiece, src + plane, a_sz[i]);
-                    cp_async16(dst + 2 * apiece, src + 2 * plane, a_sz[i]);
-                }
-            }
+            for (int i = 0; i < AU; ++i)
+                if (row0 + i * PROWS < arows)
+                    cp_async16(sa + a_unit(row0 + i * PROWS, unit), xk + (int64_t)max(a_row[i], 0) * xrow,
+                               a_row[i] >= 0 ? 16u : 0u);
             asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[st])) : "memory");
         }
         cp_async_wait<0>();  // nothing of this thread in flight past this point
@@ -349,7 +363,7 @@ void build_tc_tables(Context &c, Operators &o) {
 // the multipoles, split once for all translations of a product
 static __nv_bfloat16 *split_multipoles(Context &c, const Operators &o, const float *X, int64_t xrows, cudaStream_t st) {
     const int Npad = o.tc_Npad;
-    c.xsplit.resize((size_t)3 * xrows * Npad);
+    c.xsplit.resize((size_t)xrows * (Npad / TC_K) * XS_STEP);
     __nv_bfloat16 *xs = reinterpret_cast<__nv_bfloat16 *>(c.xsplit.p);
     const int nb = (int)std::min<int64_t>(div_up(xrows * (Npad / 4), 256), 152 * 16);
     k_split_x<<<nb, 256, 0, st>>>(xrows, o.P, Npad, X, xs);
@@ -370,7 +384,7 @@ void launch_m2l_tc(Context &c, const Operators &o, const XChunk *chunks, int64_t
     // set on every launch: the attribute belongs to the current device (~1 us against a ms kernel)
     BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     kern<<<(unsigned)nchunks, TC_THREADS, sm, st>>>(o.P, Npad, reinterpret_cast<const __nv_bfloat16 *>(o.m2l_tc.p),
-                                                   chunks, c.tree.m2l_src.p, xrows, xs, Ypair,
+                                                   chunks, c.tree.m2l_src.p, xs, Ypair,
                                                    o.margin >= 0 ? o.cls_K.p : nullptr, err);
     BEM_LAUNCH_CHECK();
 }
@@ -401,7 +415,7 @@ namespace {
 
 constexpr int TM_ROWS = 2 * TC_M;  // rows per tile: (target, rhs)
 constexpr int TM_MAXCLS = 32;      // classes per item at most (an item's cost limits them before)
-constexpr size_t TM_STAGE_BYTES = 3 * TM_ROWS * 16 * 2 + 3 * 256 * 16 * 2;  // A (two tiles) + B (K_c <= 256)
+constexpr size_t TM_STAGE_BYTES = 2 * TC_ATILE + 3 * 256 * 16 * 2;  // A (two tiles) + B (K_c <= 256)
 
 // target boxes: the boxes of levels 2.. with at least one M2L translation, key = octant
 __global__ void k_tm_flags(int64_t first, int64_t n, const int32_t *__restrict__ tgt_off, int32_t *__restrict__ flag) {
@@ -555,7 +569,7 @@ __global__ void k_tm_reduce(int P, int Npad, const int32_t *__restrict__ tm_box,
 template <int R, int TC_STAGES>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const __nv_bfloat16 *__restrict__ tcB,
                                                        const int4 *__restrict__ items, const int32_t *__restrict__ tab,
-                                                       const int32_t *__restrict__ tcls, int64_t xrows,
+                                                       const int32_t *__restrict__ tcls,
                                                        const __nv_bfloat16 *__restrict__ Xs, float *__restrict__ part,
                                                        const int32_t *__restrict__ cls_K, int *__restrict__ err) {
     constexpr int TT = TM_ROWS / R;  // target slots per tile
@@ -618,11 +632,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
     }
     int nsteps = 0;
     for (int j = 0; j < nc; ++j) nsteps += s_K[j] / TC_K;
-    const int Kp = Npad;
-    const int64_t plane = xrows * Kp;
+    const int xrow = Npad / TC_K * XS_STEP;  // elements of one row of Xs
     const uint32_t sbase = smem_u32(smem);
-    const uint32_t atile = TC_M * TC_K * 2, apiece = 2 * atile;
-    const uint32_t a_bytes = 3 * apiece;
+    const uint32_t a_bytes = 2 * TC_ATILE;
     const size_t bpiece_g = (size_t)Npad * TC_K * 2;
     const size_t cls_stride = (size_t)(Npad / TC_K) * 3 * Npad * TC_K;  // elements of one class's table
 
@@ -649,13 +661,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
                     const uint32_t sb = sa + a_bytes;
                     for (int t = 0; t < 2; ++t) {
                         const uint32_t d = tmem + (uint32_t)t * 256u;
-                        const uint32_t a0 = sa + t * atile;
-                        mma_bf16(d, make_desc(a0 + 2 * apiece), make_desc(sb), idesc, 1u);
-                        mma_bf16(d, make_desc(a0 + apiece), make_desc(sb + bpiece), idesc, 1u);
-                        mma_bf16(d, make_desc(a0), make_desc(sb + 2 * bpiece), idesc, 1u);
-                        mma_bf16(d, make_desc(a0 + apiece), make_desc(sb), idesc, 1u);
-                        mma_bf16(d, make_desc(a0), make_desc(sb + bpiece), idesc, 1u);
-                        mma_bf16(d, make_desc(a0), make_desc(sb), idesc, 1u);
+                        const uint32_t at = sa + t * TC_ATILE;
+                        mma_bf16(d, make_desc_a(at, 2), make_desc(sb), idesc, 1u);
+                        mma_bf16(d, make_desc_a(at, 1), make_desc(sb + bpiece), idesc, 1u);
+                        mma_bf16(d, make_desc_a(at, 0), make_desc(sb + 2 * bpiece), idesc, 1u);
+                        mma_bf16(d, make_desc_a(at, 1), make_desc(sb), idesc, 1u);
+                        mma_bf16(d, make_desc_a(at, 0), make_desc(sb + bpiece), idesc, 1u);
+                        mma_bf16(d, make_desc_a(at, 0), make_desc(sb), idesc, 1u);
                     }
                     mma_commit(smem_u32(&empty[st]));
                 }
@@ -665,21 +677,16 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
         __syncwarp();
     } else {
         const int pt = tid - 32;
-        constexpr int AU = (TM_ROWS * 2 + NPROD - 1) / NPROD;
-        uint32_t a_dst[AU];
-#pragma unroll
-        for (int i = 0; i < AU; ++i) {
-            const int u = pt + i * NPROD;
-            const int row2 = u >> 1, jh = u & 1;
-            a_dst[i] = (uint32_t)((row2 / TC_M) * atile + kmajor_off(row2 % TC_M, jh * 8) * 2);
-        }
+        // unit pt % 6 = (piece, 8-element half) of the rows pt / 6 + PROWS i, as in k_m2l_tc
+        constexpr int PROWS = NPROD / XS_UNITS, AU = (TM_ROWS + PROWS - 1) / PROWS;
+        const int unit = pt % XS_UNITS, row0 = pt < PROWS * XS_UNITS ? pt / XS_UNITS : TM_ROWS;
         // rows of Xs of the next class, read while the current one is moved; -1: a target without the
         // class, a zero row
         int nxt[AU];
         auto rows_of = [&](int j) {
 #pragma unroll
             for (int i = 0; i < AU; ++i) {
-                const int row2 = (pt + i * NPROD) >> 1;  // (target slot, rhs) = (row2 / R, row2 % R)
+                const int row2 = row0 + i * PROWS;  // (target slot, rhs) = (row2 / R, row2 % R)
                 nxt[i] = row2 < TM_ROWS && j < nc ? tab[(tile * kNumM2LClasses + s_cls[j]) * TT + row2 / R] : -1;
             }
         };
@@ -691,14 +698,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
             const int Kj = s_K[j];
             const uint32_t bpiece = (uint32_t)Kj * TC_K * 2;
             const __nv_bfloat16 *Bc = tcB + (size_t)s_cls[j] * cls_stride;
-            const __nv_bfloat16 *a_src[AU];
-            uint32_t a_sz[AU];
+            int a_row[AU];
 #pragma unroll
-            for (int i = 0; i < AU; ++i) {
-                const int u = pt + i * NPROD, row2 = u >> 1;
-                a_src[i] = Xs + ((size_t)max(nxt[i], 0) * R + row2 % R) * Kp + (u & 1) * 8;
-                a_sz[i] = nxt[i] >= 0 ? 16u : 0u;
-            }
+            for (int i = 0; i < AU; ++i) a_row[i] = nxt[i] >= 0 ? nxt[i] * R + (row0 + i * PROWS) % R : -1;
             rows_of(j + 1);
             for (int s = 0; s < Kj / TC_K; ++s, ++ks) {
                 const int st = ks % TC_STAGES;
@@ -719,16 +721,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tm(int P, int Npad, const
                         bulk_g2s(sa + a_bytes + piece * bpiece, bsrc + (size_t)piece * bpiece_g, bpiece, bb);
                     issued = ks;
                 }
+                const __nv_bfloat16 *xk = Xs + unit * 8 + kstep * XS_STEP;
 #pragma unroll
-                for (int i = 0; i < AU; ++i) {
-                    if (pt + i * NPROD < 2 * TM_ROWS) {
-                        const __nv_bfloat16 *src = a_src[i] + kstep * TC_K;
-                        const uint32_t dst = sa + a_dst[i];
-                        cp_async16(dst, src, a_sz[i]);
-                        cp_async16(dst + apiece, src + plane, a_sz[i]);
-                        cp_async16(dst + 2 * apiece, src + 2 * plane, a_sz[i]);
-                    }
-                }
+                for (int i = 0; i < AU; ++i)
+                    if (row0 + i * PROWS < TM_ROWS)
+                        cp_async16(sa + a_unit(row0 + i * PROWS, unit), xk + (int64_t)max(a_row[i], 0) * xrow,
+                                   a_row[i] >= 0 ? 16u : 0u);
                 asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full[st])) : "memory");
             }
         }
@@ -906,7 +904,7 @@ void launch_m2l_tm(Context &c, const Operators &o, const float *X, int64_t xrows
     const size_t sm = (stages * TM_STAGE_BYTES > epi ? stages * TM_STAGE_BYTES : epi) + 3 * stages * 8 + 16 + 1024;
     BEM_CUDA(cudaFuncSetAttribute(k_m2l_tm<R, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     k_m2l_tm<R, 3><<<(unsigned)S.nitems, TC_THREADS, sm, st>>>(
-        o.P, Npad, reinterpret_cast<const __nv_bfloat16 *>(o.m2l_tc.p), S.items.p, S.src.p, S.cls.p, xrows, xs, S.part.p,
+        o.P, Npad, reinterpret_cast<const __nv_bfloat16 *>(o.m2l_tc.p), S.items.p, S.src.p, S.cls.p, xs, S.part.p,
         o.margin >= 0 ? o.cls_K.p : nullptr, err);
     BEM_LAUNCH_CHECK();
 }
