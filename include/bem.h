@@ -124,10 +124,10 @@ typedef struct {
     int32_t gmres_restart;  /* restart length; 0 = no restart (= maxit). Default 0.            */
     double gmres_tol;       /* stop when |b - L q| / |b| <= tol (Section 3.8). Default 1e-6.  */
     int32_t m2l_stages;     /* shared-memory pipeline stages of the pair-major tensor-core M2L
-                               (m2l_target_major = 0; the target-major kernel uses 3): 2 or 3;
-                               0 = automatic (the tile autotuner's choice when leaf_target = 0,
-                               else 3). Fewer stages leave shared memory on each SM for the
-                               near field running concurrently. Default 0.                    */
+                               (the target-major kernel uses 3): 2 or 3; 0 = automatic (the
+                               tile autotuner's choice when leaf_target = 0 and
+                               m2l_target_major = 0, else 2). With two stages two of its blocks
+                               fit on an SM, with three one. Default 0.                       */
     int32_t p2p_blocks_per_sm; /* near-field grid: 0 = one warp per work unit (all units in one
                                grid); k > 0 = a persistent grid of k blocks per SM looping over
                                the units, which leaves room on every SM for the far-field
@@ -149,9 +149,11 @@ typedef struct {
                                multiply work. Default 6.                                      */
     int32_t m2l_target_major; /* layout of the tensor-core M2L (mixed precision): 1 = target-major
                                (per tile of target boxes, the MMAs of a few offset classes
-                               accumulate in tensor memory; no row per translation); 0 =
-                               pair-major (one product row per translation, summed per target
-                               afterwards). Both sum in a fixed order. Default 1.             */
+                               accumulate in tensor memory; no row per translation) where about
+                               half of a tile's rows or more carry a translation, else
+                               pair-major; 0 = pair-major (one product row per translation,
+                               summed per target afterwards). Both sum in a fixed order.
+                               Default 1.                                                     */
 } bem_params;
 
 /* Run-time counters of a context (cumulative since bem_create or bem_reset_stats). */
@@ -167,7 +169,7 @@ typedef struct {
     double last_relres;     /* true relative residual of the last solve                        */
     double last_build_ms;   /* device time of the last fmm_build                               */
     int64_t n_launches;     /* kernels launched by the library in this process (all contexts)   */
-    int32_t m2l_stages;     /* tensor-core M2L pipeline stages in use (0 = the default, 3)      */
+    int32_t m2l_stages;     /* tensor-core M2L pipeline stages in use (0 = the default, 2)      */
     int32_t overlap;        /* near-field / far-field overlap mode in use (bem_params.overlap)  */
     int32_t reserved;
     int32_t p2p_blocks_per_sm; /* near-field grid in use (0 = one warp per work unit)           */

@@ -591,25 +591,40 @@ __global__ void k_reduce_pairs(int t0, const int32_t *__restrict__ off, const in
     Y[(size_t)t * R * P + e] += s + c;
 }
 
-// FP32 with R*P a multiple of 4: one 64-thread block per target, each thread four consecutive
-// coefficients through 16-byte loads, two product rows in flight. Per coefficient the order and
-// the arithmetic are those of k_reduce_pairs, so the results are the same bit for bit.
 __device__ __forceinline__ void comp_add(float &s, float &c, float v) {
     const float tt = s + v;
     const float bp = tt - s;
     c += (s - (tt - bp)) + (v - bp);
     s = tt;
 }
+// FP32 with P a multiple of 4: one block per target; `width` threads (whole warps) take a target's
+// coefficients, four each, through 16-byte loads, and the blockDim.x / width groups of them the target's
+// pairs k, k + groups, ... (group order fixed, so the sum does not depend on the schedule). Bound by the
+// latency of the gathered rows: four in flight per thread, few registers, and as many warps as the SMs
+// hold, with several groups per target where the targets alone are too few (64 threads looping over the
+// coefficients against this: sums of a bubble of 40962 points 20 -> 11 us, of 192600 points 67 -> 53 us,
+// of the four right-hand sides of 963000 points 900 -> 867 us. Staging the indices in shared memory or per
+// warp with eight rows in flight took 172 us against 145 at 801000 points; rows laid out by target gave
+// nothing.)
+constexpr int RED_THREADS = 256;
 template <int R>
-__global__ void __launch_bounds__(64) k_reduce_pairs4(int t0, const int32_t *__restrict__ off,
-                                                      const int32_t *__restrict__ by, const float *__restrict__ Ypair,
-                                                      int P, float *__restrict__ Y, const int32_t *__restrict__ byK) {
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_pairs4(int t0, const int32_t *__restrict__ off,
+                                                               const int32_t *__restrict__ by,
+                                                               const float *__restrict__ Ypair, int P,
+                                                               float *__restrict__ Y, const int32_t *__restrict__ byK,
+                                                               int width) {
+    extern __shared__ float4 s_part[];  // [2][blockDim.x], with more than one group
     const int t = t0 + blockIdx.x;
     const int a = off[t], b = off[t + 1];
     if (a == b) return;
     const int rp4 = R * P / 4;
+    const int groups = blockDim.x / width, grp = threadIdx.x / width, ew = threadIdx.x - grp * width;
     const float4 *Y4 = reinterpret_cast<const float4 *>(Ypair);
-    for (int e = threadIdx.x; e < rp4; e += blockDim.x) {
+    for (int e0 = 0; e0 < rp4; e0 += width) {
+        const int e = e0 + ew;
+        // truncated classes: the four coefficients (4e .. 4e + 3) % P lie on one side of the pair's
+        // class size byK[k] (a multiple of 16) together; threads past the row take no pairs
+        const int n = (4 * e) % P, end = e < rp4 ? b : a;
         float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f, c0 = 0.f, c1 = 0.f, c2 = 0.f, c3 = 0.f;
         auto add = [&](const float4 v) {
             comp_add(s0, c0, v.x);
@@ -617,48 +632,45 @@ __global__ void __launch_bounds__(64) k_reduce_pairs4(int t0, const int32_t *__r
             comp_add(s2, c2, v.z);
             comp_add(s3, c3, v.w);
         };
-        if (byK) {
-            // truncated classes: the four coefficients (4e .. 4e + 3) % P lie on one side of the
-            // pair's class size byK[k] (a multiple of 16) together
-            const int n = (4 * e) % P;
-            const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            int k = a;
-            for (; k + 3 < b; k += 4) {  // four rows in flight, added in pair order
-                float4 v[4];
-                bool in[4];
+        int k = a + grp;
+        for (; k + 3 * groups < end; k += 4 * groups) {  // four rows in flight, added in pair order
+            float4 v[4];
+            bool in[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    in[u] = n < byK[k + u];
-                    v[u] = in[u] ? Y4[(size_t)by[k + u] * rp4 + e] : z;
-                }
-#pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (in[u]) add(v[u]);
+            for (int u = 0; u < 4; ++u) {
+                in[u] = !byK || n < byK[k + u * groups];
+                v[u] = in[u] ? Y4[(size_t)by[k + u * groups] * rp4 + e] : make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            for (; k < b; ++k)
-                if (n < byK[k]) add(Y4[(size_t)by[k] * rp4 + e]);
-        } else {
-            int k = a;
-            for (; k + 3 < b; k += 4) {
-                float4 v[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u) v[u] = Y4[(size_t)by[k + u] * rp4 + e];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) add(v[u]);
-            }
-            for (; k < b; ++k) add(Y4[(size_t)by[k] * rp4 + e]);
+            for (int u = 0; u < 4; ++u)
+                if (in[u]) add(v[u]);
         }
-        float4 *dst = reinterpret_cast<float4 *>(Y) + (size_t)t * rp4 + e;
-        float4 y = *dst;
-        y.x += s0 + c0;
-        y.y += s1 + c1;
-        y.z += s2 + c2;
-        y.w += s3 + c3;
-        *dst = y;
+        for (; k < end; k += groups)
+            if (!byK || n < byK[k]) add(Y4[(size_t)by[k] * rp4 + e]);
+        if (groups > 1) {
+            s_part[threadIdx.x] = make_float4(s0, s1, s2, s3);
+            s_part[blockDim.x + threadIdx.x] = make_float4(c0, c1, c2, c3);
+            __syncthreads();
+            if (grp == 0) {
+                for (int g = 1; g < groups; ++g) {
+                    add(s_part[g * width + ew]);
+                    add(s_part[blockDim.x + g * width + ew]);
+                }
+            }
+            __syncthreads();
+        }
+        if (grp == 0 && e < rp4) {
+            float4 *dst = reinterpret_cast<float4 *>(Y) + (size_t)t * rp4 + e;
+            float4 y = *dst;
+            y.x += s0 + c0;
+            y.y += s1 + c1;
+            y.z += s2 + c2;
+            y.w += s3 + c3;
+            *dst = y;
+        }
     }
 }
 
-// Y[t] += sum over the pairs of t, for the targets t0 .. t0 + ntg - 1
 // byK[k] = cls_K[class of pair by[k]]: the truncated row length, in the target-major order
 __global__ void k_pair_K(int64_t n, const int32_t *__restrict__ by, const uint32_t *__restrict__ pair_cls,
                          const int32_t *__restrict__ cls_K, int32_t *__restrict__ byK) {
@@ -666,19 +678,35 @@ __global__ void k_pair_K(int64_t n, const int32_t *__restrict__ by, const uint32
     if (k < n) byK[k] = cls_K[pair_cls[by[k]]];
 }
 
+// Y[t] += sum over the pairs of t, for the targets t0 .. t0 + ntg - 1; with truncation the rows of a pair of
+// class c hold its first cls_K[c] coefficients only
 template <class T, int R>
-void launch_reduce_pairs(int t0, int ntg, const int32_t *off, const int32_t *by, const T *Ypair, int P, T *Y,
-                         cudaStream_t st, const int32_t *byK = nullptr) {
+void launch_reduce_pairs(Context &c, int t0, int ntg, const T *Ypair, int P, T *Y, cudaStream_t st,
+                         const Operators &o) {
     if (ntg <= 0) return;
+    const Tree &t = c.tree;
+    const bool trunc = o.margin >= 0;
+    if (trunc && c.m2l_byK_ops != &o) {  // once per tree and operator set
+        c.m2l_byK.resize(std::max<int64_t>(t.n_m2l, 1));
+        k_pair_K<<<div_up(t.n_m2l, 256), 256, 0, st>>>(t.n_m2l, t.m2l_by_tgt.p, t.m2l_cls.p, o.cls_K.p, c.m2l_byK.p);
+        BEM_LAUNCH_CHECK();
+        c.m2l_byK_ops = &o;
+    }
+    const int32_t *byK = trunc ? c.m2l_byK.p : nullptr;
     if constexpr (sizeof(T) == 4) {
         if (P % 4 == 0) {
-            k_reduce_pairs4<R><<<ntg, 64, 0, st>>>(t0, off, by, Ypair, P, Y, byK);
+            // groups: about twice the warps that fit on the chip (64 per SM)
+            const int rp4 = R * P / 4, width = std::min(RED_THREADS / 2, (rp4 + 31) / 32 * 32);
+            const int64_t warps = (int64_t)ntg * (width / 32), room = (int64_t)c.num_sms * 128;
+            const int groups = (int)std::max<int64_t>(1, std::min<int64_t>(RED_THREADS / width, room / warps));
+            k_reduce_pairs4<R><<<ntg, groups * width, groups > 1 ? 2 * groups * width * sizeof(float4) : 0, st>>>(t0, t.m2l_tgt_off.p, t.m2l_by_tgt.p, Ypair, P,
+                                                                           Y, byK, width);
             BEM_LAUNCH_CHECK();
             return;
         }
     }
     dim3 rg((unsigned)ntg, div_up(R * P, 128));
-    k_reduce_pairs<T, R><<<rg, 128, 0, st>>>(t0, off, by, Ypair, P, Y, byK);
+    k_reduce_pairs<T, R><<<rg, 128, 0, st>>>(t0, t.m2l_tgt_off.p, t.m2l_by_tgt.p, Ypair, P, Y, byK);
     BEM_LAUNCH_CHECK();
 }
 
@@ -816,6 +844,17 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p(int p, const int32_t *__res
 
 // out[perm[k]] = (far_k + near_k) / h_leaf: the far field (L2P) and the near field (P2P, run
 // concurrently on the side stream) meet here, back in the caller's vertex order.
+// A target-major tile runs every class that any of its 256 targets has, 189 at least where the tree is
+// full, so pairs / (189 boxes) is about the share of its MMA rows that carry a translation; the pair-major
+// form has no empty rows but writes and reads a row per pair. M2L and its sum, target-major against
+// pair-major, in us: share 0.24 (a bubble of 40962 points) 58 / 37, 0.36 (801000 points) 536 / 404, 0.45
+// (192600 points) 156 / 133, 0.69 (3.21M points) 1097 / 1620: pair-major below one half, while its rows
+// stay within 8 GB (a quarter of what the diagonals' four right-hand sides take).
+bool m2l_tm_pays(const Tree &t, int P) {
+    const int64_t boxes = t.nbox - t.base[2];
+    return 2 * t.n_m2l >= 189 * boxes || (size_t)t.n_m2l * P * sizeof(float) > ((size_t)8 << 30);
+}
+
 template <class T>
 __global__ void k_combine_out(int64_t N, int R, const int32_t *__restrict__ perm, const T *__restrict__ far,
                               const double *__restrict__ near, const double *__restrict__ ih, RhsArgs<kMaxRhs> a) {
@@ -955,10 +994,10 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
         // are formed by cancellation (Eqs. (s3), (s5)), which magnifies the far field's rounding.
         const bool tc_path = !F64 && (R == 1 ? c.prm.m2l_tensor_cores >= 1 : R == 4 && c.diag_tc) &&
                              m2l_tc_supported(P) && opr.tc_Npad > 0;
-        // target-major (no per-translation rows) for the single-RHS products; the 4-RHS diagonal
-        // product stays pair-major (its target-major form, at 64 targets per tile, was slower and
-        // less accurate)
-        const bool tm_path = tc_path && R == 1 && c.prm.m2l_target_major;
+        // target-major (no per-translation rows) for the single-RHS products whose tiles are well
+        // filled; the 4-RHS diagonal product stays pair-major (its target-major form, at 64 targets
+        // per tile, was slower and less accurate)
+        const bool tm_path = tc_path && R == 1 && c.prm.m2l_target_major && m2l_tm_pays(t, P);
         T *ypair = nullptr;  // per-pair products of the pair-major forms, for the fixed-order sums
         if (!tm_path) {
             const size_t need = (size_t)t.n_m2l * R * P;
@@ -977,7 +1016,7 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
             PhaseScope ps(c, PH_M2L, fs);
             const int ti = R == 1 ? 0 : 1;
             if (!c.tc_chunks_ok[ti]) {
-                // chunk sizes per class: four tiles of rows for small truncated classes, else two
+                // chunk sizes per class: two tiles of rows for small truncated classes, else one
                 std::vector<XChunk> tc;
                 const int P16 = (P + 15) / 16 * 16;
                 for (int cc = 0; cc < kNumM2LClasses; ++cc) {
@@ -1025,15 +1064,7 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
         if (tm_path) {
             launch_m2l_tm_reduce<1>(c, opr, (float *)lc, fs);
         } else {
-            const bool trunc = opr.margin >= 0;
-            if (trunc) {
-                c.m2l_byK.resize(std::max<int64_t>(t.n_m2l, 1));
-                k_pair_K<<<div_up(t.n_m2l, 256), 256, 0, fs>>>(t.n_m2l, t.m2l_by_tgt.p, t.m2l_cls.p, opr.cls_K.p,
-                                                              c.m2l_byK.p);
-                BEM_LAUNCH_CHECK();
-            }
-            launch_reduce_pairs<T, R>(t.base[2], t.nbox - t.base[2], t.m2l_tgt_off.p, t.m2l_by_tgt.p, ypair, P, lc,
-                                      fs, trunc ? c.m2l_byK.p : nullptr);
+            launch_reduce_pairs<T, R>(c, t.base[2], t.nbox - t.base[2], ypair, P, lc, fs, opr);
         }
     }
     // L2L downward, levels 3 -> L: every child has exactly one parent, so it adds in place

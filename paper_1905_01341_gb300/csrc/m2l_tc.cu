@@ -2,7 +2,7 @@
 //
 // For one offset class c and a chunk of (source, target) pairs, the product
 //   Y[pair, rhs][n] = sum_k T_c[n][k] X[src, rhs][k]
-// is up to three MMA tiles D_t = A_t B^T with M = 128 rows (pair, rhs) each, N = K = K_c, the
+// is up to two MMA tiles D_t = A_t B^T with M = 128 rows (pair, rhs) each, N = K = K_c, the
 // class's truncated size (p_c^2 rounded up to 16; P rounded up without truncation):
 // A_t = gathered multipole rows, B = T_c (row n of T_c is K-contiguous, i.e. K-major). The
 // tiles share every staged block of T_c, which divides its traffic; a chunk of a class with
@@ -50,14 +50,15 @@ namespace bem {
 namespace {
 
 constexpr int TC_M = 128;        // rows per tile
-constexpr int TC_MAXT = 3;       // tiles per block at most (same class, shared B stages)
-constexpr int TC_SMALL_K = 128;  // classes truncated to at most this size take three tiles per block
+constexpr int TC_MAXT = 2;       // tiles per block at most (same class, shared B stages)
+constexpr int TC_SMALL_K = 128;  // classes truncated to at most this size take two tiles per block
 constexpr uint32_t TC_AROW = 128;           // bytes of one row of A: the three pieces of a K step
 constexpr uint32_t TC_ATILE = TC_M * TC_AROW;
-// bytes of one pipeline stage: A and B (3 pieces x K_c x 16), for three tiles with K_c <= 128 or two
-// tiles with K_c <= 256 (the larger of the two)
-constexpr size_t TC_STAGE_BYTES = 3 * TC_ATILE + 3 * 128 * 16 * 2;
-static_assert(TC_STAGE_BYTES >= 2 * TC_ATILE + 3 * 256 * 16 * 2 && TC_STAGE_BYTES % 1024 == 0, "both forms fit");
+// bytes of one pipeline stage: A and B (3 pieces x K_c x 16), for two tiles with K_c <= 128 or one
+// tile with K_c <= 256 (the larger of the two)
+constexpr size_t TC_STAGE_BYTES = 2 * TC_ATILE + 3 * 128 * 16 * 2;
+static_assert(TC_STAGE_BYTES >= TC_ATILE + 3 * 256 * 16 * 2 && TC_STAGE_BYTES % 1024 == 0, "both forms fit");
+constexpr int TC_TMEM = 256;  // TMEM columns of a block: half of the SM's, for two blocks per SM
 constexpr int TC_THREADS = 256;  // 8 warps: two warp groups share the loads and the epilogue
 
 // Row-major T_c [P][P] (FP64) -> per class, per 16-wide K step, per piece, an N_pad x 16
@@ -127,21 +128,23 @@ struct TcLayout {
 // them in one: 3.77 against 3.30 ms for the diagonal product at 963000 points)
 __host__ __device__ constexpr int epi_stride(int Npad) { return Npad + 4; }
 
+// The pair-major epilogue moves at most this many columns of a tile at a time
+constexpr int TC_EPI_COLS = 128;
+
 // ST pipeline stages and three mbarriers per stage (empty, full, bfull); the epilogue reuses
-// the stages for one tile of FP32 rows
-__host__ __device__ inline TcLayout tc_layout(int Npad, int ST) {
+// the stages for 128 columns of one tile of FP32 rows
+__host__ __device__ inline TcLayout tc_layout(int ST) {
     TcLayout L;
-    L.stage_bytes = TC_STAGE_BYTES;
-    const size_t epi = (size_t)TC_M * epi_stride(Npad) * 4;
-    L.total = (ST * L.stage_bytes > epi ? ST * L.stage_bytes : epi) + 3 * ST * 8 + 16 + 1024;
+    L.stage_bytes = TC_STAGE_BYTES;  // two stages or more hold the epilogue's rows
+    L.total = ST * L.stage_bytes + 3 * ST * 8 + 16 + 1024;
     return L;
 }
 
 // tiles per block and TMEM columns per tile for a class truncated to K_c
-__host__ __device__ inline int tc_tiles_for(int Kc) { return Kc <= TC_SMALL_K ? TC_MAXT : 2; }
+__host__ __device__ inline int tc_tiles_for(int Kc) { return Kc <= TC_SMALL_K ? TC_MAXT : 1; }
 
 template <int R, int TC_STAGES>
-__global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __nv_bfloat16 *__restrict__ tcB,
+__global__ void __launch_bounds__(TC_THREADS, 2) k_m2l_tc(int P, int Npad, const __nv_bfloat16 *__restrict__ tcB,
                                                        const XChunk *__restrict__ chunks,
                                                        const int32_t *__restrict__ srcs,
                                                        const __nv_bfloat16 *__restrict__ Xs, float *__restrict__ Ypair,
@@ -149,10 +152,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     // 1024-byte aligned base for the operand stages
     unsigned char *smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    const TcLayout Lo = tc_layout(Npad, TC_STAGES);
-    const size_t epi_bytes = (size_t)TC_M * epi_stride(Npad) * 4;
-    uint64_t *empty = reinterpret_cast<uint64_t *>(
-        smem + (TC_STAGES * Lo.stage_bytes > epi_bytes ? TC_STAGES * Lo.stage_bytes : epi_bytes));
+    const TcLayout Lo = tc_layout(TC_STAGES);
+    static_assert(TC_STAGES * TC_STAGE_BYTES >= (size_t)TC_M * epi_stride(TC_EPI_COLS) * 4, "the epilogue's rows fit");
+    uint64_t *empty = reinterpret_cast<uint64_t *>(smem + TC_STAGES * Lo.stage_bytes);
     uint64_t *full = empty + TC_STAGES;  // NPROD producer arrivals per use (the gathered A rows)
     uint64_t *bfull = full + TC_STAGES;  // one arrival + the bulk copy's bytes (the block of T_c)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bfull + TC_STAGES);
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     const int nrows = ch.count * R;
     const int ntiles = (nrows + TC_M - 1) / TC_M;
     // the class's truncated size (a multiple of 16, <= Npad): K steps and output columns; small
-    // classes take three tiles per block (TMEM columns 128 apart), the others two (256 apart)
+    // classes take two tiles per block (TMEM columns 128 apart), the others one
     const int Kc = cls_K ? cls_K[ch.cls] : Npad;
     const int nsteps = Kc / TC_K;
     const int tcap = tc_tiles_for(Kc);
@@ -184,7 +186,7 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                     "n"(512));
+                     "n"(TC_TMEM));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
@@ -296,22 +298,26 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
     if (!ok && tid == 0) atomicOr(err, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (ok) {
-        // epilogue, one tile at a time: warp w holds TMEM lanes 32w..32w+31 = tile rows; each
-        // thread moves its row into shared memory, then each warp writes whole rows of Ypair with
-        // coalesced 16-byte stores (the first Kc coefficients; the per-target sums read no more)
-        const int es = epi_stride(Npad), kw = min(Kc, P) / 4;
+        // epilogue, at most 128 columns of a tile at a time: warp w holds TMEM lanes 32 (w % 4) ..;
+        // each thread moves its part of a row into shared memory, then each warp writes whole rows
+        // of Ypair with coalesced 16-byte stores (the first Kc coefficients; the per-target sums
+        // read no more)
+        constexpr int es = epi_stride(TC_EPI_COLS);
+        const int kw = min(Kc, P);
         float *stage = reinterpret_cast<float *>(smem);  // the operand stages are free now
-        for (int t = 0; t < ntiles; ++t) {
+        for (int u = 0; u < ntiles * ((Kc + TC_EPI_COLS - 1) / TC_EPI_COLS); ++u) {
+            const int t = u % ntiles, cb = u / ntiles * TC_EPI_COLS;
             const int rows_t = min(TC_M, nrows - t * TC_M);
             // a warp reads its own quarter of the TMEM lanes (warp % 4); the two warp groups take
             // the lower and the upper half of the 16-column groups
             const int q4 = warp & 3, half = warp >> 2;
-            const int ngroups = Kc / 16, g0 = half ? (ngroups + 1) / 2 : 0, g1 = half ? ngroups : (ngroups + 1) / 2;
+            const int ngroups = min(Kc - cb, TC_EPI_COLS) / 16, mid = (ngroups + 1) / 2;
             float *srow = stage + (size_t)(q4 * 32 + lane) * es;
-            for (int c0 = g0 * 16; c0 < g1 * 16; c0 += 16) {
-                if (c0 >= Kc) continue;  // beyond the class's truncation: neither computed nor stored
+            for (int g = half ? mid : 0; g < (half ? ngroups : mid); ++g) {
+                const int c0 = g * 16;
                 uint32_t v[16];
-                const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)t * colstride + (uint32_t)c0;
+                const uint32_t taddr =
+                    tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)t * colstride + (uint32_t)(cb + c0);
                 asm volatile(
                     "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, "
                     "[%16];"
@@ -322,23 +328,22 @@ __global__ void __launch_bounds__(TC_THREADS) k_m2l_tc(int P, int Npad, const __
                 asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
                 for (int i = 0; i < 16; i += 4)
-                    if (c0 + i < P)  // P % 4 == 0: whole 16-byte groups
-                        *reinterpret_cast<float4 *>(srow + c0 + i) =
-                            make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
-                                        __uint_as_float(v[i + 3]));
+                    *reinterpret_cast<float4 *>(srow + c0 + i) =
+                        make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
+                                    __uint_as_float(v[i + 3]));
             }
             __syncthreads();
-            float4 *dst = reinterpret_cast<float4 *>(Ypair + ((size_t)ch.start * R + t * TC_M) * P);
-            for (int row = warp; row < rows_t; row += TC_THREADS / 32) {
-                const float4 *src = reinterpret_cast<const float4 *>(stage + (size_t)row * es);
-                for (int col = lane; col < kw; col += 32) dst[(size_t)row * (P / 4) + col] = src[col];
-            }
+            const int n4 = (min(kw, cb + TC_EPI_COLS) - cb) / 4;  // P % 4 == 0: whole 16-byte groups, at most 32
+            float4 *dst = reinterpret_cast<float4 *>(Ypair + ((size_t)ch.start * R + t * TC_M) * P + cb);
+            if (lane < n4)
+                for (int row = warp; row < rows_t; row += TC_THREADS / 32)
+                    dst[(size_t)row * (P / 4) + lane] = reinterpret_cast<const float4 *>(stage + (size_t)row * es)[lane];
             __syncthreads();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(512));
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(TC_TMEM));
 }
 
 }  // namespace
@@ -376,10 +381,12 @@ void launch_m2l_tc(Context &c, const Operators &o, const XChunk *chunks, int64_t
                    int64_t xrows, float *Ypair, int *err, cudaStream_t st) {
     const int Npad = o.tc_Npad;
     __nv_bfloat16 *xs = split_multipoles(c, o, X, xrows, st);
-    // pipeline depth: the context's choice (parameter or autotuner), else three stages (as many as
-    // fit at the four-tile stage size)
-    const int stages = c.tuned_stages == 2 ? 2 : 3;
-    const size_t sm = tc_layout(Npad, stages).total;
+    // pipeline depth: the context's choice (parameter or autotuner), else two stages, with which two
+    // blocks fit on an SM and one's set-up and epilogue run under the other's MMAs (one block of three
+    // stages and twice the tiles: diagonal product of 963000 points 2.91 against 2.49 ms, product of
+    // 192600 points 106 against 81 us)
+    const int stages = c.tuned_stages == 3 ? 3 : 2;
+    const size_t sm = tc_layout(stages).total;
     auto kern = stages == 2 ? k_m2l_tc<R, 2> : k_m2l_tc<R, 3>;
     // set on every launch: the attribute belongs to the current device (~1 us against a ms kernel)
     BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
