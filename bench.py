@@ -454,8 +454,8 @@ def run_ours(args):
         t_launch = ms_i / 1e3 / n_i
         achieved = P2P_FLOPS_SL * st_iso["p2p_pairs"] / t_launch / 1e12
         peak = FP32_ALU_PEAK_TFLOPS if prec == bem.BEM_PREC_MIXED else None
-        kname = ("k_p2p_units_x2 + k_p2p_back_gather (near field, single layer, symmetric)"
-                 if prec == bem.BEM_PREC_MIXED else "k_p2p_units (near field, single layer)")
+        kname = ("k_p2p_items_x2 + k_p2p_gather (near field, single layer, symmetric)"
+                 if prec == bem.BEM_PREC_MIXED else "k_p2p_items + k_p2p_gather (near field, single layer)")
         return {"kernel": kname, "bound": "alu", "achieved": achieved,
                 "peak": peak, "unit": "TFLOP/s", "frac": (achieved / peak) if peak else None,
                 "traffic": P2P_DRAM_BYTES_PER_POINT * N if prec == bem.BEM_PREC_MIXED else None,

@@ -142,9 +142,10 @@ struct Tree {
     DevBuf<int2> p2p_units;
     int64_t n_p2p_units = 0;
     DevBuf<int32_t> p2p_ucnt;  // [nleaf] units per leaf
-    // FP32 near-field work items (leaf, first receiver, first and end position in the unit's list of
-    // neighbour points; first = -1: the list from 0 and the leaf's own points): [0] symmetric (the neighbours f > leaf), [1] one-way (all but the leaf); the
-    // items of unit u are p2p_ioff[u] .. p2p_ioff[u + 1] - 1
+    // near-field work items (leaf, first receiver, first and end position in the unit's list of neighbour
+    // points; first = -1: the list from 0 and the leaf's own points): [0] symmetric (the neighbours
+    // f > leaf; FP32), [1] one-way (all but the leaf; FP32 and FP64); the items of unit u are
+    // p2p_ioff[u] .. p2p_ioff[u + 1] - 1
     DevBuf<int4> p2p_items[2];
     DevBuf<int32_t> p2p_ioff[2];
     int64_t n_p2p_items[2] = {0, 0};
@@ -326,6 +327,7 @@ struct Context {
     DevBuf<float> far32;
     DevBuf<double> near_out;       // combined potential [R][N] (sorted)
     DevBuf<float2> p2p_fwd;        // FP32 near field: sums of every item [items][R][64]
+    DevBuf<double2> p2p_fwd64;     // the same of the FP64 near field
     DevBuf<XChunk> m2l_chunks;
     std::vector<XChunk> m2l_chunks_h;
     // M2L chunks of <= 256/R pairs for the tensor-core kernel: [0] for R = 1, [1] for R = 4

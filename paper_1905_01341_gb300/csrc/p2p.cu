@@ -59,6 +59,14 @@ template <>
 struct V4<double> {
     using type = double4;
 };
+template <class T>
+struct V2 {
+    using type = float2;
+};
+template <>
+struct V2<double> {
+    using type = double2;
+};
 
 // Near-field work is split into units of up to 64 receivers of one leaf (Tree::p2p_units);
 // one warp owns a unit and each lane keeps two receivers in registers, so a staged source feeds
@@ -81,6 +89,8 @@ struct P2PStage {
     T4 b[HW ? 32 : 1];                         // n_x, n_y, n_z, w (first RHS)
     T q[(R > 1 && HQ) ? R - 1 : 1][32];        // q of the other RHS
     T w[(R > 1 && HW) ? R - 1 : 1][32];        // w of the other RHS
+    int4 tab[27];                              // per neighbour: its offset, its points less its list positions
+    int tend[27];                              // its end in the item's list
 };
 
 template <class T, int R, int KR, bool HQ, bool HW, bool SELF>
@@ -95,6 +105,13 @@ __device__ __forceinline__ void p2p_source(const P2PStage<T, R, HQ, HW> &sg, int
         const T dx = xi[k] - a.x, dy = yi[k] - a.y, dz = zi[k] - a.z;
         const T r2 = dx * dx + dy * dy + dz * dz;
         const T rinv = SELF ? (r2 > (T)0 ? rsqrt_t<T>(r2) : (T)0) : rsqrt_t<T>(r2);
+        if constexpr (R == 1 && HW) {
+            // both layers as (q + w n.d / r^2) / r, the normal staged times its strength
+            const T nd = bb.x * dx + bb.y * dy + bb.z * dz;
+            const T ri2 = rinv * rinv;
+            part[k][0] += (HQ ? a.w + nd * ri2 : nd * ri2) * rinv;
+            continue;
+        }
         if (HQ) {
             part[k][0] += a.w * rinv;
 #pragma unroll
@@ -137,18 +154,23 @@ __device__ __forceinline__ void p2p_tile(const P2PStage<T, R, HQ, HW> &sg, int n
         for (int r = 0; r < R; ++r) acc[k][r].add(part[k][r]);
 }
 
-// One work unit (up to 64 receivers of one leaf) by one warp, its lanes split into G groups
-// (G = 1 for 33..64 receivers, 2 for 17..32, 4 for 9..16, 8 for 1..8): lane = gi * (32/G) + rs
-// holds the receivers rs and rs + 32/G and takes group gi's share of every source tile.
+// One FP64 work item (see the packed form below: up to 64 receivers of one leaf and a range of its list
+// of neighbour sources) by one warp, its lanes split into G groups (G = 1 for 33..64 receivers, 2 for
+// 17..32, 4 for 9..16, 8 for 1..8): lane = gi * (32/G) + rs holds the receivers rs and rs + 32/G and takes
+// group gi's share of every source tile. Bound by the FP64 pipe (two lanes per clock and SM). With a warp
+// per unit and all its neighbours, 784 warps at 40962 points, a part of the SMs ran two rounds and the SMs
+// were active 59 % of the kernel's time: 5.62 -> 3.32 ms (both layers of 40962 points, p 16;
+// with the layers taken as one factor of 1/r, two operations a pair fewer, 6.27 -> 5.62 before).
 template <class T, int R, int G, bool HQ, bool HW>
-__device__ __forceinline__ void p2p_unit_g(P2PStage<T, R, HQ, HW> &sg, int lane, int b, int r0, int nr,
+__device__ __forceinline__ void p2p_item_g(P2PStage<T, R, HQ, HW> &sg, int lane, int4 it, int nr,
                                            const int32_t *__restrict__ bstart, const int32_t *__restrict__ bcount,
                                            const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
                                            const int8_t *__restrict__ nd, int64_t N, const T *__restrict__ loc,
                                            const T *__restrict__ nrm, const T *__restrict__ q, const T *__restrict__ w,
-                                           double *__restrict__ out) {
+                                           double2 *__restrict__ fwd) {
     constexpr int LG = 32 / G;  // lanes per group
     const int rs = lane & (LG - 1), gi = lane / LG;
+    const int b = it.x, r0 = it.y;
     const int s0 = bstart[b];
     T xi[2], yi[2], zi[2];
     Comp<T> acc[2][R];
@@ -160,38 +182,67 @@ __device__ __forceinline__ void p2p_unit_g(P2PStage<T, R, HQ, HW> &sg, int lane,
         yi[k] = loc[N + i];
         zi[k] = loc[2 * N + i];
     }
-    // neighbour table of the target leaf, one entry per lane, broadcast by shuffles
-    const int nn = ncnt[b];
-    int my_f = 0;
-    T my_d[3] = {(T)0, (T)0, (T)0};
-    if (lane < nn) {
-        my_f = nbr[b * 27 + lane];
+    auto stage = [&](int64_t j, int ox, int oy, int oz) {
+        sg.a[lane] = typename V4<T>::type{loc[j] + (T)ox, loc[N + j] + (T)oy, loc[2 * N + j] + (T)oz, HQ ? q[j] : (T)0};
+        if (HW) {
+            const T wn = R == 1 ? w[j] : (T)1;
+            sg.b[lane] = typename V4<T>::type{nrm[j] * wn, nrm[N + j] * wn, nrm[2 * N + j] * wn, w[j]};
+        }
 #pragma unroll
-        for (int d = 0; d < 3; ++d) my_d[d] = (T)nd[(b * 27 + lane) * 4 + d];
-    }
-    for (int k = 0; k < nn; ++k) {
-        const int f = __shfl_sync(0xffffffffu, my_f, k);
-        const T ox = __shfl_sync(0xffffffffu, my_d[0], k);
-        const T oy = __shfl_sync(0xffffffffu, my_d[1], k);
-        const T oz = __shfl_sync(0xffffffffu, my_d[2], k);
-        const int fs = bstart[f], fc = bcount[f];
-        const bool self = (f == b);
+        for (int r = 1; r < R; ++r) {
+            if (HQ) sg.q[r - 1][lane] = q[r * N + j];
+            if (HW) sg.w[r - 1][lane] = w[r * N + j];
+        }
+    };
+    if (it.z < 0) {  // the unit's first item: its own leaf, then the list from 0
+        const int fc = bcount[b];
         for (int t0 = 0; t0 < fc; t0 += 32) {
-            if (t0 + lane < fc) {
-                const int64_t j = fs + t0 + lane;
-                sg.a[lane] = typename V4<T>::type{loc[j] + ox, loc[N + j] + oy, loc[2 * N + j] + oz,
-                                                  HQ ? q[j] : (T)0};
-                if (HW) sg.b[lane] = typename V4<T>::type{nrm[j], nrm[N + j], nrm[2 * N + j], w[j]};
+            if (t0 + lane < fc) stage((int64_t)s0 + t0 + lane, 0, 0, 0);
+            __syncwarp();
+            p2p_tile<T, R, G, HQ, HW, true>(sg, min(32, fc - t0), gi, xi, yi, zi, acc);
+            __syncwarp();
+        }
+    }
+    const int lbeg = max(it.z, 0), lend = it.w;
+    if (lbeg < lend) {
+        // the list: per neighbour its end position and the shift from positions to points
+        const int nn = ncnt[b];
+        int cnt = 0, st = 0;
+        int4 tb = make_int4(0, 0, 0, 0);
+        if (lane < nn) {
+            const int f = nbr[b * 27 + lane];
+            if (f != b) cnt = bcount[f];
+            st = bstart[f];
+            tb.x = nd[(b * 27 + lane) * 4];
+            tb.y = nd[(b * 27 + lane) * 4 + 1];
+            tb.z = nd[(b * 27 + lane) * 4 + 2];
+        }
+        int end = cnt;
 #pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    if (HQ) sg.q[r - 1][lane] = q[r * N + j];
-                    if (HW) sg.w[r - 1][lane] = w[r * N + j];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, end, o);
+            if (lane >= o) end += v;
+        }
+        if (lane < 27) {
+            tb.w = st - (end - cnt);
+            sg.tab[lane] = tb;
+            sg.tend[lane] = end;
+        }
+        __syncwarp();
+        int k = 0, kend = sg.tend[0];
+        int4 cur = sg.tab[0];
+        for (int t0 = lbeg; t0 < lend; t0 += 32) {
+            const int s = t0 + lane;
+            if (s < lend) {
+                if (s >= kend) {
+                    do kend = sg.tend[++k];
+                    while (s >= kend);
+                    cur = sg.tab[k];
                 }
+                stage((int64_t)cur.w + s, cur.x, cur.y, cur.z);
             }
             __syncwarp();
-            const int ns = min(32, fc - t0);
-            if (self) p2p_tile<T, R, G, HQ, HW, true>(sg, ns, gi, xi, yi, zi, acc);
-            else p2p_tile<T, R, G, HQ, HW, false>(sg, ns, gi, xi, yi, zi, acc);
+            p2p_tile<T, R, G, HQ, HW, false>(sg, min(32, lend - t0), gi, xi, yi, zi, acc);
             __syncwarp();
         }
     }
@@ -212,27 +263,11 @@ __device__ __forceinline__ void p2p_unit_g(P2PStage<T, R, HQ, HW> &sg, int lane,
         for (int k = 0; k < 2; ++k) {
             const int li = rs + k * LG;
             if (li < nr) {
-                const int64_t i = s0 + r0 + li;
 #pragma unroll
-                for (int r = 0; r < R; ++r) out[r * N + i] = acc[k][r].get();  // the far field is added later
+                for (int r = 0; r < R; ++r) fwd[r * P2P_UNIT + li] = make_double2(acc[k][r].s, acc[k][r].c);
             }
         }
     }
-}
-
-template <class T, int R, bool HQ, bool HW>
-__device__ __forceinline__ void p2p_unit(P2PStage<T, R, HQ, HW> &sg, int lane, int2 un,
-                                         const int32_t *__restrict__ bstart, const int32_t *__restrict__ bcount,
-                                         const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
-                                         const int8_t *__restrict__ nd, int64_t N, const T *__restrict__ loc,
-                                         const T *__restrict__ nrm, const T *__restrict__ q, const T *__restrict__ w,
-                                         double *__restrict__ out) {
-    const int b = un.x, r0 = un.y;
-    const int nr = min(P2P_UNIT, bcount[b] - r0);  // uniform in the warp
-    if (nr > 32) p2p_unit_g<T, R, 1, HQ, HW>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out);
-    else if (nr > 16) p2p_unit_g<T, R, 2, HQ, HW>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out);
-    else if (nr > 8) p2p_unit_g<T, R, 4, HQ, HW>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out);
-    else p2p_unit_g<T, R, 8, HQ, HW>(sg, lane, b, r0, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out);
 }
 
 // FP32 form with packed two-wide arithmetic (add/mul/fma .f32x2: one instruction for two
@@ -614,9 +649,10 @@ __global__ void __launch_bounds__(P2P_WARPS * 32, SYM ? 6 : (R == 1 ? 5 : 4)) k_
 // (TwoSum; FP64 arithmetic is slow on this part). Lane k first looks up neighbour k's region;
 // shuffles broadcast it.
 constexpr int GATHER_WARPS = 8;
-template <int R, bool SYM>
+template <class T, int R, bool SYM>
 __global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_gather(
-    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ ioff, const float2 *__restrict__ fwd,
+    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ ioff,
+    const typename V2<T>::type *__restrict__ fwd,
     const int32_t *__restrict__ bstart, const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr,
     const int32_t *__restrict__ ncnt, const int32_t *__restrict__ gofs, const int32_t *__restrict__ ucnt,
     const int32_t *__restrict__ S, const int64_t *__restrict__ base, const float *__restrict__ back, int64_t N,
@@ -629,18 +665,19 @@ __global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_gather(
     const int nr = min(P2P_UNIT, bcount[b] - r0);
     const bool v0 = lane < nr, v1 = lane + 32 < nr;
     const int64_t i0 = (int64_t)bstart[b] + r0 + lane;
-    Comp<float> a0[R], a1[R];
+    using T2 = typename V2<T>::type;
+    Comp<T> a0[R], a1[R];
     for (int i = ioff[uw], e = ioff[uw + 1]; i < e; ++i) {
-        const float2 *f = fwd + (int64_t)i * (R * P2P_UNIT) + lane;
+        const T2 *f = fwd + (int64_t)i * (R * P2P_UNIT) + lane;
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (v0) {
-                const float2 x = f[r * P2P_UNIT];
+                const T2 x = f[r * P2P_UNIT];
                 a0[r].add(x.x);
                 a0[r].c += x.y;
             }
             if (v1) {
-                const float2 x = f[r * P2P_UNIT + 32];
+                const T2 x = f[r * P2P_UNIT + 32];
                 a1[r].add(x.x);
                 a1[r].c += x.y;
             }
@@ -690,23 +727,27 @@ __global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_gather(
     }
 }
 
-// Each warp takes the units u = blockIdx.x * P2P_WARPS + warp, then every gridDim.x * P2P_WARPS
-// further: one unit per warp when the grid covers all units, or a persistent grid of a fixed
-// number of blocks per SM (leaving room on every SM for the far-field kernels that run
-// concurrently on the other stream). Every unit writes its own receivers, so the result does
-// not depend on the grid.
+// The FP64 items, as k_p2p_items_x2
 template <class T, int R, bool HQ, bool HW>
-__global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p_units(
-    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ bstart,
+__global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p_items(
+    const int4 *__restrict__ items, int64_t nitems, const int32_t *__restrict__ bstart,
     const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
     const int8_t *__restrict__ nd, int64_t N, const T *__restrict__ loc, const T *__restrict__ nrm,
-    const T *__restrict__ q, const T *__restrict__ w, double *__restrict__ out) {
+    const T *__restrict__ q, const T *__restrict__ w, double2 *__restrict__ fwd) {
     __shared__ P2PStage<T, R, HQ, HW> stage[P2P_WARPS];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * P2P_WARPS;
+    auto &sg = stage[warp];
     // the loop bound is uniform in the warp; only warp-level barriers follow
-    for (int64_t u = (int64_t)blockIdx.x * P2P_WARPS + warp; u < nunits; u += stride)
-        p2p_unit<T, R, HQ, HW>(stage[warp], lane, units[u], bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, out);
+    for (int64_t u = (int64_t)blockIdx.x * P2P_WARPS + warp; u < nitems; u += stride) {
+        const int4 it = items[u];
+        const int nr = min(P2P_UNIT, bcount[it.x] - it.y);  // uniform in the warp
+        double2 *f = fwd + u * (R * P2P_UNIT);
+        if (nr > 32) p2p_item_g<T, R, 1, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
+        else if (nr > 16) p2p_item_g<T, R, 2, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
+        else if (nr > 8) p2p_item_g<T, R, 4, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
+        else p2p_item_g<T, R, 8, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
+    }
 }
 
 }  // namespace
@@ -719,8 +760,6 @@ static void launch_units(Context &c, const T *q, const T *w, double *out_sorted,
     const T *nrm = sizeof(T) == 8 ? (const T *)t.nrm64.p : (const T *)t.nrm32.p;
     const int64_t nu = t.n_p2p_units;
     if (nu == 0) return;
-    int64_t blocks = div_up(nu, P2P_WARPS);
-    if (c.tuned_p2p_blocks > 0) blocks = std::min<int64_t>(blocks, (int64_t)c.num_sms * c.tuned_p2p_blocks);
     // With the far field running concurrently, ask for the SM configuration with the most shared
     // memory: the tensor-core M2L needs it, and an SM whose resident near-field blocks had it
     // configured for more L1 would first have to drain them. (A per-device attribute, set on
@@ -735,22 +774,30 @@ static void launch_units(Context &c, const T *q, const T *w, double *out_sorted,
             BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
                                           (int)cudaSharedmemCarveoutMaxShared));
         const int64_t ni = t.n_p2p_items[li];
-        blocks = div_up(ni, P2P_WARPS);
+        int64_t blocks = div_up(ni, P2P_WARPS);
         if (c.tuned_p2p_blocks > 0) blocks = std::min<int64_t>(blocks, (int64_t)c.num_sms * c.tuned_p2p_blocks);
         c.p2p_fwd.resize((size_t)ni * R * P2P_UNIT);
         const BackArgs ba{SYM ? t.back.p : nullptr, t.back_S.p, t.back_base.p};
         kern<<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(t.p2p_items[li].p, ni, bst, bcn, t.nbr.p, t.nbr_cnt.p,
                                                            t.nbr_d.p, c.N, loc, nrm, q, w, c.p2p_fwd.p, ba);
         BEM_LAUNCH_CHECK();
-        k_p2p_gather<R, SYM><<<(unsigned)div_up(nu, GATHER_WARPS), GATHER_WARPS * 32, 0, st>>>(
+        k_p2p_gather<float, R, SYM><<<(unsigned)div_up(nu, GATHER_WARPS), GATHER_WARPS * 32, 0, st>>>(
             t.p2p_units.p, nu, t.p2p_ioff[li].p, c.p2p_fwd.p, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.back_gofs.p, t.p2p_ucnt.p,
             t.back_S.p, t.back_base.p, t.back.p, c.N, out_sorted);
     } else {
         if (c.tuned_overlap)
-            BEM_CUDA(cudaFuncSetAttribute(k_p2p_units<T, R, HQ, HW>, cudaFuncAttributePreferredSharedMemoryCarveout,
+            BEM_CUDA(cudaFuncSetAttribute(k_p2p_items<T, R, HQ, HW>, cudaFuncAttributePreferredSharedMemoryCarveout,
                                           (int)cudaSharedmemCarveoutMaxShared));
-        k_p2p_units<T, R, HQ, HW><<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(
-            t.p2p_units.p, nu, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.nbr_d.p, c.N, loc, nrm, q, w, out_sorted);
+        const int64_t ni = t.n_p2p_items[1];
+        int64_t blocks = div_up(ni, P2P_WARPS);
+        if (c.tuned_p2p_blocks > 0) blocks = std::min<int64_t>(blocks, (int64_t)c.num_sms * c.tuned_p2p_blocks);
+        c.p2p_fwd64.resize((size_t)ni * R * P2P_UNIT);
+        k_p2p_items<T, R, HQ, HW><<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(
+            t.p2p_items[1].p, ni, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.nbr_d.p, c.N, loc, nrm, q, w, c.p2p_fwd64.p);
+        BEM_LAUNCH_CHECK();
+        k_p2p_gather<double, R, false><<<(unsigned)div_up(nu, GATHER_WARPS), GATHER_WARPS * 32, 0, st>>>(
+            t.p2p_units.p, nu, t.p2p_ioff[1].p, c.p2p_fwd64.p, bst, bcn, t.nbr.p, t.nbr_cnt.p, nullptr, nullptr, nullptr,
+            nullptr, nullptr, c.N, out_sorted);
     }
     BEM_LAUNCH_CHECK();
 }

@@ -864,7 +864,7 @@ void build_tree(Context &c) {
         BEM_CUDA(cudaMemcpyAsync(t.p2p_ucnt.p, ucnt.p, nleaf * sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
         t.n_back = 32 * (int64_t)tot2[1];
         t.back.resize(std::max<int64_t>(t.n_back, 1));
-        // FP32 items. The list length of an item: enough items for about six rounds of the warps that
+        // Near-field items (one-way list: also FP64). The list length of an item: enough items for about six rounds of the warps that
         // the chip holds (24 per SM), so that the last round is a small part, but at least 64 and at
         // most 4096 positions (an item's set-up is about a quarter of a 64-source item's time, and
         // beyond 4096 nearly every unit is one item). Half the pairs in the symmetric list.
