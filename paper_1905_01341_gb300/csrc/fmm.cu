@@ -711,8 +711,8 @@ void launch_reduce_pairs(Context &c, int t0, int ntg, const T *Ypair, int P, T *
 }
 
 // ------------------------------------------------------------------------------ L2P (FP64)
-// One warp per leaf (the FP32 form is in p2m_l2p.cu): leaves hold about 70-150 points, and a 128-thread block left most of its
-// lanes idle on the second pass over a leaf's points.
+// One-warp blocks, one or more per leaf (the FP32 form is in p2m_l2p.cu): leaves hold about 70-150 points,
+// and a 128-thread block left most of its lanes idle on the second pass over a leaf's points.
 constexpr int L2P_THREADS = 32;
 
 // TwoSum-compensated accumulation in T; for double the compensation is harmless.
@@ -742,6 +742,7 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p(int p, const int32_t *__res
     T *tk = Ls + R * P;                     // [p]: -1 / (2k)
     T *tnm = tk + p;                        // [ntri]: 1 / ((n + m)(n - m)), n >= m + 2
     int b = blockIdx.x;
+    if ((int)blockIdx.y * 2 * L2P_THREADS >= bcount[b]) return;
     for (int e = threadIdx.x; e < R * P; e += L2P_THREADS) Ls[e] = lc[(size_t)b * R * P + e];
     for (int e = threadIdx.x; e < p; e += L2P_THREADS) tk[e] = e > 0 ? (T)(-0.5) / (T)e : (T)0;
     for (int e = threadIdx.x; e < ntri; e += L2P_THREADS) {
@@ -754,7 +755,7 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p(int p, const int32_t *__res
     int s0 = bstart[b], cnt = bcount[b];
     // each lane evaluates two points at once (c0 and c0 + 32): two independent recurrence chains,
     // and every coefficient read from shared memory serves both
-    for (int c0 = threadIdx.x; c0 < cnt; c0 += 2 * L2P_THREADS) {
+    for (int c0 = blockIdx.y * 2 * L2P_THREADS + threadIdx.x; c0 < cnt; c0 += gridDim.y * 2 * L2P_THREADS) {
         const bool two = c0 + L2P_THREADS < cnt;
         const int64_t i0 = s0 + c0, i1 = s0 + (two ? c0 + L2P_THREADS : c0);
         T x[2] = {loc[i0], loc[i1]}, y[2] = {loc[N + i0], loc[N + i1]}, z[2] = {loc[2 * N + i0], loc[2 * N + i1]};
@@ -1079,7 +1080,10 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
         const T *leaf_lc = lc + (size_t)t.base[L] * R * P;
         if constexpr (F64) {
             const size_t sm = ((size_t)R * P + p + (size_t)p * (p + 1) / 2) * sizeof(T);  // expansion + divisor tables
-            k_l2p<T, R><<<nleaf, L2P_THREADS, sm, fs>>>(p, bst, bcn, N, loc, leaf_lc, far);
+            // few leaves: several warps per leaf, up to eight leaves' worth per SM (272 leaves of 150
+            // points, p 16: 504 -> 272 us with one warp and with four per leaf)
+            const int parts = std::max(1, std::min(8, 8 * c.num_sms / std::max(nleaf, 1)));
+            k_l2p<T, R><<<dim3((unsigned)nleaf, (unsigned)parts), L2P_THREADS, sm, fs>>>(p, bst, bcn, N, loc, leaf_lc, far);
             BEM_LAUNCH_CHECK();
         } else {
             launch_l2p32<R>(p, nleaf, bst, bcn, N, loc, leaf_lc, far, fs);
