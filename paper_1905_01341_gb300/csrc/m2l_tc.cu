@@ -6,8 +6,9 @@
 // class's truncated size (p_c^2 rounded up to 16; P rounded up without truncation):
 // A_t = gathered multipole rows, B = T_c (row n of T_c is K-contiguous, i.e. K-major). The
 // tiles share every staged block of T_c, which divides its traffic; a chunk of a class with
-// K_c <= 128 has three tiles (TMEM columns 128 apart), the others two (256 apart), so the small
-// truncated classes amortise a block's set-up and pipeline fill over more rows.
+// K_c <= 128 has two tiles (TMEM columns 128 apart), the others one, so the small truncated
+// classes amortise a block's set-up and pipeline fill over more rows; a block takes half the SM's
+// tensor memory, for two blocks per SM.
 //
 // Accuracy: both operands are split into three BF16 pieces, x = x0 + x1 + x2 (x0 = bf16(x),
 // x1 = bf16(x - x0), x2 = bf16(x - x0 - x1)), and D accumulates in FP32 the six products with
@@ -23,14 +24,14 @@
 // apart, 8-row groups 256 B apart). The split multipoles lie in memory as they are gathered: per box
 // and right-hand side, per K step, the three pieces side by side in one 128-byte line (96 bytes
 // used); A keeps them so, one 128-byte row per tile row in the 128-byte-swizzled K-major layout (16-byte
-// unit u of row r at u ^ (r % 8)), and an MMA takes piece i by starting 32 i bytes into the rows. A
-// gathered line then arrives in one shared-memory write. With a plane per piece and no swizzle a
-// line brought one 32-byte sector whose halves fell into the same banks: 1536 writes per K step
-// against about 1200 operand reads, which filled the shared-memory pipe to 93 % (M2L of 192600
-// points 144 against 128 us, of 3.21M points 1268 against 963, of the diagonal product at 963000
-// points 3303 against 2908). The block is warp-specialised: warps 1-7
-// fill the stages with cp.async (16-byte copies; rows past the chunk read as zeros), three
-// stages deep (two on request), and let each stage's "full"
+// unit u of row r at u ^ (r % 8)), and an MMA takes piece i by starting 32 i bytes into the rows. With
+// a plane per piece and no swizzle a copy brought one 32-byte sector of each of 16 rows, whose halves fell
+// into the same banks: the target-major kernel at 192600 points wrote 20.6M wavefronts of copies where
+// it now writes 13.9M, next to 16.2M of operand reads that fill the same pipe (M2L of 192600 points 144 ->
+// 128 us, of 3.21M points 1268 -> 963, of the diagonal product at 963000 points 3303 -> 2908; the pipe is
+// still 89 % busy and bounds the kernel). The block is warp-specialised: warps 1-7
+// fill the stages with cp.async (16-byte copies; rows past the chunk read as zeros), two
+// stages deep (three in the target-major kernel), and let each stage's "full"
 // mbarrier count their copies' arrival (cp.async.mbarrier.arrive.noinc); one thread of warp 0
 // waits on "full", issues the stage's MMAs and commits them to the stage's "empty" mbarrier,
 // which releases the stage for refilling. No block-wide barrier runs inside the K loop. Every
