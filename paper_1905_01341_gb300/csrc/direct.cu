@@ -177,7 +177,8 @@ __device__ __forceinline__ float dir_rsqrt(float x) {
     return y;
 }
 
-// Sources j0 <= j < j1 against the thread's receivers i[0], i[1]; (accs, accc) the compensated sums.
+// Sources j0 <= j < j1 against the thread's receivers base + tid + 128 k, k < D32_RI (past the end: the
+// last point); (accs, accc) the compensated sums.
 // The pair i = j is left out by index, in the tiles that can hold it.
 template <int R, bool HQ, bool HW, bool SAFE>
 __device__ __forceinline__ void dir32_sources(D32Stage<R, HQ, HW> &sg, int64_t N, int64_t j0, int64_t j1, int64_t base,
@@ -317,11 +318,14 @@ __global__ void __launch_bounds__(D32_THREADS) k_direct32(int64_t N, const float
     };
     clear();
     dir32_sources<R, HQ, HW, false>(sg, N, j0, j1, base, hi, lo, s, nrm, a, accs, accc);
-    bool odd = false;  // a sum that is not finite: points closer than 1e-19, or such inputs
+    // A sum that is not finite: points closer than 1e-19, or such inputs. Threads past the last receiver
+    // hold a copy of it that meets its own source at r = 0: they have no say (with it, one CTA of every
+    // product of N % 128 != 0 points took its share twice: 9600 points 64 us, 9601 points 103 us).
+    bool odd = false;
 #pragma unroll
     for (int k = 0; k < D32_RI; ++k)
 #pragma unroll
-        for (int r = 0; r < R; ++r) odd = odd || !isfinite(accs[k][r]);
+        for (int r = 0; r < R; ++r) odd = odd || (base + tid + k * D32_THREADS < N && !isfinite(accs[k][r]));
     if (__syncthreads_or(odd)) {
         clear();
         dir32_sources<R, HQ, HW, true>(sg, N, j0, j1, base, hi, lo, s, nrm, a, accs, accc);
