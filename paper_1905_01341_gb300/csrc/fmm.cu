@@ -986,7 +986,7 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
     // M2M upward, levels L -> 2: each parent sums its children
     for (int l = L; l >= 3; --l) {
         PhaseScope ps(c, PH_M2M, fs);
-        launch_m2m<T, R>(P, t.base[l - 1], t.nb[l - 1], m2m, t.child8.p, mp, fs);
+        launch_m2m<T, R>(P, t.base[l - 1], t.nb[l - 1], t.nb[l], c.num_sms, m2m, t.child8.p, mp, fs);
     }
     // M2L, all levels at once, then each target sums its sources
     if (t.n_m2l > 0) {
@@ -1071,7 +1071,7 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
     // L2L downward, levels 3 -> L: every child has exactly one parent, so it adds in place
     for (int l = 3; l <= L; ++l) {
         PhaseScope ps(c, PH_L2L, fs);
-        launch_l2l<T, R>(P, t.base[l - 1], t.nb[l - 1], l2l, t.child8.p, lc, fs);
+        launch_l2l<T, R>(P, t.base[l - 1], t.nb[l - 1], t.nb[l], c.num_sms, l2l, t.child8.p, lc, fs);
     }
     // L2P
     {

@@ -442,12 +442,12 @@ void offdiag_apply(Context &c, int R, const double *f, const double *const *xL,
                    const double *g, const double *const *xM, double *const *out, int prec,
                    const Operators *ops = nullptr);
 
-// updown.cu: M2M into the parents pbase .. pbase + np - 1 (global boxes of one level) and L2L out
-// of them; mats [8][P][P] by child octant, child8 as in Tree
+// updown.cu: M2M into the parents pbase .. pbase + np - 1 (global boxes of one level, with nchild children
+// in all) and L2L out of them; mats [8][P][P] by child octant, child8 as in Tree
 template <class T, int R>
-void launch_m2m(int P, int pbase, int np, const T *mats, const int32_t *child8, T *mp, cudaStream_t st);
+void launch_m2m(int P, int pbase, int np, int nchild, int num_sms, const T *mats, const int32_t *child8, T *mp, cudaStream_t st);
 template <class T, int R>
-void launch_l2l(int P, int pbase, int np, const T *mats, const int32_t *child8, T *lc, cudaStream_t st);
+void launch_l2l(int P, int pbase, int np, int nchild, int num_sms, const T *mats, const int32_t *child8, T *lc, cudaStream_t st);
 
 // p2m_l2p.cu: FP32 points -> leaf multipoles [leaf][R][p^2] (hq / hw: any single- / double-layer
 // strengths) and leaf local expansions -> far-field potential [R][N]

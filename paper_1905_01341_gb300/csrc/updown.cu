@@ -2,13 +2,17 @@
 // parent, M_parent = sum_o T_o M_child(o), and local expansions handed down, L_child(o) += S_o
 // L_parent, one dense P x P matrix per child octant o and level.
 //
-// One block takes 64 columns (64 / R parents x R right-hand sides) of one octant against 64
+// One block takes up to 64 columns (64 / R children x R right-hand sides) of one octant against 64
 // coefficients of the result. Degree n of the result needs only the degrees k <= n (M2M) or k >= n
 // (L2L) of the source, so a block walks the columns of T_o that can be non-zero: half of the
 // matrix. M2M runs as clusters of 8 blocks, one per octant, that join their sums through
 // distributed shared memory in octant order (TwoSum): no row per translation in global memory, no
 // reduction launch. Before, one level of a 192600-point cluster took 33 us up and 71 us down (44
 // blocks of 128 x 128 outputs over all P columns, the operator loaded element by element).
+//
+// A block's columns are the children that exist in its octant, moved together, in groups of 16: a
+// surface's tree has about four children per parent, a tree deeper than its points are dense has one. (A
+// warp holds eight columns of every group and skips its half of the last one where that is empty.)
 //
 // The blocks are bound by the latency of a few K chunks where a level is small and by the FP32 pipe
 // where it is large; the products run as packed pairs (fma.f32x2) over even and odd k, which both
@@ -25,6 +29,7 @@ namespace bem {
 namespace {
 
 constexpr int UD_THREADS = 256, UD_ROWS = 64, UD_COLS = 64, UD_STAGES = 3;
+constexpr int UD_MAXF = 4;  // column tiles' worth of parents that a block looks through at most
 constexpr int UD_PITCH_BYTES = 144;  // 128 bytes of one row's K chunk; 8 consecutive rows fall in different banks
 template <class T>
 constexpr int ud_kc() { return 128 / (int)sizeof(T); }
@@ -81,145 +86,225 @@ struct UdTypes<double> {
     using Acc = Acc64;
 };
 
-// one staged K chunk: rows ty + 16 i (i < NI), columns tx + 16 j
-template <class T, int NI>
+// one staged K chunk: rows ty + 16 i (i < NI), columns tx + 16 j (j < NJ)
+template <class T, int NI, int NJ>
 __device__ __forceinline__ void ud_chunk(const unsigned char *st, int tx, int ty, typename UdTypes<T>::Acc (*acc)[4]) {
     using Vec = typename UdTypes<T>::Vec;
     const unsigned char *A = st + ty * UD_PITCH_BYTES, *B = st + (UD_ROWS + tx) * UD_PITCH_BYTES;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-        Vec a[NI], b[4];
+        Vec a[NI];
 #pragma unroll
         for (int i = 0; i < NI; ++i) a[i] = *reinterpret_cast<const Vec *>(A + 16 * i * UD_PITCH_BYTES + q * 16);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const Vec *>(B + 16 * j * UD_PITCH_BYTES + q * 16);
+        for (int j = 0; j < NJ; ++j) {
+            const Vec b = *reinterpret_cast<const Vec *>(B + 16 * j * UD_PITCH_BYTES + q * 16);
 #pragma unroll
-        for (int i = 0; i < NI; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j].fma4(a[i], b[j]);
+            for (int i = 0; i < NI; ++i) acc[i][j].fma4(a[i], b);
+        }
     }
+}
+
+template <class T, int NI>
+__device__ __forceinline__ void ud_cols(const unsigned char *st, int tx, int ty, int nj, typename UdTypes<T>::Acc (*acc)[4]) {
+    if (nj == 4) ud_chunk<T, NI, 4>(st, tx, ty, acc);
+    else if (nj == 3) ud_chunk<T, NI, 3>(st, tx, ty, acc);
+    else if (nj == 2) ud_chunk<T, NI, 2>(st, tx, ty, acc);
+    else if (nj == 1) ud_chunk<T, NI, 1>(st, tx, ty, acc);
+}
+template <class T>
+__device__ __forceinline__ void ud_rows(const unsigned char *st, int tx, int ty, int ni, int nj,
+                                        typename UdTypes<T>::Acc (*acc)[4]) {
+    if (ni == 4) ud_cols<T, 4>(st, tx, ty, nj, acc);
+    else if (ni == 3) ud_cols<T, 3>(st, tx, ty, nj, acc);
+    else if (ni == 2) ud_cols<T, 2>(st, tx, ty, nj, acc);
+    else ud_cols<T, 1>(st, tx, ty, nj, acc);
 }
 
 // UP: Y[parent] = sum over octants (M2M); else Y[child] += the parent's share (L2L). Parents:
 // global boxes pbase .. pbase + np - 1; child8[box][8]: their children by octant, -1 where empty.
-// Blocks: x = 8 (tile of parents) + octant, y = tile of result coefficients.
+// Blocks: x = 8 (tile of parents) + octant, y = tile of result coefficients. A tile has F x 64 / R
+// parents. Its columns are the children that exist: all in one pass where no octant (L2L: not the block's
+// own) has more than 64 / R of them, else in F passes over 64 / R parents each.
 template <class T, int R, bool UP, bool VEC>
-__global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2) k_updown(int P, int pbase, int np, const T *__restrict__ mats,
-                                                        const int32_t *__restrict__ child8, const T *X, T *Y) {
+__global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
+    k_updown(int P, int pbase, int np, int F, const T *__restrict__ mats, const int32_t *__restrict__ child8, const T *X,
+             T *Y) {
     extern __shared__ __align__(16) unsigned char ud_smem[];
-    __shared__ int s_child[UD_COLS];
-    constexpr int KC = ud_kc<T>(), TP = UD_COLS / R;
-    const int oct = blockIdx.x & 7, tile = blockIdx.x >> 3, r0 = blockIdx.y * UD_ROWS;
+    constexpr int KC = ud_kc<T>(), TP = UD_COLS / R, NO = UP ? 8 : 1, WARPS = UD_THREADS / 32;
+    static_assert(TP * UD_MAXF <= UD_THREADS && (TP == 64 || TP == 16), "a thread per parent; whole or half warps per pass");
+    __shared__ int16_t s_rank[NO][TP * UD_MAXF];  // a parent's place among its pass's columns, -1: no child
+    __shared__ int s_cnt[NO][WARPS];
+    __shared__ int s_par[TP], s_ch[TP];  // the block's own octant, by place: parent (in the tile) and child
+    const int oct = blockIdx.x & 7, q0 = (int)(blockIdx.x >> 3) * TP * F, r0 = blockIdx.y * UD_ROWS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // a warp is 8 column x 4 row groups: its 16-byte loads read 8 (4) different rows, conflict-free
     const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
-    if (tid < UD_COLS) {
-        const int q = tile * TP + tid / R;
-        s_child[tid] = q < np ? child8[(int64_t)(pbase + q) * 8 + oct] : -1;
-    }
-    __syncthreads();
-    const bool any = __syncthreads_or(tid < UD_COLS && s_child[tid] >= 0);
     const int rows = min(UD_ROWS, P - r0), ni = (rows + 15) / 16;
-    typename UdTypes<T>::Acc acc[4][4];
-    if (any) {
-        // the columns of the matrix that rows r0 .. r0 + rows - 1 can need
-        int kbeg = 0, kend = P;
-        if (UP) {
-            int n = 1;
-            while (n * n < r0 + rows) ++n;  // rows of degree < n
-            kend = min(P, n * n);
-        } else {
-            int n = 0;
-            while ((n + 1) * (n + 1) <= r0) ++n;  // degree of row r0
-            kbeg = n * n / KC * KC;
-        }
-        const T *A = mats + (size_t)oct * P * P;
-        // this thread's copies of every chunk: two 16-byte units of the matrix and two of the sources
-        constexpr int V = 16 / (int)sizeof(T);
-        const T *src[4];
-        int off[4], kk[4];
-        bool ok[4];
+    int own = -1, passes = 1;  // own: the child of this thread's parent in the block's octant
+    {
+        unsigned has[NO];
+        int most = 0;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int e = tid + u * UD_THREADS, row = e >> 3;  // 8 units per row, 64 + 64 rows
-            kk[u] = (e & 7) * V;
-            off[u] = row * UD_PITCH_BYTES + (e & 7) * 16;
-            if (row < UD_ROWS) {
-                ok[u] = r0 + row < P;
-                src[u] = A + (ok[u] ? (size_t)(r0 + row) * P : 0);
-            } else {
-                const int c = row - UD_ROWS, ch = s_child[c];
-                ok[u] = ch >= 0;
-                const int64_t box = UP ? ch : pbase + tile * TP + c / R;
-                src[u] = X + (ok[u] ? ((size_t)box * R + c % R) * P : 0);
+        for (int o = 0; o < NO; ++o) {
+            const int ch = tid < TP * F && q0 + tid < np ? child8[(int64_t)(pbase + q0 + tid) * 8 + (UP ? o : oct)] : -1;
+            if (!UP || o == oct) own = ch;
+            has[o] = __ballot_sync(0xffffffffu, ch >= 0);
+            if (lane == 0) s_cnt[o][warp] = __popc(has[o]);
+        }
+        __syncthreads();
+        if (F > 1) {
+#pragma unroll
+            for (int o = 0; o < NO; ++o) {
+                int n = 0;
+                for (int w = 0; w < WARPS; ++w) n += s_cnt[o][w];
+                most = max(most, n);
+            }
+            if (most > TP) passes = F;  // the same in all blocks of a cluster
+        }
+        if (tid < TP * F) {
+#pragma unroll
+            for (int o = 0; o < NO; ++o) {
+                unsigned before = (1u << lane) - 1u;
+                int n = 0;
+                if (passes == 1) {
+                    for (int w = 0; w < warp; ++w) n += s_cnt[o][w];
+                } else if (TP == 64) {  // a pass is two warps
+                    if (warp & 1) n = s_cnt[o][warp - 1];
+                } else if (lane >= 16) {  // a pass is half a warp
+                    before &= 0xffff0000u;
+                }
+                s_rank[o][tid] = (int16_t)((has[o] >> lane) & 1u ? n + __popc(has[o] & before) : -1);
             }
         }
-        const int nk = (kend - kbeg + KC - 1) / KC;
-        auto load = [&](int t) {
-            if (t < nk) {
-                unsigned char *st = ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) ud_copy<T, VEC>(st + off[u], src[u], kbeg + t * KC + kk[u], P, ok[u]);
-            }
-            asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk, empty past the end
-        };
-#pragma unroll
-        for (int t = 0; t < UD_STAGES - 1; ++t) load(t);
-        for (int t = 0; t < nk; ++t) {
-            asm volatile("cp.async.wait_group %0;" ::"n"(UD_STAGES - 2) : "memory");
-            __syncthreads();  // chunk t is there for everyone; the stage of chunk t - 1 is free
-            load(t + UD_STAGES - 1);
-            const unsigned char *st = ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES;
-            if (ni == 4) ud_chunk<T, 4>(st, tx, ty, acc);
-            else if (ni == 3) ud_chunk<T, 3>(st, tx, ty, acc);
-            else if (ni == 2) ud_chunk<T, 2>(st, tx, ty, acc);
-            else ud_chunk<T, 1>(st, tx, ty, acc);
-        }
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
     }
-    __syncthreads();
+    const int pp = TP * F / passes;  // parents of a pass
+    // the columns of the matrix that rows r0 .. r0 + rows - 1 can need
+    int kbeg = 0, kend = P;
+    if (UP) {
+        int n = 1;
+        while (n * n < r0 + rows) ++n;  // rows of degree < n
+        kend = min(P, n * n);
+    } else {
+        int n = 0;
+        while ((n + 1) * (n + 1) <= r0) ++n;  // degree of row r0
+        kbeg = n * n / KC * KC;
+    }
     constexpr int RP = UD_ROWS + 4;
     T *red = reinterpret_cast<T *>(ud_smem);  // [column][RP]
-    if (any || UP) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) red[(tx + 16 * j) * RP + ty + 16 * i] = acc[i][j].get();
-    }
-    if constexpr (UP) {
-        cg::cluster_group cl = cg::this_cluster();  // its 8 blocks are the octants of one tile
-        cl.sync();
-        for (int e = tid; e < (UD_COLS / 8) * UD_ROWS; e += UD_THREADS) {
-            const int c = oct * (UD_COLS / 8) + e / UD_ROWS, row = e % UD_ROWS;
-            const int q = tile * TP + c / R;
-            if (row >= rows || q >= np) continue;
-            T s = 0, comp = 0;
-#pragma unroll
-            for (int o = 0; o < 8; ++o) {
-                const T v = cl.map_shared_rank(red, o)[c * RP + row];
-                const T t = s + v, bp = t - s;
-                comp += (s - (t - bp)) + (v - bp);
-                s = t;
-            }
-            Y[((size_t)(pbase + q) * R + c % R) * P + r0 + row] = s + comp;
+    for (int p0 = 0; p0 < TP * F && q0 + p0 < np; p0 += pp) {
+        const bool mine = own >= 0 && tid >= p0 && tid < p0 + pp;
+        if (mine) {
+            const int c = s_rank[UP ? oct : 0][tid];
+            s_par[c] = tid;
+            s_ch[c] = own;
         }
-        cl.sync();  // no block leaves while another still reads its sums
-    } else {
-        __syncthreads();
-        if (!any) return;
-        for (int e = tid; e < UD_COLS * UD_ROWS; e += UD_THREADS) {
-            const int c = e / UD_ROWS, row = e % UD_ROWS, ch = s_child[c];
-            if (ch >= 0 && row < rows) Y[((size_t)ch * R + c % R) * P + r0 + row] += red[c * RP + row];
+        const int cols = __syncthreads_count(mine) * R;
+        const int nj = (cols - 8 * (warp & 1) + 15) / 16;  // column groups that this warp has a part in
+        if (cols) {
+            const T *A = mats + (size_t)oct * P * P;
+            // this thread's copies of every chunk: a 16-byte unit of the rows tid / 8 + 32 u, two of the
+            // matrix and two of the sources (8 units per row, 64 + 64 rows; zeros past the last column, up to
+            // the last group of 16)
+            constexpr int V = 16 / (int)sizeof(T);
+            const T *src[4];
+            const int row0 = tid >> 3, off = row0 * UD_PITCH_BYTES + (tid & 7) * 16, kk = kbeg + (tid & 7) * V;
+            bool ok[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int row = row0 + 32 * u;
+                if (u < 2) {
+                    ok[u] = r0 + row < P;
+                    src[u] = A + (ok[u] ? (size_t)(r0 + row) * P : 0);
+                } else {
+                    const int c = row - UD_ROWS;
+                    ok[u] = c < cols;
+                    const int64_t box = !ok[u] ? 0 : (UP ? s_ch[c / R] : pbase + q0 + s_par[c / R]);
+                    src[u] = X + (ok[u] ? ((size_t)box * R + c % R) * P : 0);
+                }
+            }
+            const int nk = (kend - kbeg + KC - 1) / KC;
+            auto load = [&](int t) {
+                if (t < nk) {
+                    unsigned char *st = ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (u < 2 || row0 + 32 * (u - 2) < (cols + 15) / 16 * 16)
+                            ud_copy<T, VEC>(st + off + 32 * u * UD_PITCH_BYTES, src[u], kk + t * KC, P, ok[u]);
+                }
+                asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk, empty past the end
+            };
+            typename UdTypes<T>::Acc acc[4][4];
+#pragma unroll
+            for (int t = 0; t < UD_STAGES - 1; ++t) load(t);
+            for (int t = 0; t < nk; ++t) {
+                asm volatile("cp.async.wait_group %0;" ::"n"(UD_STAGES - 2) : "memory");
+                __syncthreads();  // chunk t is there for everyone; the stage of chunk t - 1 is free
+                load(t + UD_STAGES - 1);
+                ud_rows<T>(ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES, tx, ty, ni, nj, acc);
+            }
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) red[(tx + 16 * j) * RP + ty + 16 * i] = acc[i][j].get();
+        }
+        if constexpr (UP) {
+            cg::cluster_group cl = cg::this_cluster();  // its 8 blocks are the octants of one tile
+            cl.sync();
+            for (int e = oct * UD_THREADS + tid; e < pp * R * UD_ROWS; e += 8 * UD_THREADS) {
+                const int q = p0 + e / (UD_ROWS * R), r = e / UD_ROWS % R, row = e % UD_ROWS;
+                if (row >= rows || q0 + q >= np) continue;
+                T v[8], s = 0, comp = 0;
+                bool first = true;
+#pragma unroll
+                for (int o = 0; o < 8; ++o) {
+                    const int c = s_rank[o][q];
+                    v[o] = c >= 0 ? cl.map_shared_rank(red, o)[(c * R + r) * RP + row] : (T)0;
+                }
+#pragma unroll
+                for (int o = 0; o < 8; ++o) {
+                    if (s_rank[o][q] < 0) continue;  // uniform in the warp
+                    if (first) {
+                        s = v[o];
+                        first = false;
+                        continue;
+                    }
+                    const T t = s + v[o], bp = t - s;
+                    comp += (s - (t - bp)) + (v[o] - bp);
+                    s = t;
+                }
+                Y[((size_t)(pbase + q0 + q) * R + r) * P + r0 + row] = s + comp;
+            }
+            cl.sync();  // no block leaves, or takes its next pass, while another still reads its sums
+        } else {
+            __syncthreads();
+            for (int e = tid; e < cols * UD_ROWS; e += UD_THREADS) {
+                const int c = e / UD_ROWS, row = e % UD_ROWS;
+                if (row < rows) Y[((size_t)s_ch[c / R] * R + c % R) * P + r0 + row] += red[c * RP + row];
+            }
+            __syncthreads();
         }
     }
 }
 
 template <class T, int R, bool UP, bool VEC>
-void launch_vec(int P, int pbase, int np, const T *mats, const int32_t *child8, const T *X, T *Y, cudaStream_t st) {
+void launch_vec(int P, int pbase, int np, int nchild, int num_sms, const T *mats, const int32_t *child8, const T *X, T *Y,
+                cudaStream_t st) {
     auto kern = k_updown<T, R, UP, VEC>;
     BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, UD_SMEM));
+    // Wider tiles where parents have few children: the expected columns of an octant, F x 64 / 8 children per
+    // parent, stay within 48 of its 64 (more would mean F passes), and four blocks per SM are left.
+    // 40962 points of a sphere at depth 10, one child per parent at most levels: all columns multiplied M2M 2.65
+    // and L2L 2.26 ms, those with a child 1.88 and 1.68 ms, with wider tiles 1.03 and 0.72 ms (FP32, p 14);
+    // FP64, p 8: 9.2 and 7.7, 3.8 and 2.6, 2.3 and 1.7 ms. 3.21M points on 5000 spheres, 4 children per parent
+    // and F = 1: 0.13 and 0.14 ms in every form.
+    const int ry = div_up(P, UD_ROWS);
+    int F = UD_MAXF;
+    while (F > 1 && (F * (int64_t)nchild > 6 * (int64_t)np || (int64_t)8 * div_up(np, F * UD_COLS / R) * ry < 4 * num_sms)) F /= 2;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(8 * div_up(np, UD_COLS / R)), (unsigned)div_up(P, UD_ROWS));
+    cfg.gridDim = dim3((unsigned)(8 * div_up(np, F * UD_COLS / R)), (unsigned)ry);
     cfg.blockDim = dim3(UD_THREADS);
     cfg.dynamicSmemBytes = UD_SMEM;
     cfg.stream = st;
@@ -229,35 +314,36 @@ void launch_vec(int P, int pbase, int np, const T *mats, const int32_t *child8, 
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = UP ? 1 : 0;
-    BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, P, pbase, np, mats, child8, X, Y));
+    BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, P, pbase, np, F, mats, child8, X, Y));
     BEM_LAUNCH_CHECK();
 }
 
 template <class T, int R, bool UP>
-void launch(int P, int pbase, int np, const T *mats, const int32_t *child8, const T *X, T *Y, cudaStream_t st) {
+void launch(int P, int pbase, int np, int nchild, int num_sms, const T *mats, const int32_t *child8, const T *X, T *Y,
+            cudaStream_t st) {
     if (np <= 0) return;
-    if (P % (16 / (int)sizeof(T)) == 0) launch_vec<T, R, UP, true>(P, pbase, np, mats, child8, X, Y, st);
-    else launch_vec<T, R, UP, false>(P, pbase, np, mats, child8, X, Y, st);
+    if (P % (16 / (int)sizeof(T)) == 0) launch_vec<T, R, UP, true>(P, pbase, np, nchild, num_sms, mats, child8, X, Y, st);
+    else launch_vec<T, R, UP, false>(P, pbase, np, nchild, num_sms, mats, child8, X, Y, st);
 }
 
 }  // namespace
 
 template <class T, int R>
-void launch_m2m(int P, int pbase, int np, const T *mats, const int32_t *child8, T *mp, cudaStream_t st) {
-    launch<T, R, true>(P, pbase, np, mats, child8, mp, mp, st);
+void launch_m2m(int P, int pbase, int np, int nchild, int num_sms, const T *mats, const int32_t *child8, T *mp, cudaStream_t st) {
+    launch<T, R, true>(P, pbase, np, nchild, num_sms, mats, child8, mp, mp, st);
 }
 template <class T, int R>
-void launch_l2l(int P, int pbase, int np, const T *mats, const int32_t *child8, T *lc, cudaStream_t st) {
-    launch<T, R, false>(P, pbase, np, mats, child8, lc, lc, st);
+void launch_l2l(int P, int pbase, int np, int nchild, int num_sms, const T *mats, const int32_t *child8, T *lc, cudaStream_t st) {
+    launch<T, R, false>(P, pbase, np, nchild, num_sms, mats, child8, lc, lc, st);
 }
 
-template void launch_m2m<float, 1>(int, int, int, const float *, const int32_t *, float *, cudaStream_t);
-template void launch_m2m<float, 4>(int, int, int, const float *, const int32_t *, float *, cudaStream_t);
-template void launch_m2m<double, 1>(int, int, int, const double *, const int32_t *, double *, cudaStream_t);
-template void launch_m2m<double, 4>(int, int, int, const double *, const int32_t *, double *, cudaStream_t);
-template void launch_l2l<float, 1>(int, int, int, const float *, const int32_t *, float *, cudaStream_t);
-template void launch_l2l<float, 4>(int, int, int, const float *, const int32_t *, float *, cudaStream_t);
-template void launch_l2l<double, 1>(int, int, int, const double *, const int32_t *, double *, cudaStream_t);
-template void launch_l2l<double, 4>(int, int, int, const double *, const int32_t *, double *, cudaStream_t);
+template void launch_m2m<float, 1>(int, int, int, int, int, const float *, const int32_t *, float *, cudaStream_t);
+template void launch_m2m<float, 4>(int, int, int, int, int, const float *, const int32_t *, float *, cudaStream_t);
+template void launch_m2m<double, 1>(int, int, int, int, int, const double *, const int32_t *, double *, cudaStream_t);
+template void launch_m2m<double, 4>(int, int, int, int, int, const double *, const int32_t *, double *, cudaStream_t);
+template void launch_l2l<float, 1>(int, int, int, int, int, const float *, const int32_t *, float *, cudaStream_t);
+template void launch_l2l<float, 4>(int, int, int, int, int, const float *, const int32_t *, float *, cudaStream_t);
+template void launch_l2l<double, 1>(int, int, int, int, int, const double *, const int32_t *, double *, cudaStream_t);
+template void launch_l2l<double, 4>(int, int, int, int, int, const double *, const int32_t *, double *, cudaStream_t);
 
 }  // namespace bem

@@ -6,8 +6,9 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
+import synth  # noqa: E402
 from test_gpu_mlp import make_stepper, small_system  # noqa: E402
-from test_gpu_parity import _bem  # noqa: E402
+from test_gpu_parity import _bem, make_ctx, rel  # noqa: E402
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -82,3 +83,76 @@ def test_network_takes_more_rows_than_a_grid_has_in_y():
     want = 0.5 * float(((Y - T.float()) ** 2).sum()) / rows
     assert abs(loss - want) < 1e-5 * want and bool(torch.isfinite(grads).all())
     ctx.close()
+
+
+# Every box of level 4 with all its children at level 5, or with one of them at random: the levels above
+# are the same, so the second tree has 4096 translations at the leaves where the first has 32768. FP64 is
+# bound by its operations: 64 parents of a block that have 8 children on average in its octant instead of
+# 64 need one of four groups of 16 columns, and the levels above (585 of 4681 full parents) stay, so the
+# second takes about (0.25 x 4096 + 585) / 4681 = 0.34 of the first's time, and all of it when the columns
+# without a child are multiplied too. The line lies between.
+def test_translations_up_and_down_cost_what_the_children_are():
+    bem = _bem()
+    rng = np.random.Generator(np.random.PCG64(5))
+    box = np.stack(np.meshgrid(*[np.arange(16)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    octs = np.stack(np.meshgrid(*[np.arange(2)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    ms = {}
+    for name, child in (("all", np.broadcast_to(octs, (4096, 8, 3))), ("one", rng.integers(0, 2, (4096, 1, 3)))):
+        x = ((box[:, None] + 0.25 + 0.5 * child) / 16.0).reshape(-1, 3)
+        x = np.concatenate([x, [[0.0] * 3, [1.0] * 3]])  # the cube
+        ctx = bem.BemContext(precision=bem.BEM_PREC_FP64, p_fmm=16, fixed_level=5, overlap=0)
+        bem.bem_points_upload(ctx.ctx, len(x), torch.from_numpy(np.ascontiguousarray(x.T)).cuda())
+        ctx.build()
+        q = torch.ones(len(x), dtype=torch.float64, device="cuda")
+        out = torch.empty_like(q)
+        ctx.apply(1.0, q, 0.0, None, out)
+        bem.bem_profile_enable(ctx.ctx)
+        bem.bem_profile_read(ctx.ctx)
+        for _ in range(5):
+            ctx.apply(1.0, q, 0.0, None, out)
+        prof = bem.bem_profile_read(ctx.ctx)
+        ms[name] = np.array([prof["m2m"][0], prof["l2l"][0]])
+        ctx.close()
+    assert np.all(ms["one"] < 0.65 * ms["all"]), ms
+
+
+# Trees whose lowest levels have one child per parent, in one octant for all (a tile's columns are then
+# one octant's, in several passes) or in any: products of points (one right-hand side) against the sum
+# over all pairs, and the diagonals of tiny bubbles (four) against the direct FP64 path. 1e-6: the bound
+# of the FP64 multipole path at p >= 14.
+@pytest.mark.parametrize("octants", ["one", "any"])
+@pytest.mark.parametrize("p", [16, 17])
+def test_one_child_per_parent_products(octants, p):
+    bem = _bem()
+    rng = np.random.Generator(np.random.PCG64(6))
+    box = np.stack(np.meshgrid(*[np.arange(16)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    child = np.zeros((4096, 3)) if octants == "one" else rng.integers(0, 2, (4096, 3))
+    x = np.concatenate([(box + 0.25 + 0.5 * child) / 16.0, [[0.0] * 3, [1.0] * 3]])
+    q = torch.from_numpy(rng.random(len(x))).cuda()
+    t = torch.from_numpy(x).cuda()
+    inv = 1.0 / (t[:, None] - t[None]).norm(dim=2).fill_diagonal_(np.inf)
+    ctx = bem.BemContext(precision=bem.BEM_PREC_FP64, p_fmm=p, fixed_level=6)
+    bem.bem_points_upload(ctx.ctx, len(x), t.T.contiguous())
+    ctx.build()
+    out = torch.empty_like(q)
+    ctx.apply(1.0, q, 0.0, None, out)
+    assert rel(out.cpu(), (inv @ q / (4.0 * np.pi)).cpu()) < 1e-6
+    ctx.close()
+
+
+def test_one_child_per_parent_diagonals():
+    bem = _bem()
+    i = np.stack(np.meshgrid(np.arange(16), np.arange(16), np.arange(4), indexing="ij"), -1).reshape(-1, 3)
+    centres = np.concatenate([(i + 0.3) / 16.0, [[0.0] * 3, [1.0] * 3]])
+    mesh = synth.cluster(0, np.full(len(centres), 1e-3), centres)
+    geo = []
+    for par in ({"mvp": bem.BEM_MVP_DIRECT}, {"p_fmm": 17, "fixed_level": 6}):
+        ctx = make_ctx(mesh, precision=bem.BEM_PREC_FP64, **par)
+        d = [torch.empty(k * mesh.n, dtype=torch.float64, device="cuda") for k in (1, 3, 1, 1)]
+        bem.bem_get_geometry(ctx.ctx, *d)
+        out = torch.empty(mesh.n, dtype=torch.float64, device="cuda")
+        ctx.apply(1.0, torch.ones_like(out), 0.5, torch.ones_like(out), out)
+        geo.append([v.cpu() for v in (*d[2:], out)])
+        ctx.close()
+    for a, b in zip(*geo):
+        assert rel(b, a) < 1e-6
