@@ -145,10 +145,11 @@ struct Tree {
     // near-field work items (leaf, first receiver, first and end position in the unit's list of neighbour
     // points; first = -1: the list from 0 and the leaf's own points): [0] symmetric (the neighbours
     // f > leaf; FP32), [1] one-way (all but the leaf; FP32 and FP64); the items of unit u are
-    // p2p_ioff[u] .. p2p_ioff[u + 1] - 1
+    // p2p_ioff[u] .. p2p_ioff[u + 1] - 1. Item i's sums take R x its unit's receivers rounded up to 8 entries of
+    // the products' scratch from entry 8 R p2p_irow[i] on, 8 R n_p2p_rows in all
     DevBuf<int4> p2p_items[2];
-    DevBuf<int32_t> p2p_ioff[2];
-    int64_t n_p2p_items[2] = {0, 0};
+    DevBuf<int32_t> p2p_ioff[2], p2p_irow[2];
+    int64_t n_p2p_items[2] = {0, 0}, n_p2p_rows[2] = {0, 0};
     // symmetric near field (FP32 single-RHS products): a pair of neighbour leaves A < B is
     // evaluated once, by A's units; each unit of A writes B's share (one float per point of B)
     // into its own region of `back`, and a gather adds those shares to B's points in a fixed order
@@ -326,8 +327,8 @@ struct Context {
     DevBuf<double> far64;          // far-field potential [R][N] (sorted)
     DevBuf<float> far32;
     DevBuf<double> near_out;       // combined potential [R][N] (sorted)
-    DevBuf<float2> p2p_fwd;        // FP32 near field: sums of every item [items][R][64]
-    DevBuf<double2> p2p_fwd64;     // the same of the FP64 near field
+    DevBuf<float2> p2p_fwd;        // FP32 near field: sums of every item (Tree::p2p_irow)
+    DevBuf<double2> p2p_fwd64;     // ... of the FP64 near field
     DevBuf<XChunk> m2l_chunks;
     std::vector<XChunk> m2l_chunks_h;
     // M2L chunks of <= 256/R pairs for the tensor-core kernel: [0] for R = 1, [1] for R = 4

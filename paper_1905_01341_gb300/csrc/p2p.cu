@@ -81,6 +81,9 @@ struct V2<double> {
 // quadrature excludes j = i, Eq. (ns1); distinct vertices never coincide on a valid mesh).
 constexpr int P2P_WARPS = 4;   // warps (work units) per block
 constexpr int P2P_UNIT = 64;   // receivers per work unit
+// receivers in an item's row of sums [receiver][R]: a multiple of 8 (with 64 for every item, leaves of one or
+// two points took 1 KB a leaf and right-hand side in FP64)
+__device__ __forceinline__ int p2p_row(int nr) { return (nr + 7) & ~7; }
 
 template <class T, int R, bool HQ, bool HW>
 struct P2PStage {
@@ -167,7 +170,7 @@ __device__ __forceinline__ void p2p_item_g(P2PStage<T, R, HQ, HW> &sg, int lane,
                                            const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
                                            const int8_t *__restrict__ nd, int64_t N, const T *__restrict__ loc,
                                            const T *__restrict__ nrm, const T *__restrict__ q, const T *__restrict__ w,
-                                           double2 *__restrict__ fwd) {
+                                           double2 *__restrict__ fwd, const int32_t *__restrict__ row) {
     constexpr int LG = 32 / G;  // lanes per group
     const int rs = lane & (LG - 1), gi = lane / LG;
     const int b = it.x, r0 = it.y;
@@ -259,12 +262,13 @@ __device__ __forceinline__ void p2p_item_g(P2PStage<T, R, HQ, HW> &sg, int lane,
                 acc[k][r].c += oc;
             }
     if (gi == 0) {
+        fwd += (int64_t)*row * (8 * R);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int li = rs + k * LG;
             if (li < nr) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) fwd[r * P2P_UNIT + li] = make_double2(acc[k][r].s, acc[k][r].c);
+                for (int r = 0; r < R; ++r) fwd[li * R + r] = make_double2(acc[k][r].s, acc[k][r].c);
             }
         }
     }
@@ -516,7 +520,8 @@ __device__ __forceinline__ void p2p_item_gx2(P2PStageSym<R, HQ, HW, SYM> &sg, in
                                              const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
                                              const int8_t *__restrict__ nd, int64_t N, const float *__restrict__ loc,
                                              const float *__restrict__ nrm, const float *__restrict__ q,
-                                             const float *__restrict__ w, float2 *__restrict__ fwd, BackArgs ba) {
+                                             const float *__restrict__ w, float2 *__restrict__ fwd, const int32_t *__restrict__ row,
+                                             BackArgs ba) {
     constexpr int LG = 32 / G;
     const int rs = lane & (LG - 1), gi = lane / LG;
     const int b = it.x, r0 = it.y;
@@ -606,12 +611,13 @@ __device__ __forceinline__ void p2p_item_gx2(P2PStageSym<R, HQ, HW, SYM> &sg, in
                 acc[k][r].c += oc;
             }
     if (gi == 0) {
+        if (!SYM) fwd += (int64_t)*row * (8 * R);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int li = rs + k * LG;
             if (li < nr) {
 #pragma unroll
-                for (int r = 0; r < R; ++r) fwd[r * P2P_UNIT + li] = make_float2(acc[k][r].s, acc[k][r].c);
+                for (int r = 0; r < R; ++r) fwd[li * R + r] = make_float2(acc[k][r].s, acc[k][r].c);
             }
         }
     }
@@ -623,7 +629,7 @@ __device__ __forceinline__ void p2p_item_gx2(P2PStageSym<R, HQ, HW, SYM> &sg, in
 // other stream). Every item writes its own row, so the result does not depend on the grid.
 template <int R, bool HQ, bool HW, bool SYM>
 __global__ void __launch_bounds__(P2P_WARPS * 32, SYM ? 6 : (R == 1 ? 5 : 4)) k_p2p_items_x2(
-    const int4 *__restrict__ items, int64_t nitems, const int32_t *__restrict__ bstart,
+    const int4 *__restrict__ items, const int32_t *__restrict__ irow, int64_t nitems, const int32_t *__restrict__ bstart,
     const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
     const int8_t *__restrict__ nd, int64_t N, const float *__restrict__ loc, const float *__restrict__ nrm,
     const float *__restrict__ q, const float *__restrict__ w, float2 *__restrict__ fwd, BackArgs ba) {
@@ -635,11 +641,13 @@ __global__ void __launch_bounds__(P2P_WARPS * 32, SYM ? 6 : (R == 1 ? 5 : 4)) k_
     for (int64_t u = (int64_t)blockIdx.x * P2P_WARPS + warp; u < nitems; u += stride) {
         const int4 it = items[u];
         const int nr = min(P2P_UNIT, bcount[it.x] - it.y);  // uniform in the warp
-        float2 *f = fwd + u * (R * P2P_UNIT);
-        if (nr > 32) p2p_item_gx2<R, 1, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
-        else if (nr > 16) p2p_item_gx2<R, 2, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
-        else if (nr > 8) p2p_item_gx2<R, 4, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
-        else p2p_item_gx2<R, 8, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, ba);
+        // where the row lies: the symmetric form looks it up first, the others, short of registers, at the end
+        // (the other way round costs each about 1 %)
+        float2 *f = SYM ? fwd + (int64_t)irow[u] * (8 * R) : fwd;
+        if (nr > 32) p2p_item_gx2<R, 1, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, irow + u, ba);
+        else if (nr > 16) p2p_item_gx2<R, 2, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, irow + u, ba);
+        else if (nr > 8) p2p_item_gx2<R, 4, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, irow + u, ba);
+        else p2p_item_gx2<R, 8, HQ, HW, SYM>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f, irow + u, ba);
     }
 }
 
@@ -651,7 +659,7 @@ __global__ void __launch_bounds__(P2P_WARPS * 32, SYM ? 6 : (R == 1 ? 5 : 4)) k_
 constexpr int GATHER_WARPS = 8;
 template <class T, int R, bool SYM>
 __global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_gather(
-    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ ioff,
+    const int2 *__restrict__ units, int64_t nunits, const int32_t *__restrict__ ioff, const int32_t *__restrict__ irow,
     const typename V2<T>::type *__restrict__ fwd,
     const int32_t *__restrict__ bstart, const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr,
     const int32_t *__restrict__ ncnt, const int32_t *__restrict__ gofs, const int32_t *__restrict__ ucnt,
@@ -667,17 +675,18 @@ __global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_gather(
     const int64_t i0 = (int64_t)bstart[b] + r0 + lane;
     using T2 = typename V2<T>::type;
     Comp<T> a0[R], a1[R];
-    for (int i = ioff[uw], e = ioff[uw + 1]; i < e; ++i) {
-        const T2 *f = fwd + (int64_t)i * (R * P2P_UNIT) + lane;
+    const int row = p2p_row(nr) * R;  // the unit's items lie one after another
+    const T2 *f = fwd + (int64_t)irow[ioff[uw]] * (8 * R) + lane * R;
+    for (int i = ioff[uw], e = ioff[uw + 1]; i < e; ++i, f += row) {
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if (v0) {
-                const T2 x = f[r * P2P_UNIT];
+                const T2 x = f[r];
                 a0[r].add(x.x);
                 a0[r].c += x.y;
             }
             if (v1) {
-                const T2 x = f[r * P2P_UNIT + 32];
+                const T2 x = f[32 * R + r];
                 a1[r].add(x.x);
                 a1[r].c += x.y;
             }
@@ -730,7 +739,7 @@ __global__ void __launch_bounds__(GATHER_WARPS * 32) k_p2p_gather(
 // The FP64 items, as k_p2p_items_x2
 template <class T, int R, bool HQ, bool HW>
 __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p_items(
-    const int4 *__restrict__ items, int64_t nitems, const int32_t *__restrict__ bstart,
+    const int4 *__restrict__ items, const int32_t *__restrict__ irow, int64_t nitems, const int32_t *__restrict__ bstart,
     const int32_t *__restrict__ bcount, const int32_t *__restrict__ nbr, const int32_t *__restrict__ ncnt,
     const int8_t *__restrict__ nd, int64_t N, const T *__restrict__ loc, const T *__restrict__ nrm,
     const T *__restrict__ q, const T *__restrict__ w, double2 *__restrict__ fwd) {
@@ -742,15 +751,21 @@ __global__ void __launch_bounds__(P2P_WARPS * 32) k_p2p_items(
     for (int64_t u = (int64_t)blockIdx.x * P2P_WARPS + warp; u < nitems; u += stride) {
         const int4 it = items[u];
         const int nr = min(P2P_UNIT, bcount[it.x] - it.y);  // uniform in the warp
-        double2 *f = fwd + u * (R * P2P_UNIT);
-        if (nr > 32) p2p_item_g<T, R, 1, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
-        else if (nr > 16) p2p_item_g<T, R, 2, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
-        else if (nr > 8) p2p_item_g<T, R, 4, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
-        else p2p_item_g<T, R, 8, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, f);
+        if (nr > 32) p2p_item_g<T, R, 1, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, fwd, irow + u);
+        else if (nr > 16) p2p_item_g<T, R, 2, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, fwd, irow + u);
+        else if (nr > 8) p2p_item_g<T, R, 4, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, fwd, irow + u);
+        else p2p_item_g<T, R, 8, HQ, HW>(sg, lane, it, nr, bstart, bcount, nbr, ncnt, nd, N, loc, nrm, q, w, fwd, irow + u);
     }
 }
 
 }  // namespace
+
+// scratch that follows the tree: an eighth more than asked for, so that a tree that changes slowly (time
+// steps) does not allocate in every product
+template <class T>
+static void grow(DevBuf<T> &b, size_t n) {
+    if (n > b.cap) b.resize(n + n / 8);
+}
 
 template <class T, int R, bool HQ, bool HW>
 static void launch_units(Context &c, const T *q, const T *w, double *out_sorted, cudaStream_t st) {
@@ -776,13 +791,13 @@ static void launch_units(Context &c, const T *q, const T *w, double *out_sorted,
         const int64_t ni = t.n_p2p_items[li];
         int64_t blocks = div_up(ni, P2P_WARPS);
         if (c.tuned_p2p_blocks > 0) blocks = std::min<int64_t>(blocks, (int64_t)c.num_sms * c.tuned_p2p_blocks);
-        c.p2p_fwd.resize((size_t)ni * R * P2P_UNIT);
+        grow(c.p2p_fwd, (size_t)t.n_p2p_rows[li] * 8 * R);
         const BackArgs ba{SYM ? t.back.p : nullptr, t.back_S.p, t.back_base.p};
-        kern<<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(t.p2p_items[li].p, ni, bst, bcn, t.nbr.p, t.nbr_cnt.p,
+        kern<<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(t.p2p_items[li].p, t.p2p_irow[li].p, ni, bst, bcn, t.nbr.p, t.nbr_cnt.p,
                                                            t.nbr_d.p, c.N, loc, nrm, q, w, c.p2p_fwd.p, ba);
         BEM_LAUNCH_CHECK();
         k_p2p_gather<float, R, SYM><<<(unsigned)div_up(nu, GATHER_WARPS), GATHER_WARPS * 32, 0, st>>>(
-            t.p2p_units.p, nu, t.p2p_ioff[li].p, c.p2p_fwd.p, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.back_gofs.p, t.p2p_ucnt.p,
+            t.p2p_units.p, nu, t.p2p_ioff[li].p, t.p2p_irow[li].p, c.p2p_fwd.p, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.back_gofs.p, t.p2p_ucnt.p,
             t.back_S.p, t.back_base.p, t.back.p, c.N, out_sorted);
     } else {
         if (c.tuned_overlap)
@@ -791,12 +806,12 @@ static void launch_units(Context &c, const T *q, const T *w, double *out_sorted,
         const int64_t ni = t.n_p2p_items[1];
         int64_t blocks = div_up(ni, P2P_WARPS);
         if (c.tuned_p2p_blocks > 0) blocks = std::min<int64_t>(blocks, (int64_t)c.num_sms * c.tuned_p2p_blocks);
-        c.p2p_fwd64.resize((size_t)ni * R * P2P_UNIT);
+        grow(c.p2p_fwd64, (size_t)t.n_p2p_rows[1] * 8 * R);
         k_p2p_items<T, R, HQ, HW><<<(unsigned)blocks, P2P_WARPS * 32, 0, st>>>(
-            t.p2p_items[1].p, ni, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.nbr_d.p, c.N, loc, nrm, q, w, c.p2p_fwd64.p);
+            t.p2p_items[1].p, t.p2p_irow[1].p, ni, bst, bcn, t.nbr.p, t.nbr_cnt.p, t.nbr_d.p, c.N, loc, nrm, q, w, c.p2p_fwd64.p);
         BEM_LAUNCH_CHECK();
         k_p2p_gather<double, R, false><<<(unsigned)div_up(nu, GATHER_WARPS), GATHER_WARPS * 32, 0, st>>>(
-            t.p2p_units.p, nu, t.p2p_ioff[1].p, c.p2p_fwd64.p, bst, bcn, t.nbr.p, t.nbr_cnt.p, nullptr, nullptr, nullptr,
+            t.p2p_units.p, nu, t.p2p_ioff[1].p, t.p2p_irow[1].p, c.p2p_fwd64.p, bst, bcn, t.nbr.p, t.nbr_cnt.p, nullptr, nullptr, nullptr,
             nullptr, nullptr, c.N, out_sorted);
     }
     BEM_LAUNCH_CHECK();

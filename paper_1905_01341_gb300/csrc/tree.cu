@@ -607,24 +607,42 @@ __device__ __forceinline__ UnitCut unit_cut(int own, int r0, int len, int chunk)
     const int first = min(len, max(0, c - (own + 31) / 32 * 32));
     return {first, c, 1 + (len - first + c - 1) / c};
 }
+// receivers of a unit rounded up to 8, in eights
+__device__ __forceinline__ int unit_row8(int own, int r0) { return (min(64, own - r0) + 7) / 8; }
+// cnt[4][nu] + 1: per unit the items of the symmetric and of the one-way list, then the eights of their rows
 __global__ void k_p2p_item_count(int64_t nu, const int2 *__restrict__ units, const int32_t *__restrict__ bcount,
-                                 const int32_t *__restrict__ len, int chunk, int32_t *__restrict__ cnt) {
+                                 const int32_t *__restrict__ len0, const int32_t *__restrict__ len1, int chunk0, int chunk1,
+                                 int32_t *__restrict__ cnt) {
     const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (u >= nu) return;
     const int2 un = units[u];
-    cnt[u] = unit_cut(bcount[un.x], un.y, len[un.x], chunk).n;
+    const int own = bcount[un.x], w8 = unit_row8(own, un.y);
+    const int n0 = unit_cut(own, un.y, len0[un.x], chunk0).n, n1 = unit_cut(own, un.y, len1[un.x], chunk1).n;
+    cnt[u] = n0;
+    cnt[nu + u] = n1;
+    cnt[2 * nu + u] = n0 * w8;
+    cnt[3 * nu + u] = n1 * w8;
+    if (u == 0) cnt[4 * nu] = 0;
 }
+// items, their rows and the units' first items, list by list, from the sums over cnt
 __global__ void k_p2p_item_emit(int64_t nu, const int2 *__restrict__ units, const int32_t *__restrict__ bcount,
-                                const int32_t *__restrict__ len, int chunk, const int32_t *__restrict__ off,
-                                int4 *__restrict__ items) {
+                                const int32_t *__restrict__ len, int chunk, const int32_t *__restrict__ ex, int list,
+                                int32_t *__restrict__ ioff, int4 *__restrict__ items, int32_t *__restrict__ irow) {
     const int64_t u = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (u >= nu) return;
     const int2 un = units[u];
-    const int L = len[un.x];
-    const UnitCut uc = unit_cut(bcount[un.x], un.y, L, chunk);
-    items[off[u]] = make_int4(un.x, un.y, -1, uc.first);  // -1: from 0, and the leaf's own points
-    for (int i = 1; i < uc.n; ++i)
-        items[off[u] + i] = make_int4(un.x, un.y, uc.first + (i - 1) * uc.chunk, min(L, uc.first + i * uc.chunk));
+    const int L = len[un.x], own = bcount[un.x], w8 = unit_row8(own, un.y);
+    const UnitCut uc = unit_cut(own, un.y, L, chunk);
+    const int32_t *ei = ex + list * nu, *er = ex + (2 + list) * nu;
+    const int i0 = ei[u] - ei[0], row = er[u] - er[0];
+    ioff[u] = i0;
+    if (u + 1 == nu) ioff[nu] = i0 + uc.n;
+    items[i0] = make_int4(un.x, un.y, -1, uc.first);  // -1: from 0, and the leaf's own points
+    irow[i0] = row;
+    for (int i = 1; i < uc.n; ++i) {
+        items[i0 + i] = make_int4(un.x, un.y, uc.first + (i - 1) * uc.chunk, min(L, uc.first + i * uc.chunk));
+        irow[i0 + i] = row + i * w8;
+    }
 }
 
 __global__ void k_back_base(int nleaf, const int32_t *__restrict__ blkoff, int64_t *__restrict__ base) {
@@ -828,7 +846,7 @@ void build_tree(Context &c) {
         DevBuf<int32_t> &ucnt = t.s_i32[4], &uoff = t.s_i32[5], &utot = t.s_i32[6];
         ucnt.resize(nleaf + 1);
         uoff.resize(nleaf + 1);
-        utot.resize(4);  // units, 32-float blocks of shares, items of either list
+        utot.resize(2);  // units, 32-float blocks of shares
         k_p2p_unit_count<<<div_up(nleaf, tb), tb, 0, st>>>(nleaf, t.bcount.p + t.base[L], ucnt.p);
         BEM_LAUNCH_CHECK();
         exclusive_scan_i32(ucnt.p, uoff.p, nleaf, utot.p, st);
@@ -869,28 +887,31 @@ void build_tree(Context &c) {
         // most 4096 positions (an item's set-up is about a quarter of a 64-source item's time, and
         // beyond 4096 nearly every unit is one item). Half the pairs in the symmetric list.
         const double per_item = (double)t.p2p_pairs / P2P_ITEM_RECV / ((double)c.num_sms * 24 * 6);
-        DevBuf<int32_t> &icnt = t.s_i32[23];
-        icnt.resize(std::max<int64_t>(nu, 1));
+        DevBuf<int32_t> &icnt = t.s_i32[23], &iex = t.s_i32[18];
+        icnt.resize(4 * nu + 1);
+        iex.resize(4 * nu + 1);
         int chunk[2];
         const int32_t *len[2] = {t.back_S.p, all.p};
         for (int k = 0; k < 2; ++k) {
             const double want = k == 0 ? 0.5 * per_item : per_item;
             chunk[k] = std::min(4096, std::max(64, ((int)std::min(want, 1e6) + 31) / 32 * 32));
-            t.p2p_ioff[k].resize(nu + 1);
-            k_p2p_item_count<<<div_up(nu, tb), tb, 0, st>>>(nu, t.p2p_units.p, t.bcount.p + t.base[L], len[k], chunk[k],
-                                                            icnt.p);
-            BEM_LAUNCH_CHECK();
-            exclusive_scan_i32(icnt.p, t.p2p_ioff[k].p, nu, utot.p + 2 + k, st);
-            BEM_CUDA(cudaMemcpyAsync(t.p2p_ioff[k].p + nu, utot.p + 2 + k, sizeof(int32_t), cudaMemcpyDeviceToDevice, st));
         }
-        int32_t ni[2] = {0, 0};
-        BEM_CUDA(cudaMemcpyAsync(ni, utot.p + 2, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+        k_p2p_item_count<<<div_up(nu, tb), tb, 0, st>>>(nu, t.p2p_units.p, t.bcount.p + t.base[L], len[0], len[1], chunk[0],
+                                                        chunk[1], icnt.p);
+        BEM_LAUNCH_CHECK();
+        exclusive_scan_i32(icnt.p, iex.p, 4 * nu + 1, nullptr, st);
+        int32_t at[5];  // where each of the four lists begins, and the end
+        BEM_CUDA(cudaMemcpy2DAsync(at, sizeof(int32_t), iex.p, nu * sizeof(int32_t), sizeof(int32_t), 5, cudaMemcpyDeviceToHost,
+                                   st));
         BEM_CUDA(cudaStreamSynchronize(st));
         for (int k = 0; k < 2; ++k) {
-            t.n_p2p_items[k] = ni[k];
-            t.p2p_items[k].resize(std::max<int64_t>(ni[k], 1));
-            k_p2p_item_emit<<<div_up(nu, tb), tb, 0, st>>>(nu, t.p2p_units.p, t.bcount.p + t.base[L], len[k], chunk[k],
-                                                           t.p2p_ioff[k].p, t.p2p_items[k].p);
+            t.n_p2p_items[k] = at[k + 1] - at[k];
+            t.n_p2p_rows[k] = at[k + 3] - at[k + 2];
+            t.p2p_items[k].resize(std::max<int64_t>(t.n_p2p_items[k], 1));
+            t.p2p_irow[k].resize(std::max<int64_t>(t.n_p2p_items[k], 1));
+            t.p2p_ioff[k].resize(nu + 1);
+            k_p2p_item_emit<<<div_up(nu, tb), tb, 0, st>>>(nu, t.p2p_units.p, t.bcount.p + t.base[L], len[k], chunk[k], iex.p,
+                                                           k, t.p2p_ioff[k].p, t.p2p_items[k].p, t.p2p_irow[k].p);
             BEM_LAUNCH_CHECK();
         }
     }

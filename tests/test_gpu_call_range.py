@@ -156,3 +156,32 @@ def test_one_child_per_parent_diagonals():
         ctx.close()
     for a, b in zip(*geo):
         assert rel(b, a) < 1e-6
+
+
+# A sheet of 512 x 512 points, each in a leaf box of its own. What the first product may allocate, in bytes:
+# strengths and potentials (4 N doubles), expansions of all boxes (two of p^2), a row of p^2 and the target-major
+# index per translation, and the near field's sums, 8 receivers of 16 bytes per leaf for up to two items
+# and an eighth more; 64 MB for the chunk tables and the rounding of 16 allocations. 64 slots per leaf and
+# item would be 268 MB, not 75.
+def test_near_field_scratch_of_small_leaves():
+    bem = _bem()
+    n, p = 512 * 512, 2
+    g = (np.arange(512) + 0.5) / 512.0
+    xy = np.stack(np.meshgrid(g, g, indexing="ij"), -1).reshape(-1, 2)
+    xyz = torch.from_numpy(np.concatenate([xy, np.full((n, 1), 0.5)], axis=1).T.copy()).cuda()
+    ctx = bem.BemContext(precision=bem.BEM_PREC_FP64, p_fmm=p, fixed_level=10)
+    bem.bem_points_upload(ctx.ctx, n, xyz)
+    ctx.build()
+    st = ctx.stats()
+    q = torch.ones(n, dtype=torch.float64, device="cuda")
+    out = torch.empty_like(q)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    ctx.apply(1.0, q, 0.0, None, out)
+    torch.cuda.synchronize()
+    used = free - torch.cuda.mem_get_info()[0]
+    assert st["leaves"] == n
+    boxes = 2 * n + n // 3
+    bound = 32 * n + 16 * p * p * boxes + (8 * p * p + 4) * st["m2l_pairs"] + 2 * 128 * n * 9 // 8 + (64 << 20)
+    ctx.close()
+    assert used < bound, (used, bound, st["m2l_pairs"])
