@@ -182,7 +182,8 @@ __global__ void k_build_ops(int kind, int p, double *__restrict__ out64, float *
             else val = (pi == 0) ? A.im : B.re;
         }
         out64[mbase + e] = val;
-        out32[mbase + e] = (float)val;
+        const int en = expo32(p, n), ek = expo32(p, k);
+        out32[mbase + e] = (float)ldexp(val, kind == kOpM2L ? -en - ek : (kind == kOpM2M ? en - ek : ek - en));
     }
 }
 
@@ -385,6 +386,10 @@ __global__ void __launch_bounds__(256) k_p2m(int p, int nleaf, const int32_t *__
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             T *dst = mp + ((size_t)b * R + r) * P;
+            if (sizeof(T) == 4 && p > kPlainP32) {
+                are[o][r] = ldexp(are[o][r], expo32(p, n));
+                aim[o][r] = ldexp(aim[o][r], expo32(p, n));
+            }
             if (m == 0) {
                 dst[n * n] = are[o][r];
             } else {

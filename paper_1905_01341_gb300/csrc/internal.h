@@ -94,6 +94,16 @@ inline int div_up(long long a, long long b) { return (int)((a + b - 1) / b); }
 constexpr int kMaxRhs = 4;
 constexpr int kDeepLevel = 10;       // Morton keys are computed at this depth (30 bits)
 constexpr int kMaxPfmm = 20;
+// FP32 expansions of orders above kPlainP32 hold M_n 2^e_n and L_n 2^-e_n, e_n = round(log2 n!), e_n below; up to
+// it e_n = 0. The M2L of degrees n and k is an irregular harmonic of degree n + k, up to (2n + 2k - 1)!! / 2^(n + k + 1)
+// at the nearest offset: 1.4e37 at p = 18 and 1.7e40, past FP32's range, at 19. Powers of two, so that nothing is rounded;
+// with them its entries stay below 1e10 at p = 20. The tensor-core M2L ends at p = 16 and needs none.
+constexpr int kPlainP32 = 16;
+__host__ __device__ constexpr int expo32(int p, int n) {
+    const int e[kMaxPfmm] = {0, 0, 1, 3, 5, 7, 9, 12, 15, 18, 22, 25, 29, 33, 36, 40, 44, 48, 53, 57};
+    return p > kPlainP32 ? e[n] : 0;
+}
+
 // largest bubble (vertices; icosphere level 4) for which the automatic mode runs the diagonal
 // product's M2L on the tensor cores
 constexpr int64_t kDiagTcMaxVerts = 2562;

@@ -39,6 +39,7 @@ struct Pair {
 struct Tables {
     Pair beta[kMaxPfmm][kMaxPfmm + 1];    // [m][n], broadcast pairs
     float gamma[kMaxPfmm][kMaxPfmm];      // [m][n]
+    float scale[kMaxPfmm];                // 2^e_n of the orders above kPlainP32
 };
 constexpr Tables make_tables() {
     Tables t{};
@@ -54,6 +55,10 @@ constexpr Tables make_tables() {
             const float b = (float)(((double)(n - 1) * (n - 1) - (double)m * m) / ((2.0 * n - 1.0) * (2.0 * n - 3.0)));
             t.beta[m][n] = {b, b};
         }
+    }
+    for (int n = 0; n < kMaxPfmm; ++n) {
+        t.scale[n] = 1.f;
+        for (int i = 0; i < expo32(kMaxPfmm, n); ++i) t.scale[n] *= 2.f;
     }
     return t;
 }
@@ -282,6 +287,10 @@ __global__ void __launch_bounds__(PL_WARPS * 32) k_p2m32(int p, const int32_t *_
                 re += gr;
                 im += gi;
             }
+            if (p > kPlainP32) {
+                re *= kTabG.scale[n];
+                im *= kTabG.scale[n];
+            }
             mp[((size_t)b * R + r) * P + e] = part ? -im : re;  // conjugate
         }
     }
@@ -377,7 +386,8 @@ __global__ void __launch_bounds__(PL_WARPS * 32) k_l2p32(int p, const int32_t *_
     for (int e = threadIdx.x; e < P; e += PL_WARPS * 32) {
         int n, m, part;
         coef_nm(e, n, m, part);
-        const float f = kTabG.gamma[m][n] * (m == 0 ? 1.f : (part ? -2.f : 2.f));
+        float f = kTabG.gamma[m][n] * (m == 0 ? 1.f : (part ? -2.f : 2.f));
+        if (p > kPlainP32) f *= kTabG.scale[n];
         float2 *dst = reinterpret_cast<float2 *>(Ls + (size_t)col_idx(p, n, m) * R) + part;
 #pragma unroll
         for (int r = 0; r < R; ++r) {

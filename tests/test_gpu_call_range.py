@@ -8,7 +8,7 @@ pytestmark = pytest.mark.gpu
 
 import synth  # noqa: E402
 from test_gpu_mlp import make_stepper, small_system  # noqa: E402
-from test_gpu_parity import _bem, make_ctx, rel  # noqa: E402
+from test_gpu_parity import _bem, dev, make_ctx, rel, small_cluster  # noqa: E402
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -185,3 +185,26 @@ def test_near_field_scratch_of_small_leaves():
     bound = 32 * n + 16 * p * p * boxes + (8 * p * p + 4) * st["m2l_pairs"] + 2 * 128 * n * 9 // 8 + (64 << 20)
     ctx.close()
     assert used < bound, (used, bound, st["m2l_pairs"])
+
+
+# Orders whose FP32 M2L leaves the range of FP32 (19, 20, and 17, 18 through the diagonals' p + 2), beside
+# the last ones that do not: mixed against FP64 at the same order (the same truncation), with the mixed
+# path's bound 1e-5, the diagonals in FP64 and at the default, in the mixed precision.
+@pytest.mark.parametrize("p", [15, 16, 17, 18, 19, 20])
+@pytest.mark.parametrize("diag", [0, -1])
+def test_mixed_products_of_high_order(p, diag):
+    bem = _bem()
+    mesh = small_cluster(20, 3, seed=11)
+    rng = np.random.Generator(np.random.PCG64(12))
+    xL, xM = dev(rng.standard_normal(mesh.n)), dev(rng.standard_normal(mesh.n))
+    out = {}
+    for prec in (0, 1):
+        ctx = make_ctx(mesh, mvp=bem.BEM_MVP_FMM, precision=prec, p_fmm=p, leaf_target=32, diag_precision=diag)
+        out[prec] = []
+        for f, g in ((1.0, 0.0), (0.0, 1.0), (0.7, -1.3)):
+            o = torch.zeros(mesh.n, dtype=torch.float64, device="cuda")
+            ctx.apply(f, xL, g, xM, o)
+            out[prec].append(o.cpu())
+        ctx.close()
+    for a, b in zip(out[1], out[0]):
+        assert rel(a, b) < 1e-5
