@@ -571,9 +571,16 @@ void gmres_solve(Context &c, const double *b, double *x, int *iters_out, double 
     };
     c.wv.resize(N);
     c.rv.resize(N);
-    // fused Arnoldi step: CTAs of at least AR_MIN and at most AR_SLICE elements, at most one per SM
+    // fused Arnoldi step: CTAs of at least AR_MIN and at most AR_SLICE elements, at most one per SM, where the
+    // device can hold them all at a time; else, and when the launch is refused after all, the separate launches
     const int ar_ctas = (int)std::min<int64_t>(c.num_sms, (N + AR_MIN - 1) / AR_MIN);
-    const bool fused = N <= (int64_t)c.num_sms * AR_SLICE;
+    const void *ar_kern = b32 ? (const void *)k_arnoldi<float> : (const void *)k_arnoldi<double>;
+    bool fused = N <= (int64_t)c.num_sms * AR_SLICE;
+    if (fused) {
+        int per_sm = 0;
+        BEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ar_kern, AR_THREADS, 0));
+        fused = (int64_t)per_sm * c.num_sms >= ar_ctas;
+    }
     c.partial.resize(std::max((size_t)(m + 2) * RED_BLOCKS, fused ? (size_t)(2 * 128 + 1) * ar_ctas : 0));
     c.bar.resize(1);
     if (fused) BEM_CUDA(cudaMemsetAsync(c.bar.p, 0, sizeof(unsigned), c.stream));
@@ -647,11 +654,17 @@ void gmres_solve(Context &c, const double *b, double *x, int *iters_out, double 
                 double *Vd = c.V.p;
                 float *Vf = c.V32.p;
                 void *args[2] = {&ar, b32 ? (void *)&Vf : (void *)&Vd};
-                BEM_CUDA(cudaLaunchCooperativeKernel(b32 ? (const void *)k_arnoldi<float> : (const void *)k_arnoldi<double>,
-                                                     dim3(ar_ctas), dim3(AR_THREADS), args, 0, c.stream));
-                BEM_LAUNCH_CHECK();
-                bar_base += 3u * ar_ctas;
-            } else {
+                const cudaError_t e = cudaLaunchCooperativeKernel(ar_kern, dim3(ar_ctas), dim3(AR_THREADS), args, 0, c.stream);
+                if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+                    (void)cudaGetLastError();  // nothing was launched: the separate launches take this step and the rest
+                    fused = false;
+                } else {
+                    BEM_CUDA(e);
+                    BEM_LAUNCH_CHECK();
+                    bar_base += 3u * ar_ctas;
+                }
+            }
+            if (!fused) {
                 // classical Gram-Schmidt, twice
                 project(k + 1, c.wv.p, c.hcol.p);
                 update(k + 1, c.hcol.p, -1.0, c.wv.p);

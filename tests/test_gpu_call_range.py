@@ -208,3 +208,43 @@ def test_mixed_products_of_high_order(p, diag):
         ctx.close()
     for a, b in zip(out[1], out[0]):
         assert rel(a, b) < 1e-5
+
+
+# The Arnoldi step by one cooperative kernel takes up to 2048 unknowns per SM, more by separate launches:
+# cycles of a solve at either side of that line (full slices below it), in both precisions. A broken
+# Arnoldi relation or a wrong column or rotation shows in a cycle's last estimate, which is the residual to
+# rounding when all are right (r_0 - A d is evaluated with the same products; its own rounding is below
+# 1e-7 of |b| in the mixed precision and 1e-13 in FP64).
+@pytest.mark.parametrize("prec,p,slack", [(0, 6, 1e-12), (1, 8, 2e-7)])
+def test_solves_either_side_of_the_fused_step(prec, p, slack):
+    bem = _bem()
+    limit = 2048 * torch.cuda.get_device_properties(0).multi_processor_count
+    for nb in (limit // 642, limit // 642 + 1):
+        r = int(np.ceil(nb ** (1.0 / 3.0)))
+        centres = 4.0 * np.stack(np.meshgrid(*[np.arange(r)] * 3, indexing="ij"), -1).reshape(-1, 3)[:nb]
+        mesh = synth.cluster(3, 0.6 + 0.8 * np.random.Generator(np.random.PCG64(4)).random(nb), centres)
+        assert (mesh.n <= limit) == (nb == limit // 642)
+        ctx = make_ctx(mesh, precision=prec, p_fmm=p, gmres_precond=1, gmres_restart=12, gmres_maxit=24, gmres_tol=1e-9)
+        phi = dev(np.cos(mesh.xyz @ np.array([0.3, 0.2, 0.1])))
+        q = torch.zeros(mesh.n, dtype=torch.float64, device="cuda")
+        it, rr = ctx.solve(phi, q, raise_on_noconv=False)
+        hist = bem.bem_get_residual_history(ctx.ctx)  # residual, 12 estimates, residual, 12 estimates, residual
+        ctx.close()
+        assert it == 24 and len(hist) == 27 and rr == hist[26] and bool(torch.isfinite(q).all())
+        for e in (12, 25):
+            assert abs(hist[e + 1] - hist[e]) <= slack + 1e-6 * hist[e], hist
+            assert hist[e] < 0.5 * hist[e - 12], hist
+
+
+# one cycle of 75 basis vectors (the residual falls by about 0.6 an iteration), FP64
+def test_solve_with_more_than_64_basis_vectors():
+    bem = _bem()
+    mesh = small_cluster(12, 2, seed=3)
+    ctx = make_ctx(mesh, mvp=bem.BEM_MVP_DIRECT, precision=bem.BEM_PREC_FP64, gmres_tol=1e-18, gmres_maxit=75)
+    q = torch.zeros(mesh.n, dtype=torch.float64, device="cuda")
+    phi = dev(1.0 + 0.1 * np.random.Generator(np.random.PCG64(4)).standard_normal(mesh.n))
+    it, rr = ctx.solve(phi, q, raise_on_noconv=False)
+    hist = np.array(bem.bem_get_residual_history(ctx.ctx))
+    ctx.close()
+    assert it == 75 and len(hist) == 77
+    assert np.all(np.diff(hist[:76]) <= 0.0) and abs(hist[76] - hist[75]) < 1e-12 and rr < 1e-12
