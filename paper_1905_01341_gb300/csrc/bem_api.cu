@@ -360,6 +360,7 @@ void build_all(Context &c) {
         c.tc_chunks_ok[0] = c.tc_chunks_ok[1] = false;
         c.m2l_byK_ops = nullptr;
         c.tm[0].ok = c.tm[1].ok = false;  // chunk tables follow the tree (the autotuner built others)
+        c.tm_only = false;
         c.stats.p2p_pairs = c.tree.p2p_pairs;
         c.stats.m2l_pairs = c.tree.n_m2l;
         c.stats.levels = c.tree.L;

@@ -852,10 +852,12 @@ __global__ void __launch_bounds__(L2P_THREADS) k_l2p(int p, const int32_t *__res
 // concurrently on the side stream) meet here, back in the caller's vertex order.
 // A target-major tile runs every class that any of its 256 targets has, 189 at least where the tree is
 // full, so pairs / (189 boxes) is about the share of its MMA rows that carry a translation; the pair-major
-// form has no empty rows but writes and reads a row per pair. M2L and its sum, target-major against
-// pair-major, in us: share 0.24 (a bubble of 40962 points) 58 / 37, 0.36 (801000 points) 536 / 404, 0.45
-// (192600 points) 156 / 133, 0.69 (3.21M points) 1097 / 1620: pair-major below one half, while its rows
-// stay within 8 GB (a quarter of what the diagonals' four right-hand sides take).
+// form has no empty rows but writes and reads a row per pair. M2L and its sum at p = 14, target-major against
+// pair-major, in us: share 0.24 (a bubble of 40962 points) 57 / 36, 0.36 (801000 points) 541 / 427, 0.45
+// (192600 points) 156 / 140, 0.58 (1.6M points) 910 / 1080, 0.64 (802500 points) 204 / 234. The line lies at the same
+// place from p = 8 (192600 points 78 / 78, 802500 points 103 / 124) to 16 (184 / 147, 240 / 251); at p = 4 it would lie
+// at 0.3 (192600 points 44 / 60, 7 % of the product). Pair-major below one half, while its rows stay within 8 GB (a
+// quarter of what the diagonals' four right-hand sides take) and there is room for them.
 bool m2l_tm_pays(const Tree &t, int P) {
     const int64_t boxes = t.nbox - t.base[2];
     return 2 * t.n_m2l >= 189 * boxes || (size_t)t.n_m2l * P * sizeof(float) > ((size_t)8 << 30);
@@ -1003,13 +1005,16 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
         // target-major (no per-translation rows) for the single-RHS products whose tiles are well
         // filled; the 4-RHS diagonal product stays pair-major (its target-major form, at 64 targets
         // per tile, was slower and less accurate)
-        const bool tm_path = tc_path && R == 1 && c.prm.m2l_target_major && m2l_tm_pays(t, P);
+        const bool tm_can = tc_path && R == 1 && c.prm.m2l_target_major;
+        bool tm_path = tm_can && (c.tm_only || m2l_tm_pays(t, P));
         T *ypair = nullptr;  // per-pair products of the pair-major forms, for the fixed-order sums
         if (!tm_path) {
             const size_t need = (size_t)t.n_m2l * R * P;
             if (F64) {
                 c.ypair64.resize(need);
                 ypair = (T *)c.ypair64.p;
+            } else if (tm_can && !c.ypair32.try_resize(need)) {
+                c.tm_only = tm_path = true;  // no room for the rows: the tiles take about half as much
             } else {
                 c.ypair32.resize(need);
                 ypair = (T *)c.ypair32.p;

@@ -64,6 +64,24 @@ struct DevBuf {
         }
         n = m;
     }
+    // the same, but false where the device has no room (the buffer is then empty, the error cleared)
+    bool try_resize(size_t m) {
+        if (m > cap) {
+            if (p) cudaFree(p);
+            p = nullptr;
+            n = cap = 0;
+            const cudaError_t e = cudaMalloc(&p, m * sizeof(T));
+            if (e == cudaErrorMemoryAllocation) {
+                p = nullptr;
+                (void)cudaGetLastError();
+                return false;
+            }
+            BEM_CUDA(e);
+            cap = m;
+        }
+        n = m;
+        return true;
+    }
     T *get() const { return p; }
 };
 
@@ -367,6 +385,7 @@ struct Context {
         DevBuf<uint8_t> has;
     };
     TmState tm[2];
+    bool tm_only = false;            // no room for the pair-major rows of a single-RHS product (this tree)
     DevBuf<int> tc_err;              // set by a tensor-core block whose wait ran out
     DevBuf<double2> tri_tmp;         // [2T] per-triangle pairs: area vectors, then (n x v)_k A_k
     // per-build and per-step scratch kept in the context (a cudaFree synchronises the device):

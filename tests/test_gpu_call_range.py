@@ -248,3 +248,41 @@ def test_solve_with_more_than_64_basis_vectors():
     ctx.close()
     assert it == 75 and len(hist) == 77
     assert np.all(np.diff(hist[:76]) <= 0.0) and abs(hist[76] - hist[75]) < 1e-12 and rr < 1e-12
+
+
+# A tree whose single-layer M2L takes the pair-major rows (p = 16: 1 KB a translation, 0.9 GB), on a device with
+# less room than those: the target-major tiles take half as much. A first product allocates 1.0 GB with the
+# rows and 0.5 GB with the tiles; 0.7 GB are left.
+def test_product_without_room_for_pair_rows():
+    bem = _bem()
+    rng = np.random.Generator(np.random.PCG64(9))
+    radii = np.exp(0.3 * rng.standard_normal(500))
+    mesh = synth.cluster(np.resize([3, 4], 500), radii, synth._place_centres(radii, 4.0 * 500 ** (1 / 3), 0.5, rng))
+    par = dict(precision=bem.BEM_PREC_MIXED, p_fmm=16, diag_precision=0)
+    x = dev(rng.standard_normal(mesh.n))
+    outs = []
+    # every kernel is loaded before memory is short: both forms, the tiles on a dense tree
+    warm = point_ctx(points(100000), **par)
+    warm.apply(1.0, torch.ones(100000, dtype=torch.float64, device="cuda"), 0.0, None,
+               torch.empty(100000, dtype=torch.float64, device="cuda"))
+    warm.close()
+    for short in (False, True):
+        ctx = make_ctx(mesh, **par)
+        pairs = ctx.stats()["m2l_pairs"]
+        out = torch.empty_like(x)
+        torch.cuda.empty_cache()
+        fill = None
+        if short:
+            assert 1024 * pairs > 700 << 20  # the rows alone have no room
+            free = torch.cuda.mem_get_info()[0]
+            fill = torch.empty(free - (700 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            ctx.apply(1.0, x, 0.0, None, out)
+            ctx.apply(1.0, x, 0.0, None, out)
+            outs.append(out.cpu().numpy())
+        finally:
+            del fill
+            ctx.close()
+            torch.cuda.empty_cache()
+    # other sums of the same translations: the mixed path's bound, and not the same bits
+    assert 0.0 < rel(outs[1], outs[0]) < 1e-5
