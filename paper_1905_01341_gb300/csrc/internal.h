@@ -23,10 +23,12 @@ struct Error {
 #define BEM_CUDA(expr)                                                                     \
     do {                                                                                   \
         cudaError_t e_ = (expr);                                                           \
-        if (e_ != cudaSuccess)                                                             \
+        if (e_ != cudaSuccess) {                                                           \
+            (void)cudaGetLastError(); /* reported here, not again by a later launch check */ \
             ::bem::fail(e_ == cudaErrorMemoryAllocation ? BEM_ERR_NOMEM : BEM_ERR_CUDA,    \
                         std::string(#expr) + " -> " + cudaGetErrorString(e_) + " at " +    \
                             __FILE__ + ":" + std::to_string(__LINE__));                    \
+        }                                                                                  \
     } while (0)
 
 // Message of the last failure that has no context (bem_create, context-free entry points),

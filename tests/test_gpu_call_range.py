@@ -286,3 +286,26 @@ def test_product_without_room_for_pair_rows():
             torch.cuda.empty_cache()
     # other sums of the same translations: the mixed path's bound, and not the same bits
     assert 0.0 < rel(outs[1], outs[0]) < 1e-5
+
+
+# 3 x 8 bytes of a million points have no room in 8 MB; once there is room, the next calls work.
+def test_calls_after_a_refused_allocation():
+    bem = _bem()
+    xyz = points(1000000)
+    q = torch.ones(xyz.shape[1], dtype=torch.float64, device="cuda")
+    out = torch.empty_like(q)
+    ctx = bem.BemContext(p_fmm=8)
+    torch.cuda.empty_cache()
+    fill = torch.empty(torch.cuda.mem_get_info()[0] - (8 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(bem.BemError) as ei:
+            bem.bem_points_upload(ctx.ctx, xyz.shape[1], xyz)
+    finally:
+        del fill
+        torch.cuda.empty_cache()
+    assert ei.value.code == bem.BEM_ERR_NOMEM
+    bem.bem_points_upload(ctx.ctx, xyz.shape[1], xyz)
+    ctx.build()
+    ctx.apply(1.0, q, 0.0, None, out)
+    assert bool(torch.isfinite(out).all())
+    ctx.close()
