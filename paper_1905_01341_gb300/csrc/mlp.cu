@@ -87,7 +87,7 @@ constexpr int G_SPLIT = 8;        // CTAs sharing a long K (one cluster)
 constexpr int G_SPLIT_K = 512;    // from this K on
 constexpr int LOSS_BLOCKS = 128;
 constexpr uint32_t G_LBO = 128, G_SBO = 1024;
-constexpr long long kWait = 1ll << 20;
+constexpr long long kWait = 1ll << 20;  // polls before a wait gives up, as in the other tensor-core kernels
 
 constexpr int64_t ld8(int64_t n) { return (n + 7) / 8 * 8; }  // row length padded to 16 bytes of BF16
 
@@ -487,7 +487,8 @@ Mlp &mlp_of(Context &c) {
 
 void gemm(Context &c, Mlp &m, int M, int N, int K, const __nv_bfloat16 *A, int64_t lda, const __nv_bfloat16 *B,
           int64_t ldb, const GemmOut &out) {
-    const bool split = K >= G_SPLIT_K;
+    // the split form stores plain sums only (weight gradients; the layers' products have K <= 363)
+    const bool split = K >= G_SPLIT_K && out.epi == EPI_STORE && !out.H && !out.HT;
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(div_up(M, GM) * (split ? G_SPLIT : 1)), (unsigned)div_up(N, GN));
     cfg.blockDim = dim3(G_THREADS);
