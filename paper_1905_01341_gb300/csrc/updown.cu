@@ -121,47 +121,186 @@ __device__ __forceinline__ void ud_rows(const unsigned char *st, int tx, int ty,
     else ud_cols<T, 1>(st, tx, ty, nj, acc);
 }
 
+// acc (zero before) = rows r0 .. r0 + rows - 1 of A times `cols` packed columns, source(c) the data of
+// column c. All threads leave together, the stages free.
+template <class T, bool UP, bool VEC, class F>
+__device__ __forceinline__ void ud_product(int P, int r0, int rows, int cols, const T *A, F source,
+                                           typename UdTypes<T>::Acc (*acc)[4]) {
+    extern __shared__ __align__(16) unsigned char ud_smem[];
+    constexpr int KC = ud_kc<T>(), V = 16 / (int)sizeof(T);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    // a warp is 8 column x 4 row groups: its 16-byte loads read 8 (4) different rows, conflict-free
+    const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
+    const int ni = (rows + 15) / 16;
+    const int nj = (cols - 8 * (warp & 1) + 15) / 16;  // column groups that this warp has a part in
+    // the columns of the matrix that the rows can need
+    int kbeg = 0, kend = P;
+    if (UP) {
+        int n = 1;
+        while (n * n < r0 + rows) ++n;  // rows of degree < n
+        kend = min(P, n * n);
+    } else {
+        int n = 0;
+        while ((n + 1) * (n + 1) <= r0) ++n;  // degree of row r0
+        kbeg = n * n / KC * KC;
+    }
+    // this thread's copies of every chunk: a 16-byte unit of the rows tid / 8 + 32 u, two of the
+    // matrix and two of the sources (8 units per row, 64 + 64 rows; zeros past the last column, up to
+    // the last group of 16)
+    const T *src[4];
+    const int row0 = tid >> 3, off = row0 * UD_PITCH_BYTES + (tid & 7) * 16, kk = kbeg + (tid & 7) * V;
+    bool ok[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int row = row0 + 32 * u;
+        if (u < 2) {
+            ok[u] = r0 + row < P;
+            src[u] = A + (ok[u] ? (size_t)(r0 + row) * P : 0);
+        } else {
+            ok[u] = row - UD_ROWS < cols;
+            src[u] = ok[u] ? source(row - UD_ROWS) : A;
+        }
+    }
+    const int nk = (kend - kbeg + KC - 1) / KC;
+    auto load = [&](int t) {
+        if (t < nk) {
+            unsigned char *st = ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES;
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (u < 2 || row0 + 32 * (u - 2) < (cols + 15) / 16 * 16)
+                    ud_copy<T, VEC>(st + off + 32 * u * UD_PITCH_BYTES, src[u], kk + t * KC, P, ok[u]);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk, empty past the end
+    };
+#pragma unroll
+    for (int t = 0; t < UD_STAGES - 1; ++t) load(t);
+    for (int t = 0; t < nk; ++t) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(UD_STAGES - 2) : "memory");
+        __syncthreads();  // chunk t is there for everyone; the stage of chunk t - 1 is free
+        load(t + UD_STAGES - 1);
+        ud_rows<T>(ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES, tx, ty, ni, nj, acc);
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+}
+
 // UP: Y[parent] = sum over octants (M2M); else Y[child] += the parent's share (L2L). Parents:
 // global boxes pbase .. pbase + np - 1; child8[box][8]: their children by octant, -1 where empty.
-// Blocks: x = 8 (tile of parents) + octant, y = tile of result coefficients. A tile has F x 64 / R
-// parents. Its columns are the children that exist: all in one pass where no octant (L2L: not the block's
-// own) has more than 64 / R of them, else in F passes over 64 / R parents each.
+// Blocks: x = 8 (tile of 64 / R parents) + octant, y = tile of result coefficients. The result tile in
+// shared memory is indexed by the tile's columns (parent, right-hand side), zero where there is no child.
+constexpr int UD_RP = UD_ROWS + 4;
 template <class T, int R, bool UP, bool VEC>
 __global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
-    k_updown(int P, int pbase, int np, int F, const T *__restrict__ mats, const int32_t *__restrict__ child8, const T *X,
-             T *Y) {
+    k_updown(int P, int pbase, int np, const T *__restrict__ mats, const int32_t *__restrict__ child8, const T *X, T *Y) {
     extern __shared__ __align__(16) unsigned char ud_smem[];
-    constexpr int KC = ud_kc<T>(), TP = UD_COLS / R, NO = UP ? 8 : 1, WARPS = UD_THREADS / 32;
+    constexpr int TP = UD_COLS / R;
+    __shared__ int s_child[UD_COLS], s_col[UD_COLS], s_half;
+    const int oct = blockIdx.x & 7, q0 = (int)(blockIdx.x >> 3) * TP, r0 = blockIdx.y * UD_ROWS;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rows = min(UD_ROWS, P - r0);
+    bool here = false;
+    int place = 0;
+    if (tid < UD_COLS) {
+        const int q = q0 + tid / R, ch = q < np ? child8[(int64_t)(pbase + q) * 8 + oct] : -1;
+        s_child[tid] = ch;
+        here = ch >= 0;
+        const unsigned mask = __ballot_sync(0xffffffffu, here), below = (1u << lane) - 1u;
+        place = here ? __popc(mask & below) : __popc(~mask & below);  // among the warp's
+        if (tid == 31) s_half = __popc(mask);
+    }
+    const int cols = __syncthreads_count(here);
+    // s_col: the columns that have a child, then the others
+    if (tid < UD_COLS) s_col[place + (here ? (warp ? s_half : 0) : cols + (warp ? 32 - s_half : 0))] = tid;
+    __syncthreads();
+    T *red = reinterpret_cast<T *>(ud_smem);  // [column][UD_RP]
+    if (cols || UP) {
+        typename UdTypes<T>::Acc acc[4][4];
+        if (cols)
+            ud_product<T, UP, VEC>(P, r0, rows, cols, mats + (size_t)oct * P * P, [&](int c) {
+                const int col = s_col[c];
+                const int64_t box = UP ? s_child[col] : pbase + q0 + col / R;
+                return X + ((size_t)box * R + col % R) * P;
+            }, acc);
+        const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int col = s_col[tx + 16 * j];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) red[col * UD_RP + ty + 16 * i] = acc[i][j].get();
+        }
+    }
+    if constexpr (UP) {
+        cg::cluster_group cl = cg::this_cluster();  // its 8 blocks are the octants of one tile
+        cl.sync();
+        for (int e = tid; e < (UD_COLS / 8) * UD_ROWS; e += UD_THREADS) {
+            const int c = oct * (UD_COLS / 8) + e / UD_ROWS, row = e % UD_ROWS, q = q0 + c / R;
+            if (row >= rows || q >= np) continue;
+            T s = 0, comp = 0;
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                const T v = cl.map_shared_rank(red, o)[c * UD_RP + row];
+                const T t = s + v, bp = t - s;
+                comp += (s - (t - bp)) + (v - bp);
+                s = t;
+            }
+            Y[((size_t)(pbase + q) * R + c % R) * P + r0 + row] = s + comp;
+        }
+        cl.sync();  // no block leaves while another still reads its sums
+    } else if (cols) {
+        __syncthreads();
+        for (int e = tid; e < UD_COLS * UD_ROWS; e += UD_THREADS) {
+            const int c = e / UD_ROWS, row = e % UD_ROWS, ch = s_child[c];
+            if (ch >= 0 && row < rows) Y[((size_t)ch * R + c % R) * P + r0 + row] += red[c * UD_RP + row];
+        }
+    }
+}
+
+// The same for parents of few children (in small orders the ranks of all octants cost more than they
+// save where parents have about eight: M2M of 192600 points at p = 4, 17 us a product without and 21 with them):
+// a tile has F x 64 / R parents (F = 2, 4), and its packed columns are all
+// worked on in one pass where no octant (L2L: not the block's own) has more than 64 / R children, else in F
+// passes over 64 / R parents each. The result tile is indexed by the packed columns.
+template <class T, int R, bool UP, bool VEC>
+__global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
+    k_updown_wide(int P, int pbase, int np, int F, const T *__restrict__ mats, const int32_t *__restrict__ child8,
+                  const T *X, T *Y) {
+    extern __shared__ __align__(16) unsigned char ud_smem[];
+    constexpr int TP = UD_COLS / R, NO = UP ? 8 : 1, WARPS = UD_THREADS / 32;
     static_assert(TP * UD_MAXF <= UD_THREADS && (TP == 64 || TP == 16), "a thread per parent; whole or half warps per pass");
     __shared__ int16_t s_rank[NO][TP * UD_MAXF];  // a parent's place among its pass's columns, -1: no child
     __shared__ int s_cnt[NO][WARPS];
     __shared__ int s_par[TP], s_ch[TP];  // the block's own octant, by place: parent (in the tile) and child
     const int oct = blockIdx.x & 7, q0 = (int)(blockIdx.x >> 3) * TP * F, r0 = blockIdx.y * UD_ROWS;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    // a warp is 8 column x 4 row groups: its 16-byte loads read 8 (4) different rows, conflict-free
-    const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
-    const int rows = min(UD_ROWS, P - r0), ni = (rows + 15) / 16;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rows = min(UD_ROWS, P - r0);
     int own = -1, passes = 1;  // own: the child of this thread's parent in the block's octant
     {
         unsigned has[NO];
-        int most = 0;
+        int most = 0, ch[NO];
+#pragma unroll
+        for (int o = 0; o < NO; ++o) ch[o] = -1;
+        if (tid < TP * F && q0 + tid < np) {
+            const int32_t *row = child8 + (int64_t)(pbase + q0 + tid) * 8;
+            own = row[oct];
+            if constexpr (UP) {
+                const int4 a = reinterpret_cast<const int4 *>(row)[0], b = reinterpret_cast<const int4 *>(row)[1];
+                ch[0] = a.x, ch[1] = a.y, ch[2] = a.z, ch[3] = a.w;
+                ch[4] = b.x, ch[5] = b.y, ch[6] = b.z, ch[7] = b.w;
+            } else {
+                ch[0] = own;
+            }
+        }
 #pragma unroll
         for (int o = 0; o < NO; ++o) {
-            const int ch = tid < TP * F && q0 + tid < np ? child8[(int64_t)(pbase + q0 + tid) * 8 + (UP ? o : oct)] : -1;
-            if (!UP || o == oct) own = ch;
-            has[o] = __ballot_sync(0xffffffffu, ch >= 0);
+            has[o] = __ballot_sync(0xffffffffu, ch[o] >= 0);
             if (lane == 0) s_cnt[o][warp] = __popc(has[o]);
         }
         __syncthreads();
-        if (F > 1) {
 #pragma unroll
-            for (int o = 0; o < NO; ++o) {
-                int n = 0;
-                for (int w = 0; w < WARPS; ++w) n += s_cnt[o][w];
-                most = max(most, n);
-            }
-            if (most > TP) passes = F;  // the same in all blocks of a cluster
+        for (int o = 0; o < NO; ++o) {
+            int n = 0;
+            for (int w = 0; w < WARPS; ++w) n += s_cnt[o][w];
+            most = max(most, n);
         }
+        if (most > TP) passes = F;  // the same in all blocks of a cluster
         if (tid < TP * F) {
 #pragma unroll
             for (int o = 0; o < NO; ++o) {
@@ -179,19 +318,7 @@ __global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
         }
     }
     const int pp = TP * F / passes;  // parents of a pass
-    // the columns of the matrix that rows r0 .. r0 + rows - 1 can need
-    int kbeg = 0, kend = P;
-    if (UP) {
-        int n = 1;
-        while (n * n < r0 + rows) ++n;  // rows of degree < n
-        kend = min(P, n * n);
-    } else {
-        int n = 0;
-        while ((n + 1) * (n + 1) <= r0) ++n;  // degree of row r0
-        kbeg = n * n / KC * KC;
-    }
-    constexpr int RP = UD_ROWS + 4;
-    T *red = reinterpret_cast<T *>(ud_smem);  // [column][RP]
+    T *red = reinterpret_cast<T *>(ud_smem);  // [packed column][UD_RP]
     for (int p0 = 0; p0 < TP * F && q0 + p0 < np; p0 += pp) {
         const bool mine = own >= 0 && tid >= p0 && tid < p0 + pp;
         if (mine) {
@@ -200,58 +327,20 @@ __global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
             s_ch[c] = own;
         }
         const int cols = __syncthreads_count(mine) * R;
-        const int nj = (cols - 8 * (warp & 1) + 15) / 16;  // column groups that this warp has a part in
         if (cols) {
-            const T *A = mats + (size_t)oct * P * P;
-            // this thread's copies of every chunk: a 16-byte unit of the rows tid / 8 + 32 u, two of the
-            // matrix and two of the sources (8 units per row, 64 + 64 rows; zeros past the last column, up to
-            // the last group of 16)
-            constexpr int V = 16 / (int)sizeof(T);
-            const T *src[4];
-            const int row0 = tid >> 3, off = row0 * UD_PITCH_BYTES + (tid & 7) * 16, kk = kbeg + (tid & 7) * V;
-            bool ok[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int row = row0 + 32 * u;
-                if (u < 2) {
-                    ok[u] = r0 + row < P;
-                    src[u] = A + (ok[u] ? (size_t)(r0 + row) * P : 0);
-                } else {
-                    const int c = row - UD_ROWS;
-                    ok[u] = c < cols;
-                    const int64_t box = !ok[u] ? 0 : (UP ? s_ch[c / R] : pbase + q0 + s_par[c / R]);
-                    src[u] = X + (ok[u] ? ((size_t)box * R + c % R) * P : 0);
-                }
-            }
-            const int nk = (kend - kbeg + KC - 1) / KC;
-            auto load = [&](int t) {
-                if (t < nk) {
-                    unsigned char *st = ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        if (u < 2 || row0 + 32 * (u - 2) < (cols + 15) / 16 * 16)
-                            ud_copy<T, VEC>(st + off + 32 * u * UD_PITCH_BYTES, src[u], kk + t * KC, P, ok[u]);
-                }
-                asm volatile("cp.async.commit_group;" ::: "memory");  // one group per chunk, empty past the end
-            };
             typename UdTypes<T>::Acc acc[4][4];
-#pragma unroll
-            for (int t = 0; t < UD_STAGES - 1; ++t) load(t);
-            for (int t = 0; t < nk; ++t) {
-                asm volatile("cp.async.wait_group %0;" ::"n"(UD_STAGES - 2) : "memory");
-                __syncthreads();  // chunk t is there for everyone; the stage of chunk t - 1 is free
-                load(t + UD_STAGES - 1);
-                ud_rows<T>(ud_smem + (t % UD_STAGES) * UD_STAGE_BYTES, tx, ty, ni, nj, acc);
-            }
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-            __syncthreads();
+            ud_product<T, UP, VEC>(P, r0, rows, cols, mats + (size_t)oct * P * P, [&](int c) {
+                const int64_t box = UP ? s_ch[c / R] : pbase + q0 + s_par[c / R];
+                return X + ((size_t)box * R + c % R) * P;
+            }, acc);
+            const int tx = (warp & 1) * 8 + (lane & 7), ty = (warp >> 1) * 4 + (lane >> 3);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) red[(tx + 16 * j) * RP + ty + 16 * i] = acc[i][j].get();
+                for (int j = 0; j < 4; ++j) red[(tx + 16 * j) * UD_RP + ty + 16 * i] = acc[i][j].get();
         }
         if constexpr (UP) {
-            cg::cluster_group cl = cg::this_cluster();  // its 8 blocks are the octants of one tile
+            cg::cluster_group cl = cg::this_cluster();
             cl.sync();
             for (int e = oct * UD_THREADS + tid; e < pp * R * UD_ROWS; e += 8 * UD_THREADS) {
                 const int q = p0 + e / (UD_ROWS * R), r = e / UD_ROWS % R, row = e % UD_ROWS;
@@ -259,10 +348,8 @@ __global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
                 T v[8], s = 0, comp = 0;
                 bool first = true;
 #pragma unroll
-                for (int o = 0; o < 8; ++o) {
-                    const int c = s_rank[o][q];
-                    v[o] = c >= 0 ? cl.map_shared_rank(red, o)[(c * R + r) * RP + row] : (T)0;
-                }
+                for (int o = 0; o < 8; ++o)  // all eight in flight; an octant without the child gives column 0, left out below
+                    v[o] = cl.map_shared_rank(red, o)[(max((int)s_rank[o][q], 0) * R + r) * UD_RP + row];
 #pragma unroll
                 for (int o = 0; o < 8; ++o) {
                     if (s_rank[o][q] < 0) continue;  // uniform in the warp
@@ -282,7 +369,7 @@ __global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
             __syncthreads();
             for (int e = tid; e < cols * UD_ROWS; e += UD_THREADS) {
                 const int c = e / UD_ROWS, row = e % UD_ROWS;
-                if (row < rows) Y[((size_t)s_ch[c / R] * R + c % R) * P + r0 + row] += red[c * RP + row];
+                if (row < rows) Y[((size_t)s_ch[c / R] * R + c % R) * P + r0 + row] += red[c * UD_RP + row];
             }
             __syncthreads();
         }
@@ -292,8 +379,6 @@ __global__ void __launch_bounds__(UD_THREADS, sizeof(T) == 4 ? 3 : 2)
 template <class T, int R, bool UP, bool VEC>
 void launch_vec(int P, int pbase, int np, int nchild, int num_sms, const T *mats, const int32_t *child8, const T *X, T *Y,
                 cudaStream_t st) {
-    auto kern = k_updown<T, R, UP, VEC>;
-    BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, UD_SMEM));
     // Wider tiles where parents have few children: the expected columns of an octant, F x 64 / 8 children per
     // parent, stay within 48 of its 64 (more would mean F passes), and four blocks per SM are left.
     // 40962 points of a sphere at depth 10, one child per parent at most levels: all columns multiplied M2M 2.65
@@ -314,7 +399,13 @@ void launch_vec(int P, int pbase, int np, int nchild, int num_sms, const T *mats
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = UP ? 1 : 0;
-    BEM_CUDA(cudaLaunchKernelEx(&cfg, kern, P, pbase, np, F, mats, child8, X, Y));
+    if (F == 1) {
+        BEM_CUDA(cudaFuncSetAttribute(k_updown<T, R, UP, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, UD_SMEM));
+        BEM_CUDA(cudaLaunchKernelEx(&cfg, k_updown<T, R, UP, VEC>, P, pbase, np, mats, child8, X, Y));
+    } else {
+        BEM_CUDA(cudaFuncSetAttribute(k_updown_wide<T, R, UP, VEC>, cudaFuncAttributeMaxDynamicSharedMemorySize, UD_SMEM));
+        BEM_CUDA(cudaLaunchKernelEx(&cfg, k_updown_wide<T, R, UP, VEC>, P, pbase, np, F, mats, child8, X, Y));
+    }
     BEM_LAUNCH_CHECK();
 }
 
