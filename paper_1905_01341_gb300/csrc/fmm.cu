@@ -386,10 +386,6 @@ __global__ void __launch_bounds__(256) k_p2m(int p, int nleaf, const int32_t *__
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             T *dst = mp + ((size_t)b * R + r) * P;
-            if (sizeof(T) == 4 && p > kPlainP32) {
-                are[o][r] = ldexp(are[o][r], expo32(p, n));
-                aim[o][r] = ldexp(aim[o][r], expo32(p, n));
-            }
             if (m == 0) {
                 dst[n * n] = are[o][r];
             } else {
@@ -398,6 +394,16 @@ __global__ void __launch_bounds__(256) k_p2m(int p, int nleaf, const int32_t *__
             }
         }
     }
+}
+
+// M_n 2^e_n (expo32) for the multipoles of this kernel, in FP32 at orders that need it. (In the kernel itself,
+// after a branch that no order up to 16 takes, it cost the four-RHS P2M 20 % at 57000 points.)
+__global__ void k_scale_mp(int64_t n, int p, float *__restrict__ mp) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    int deg, m, part;
+    decode((int)(i % (p * p)), deg, m, part);
+    mp[i] = ldexpf(mp[i], expo32(p, deg));
 }
 
 // ------------------------------------------------------------------------------ translations
@@ -984,6 +990,11 @@ void run_fmm(Context &c, const RhsArgs<R> &a, const Operators &opr) {
                 BEM_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
             kern<<<nleaf, threads, sm, fs>>>(p, nleaf, bst, bcn, N, loc, nrm, q, w, leaf_mp);
             BEM_LAUNCH_CHECK();
+            if (!F64 && p > kPlainP32) {
+                const int64_t ne = (int64_t)nleaf * R * P;
+                k_scale_mp<<<div_up(ne, 256), 256, 0, fs>>>(ne, p, (float *)leaf_mp);
+                BEM_LAUNCH_CHECK();
+            }
         } else {
             launch_p2m32<R>(p, nleaf, bst, bcn, N, loc, nrm, q, w, hq, hw, leaf_mp, fs);
         }
