@@ -577,8 +577,8 @@ void gmres_solve(Context &c, const double *b, double *x, int *iters_out, double 
     const void *ar_kern = b32 ? (const void *)k_arnoldi<float> : (const void *)k_arnoldi<double>;
     bool fused = N <= (int64_t)c.num_sms * AR_SLICE;
     if (fused) {
-        int per_sm = 0;
-        BEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ar_kern, AR_THREADS, 0));
+        int &per_sm = c.ar_per_sm[b32];
+        if (per_sm < 0) BEM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ar_kern, AR_THREADS, 0));
         fused = (int64_t)per_sm * c.num_sms >= ar_ctas;
     }
     c.partial.resize(std::max((size_t)(m + 2) * RED_BLOCKS, fused ? (size_t)(2 * 128 + 1) * ar_ctas : 0));

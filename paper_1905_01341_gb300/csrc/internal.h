@@ -330,7 +330,7 @@ struct Context {
     // depth the autotuner chose for this mesh (0 = not tuned yet)
     int level_override = 0, tuned_level = 0;
     // tile choices of the products: tensor-core M2L pipeline stages (0 = deepest that fits) and
-    // near-field blocks per SM (0 = one warp per unit); set from the parameters, or by the
+    // near-field blocks per SM (0 = one warp per item); set from the parameters, or by the
     // autotuner when those are automatic
     int tuned_stages = 0, tuned_p2p_blocks = 0, tuned_overlap = 1;
     int num_sms = 1;
@@ -408,6 +408,7 @@ struct Context {
     DevBuf<double> V, wv, rv, bv, zv, hcol, hmat, givens, gvec, yvec, partial, scal;
     DevBuf<double> dv;   // a GMRES cycle's update d = P V y
     DevBuf<unsigned> bar;  // arrivals at the grid barriers of the fused Arnoldi step
+    int ar_per_sm[2] = {-1, -1};  // its CTAs that fit on an SM (FP64, FP32 basis); -1: not asked yet
     DevBuf<float> V32;   // the Krylov basis in FP32 (mixed precision)
     DevBuf<double> vk64; // the current basis vector of V32 in FP64, the product's input
     // bubble-block preconditioner (gmres_precond = 2, precond.cu): per distinct bubble mesh
