@@ -299,12 +299,13 @@ __global__ void __launch_bounds__(G_THREADS) k_gemm_bf16(int M, int N, int K, co
 }
 
 // H[r][c] = bf16(x[r][c] / scale[c]) (scale may be null), rows of ldh; HT (when set) transposed, rows of
-// ldt. Tiles of 32 x 32 through shared memory; the rows, which may be millions, on gridDim.x (y ends at 65535).
+// ldt. Tiles of 32 x 32 through shared memory, row of tiles after row of tiles on gridDim.x (the rows may be
+// millions, and a column of tiles after another reads 50000 rows 11 us slower).
 template <class T>
 __global__ void k_to_bf16(int rows, int cols, const T *__restrict__ x, const float *__restrict__ scale,
                           __nv_bfloat16 *__restrict__ H, int64_t ldh, __nv_bfloat16 *__restrict__ HT, int64_t ldt) {
     __shared__ __nv_bfloat16 t[32][34];
-    const int r0 = blockIdx.x * 32, q0 = blockIdx.y * 32;
+    const int tc = (cols + 31) / 32, r0 = (int)(blockIdx.x / tc) * 32, q0 = (int)(blockIdx.x % tc) * 32;
     for (int i = threadIdx.y; i < 32; i += blockDim.y) {
         const int r = r0 + i, q = q0 + threadIdx.x;
         if (r < rows && q < cols) {
@@ -508,7 +509,7 @@ void gemm(Context &c, Mlp &m, int M, int N, int K, const __nv_bfloat16 *A, int64
 
 template <class T>
 void to_bf16(Context &c, int rows, int cols, const T *x, const float *scale, __nv_bfloat16 *H, __nv_bfloat16 *HT) {
-    const dim3 grid(div_up(rows, 32), div_up(cols, 32));
+    const unsigned grid = (unsigned)((int64_t)div_up(rows, 32) * div_up(cols, 32));
     k_to_bf16<T><<<grid, dim3(32, 8), 0, c.stream>>>(rows, cols, x, scale, H, ld8(cols), HT, ld8(rows));
     BEM_LAUNCH_CHECK();
 }
