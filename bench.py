@@ -55,12 +55,12 @@ PEAKS = _load_peaks()
 # Tensor-core M2L: six BF16 products per translation (three-piece split of both operands).
 M2L_TC_PRODUCTS = 6
 # DRAM traffic per unit from the ncu capture of the 2000-bubble cluster at depth 5 (profiles/;
-# 1,284,000 points, 2,231,186 translations: large enough that the near field's shares and the
+# 1,284,000 points, 2,232,582 translations: large enough that the near field's rows and the
 # M2L's partial expansions leave L2), scaled to a full launch by the units it processes. Near
-# field (symmetric kernel + gather of the shares): 25.2 + 22.5 MB and 89.5 + 0.3 MB; target-major
-# M2L: 228.7 MB read (gathered multipoles, operator blocks) + 269.4 MB written (partials).
-P2P_DRAM_BYTES_PER_POINT = (25.21e6 + 22.49e6 + 89.54e6 + 0.34e6) / 1284000
-M2L_DRAM_BYTES_PER_TRANSLATION = (228.67e6 + 269.36e6) / 2231186
+# field (items and gather): 26.0 + 39.0 MB and 97.0 + 1.1 MB; target-major M2L: 362.2 MB read
+# (gathered multipoles, operator blocks) + 348.3 MB written (partials).
+P2P_DRAM_BYTES_PER_POINT = (25.98e6 + 39.02e6 + 97.03e6 + 1.09e6) / 1284000
+M2L_DRAM_BYTES_PER_TRANSLATION = (362.24e6 + 348.30e6) / 2232582
 
 
 def parse():

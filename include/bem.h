@@ -128,9 +128,9 @@ typedef struct {
                                tile autotuner's choice when leaf_target = 0 and
                                m2l_target_major = 0, else 2). With two stages two of its blocks
                                fit on an SM, with three one. Default 0.                       */
-    int32_t p2p_blocks_per_sm; /* near-field grid: 0 = one warp per work unit (all units in one
+    int32_t p2p_blocks_per_sm; /* near-field grid: 0 = one warp per work item (all items in one
                                grid); k > 0 = a persistent grid of k blocks per SM looping over
-                               the units, which leaves room on every SM for the far-field
+                               the items, which leaves room on every SM for the far-field
                                kernels of the concurrent stream. Same results either way.
                                -1 = automatic (the tile autotuner's choice when leaf_target = 0,
                                else 0). Default -1.                                           */
@@ -150,8 +150,8 @@ typedef struct {
     int32_t m2l_target_major; /* layout of the tensor-core M2L (mixed precision): 1 = target-major
                                (per tile of target boxes, the MMAs of a few offset classes
                                accumulate in tensor memory; no row per translation) where about
-                               half of a tile's rows or more carry a translation, else
-                               pair-major; 0 = pair-major (one product row per translation,
+                               half of a tile's rows or more carry a translation or the device
+                               has no room for the pair-major rows, else pair-major; 0 = pair-major (one product row per translation,
                                summed per target afterwards). Both sum in a fixed order.
                                Default 1.                                                     */
 } bem_params;
@@ -172,7 +172,7 @@ typedef struct {
     int32_t m2l_stages;     /* tensor-core M2L pipeline stages in use (0 = the default, 2)      */
     int32_t overlap;        /* near-field / far-field overlap mode in use (bem_params.overlap)  */
     int32_t reserved;
-    int32_t p2p_blocks_per_sm; /* near-field grid in use (0 = one warp per work unit)           */
+    int32_t p2p_blocks_per_sm; /* near-field grid in use (0 = one warp per work item)           */
     int64_t m2l_macs;       /* multiply-adds of one RHS's M2L, last build: sum over the pairs of
                                (truncated size)^2, the size padded to a multiple of 16 (the
                                tensor-core tiles): p_c^2 rounded up; = pairs x P^2 untruncated */

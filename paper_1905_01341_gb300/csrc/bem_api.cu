@@ -209,9 +209,9 @@ void apply_full(Context &c, double f, const double *xL, double g, const double *
 // rule gives for 64 points per leaf and at one level either side, and keeps the fastest depth
 // for this mesh: points on surfaces fill ~4x more boxes per level, not 8x, so the near-field /
 // far-field balance moves in coarse steps and is cheapest to settle by timing. At that depth it
-// then times the tile choices left automatic: the tensor-core M2L's pipeline depth (3, 4 or 5
-// shared-memory stages) and the near field's grid (one warp per unit, or a persistent grid of
-// k blocks per SM). Both decide how the near field and the far field share the SMs while they
+// then times the tile choices left automatic: the pair-major tensor-core M2L's pipeline depth (2 or 3
+// shared-memory stages, with m2l_target_major = 0) and the near field's grid (one warp per work item, or a
+// persistent grid of k blocks per SM). Both decide how the near field and the far field share the SMs while they
 // run concurrently on two streams; neither changes a result.
 void tune_tiles(Context &c) {
     const int64_t N = c.N;

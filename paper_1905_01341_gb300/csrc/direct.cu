@@ -143,11 +143,12 @@ __global__ void __launch_bounds__(D64_THREADS) k_direct64(int64_t N, const doubl
 // Coordinates as hi + lo FP32 pairs; packed two-wide arithmetic (add/mul/fma .f32x2) over two
 // sources, 128 receivers per cluster. Per pair the FP32 pipe has 9
 // additions for the difference of the split coordinates and 4 (single layer) to 11 (both) further
-// operations, the special-function unit one reciprocal square root: FP32-bound, about 0.16 clocks
-// per pair and SM for both layers. Sums run over at most 64 sources per packed half in FP32 and are
+// operations, the special-function unit one reciprocal square root; a thread reads 28 (single layer) to
+// 44 bytes (both) of shared memory a pair, and that pipe bounds the kernel (74 % busy at 13446 points, both
+// layers, 144 us; 103 us the single layer). Sums run over at most 64 sources per packed half in FP32 and are
 // merged with TwoSum; the cluster's shares are joined in FP64.
-// One receiver per thread (two save shared-memory loads, but leave half as many warps: 232 against
-// 221 us at 13446 points, 452 against 420 at 20484).
+// One receiver per thread: two halve the shared-memory reads, but leave half as many warps (both layers,
+// one against two: 34 / 41 us at 5000 points, 144 / 174 at 13446, 330 / 318 at 20484, 1129 / 1061 at 40000).
 constexpr int D32_THREADS = 128, D32_RI = 1, D32_RECV = D32_THREADS * D32_RI, D32_TILE = 128;
 
 template <int R, bool HQ, bool HW>

@@ -68,18 +68,18 @@ struct V2<double> {
     using type = double2;
 };
 
-// Near-field work is split into units of up to 64 receivers of one leaf (Tree::p2p_units);
-// one warp owns a unit and each lane keeps two receivers in registers, so a staged source feeds
-// two pairs; a unit of fewer receivers splits each source tile over groups of lanes instead of
-// leaving lanes idle. The warp
-// walks the (up to 27) neighbour leaves; each neighbour's sources are staged 32 at a time in
-// the warp's own shared-memory slice as (x, y, z, q) and (n_x, n_y, n_z, w), positions
+// Near-field work is split into units of up to 64 receivers of one leaf (Tree::p2p_units) and these
+// into items, ranges of the joined list of the (up to 27) neighbour leaves' sources
+// (Tree::p2p_items). One warp takes an item and each lane keeps two receivers in registers, so a
+// staged source feeds two pairs; a unit of fewer receivers splits each source tile over groups of
+// lanes instead of leaving lanes idle. The sources are staged 32 at a time in the warp's own
+// shared-memory slice as (x, y, z, q) and (n_x, n_y, n_z, w), positions
 // relative to the target leaf's centre in leaf-box units. HQ / HW select the single- and
 // double-layer terms, so a product with one layer only (every GMRES product) pays for that
 // layer alone. The self pair has r^2 = 0 exactly (same coordinates, zero offset) and is
 // skipped; only the target leaf's own tiles can hold it, so only they test r^2 (the paper's
 // quadrature excludes j = i, Eq. (ns1); distinct vertices never coincide on a valid mesh).
-constexpr int P2P_WARPS = 4;   // warps (work units) per block
+constexpr int P2P_WARPS = 4;   // warps (work items) per block
 constexpr int P2P_UNIT = 64;   // receivers per work unit
 // receivers in an item's row of sums [receiver][R]: a multiple of 8 (with 64 for every item, leaves of one or
 // two points took 1 KB a leaf and right-hand side in FP64)
